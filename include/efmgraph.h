@@ -313,8 +313,10 @@ int efm_fetch_results(efm_job *job, int32_t job_target_idx, uint64_t *supports, 
  *                    chunk of a first-K level)
  *  expand_bytes      algorithmic bytes those launches must move: each parent
  *                    state read once, each new distinct state written once
- *                    (state = 8 W + 4 M + 4 bytes), 16 bytes of hash slot
- *                    traffic per child
+ *                    (state = 8 W + 4 M + 4 bytes; beyond 64 internal
+ *                    metabolites a header and the payload of its columns and
+ *                    unbalanced entries), 16 bytes of hash slot traffic per
+ *                    child
  *  kernel_launches   every kernel this library launched for the target
  * Any output pointer may be NULL. */
 int efm_job_timing(const efm_job *job, int32_t job_target_idx, double *total_ms, double *expand_ms,

@@ -181,8 +181,6 @@ extern "C" int efm_load_network(int32_t n_met, int32_t n_rxn, const int32_t *row
     nv.o_keyr = prep.o_keyr;
     nv.o_hrow = prep.o_hrow;
     nv.o_colx = prep.o_colx;
-    nv.o_fixc = prep.o_fixc;
-    nv.o_fixp = prep.o_fixp;
     nv.blob_words = (int)blob.size();
     nv.M = prep.M;
     nv.N = prep.N;
@@ -252,7 +250,6 @@ extern "C" int efm_load_network(int32_t n_met, int32_t n_rxn, const int32_t *row
         vs.EPL = sub.EPL;
         vs.Mpad = sub.Mpad;
         vs.narrow = 0;
-        vs.o_fixc = vs.o_fixp = 0;
         net->has_sub = true;
     }
     *out = net;
@@ -297,8 +294,11 @@ namespace {
 struct Work {
     DevBuf U[2], B[2], meta[2], live[2];
     DevBuf sum[2];  // narrow networks: per-state summaries of the extra-flux row
-    DevBuf fx[2];   // first-K on wide networks: per-state lane masks of the rows U consumes / produces
-    int fx_words = 0;  // lane-mask words per state (0: not kept)
+    DevBuf hdr[2], pay[2];      // sparse states: headers, payload pool
+    uint64_t pay_cap[2] = {0, 0};
+    bool sparse = false;
+    DevBuf cells, ksig;         // sparse states: the superset rule's index (with cent, csingle)
+    uint64_t cell_cap = 0;
     DevBuf slots, cslots, cand, res, bcnt, bfill, bptr, bres, ctr, sortidx, rcols;
     DevBuf fp;         // fingerprints of one level's reserved child rows
     DevBuf wrec;       // narrow networks: the row pass's record per reserved row (16 B)
@@ -323,8 +323,10 @@ void free_arena(Work &w, int i, cudaStream_t s)
     dev_free(w.meta[i], s);
     dev_free(w.live[i], s);
     dev_free(w.sum[i], s);
-    dev_free(w.fx[i], s);
+    dev_free(w.hdr[i], s);
+    dev_free(w.pay[i], s);
     w.rows[i] = 0;
+    w.pay_cap[i] = 0;
 }
 
 void free_work(Work &w, cudaStream_t s)
@@ -333,21 +335,29 @@ void free_work(Work &w, cudaStream_t s)
     DevBuf *bufs[] = {&w.slots, &w.cslots, &w.cand, &w.res, &w.bcnt,    &w.bfill, &w.bptr,
                       &w.bres,  &w.ctr,    &w.sortidx, &w.rcols, &w.perm, &w.fkb,
                       &w.lx,    &w.lscore, &w.lhist,   &w.lerr, &w.band, &w.fp, &w.slow, &w.wrec,
-                      &w.ccnt,  &w.cfill,  &w.cptr,    &w.cne,  &w.csingle, &w.cent};
+                      &w.ccnt,  &w.cfill,  &w.cptr,    &w.cne,  &w.csingle, &w.cent, &w.cells, &w.ksig};
     for (DevBuf *b : bufs) dev_free(*b, s);
     for (auto &e : w.ev)
         if (e) cudaEventDestroy(e);
 }
 
-// Arena i with room for `rows` states (contents are not kept).
-bool alloc_arena(Work &w, const NetView &nv, int i, int64_t rows, cudaStream_t s)
+// Arena i with room for `rows` states and, sparse states, `units` payload
+// units (contents are not kept).
+bool alloc_arena(Work &w, const NetView &nv, int i, int64_t rows, uint64_t units, cudaStream_t s)
 {
     free_arena(w, i, s);
     const size_t F = (size_t)rows;
+    if (w.sparse) {
+        units = std::min<uint64_t>(units, 0xFFFFFFFFull);  // a header's offset has 32 bits
+        if (!dev_alloc(w.hdr[i], F * 16, s) || !dev_alloc(w.pay[i], units * 16, s) || !dev_alloc(w.live[i], F * 4, s))
+            return false;
+        w.rows[i] = rows;
+        w.pay_cap[i] = units;
+        return true;
+    }
     bool ok = dev_alloc(w.U[i], F * nv.W * 8, s) && dev_alloc(w.B[i], F * nv.Mpad * 4, s) &&
               dev_alloc(w.meta[i], F * 4, s) && dev_alloc(w.live[i], F * 4, s);
     if (ok && nv.narrow) ok = dev_alloc(w.sum[i], F * kSumWords * 8, s);
-    if (ok && w.fx_words) ok = dev_alloc(w.fx[i], F * w.fx_words * 4, s);
     if (ok) w.rows[i] = rows;
     return ok;
 }
@@ -359,7 +369,7 @@ bool ensure_level_tables(Work &w, uint64_t reserved, cudaStream_t s)
         dev_free(w.fp, s);
         dev_free(w.wrec, s);
         const int64_t cap = std::max<int64_t>((int64_t)reserved, w.fp_cap + w.fp_cap / 2);
-        if (!dev_alloc(w.fp, (size_t)cap * 8, s) || !dev_alloc(w.wrec, (size_t)cap * 16, s)) return false;
+        if (!dev_alloc(w.fp, (size_t)cap * 8, s) || (!w.sparse && !dev_alloc(w.wrec, (size_t)cap * 16, s))) return false;
         w.fp_cap = cap;
     }
     const uint64_t need = next_pow2(2 * reserved + 64);
@@ -369,6 +379,13 @@ bool ensure_level_tables(Work &w, uint64_t reserved, cudaStream_t s)
         w.slot_cap = need;
     }
     return true;
+}
+
+// CTAs of the expansion launches (kExpandWarps warps each)
+int level_grid(const NetView &nv, const efm_limits &lim, int sm_count)
+{
+    return nv.narrow ? generate_grid(nv, sm_count)
+                     : sparse_grid(lim.variant == EFM_SUBTRACTIVE, lim.first_k > 0, sm_count);
 }
 
 // The static network a traversal reads: the subtractive variant's rows
@@ -387,14 +404,18 @@ int alloc_work(Work &w, const efm_net *net, const efm_limits &lim, int total_war
     // the rows warps reserve but leave unused; a level that needs more is
     // run again with a larger arena
     w.F_cap = lim.max_frontier > 0 ? lim.max_frontier + 1 : default_cap;
-    const int64_t rows = w.F_cap + w.F_cap / 8 + 32 * (int64_t)total_warps;
+    w.sparse = !nv.narrow;
+    const int64_t rows = w.F_cap + w.F_cap / 8 + (w.sparse ? 1024 : 32 * (int64_t)total_warps);
+    // sparse states: 256 bytes of payload a row (a level that needs more is
+    // run again with a larger pool), and never less than every seed takes
+    // (the subtractive variant's states also hold their flux vector: 384)
+    const uint64_t units = std::max<uint64_t>((uint64_t)rows * (lim.variant == EFM_SUBTRACTIVE ? 24 : 16), (uint64_t)(nv.o_consptr - nv.o_colent) +
+                                                                       4ull * (uint64_t)nv.N + 1024);
     w.cand_cap = (int64_t)1 << 20;
     w.res_cap = w.cand_cap;
     w.cslot_cap = next_pow2(2 * (uint64_t)w.cand_cap);
-    // first-K on a wide network keeps the lane masks of the length-cap rule
-    w.fx_words = (lim.first_k > 0 && nv.o_fixc > 0 && !nv.narrow) ? 2 * std::min(32, 4 * nv.EPL) : 0;
     const size_t W = (size_t)nv.W;
-    bool ok = alloc_arena(w, nv, 0, rows, s) && alloc_arena(w, nv, 1, rows, s);
+    bool ok = alloc_arena(w, nv, 0, rows, units, s) && alloc_arena(w, nv, 1, rows, units, s);
     ok = ok && ensure_level_tables(w, 1024 + 32 * (uint64_t)total_warps, s);
     ok = ok && dev_alloc(w.cslots, w.cslot_cap * 8, s);
     ok = ok && dev_alloc(w.cand, (size_t)w.cand_cap * W * 8, s);
@@ -403,8 +424,10 @@ int alloc_work(Work &w, const efm_net *net, const efm_limits &lim, int total_war
     ok = ok && dev_alloc(w.bfill, (size_t)nv.N * 4, s);
     ok = ok && dev_alloc(w.bptr, (size_t)(nv.N + 1) * 4, s);
     ok = ok && dev_alloc(w.ctr, C_COUNT * 8, s);
-    if (nv.W > 2) ok = ok && dev_alloc(w.rcols, (size_t)w.res_cap * kRcolStride * 2, s);
-    if (nv.W <= 2) {
+    if (nv.W > 2 || w.sparse) ok = ok && dev_alloc(w.rcols, (size_t)w.res_cap * kRcolStride * 2, s);
+    if (w.sparse) {
+        ok = ok && dev_alloc(w.ksig, (size_t)nv.N * 8, s) && dev_alloc(w.csingle, (size_t)nv.N * 4, s);
+    } else if (nv.W <= 2) {
         const size_t cells = (size_t)nv.N * nv.N;
         ok = ok && dev_alloc(w.band, (size_t)nv.N * nv.W * 8, s) && dev_alloc(w.ccnt, cells * 4, s) &&
              dev_alloc(w.cfill, cells * 4, s) && dev_alloc(w.cptr, (cells + 1) * 4, s) &&
@@ -523,7 +546,8 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
 {
     const NetView &nv = view_of(net, lim);
     cudaStream_t s = net->stream;
-    const int grid = generate_grid(nv, net->sm_count);
+    const bool sparse = w.sparse;
+    const int grid = level_grid(nv, lim, net->sm_count);
     const int total_warps = grid * kExpandWarps;
     const int NG = 32 / std::min(32, std::max(4, 4 * nv.EPL));  // children per warp round
     unsigned long long *ctr = (unsigned long long *)w.ctr.p;
@@ -540,7 +564,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
     a.bptr = (const int32_t *)w.bptr.p;
     a.bres = nullptr;
     a.bids = nullptr;
-    a.rcols = nv.W > 2 ? (const uint16_t *)w.rcols.p : nullptr;
+    a.rcols = (const uint16_t *)w.rcols.p;
     a.band = nv.W <= 2 ? (const uint64_t *)w.band.p : nullptr;
     a.max_len = lim.max_len;
     a.max_sec = lim.max_secondary;
@@ -554,7 +578,9 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         r.meta = (uint32_t *)w.meta[i].p;
         r.cap = w.rows[i];
         r.sum = (uint64_t *)w.sum[i].p;
-        r.fx = (uint32_t *)w.fx[i].p;
+        r.hdr = (uint4 *)w.hdr[i].p;
+        r.pay = (uint4 *)w.pay[i].p;
+        r.pay_cap = w.pay_cap[i];
         return r;
     };
 
@@ -572,16 +598,16 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
     if (fs) {
         // the first parents are the caller's rows: nothing to seed
     } else if (seedset) {
-        CK(launch_seedset(nv, a, seedset, n_seedset, s));
+        CK(sparse ? launch_seedset_sparse(nv, a, seedset, n_seedset, s) : launch_seedset(nv, a, seedset, n_seedset, s));
     } else {
-        CK(launch_seed(nv, a, target, s));
+        CK(sparse ? launch_seed_sparse(nv, a, target, s) : launch_seed(nv, a, target, s));
     }
     out.kernel_launches += fs ? 0 : 1;
     AcceptArgs acc{};
     acc.cand = (const uint64_t *)w.cand.p;
     acc.res = (uint64_t *)w.res.p;
     acc.res_cap = w.res_cap;
-    acc.rcols = nv.W > 2 ? (uint16_t *)w.rcols.p : nullptr;
+    acc.rcols = (uint16_t *)w.rcols.p;
     acc.ctr = ctr;
     acc.cand_cap = w.cand_cap;
     auto read_ctr = [&]() -> int {
@@ -620,6 +646,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
     }
     int64_t n_front = fs ? fs->r1 - fs->r0 : (int64_t)h[C_NEXT];  // distinct states of the level
     int64_t n_rows = n_front;              // arena rows the next level reads (seeds are dense)
+    double row_units = 0.0;                // sparse states: payload units of the level's rows
     uint64_t deg_sum = fs ? fs->deg_sum : h[C_DEGSUM];
     int status = 0;
     bool split = false;  // the K smallest come from the parts of a split level (top)
@@ -644,6 +671,27 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         // every step adds a column or a secondary step, so depth is bounded
         if (level > lim.max_len + lim.max_secondary + 1) return EFM_ETIMEOUT;
         // buckets over every accepted result so far (all of them come from levels < `level`)
+        if (res_n != buckets_built_for && sparse) {
+            const int64_t need = std::max<int64_t>(res_n * (int64_t)lim.max_len, 1);
+            if (need > w.bres_cap) {
+                dev_free(w.cent, s);
+                dev_free(w.cells, s);
+                const int64_t cap = std::max<int64_t>(std::max<int64_t>(need, 2 * w.bres_cap), 4096);
+                w.cell_cap = next_pow2(2 * (uint64_t)cap);
+                if (!dev_alloc(w.cent, (size_t)cap * 16, s) || !dev_alloc(w.cells, w.cell_cap * 8, s)) return EFM_ENOMEM;
+                w.bres_cap = cap;
+            }
+            CellIndex &ix = a.cells;
+            ix.cells = (uint2 *)w.cells.p;
+            ix.mask = (uint32_t)std::min<uint64_t>(w.cell_cap, next_pow2(2 * (uint64_t)need)) - 1u;
+            ix.ent = (uint4 *)w.cent.p;
+            ix.ksig = (uint64_t *)w.ksig.p;
+            ix.single = (uint32_t *)w.csingle.p;
+            ix.n_res = res_n;
+            CK(launch_cells(nv, (const uint16_t *)w.rcols.p, res_n, (int32_t *)w.bcnt.p, ix, lim.max_len, s));
+            out.kernel_launches += 2;
+            buckets_built_for = res_n;
+        }
         if (res_n != buckets_built_for) {
             // bucket entries needed: sum of |E| <= res_n * max_len (grown on demand)
             const int64_t need = std::max<int64_t>(res_n * (int64_t)lim.max_len, 1);
@@ -677,8 +725,12 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             // through the list of its surviving rows
             unsigned long long n_live = 0;
             CK(cudaMemsetAsync(ctr + C_LIVE, 0, 8, s));
-            CK(launch_live_list((const uint32_t *)w.meta[cur].p, n_rows, (uint32_t *)w.live[cur].p, ctr + C_LIVE,
-                                net->sm_count, s));
+            if (sparse)
+                CK(launch_live_sparse((const uint4 *)w.hdr[cur].p, n_rows, (uint32_t *)w.live[cur].p, ctr + C_LIVE,
+                                      net->sm_count, s));
+            else
+                CK(launch_live_list((const uint32_t *)w.meta[cur].p, n_rows, (uint32_t *)w.live[cur].p, ctr + C_LIVE,
+                                    net->sm_count, s));
             CK(cudaMemcpyAsync(&n_live, ctr + C_LIVE, 8, cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
             const int64_t nl = (int64_t)n_live;
@@ -690,7 +742,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             const uint32_t *live = (const uint32_t *)w.live[cur].p;
             CK(launch_features(nv, arena(cur), live, 0, stride, cnt, level - 1, lim.max_len, lim.max_secondary,
                                (const uint64_t *)net->dep.p, m->X.p, m->n_rows, s));
-            CK(launch_labels((const uint64_t *)w.U[cur].p, nv.W, live, 0, stride, cnt, trace->ans, trace->n_ans,
+            CK(launch_labels(arena(cur), nv.W, live, 0, stride, cnt, trace->ans, trace->n_ans,
                              (float *)m->y.p, m->n_rows, s));
             m->n_rows += cnt;
         }
@@ -741,9 +793,18 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         // (a warp's unused reserved rows at the end of every launch are dead
         // weight in the arena), 32 for large ones
         const int64_t launches = (n_rows + chunk - 1) / chunk;
-        const int blk = launches > 1 ? NG
-                                     : (int)std::min<uint64_t>(32, std::max<uint64_t>((uint64_t)NG,
-                                                                                     deg_sum / (64ull * total_warps)));
+        // (sparse states: exactly what a round needs, and at large levels about
+        // a 16th of what a warp writes)
+        int blk = launches > 1 ? NG
+                               : (int)std::min<uint64_t>(32, std::max<uint64_t>((uint64_t)NG,
+                                                                                deg_sum / (64ull * total_warps)));
+        a.pay_blk = 0;
+        if (sparse) {
+            blk = launches > 1 ? 0 : (int)std::min<uint64_t>(512, deg_sum / (16ull * total_warps));
+            if (blk < 32) blk = 0;
+            const double avg = n_rows > 0 && row_units > 0.0 ? row_units / (double)n_rows : 8.0;
+            a.pay_blk = (int)(blk * (avg + 1.0));
+        }
         const uint64_t reserved = deg_sum + (uint64_t)launches * blk * total_warps + 64;
         if (!ensure_level_tables(w, reserved, s)) return EFM_ENOMEM;
         // narrow networks: room for every child of a launch in the settle list
@@ -766,6 +827,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             CK(cudaMemsetAsync(ctr + C_NEXT, 0, 2 * 8, s));
             CK(cudaMemsetAsync(ctr + C_WRITTEN, 0, 3 * 8, s));
             CK(cudaMemsetAsync(ctr + C_DEDUP_BEGIN, 0, 8, s));
+            if (sparse) CK(cudaMemsetAsync(ctr + C_PAY, 0, 8, s));
             a.par = ext ? fs->par : arena(cur);
             a.child = arena(cur ^ 1);
             a.live = (uint32_t *)w.live[cur ^ 1].p;
@@ -790,12 +852,17 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                 a.fk_sup = (const uint64_t *)w.fkb.p;
                 a.max_len = (fk && top.pc > 0) ? std::min(lim.max_len, top.pc) : lim.max_len;
                 CK(cudaEventRecord(w.ev[2], s));
-                CK(cudaMemsetAsync(ctr + C_SLOW, 0, 8, s));
-                CK(launch_generate(nv, a, grid, s));
-                CK(launch_prune_rows(nv, a, net->sm_count, s));
-                CK(launch_write_rows(nv, a, net->sm_count, s));
-                CK(launch_settle(nv, a, net->sm_count, s));
-                CK(launch_dedup(a, nv.Mpad, nv.W, net->sm_count, s));
+                if (sparse) {
+                    CK(launch_generate_sparse(nv, a, grid, s));
+                    CK(launch_dedup_sparse(a, net->sm_count, s));
+                } else {
+                    CK(cudaMemsetAsync(ctr + C_SLOW, 0, 8, s));
+                    CK(launch_generate(nv, a, grid, s));
+                    CK(launch_prune_rows(nv, a, net->sm_count, s));
+                    CK(launch_write_rows(nv, a, net->sm_count, s));
+                    CK(launch_settle(nv, a, net->sm_count, s));
+                    CK(launch_dedup(a, nv.Mpad, nv.W, net->sm_count, s));
+                }
                 CK(cudaEventRecord(w.ev[3], s));
                 // minimality test of the new candidates, range taken on the device
                 CK(launch_accept_new(nv, acc, net->sm_count, s));
@@ -809,23 +876,29 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                 CK(cudaEventElapsedTime(&ms, w.ev[2], w.ev[3]));
                 out.expand_ms += ms;
                 out.expand_launches += 1;
-                out.kernel_launches += nv.narrow ? (nv.W <= 2 && a.cptr ? 8 : 7) : 5;
+                out.kernel_launches += sparse ? 5 : (nv.W <= 2 && a.cptr ? 8 : 7);
                 {
-                    const double state_bytes = 8.0 * nv.W + 4.0 * nv.M + 4.0;
+                    // sparse states: a header and the payload units of an average row of the level
+                    const double par_bytes = !sparse ? 8.0 * nv.W + 4.0 * nv.M + 4.0
+                                                     : 16.0 + 16.0 * row_units / (double)std::max<int64_t>(n_rows, 1);
+                    const double new_bytes = !sparse ? par_bytes
+                                                     : 16.0 + 16.0 * (double)h[C_PAY] /
+                                                                  (double)std::max<unsigned long long>(h[C_WRITTEN], 1);
                     const uint64_t next_now = h[C_NEXT];
                     const double n_new = (double)(next_now - next_before);
                     const double n_child = (double)(h[C_EXP] - exp_before);
                     // distinct parents of the chunk (its rows include later copies
                     // and unused rows, which carry no state)
                     const double n_par = (double)cn * (double)n_front_level / (double)std::max<int64_t>(n_rows, 1);
-                    out.expand_bytes += state_bytes * (n_par + n_new) + 16.0 * n_child;
+                    const double bytes = par_bytes * n_par + new_bytes * n_new + 16.0 * n_child;
+                    out.expand_bytes += bytes;
                     if (getenv("EFM_DEBUG"))
                         fprintf(stderr,
                                 "efm: level %d parents %lld items %llu children %.0f new %.0f rows %llu settled %llu "
                                 "pruned %llu bytes %.0f ms %.3f\n",
                                 level, (long long)cn, (unsigned long long)(c0 == 0 && chunk >= n_rows ? deg_sum : 0),
                                 n_child, n_new, h[C_WRITTEN], h[C_SLOW], h[C_PRUNED],
-                                state_bytes * (n_par + n_new) + 16.0 * n_child, ms);
+                                bytes, ms);
                     exp_before = h[C_EXP];
                     next_before = next_now;
                 }
@@ -856,9 +929,14 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             // not decided: grow the child arena to every reserved row and run
             // the level again (its balanced supports are already judged, so
             // only the per-child counters are rolled back)
-            if (!alloc_arena(w, nv, cur ^ 1, (int64_t)h[C_WRITTEN] + (int64_t)h[C_WRITTEN] / 8 + 1024, s))
+            const uint64_t more = h[C_PAY] + h[C_PAY] / 8 + 1024;
+            if (sparse && more > 0xFFFFFFFFull) return EFM_ENOMEM;  // past a header's 32-bit offsets
+            if (!alloc_arena(w, nv, cur ^ 1,
+                             std::max<int64_t>((int64_t)h[C_WRITTEN] + (int64_t)h[C_WRITTEN] / 8 + 1024,
+                                               w.rows[cur ^ 1]),
+                             std::max<uint64_t>(more, w.pay_cap[cur ^ 1]), s))
                 return EFM_ENOMEM;
-            const int back[] = {C_EXP, C_OVF, C_BAL, C_PRUNED};
+            const int back[] = {C_EXP, C_OVF, C_BAL, C_PRUNED, C_ZERO};
             for (int i : back) {
                 h[i] = snap[i];
                 CK(cudaMemcpyAsync(ctr + i, &snap[i], 8, cudaMemcpyHostToDevice, s));
@@ -869,6 +947,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         n_front = unwritten ? (int64_t)(h[C_NEXT] + h[C_UNV]) : (int64_t)h[C_NEXT];
         n_rows = (int64_t)std::min<unsigned long long>(h[C_WRITTEN], (unsigned long long)w.rows[cur ^ 1]);
         deg_sum = h[C_DEGSUM];
+        row_units = (double)h[C_PAY];
         c.levels = level - level0 + 1;
         cur ^= 1;
         if (lim.max_frontier > 0 && n_front > lim.max_frontier) {
@@ -1070,7 +1149,7 @@ extern "C" int efm_find_pathways(efm_net *net, const int32_t *targets, int32_t n
     job->net = net;
     job->out.resize(n_targets);
     Work w;
-    const int total_warps = generate_grid(view_of(net, lim), net->sm_count) * kExpandWarps;
+    const int total_warps = level_grid(view_of(net, lim), lim, net->sm_count) * kExpandWarps;
     int rc = alloc_work(w, net, lim, total_warps, net->stream);
     int flags = 0;
     for (int i = 0; rc == EFM_OK && i < n_targets; ++i) {
@@ -1118,7 +1197,7 @@ extern "C" int efm_find_pathways_from(efm_net *net, const int32_t *columns, int3
     cudaStream_t s = net->stream;
     Work w;
     DevBuf cols;
-    const int total_warps = generate_grid(view_of(net, lim), net->sm_count) * kExpandWarps;
+    const int total_warps = level_grid(view_of(net, lim), lim, net->sm_count) * kExpandWarps;
     int rc = alloc_work(w, net, lim, total_warps, s);
     if (rc == EFM_OK && !dev_alloc(cols, (size_t)n_columns * 4, s)) rc = EFM_ENOMEM;
     if (rc == EFM_OK && cudaMemcpyAsync(cols.p, columns, (size_t)n_columns * 4, cudaMemcpyHostToDevice, s) != cudaSuccess)
@@ -2063,7 +2142,7 @@ extern "C" int efm_model_trace(efm_model *m, efm_net *net, const int32_t *target
     for (int i = 0; i < n_targets; ++i)
         if (targets[i] < -1 || targets[i] >= net->n_met) return EFM_EINVAL;
     Work w;
-    const int total_warps = generate_grid(net->nv, net->sm_count) * kExpandWarps;
+    const int total_warps = level_grid(net->nv, lim, net->sm_count) * kExpandWarps;
     int rc = alloc_work(w, net, lim, total_warps, net->stream);
     for (int i = 0; rc == EFM_OK && i < n_targets; ++i) {
         TargetOut ans;

@@ -17,7 +17,6 @@ constexpr uint32_t kPending = 0xFFFFFFFFu;
 constexpr uint32_t kOverflowIdx = 0xFFFFFFFEu;
 constexpr int kNumPrimes = 24;
 constexpr int kStageLimitBytes = 72 * 1024;  // static network staged in smem up to this size
-constexpr int kStageSparseLimitBytes = 100 * 1024;  // generic kernel: its sparse tables staged up to this size
 constexpr int64_t kFirstKChunkMin = 8192;     // first-K search: fewest parents per expansion launch
 constexpr int64_t kFirstKChunks = 32;         // first-K search: launches per level, at most
 constexpr int64_t kResultWindow = 256;        // first-K search: new results fetched with the counters
@@ -46,8 +45,9 @@ enum {
     C_ZERO = 28,  // subtractive steps discarded: no positive flux left on the reaction (Prop. 3)
     C_SLOW,       // narrow networks: children handed to the settle pass in this launch
     C_LIVE,       // surviving rows counted by the live-list pass
-    C_CAPDEAD,    // first-K: children at the length cap that can never balance
-    C_COUNT = 32
+    C_CAPDEAD,    // unused
+    C_PAY,        // sparse states: payload units reserved so far in the level
+    C_COUNT = 40
 };
 
 // Static network, packed into one 16-byte aligned word array (the "blob").
@@ -70,9 +70,6 @@ struct NetView {
     int o_keyr;                // per rank: positive key [64], then negative key [64]
     int o_hrow;                // per row: 64-bit row hash constant R[m]
     int o_colx;                // per column: suppP, suppN, suppR, HC (u64 each), smax, gcd1 (10 words)
-    // wide networks: per column, G lane masks of the rows it consumes, then
-    // (at o_fixp) of the rows it produces, G = min(32, 4 EPL); 0: absent
-    int o_fixc, o_fixp;
     const int32_t *metptr;     // full S rows over split columns (seeds), [n_met + 1]
     const uint32_t *metent;    // packed (column, coefficient)
     int n_met;
@@ -95,10 +92,29 @@ struct Arena {
     //   sum[6 s + 4] = rows with odd EF_m
     //   sum[6 s + 5] = an upper bound of max_m |EF_m| (saturating at 2^31 - 1)
     uint64_t *sum;
-    // first-K on wide networks: per state, 2G lane masks (G = min(32, 4 EPL)):
-    // the rows some column of U consumes, then the rows some column of U
-    // produces (null: not kept)
-    uint32_t *fx;
+    // sparse states (every network but the narrow ones, and the subtractive
+    // variant; layout in efm_sparse.cu): headers per row, payload pool
+    uint4 *hdr;         // [cap]
+    uint4 *pay;         // [pay_cap] 16-byte units
+    uint64_t pay_cap;
+};
+
+// Sparse states: payload units of the column list (an 8-byte hash in front)
+__host__ __device__ inline int sparse_list_units(int pc) { return (8 + 2 * pc + 15) >> 4; }
+
+// Sparse states: the superset rule's index.  A result E is filed, for each of
+// its columns k, in cell (k, s) where s is E's other column with the fewest
+// results (its sentinel): a child adding k contains E only if it holds s, so
+// it looks up the cells (k, s) of its own columns s and no others.  Cells sit
+// in a hash table (key k << 12 | s, head of a list); an entry holds a 64-bit
+// signature of E's columns, the next entry and the result's id.
+struct CellIndex {
+    uint2 *cells;       // [mask + 1], empty: key ~0
+    uint32_t mask;
+    uint4 *ent;
+    uint64_t *ksig;     // [N]: signature of the sentinels s with a cell (k, s)
+    uint32_t *single;   // [N]: 1 if {k} itself is a result
+    int64_t n_res;      // results filed (0: no index)
 };
 
 constexpr int kSumWords = 6;
@@ -127,6 +143,7 @@ struct LevelArgs {
     const uint64_t *cent;       // cell entries: the result's W support words
     const uint64_t *cne;        // [N][W]: sentinels with a non-empty cell (k, s)
     const uint32_t *csingle;    // [N]: 1 if {k} itself is a result
+    CellIndex cells;            // sparse states
     int level, max_len, max_sec;
     int cpw;                    // parents per warp chunk (1..32)
     unsigned long long *ctr;
@@ -143,7 +160,8 @@ struct LevelArgs {
     uint64_t *fp;               // [fp_cap] fingerprint per reserved row (kDeadFp: unused)
     int64_t fp_cap;
     uint32_t *live;             // unused by the kernels (kept for the host's bookkeeping)
-    int blk;                    // rows a warp reserves at a time (NG..32)
+    int blk;                    // rows a warp reserves at a time (sparse states: at least a round's)
+    int pay_blk;                // sparse states: payload units a warp reserves at a time, at least a round's
     // subtractive variant (Eq. 5): rows hold the extra flux (M entries), then
     // the flux of every column; a state's branches also take flux away from
     // a column in U, and its meta degree counts both lists of the pivot
@@ -232,7 +250,7 @@ __host__ __device__ inline uint32_t mlp_blk_off(int row, int k)
 cudaError_t launch_features(const NetView &nv, const Arena &par, const uint32_t *map, int64_t first, int64_t stride,
                             int64_t n, int level, int max_len, int max_sec, const uint64_t *dep, void *X, int64_t row0,
                             cudaStream_t s);
-cudaError_t launch_labels(const uint64_t *U, int W, const uint32_t *map, int64_t first, int64_t stride, int64_t n,
+cudaError_t launch_labels(const Arena &par, int W, const uint32_t *map, int64_t first, int64_t stride, int64_t n,
                           const uint64_t *ans, int64_t n_ans, float *y, int64_t row0, cudaStream_t s);
 cudaError_t launch_mlp_score(const void *X, int64_t n_rows, const void *wb, const float *params, float *score,
                              unsigned *err, cudaStream_t s);
@@ -265,6 +283,18 @@ cudaError_t launch_write_rows(const NetView &nv, const LevelArgs &a, int sm_coun
 cudaError_t launch_live_list(const uint32_t *meta, int64_t n, uint32_t *live, unsigned long long *count,
                              int sm_count, cudaStream_t s);
 int generate_grid(const NetView &nv, int sm_count);
+// kernels (efm_sparse.cu): the level pass on sparse states
+int sparse_grid(bool sub, bool first_k, int sm_count);
+cudaError_t launch_generate_sparse(const NetView &nv, const LevelArgs &a, int grid, cudaStream_t s);
+cudaError_t launch_dedup_sparse(const LevelArgs &a, int sm_count, cudaStream_t s);
+cudaError_t launch_seed_sparse(const NetView &nv, const LevelArgs &a, int target, cudaStream_t s);
+cudaError_t launch_seedset_sparse(const NetView &nv, const LevelArgs &a, const int32_t *cols, int n_cols,
+                                  cudaStream_t s);
+// the superset rule's index over results [0, n_res); entries of result r start at r * ent_stride
+cudaError_t launch_cells(const NetView &nv, const uint16_t *rcols, int64_t n_res, int32_t *cnt, const CellIndex &ix,
+                         int ent_stride, cudaStream_t s);
+cudaError_t launch_live_sparse(const uint4 *hdr, int64_t n, uint32_t *live, unsigned long long *count, int sm_count,
+                               cudaStream_t s);
 cudaError_t launch_accept(const NetView &nv, const AcceptArgs &a, cudaStream_t s);
 // minimality test of the candidates appended since the last such launch (range read on the
 // device, so no host round trip is needed between expansion and test); then advance the range

@@ -20,104 +20,23 @@
 // tested by Gaussian elimination modulo primes p = 2^31 - c, with enough
 // primes that their product exceeds the Hadamard bound of the columns.
 //
-// Layout: a frontier is an arena of states, each a row of W support words,
+// Layout (narrow networks): a frontier is an arena of states, each a row of W support words,
 // a row of Mpad int32 extra-flux entries (16-byte aligned) and a meta word
 // (acting metabolite, its degree, |U|).  The expansion gives every lane its
 // own child; the seed and minimality kernels give a warp one item.  The
 // static network (CSR by column and by metabolite, twins, pivot keys) is
 // staged into shared memory with one bulk async copy (no multicast) when it
 // fits.
-#include "efm_internal.cuh"
+#include "efm_device.cuh"
 
 namespace efm {
 namespace {
 
-constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int kSpinLimit = 1 << 20;  // x ~1 us sleep: about one second
 
 // primes p = 2^31 - c (c < 2^10), the 24 largest below 2^31
 __constant__ uint32_t c_prime_c[kNumPrimes] = {1,   19,  61,  69,  85,  99,  105, 151, 159, 171, 225, 249,
                                               295, 325, 379, 399, 411, 469, 477, 511, 525, 571, 579, 589};
-
-__device__ __forceinline__ uint64_t mix64(uint64_t x)
-{
-    // splitmix64 finaliser (Steele, Lea, Flood 2014)
-    x ^= x >> 30;
-    x *= 0xbf58476d1ce4e5b9ull;
-    x ^= x >> 27;
-    x *= 0x94d049bb133111ebull;
-    x ^= x >> 31;
-    return x;
-}
-
-__device__ __forceinline__ uint64_t gcd64(uint64_t a, uint64_t b)
-{
-    // binary gcd (Stein)
-    if (a == 0) return b;
-    if (b == 0) return a;
-    const int sh = __ffsll((long long)(a | b)) - 1;
-    a >>= __ffsll((long long)a) - 1;
-    while (b != 0) {
-        b >>= __ffsll((long long)b) - 1;
-        if (a > b) {
-            const uint64_t t = a;
-            a = b;
-            b = t;
-        }
-        b -= a;
-    }
-    return a << sh;
-}
-
-__device__ __forceinline__ uint32_t gcd32(uint32_t a, uint32_t b)
-{
-    if (a == 0) return b;
-    if (b == 0) return a;
-    const int sh = __ffs((int)(a | b)) - 1;
-    a >>= __ffs((int)a) - 1;
-    while (b != 0) {
-        b >>= __ffs((int)b) - 1;
-        if (a > b) {
-            const uint32_t t = a;
-            a = b;
-            b = t;
-        }
-        b -= a;
-    }
-    return a << sh;
-}
-
-__device__ __forceinline__ uint64_t abs64(int64_t x) { return x < 0 ? (uint64_t)(-x) : (uint64_t)x; }
-
-__device__ __forceinline__ bool bit_of(const uint64_t *U, int k) { return (U[k >> 6] >> (k & 63)) & 1ull; }
-
-__device__ __forceinline__ unsigned long long load_volatile(unsigned long long *p)
-{
-    return *(volatile unsigned long long *)p;
-}
-
-__device__ __forceinline__ uint64_t global_ns()
-{
-    uint64_t t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
-
-constexpr uint64_t kWatchdogNs = 20ull * 1000000000ull;  // a level that runs longer gives up
-constexpr int kMaxRounds = 1 << 22;
-
-// Record the first failed self-check (code, offending value, its limit) and
-// raise the error bit; the caller skips the access.
-__device__ void record_diag(unsigned long long *ctr, unsigned bit, unsigned long long code, long long value,
-                            long long limit, int level)
-{
-    atomicOr(&ctr[C_ERR], (unsigned long long)bit);
-    if (atomicCAS(&ctr[C_DIAG], 0ull, code) == 0ull) {
-        ctr[C_DIAG + 1] = (unsigned long long)value;
-        ctr[C_DIAG + 2] = (unsigned long long)limit;
-        ctr[C_DIAG + 3] = (unsigned long long)level;
-    }
-}
 
 // ---------------------------------------------------------------------------
 // static network staging (a4): bulk async copy global -> shared, mbarrier
@@ -190,16 +109,6 @@ __device__ const uint32_t *stage_words(const NetView &nv, uint32_t *sblob, uint6
 // index and compares the full record; records are never compared by tag
 // alone, so the set is exact.
 // ---------------------------------------------------------------------------
-
-enum { INS_NEW = 1, INS_DUP = 0, INS_ARENA_FULL = -1, INS_TIMEOUT = -2, INS_TABLE_FULL = -3 };
-
-__device__ __forceinline__ void slot_tag_pos(uint64_t h, uint64_t mask, uint64_t &pos, uint32_t &tag)
-{
-    const uint64_t f = mix64(h);
-    pos = f & mask;
-    tag = (uint32_t)(f >> 32);
-    if (tag == 0xFFFFFFFFu) tag = 0xFFFFFFFEu;
-}
 
 // word w of the support U' = U (pu, or empty if null) plus column k
 __device__ __forceinline__ uint64_t child_word(const uint64_t *pu, int w, int k)
@@ -295,12 +204,6 @@ __device__ __forceinline__ bool result_inside_wide(const LevelArgs &a, const uin
     return sub;
 }
 
-// pivot key (degree << 16 | row) -> state meta: row | degree << 10 | |U| << 23
-__device__ __forceinline__ uint32_t pack_meta(uint32_t key, int pc)
-{
-    return (key & 0x3FFu) | ((key >> 16) << 10) | ((uint32_t)pc << 23);
-}
-
 // Pivot key of a state: min over unbalanced rows of (degree << 16 | row)
 // (warp-cooperative; lane l holds rows l + 32 e).
 template <int EPL>
@@ -316,16 +219,6 @@ __device__ __forceinline__ uint32_t pivot_key(const uint32_t *bl, const NetView 
         }
     }
     return __reduce_min_sync(FULL, kmin);
-}
-
-// The meta word's degree field counts the branches a state has: the list of
-// the pivot's side, plus (subtractive variant) the opposite list.
-__device__ __forceinline__ uint32_t branch_key(const uint32_t *bl, const NetView &nv, uint32_t key, int sub)
-{
-    if (!sub) return key;
-    const int m = (int)(key & 0xFFFFu);
-    const uint32_t deg = (bl[nv.o_consptr + m + 1] - bl[nv.o_consptr + m]) + (bl[nv.o_prodptr + m + 1] - bl[nv.o_prodptr + m]);
-    return (deg << 16) | (key & 0xFFFFu);
 }
 
 // warp-wide test: all balance rows (m < M) of a row held across the warp are 0
@@ -492,11 +385,6 @@ __device__ void seed_range(const NetView &nv, const LevelArgs &a, int target, in
             const uint32_t bkey = branch_key(bl, nv, key, a.sub);
             if (lane == 0) a.child.meta[idx] = pack_meta(bkey, 1);
             deg_sum += bkey >> 16;
-            if (a.child.fx) {  // the lane masks of {k}: column k's own
-                const int G = EPL >= 8 ? 32 : 4 * EPL;
-                for (int x = lane; x < 2 * G; x += 32)
-                    a.child.fx[(size_t)idx * (2 * G) + x] = bl[(x < G ? nv.o_fixc : nv.o_fixp) + k * G + x % G];
-            }
         }
         if (EPL <= 2 && nv.narrow && a.child.sum) {
             const NarrowSum sm = warp_summary<EPL>(bl, nv, t, lane);
@@ -736,14 +624,6 @@ __global__ void __launch_bounds__(32) seedset_kernel(NetView nv, LevelArgs a, co
     for (int x = lane; x < W; x += 32) a.child.U[x] = U[x];
 #pragma unroll
     for (int e = 0; e < EPL; ++e) a.child.B[lane + 32 * e] = t[e];
-    if (a.child.fx) {  // the lane masks of R_in: the union of its columns'
-        const int G = EPL >= 8 ? 32 : 4 * EPL;
-        for (int x = lane; x < 2 * G; x += 32) {
-            uint32_t f = 0;
-            for (int i = 0; i < n_cols; ++i) f |= nv.blob[(x < G ? nv.o_fixc : nv.o_fixp) + cols[i] * G + x % G];
-            a.child.fx[x] = f;
-        }
-    }
     const uint32_t bkey = branch_key(nv.blob, nv, key, a.sub);
     if (lane == 0) {
         a.child.meta[0] = pack_meta(bkey, n_cols);
@@ -1383,519 +1263,6 @@ __device__ void expand_range(const NetView &nv, const LevelArgs &a, const uint32
 
 
 // ---------------------------------------------------------------------------
-// a1-a5 as two passes (single-job traversal): generate, then deduplicate.
-//
-// Generate: the same per-item work as phase 1 above (branch selection, AND
-// update, balance test, superset rule, pivot key, fingerprint), but every
-// surviving unbalanced child is written straight from registers to a row of
-// the child arena that its warp reserved in advance (rows are reserved blk
-// at a time with one atomic), together with its 64-bit fingerprint.  Nothing
-// waits on another child: no hash-table probe, no publish/compare protocol.
-// Children whose reserved row lies past the arena's capacity keep only their
-// fingerprint (the level is then decided from fingerprints, or run again
-// with a larger arena).
-//
-// Dedup: one thread per reserved row inserts (tag, row) into the level's
-// hash table with a plain CAS.  Every row was written by the previous
-// launch, so a tag match is settled at once by comparing the two rows; the
-// first row of every distinct (U, EF) survives and is appended to the live
-// list, which the next level reads its parents through.
-// ---------------------------------------------------------------------------
-
-template <int G, int CPL>
-__device__ void generate_range(const NetView &nv, const LevelArgs &a, const uint32_t *bl, const uint32_t *blg,
-                               int64_t worker,
-                               int64_t nworkers)
-{
-    constexpr int NG = 32 / G;    // children per warp round
-    constexpr int EPL = 4 * CPL;  // balance entries per lane
-    const int lane = threadIdx.x & 31;
-    const int gi = lane / G;  // group in the warp
-    const int gl = lane % G;  // lane in the group
-    const int lead = gi * G;  // group leader lane
-    const int W = nv.W;
-    const int Mpad = nv.Mpad;
-    // bl: the static network (its sparse tables possibly in shared memory);
-    // blg: the same words, for the dense columns and the first-K tables
-    const int4 *dcol = reinterpret_cast<const int4 *>(blg + nv.o_dcols);
-    const int64_t row_cap = a.child.cap;
-
-    unsigned long long n_exp = 0, n_ovf = 0, n_bal = 0, n_pruned = 0, n_unwritten = 0, n_zero = 0, n_capdead = 0;
-    bool fatal = false;
-    // this warp's reserved rows: [pool_next, pool_next + pool_left)
-    uint64_t pool_next = 0;
-    int pool_left = 0;
-
-    const int cpw = a.cpw;
-    const int64_t wstride = nworkers * cpw;
-    for (int64_t p0 = worker * cpw; p0 < a.n_par; p0 += wstride) {
-        const int64_t pl = p0 + lane;
-        const bool pin = lane < cpw && pl < a.n_par;
-        const int64_t pid = pin ? (a.perm ? (int64_t)a.perm[pl] : a.par_base + pl) : 0;  // this lane's parent
-        const int64_t pn = pl + wstride;
-        if (lane < cpw && pn < a.n_par) {
-            const int64_t nid = a.perm ? (int64_t)a.perm[pn] : a.par_base + pn;
-            const char *rp = reinterpret_cast<const char *>(a.par.B + (size_t)nid * Mpad);
-            for (int off = 0; off < Mpad * 4; off += 128) prefetch_l2(rp + off);
-            prefetch_l2(a.par.U + (size_t)nid * W);
-            prefetch_l2(a.par.meta + nid);
-        }
-        const uint32_t mj = pin ? a.par.meta[pid] : 0u;
-        int dj = pin ? (int)((mj >> 10) & 0x1FFFu) : 0;
-        // first-K: a parent larger than the bound has no descendant among the K smallest
-        if (a.fk_pc > 0 && (int)((mj >> 23) & 0x7Fu) > a.fk_pc) dj = 0;
-        int incl = dj;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int x = __shfl_up_sync(FULL, incl, off);
-            if (lane >= off) incl += x;
-        }
-        const int prej = incl - dj;
-        const int T = __shfl_sync(FULL, incl, 31);
-        if (T > 32 * nv.N) {
-            if (lane == 0) record_diag(a.ctr, ERR_BOUNDS, 3, T, 32 * nv.N, a.level);
-            fatal = true;
-        }
-        for (int base = 0; base < T; base += 32) {
-            if (__any_sync(FULL, fatal)) break;
-            // --- branch selection: one (parent, branch) item per lane ---
-            const int c = base + lane;
-            int j = 0;  // largest j with pre_j <= c
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-                const int v = __shfl_sync(FULL, prej, j + step);
-                if (v <= c) j += step;
-            }
-            const uint32_t pm = __shfl_sync(FULL, mj, j);
-            const int q = c - __shfl_sync(FULL, prej, j);
-            const int64_t pl_ = __shfl_sync(FULL, pid, j);
-            bool okl = c < T;
-            int kl = 0, pcl = 0;
-            bool inl = false, subl = false;
-            int32_t Al = 0, Cl = 0;
-            if (okl) {
-                const int32_t *prow_l = a.par.B + (size_t)pl_ * Mpad;
-                const uint64_t *pu_l = a.par.U + (size_t)pl_ * W;
-                const int piv = (int)(pm & 0x3FFu);
-                pcl = (int)((pm >> 23) & 0x7Fu);
-                const int32_t bi = piv < nv.M ? prow_l[piv] : 0;
-                const bool fwd = bi > 0;  // forward flow: consume the surplus
-                const uint32_t abi = (uint32_t)(bi < 0 ? -bi : bi);
-                const int pv_ = piv < nv.M ? piv : 0;
-                const int lptr = (fwd ? nv.o_consptr : nv.o_prodptr) + pv_;
-                const int lb = (int)bl[lptr];
-                const int le = (int)bl[lptr + 1];
-                // subtractive variant: after the side list, the opposite list
-                // (Eq. 5: less flux on a column of U that moves i the same way)
-                const int optr = (fwd ? nv.o_prodptr : nv.o_consptr) + pv_;
-                const int on = a.sub ? (int)bl[optr + 1] - (int)bl[optr] : 0;
-                if (piv >= nv.M || bi == 0 || q >= (le - lb) + on) {
-                    record_diag(a.ctr, ERR_BOUNDS, 1 + (piv >= nv.M ? 10 : 0) + (bi == 0 ? 100 : 0), (long long)q,
-                                (long long)(le - lb + on), a.level);
-                    fatal = true;
-                    okl = false;
-                } else if (q >= le - lb) {
-                    const uint32_t br = bl[(fwd ? nv.o_prodent : nv.o_consent) + (int)bl[optr] + (q - (le - lb))];
-                    kl = ent_index(br);
-                    const uint32_t sik = (uint32_t)ent_coef(br);  // |S_ik|
-                    inl = bit_of(pu_l, kl);
-                    okl = inl && (a.level - pcl) + 1 <= a.max_sec;
-                    subl = true;
-                    const uint32_t g0 = (abi == 1u || sik == 1u) ? 1u : gcd32(abi, sik);
-                    Al = (int32_t)(sik / g0);
-                    Cl = (int32_t)(abi / g0);
-                } else {
-                    const uint32_t br = bl[(fwd ? nv.o_consent : nv.o_prodent) + lb + q];
-                    kl = ent_index(br);
-                    const uint32_t sik = (uint32_t)ent_coef(br);  // |S_ik|
-                    const int tw = (int)bl[nv.o_twin + kl];
-                    inl = bit_of(pu_l, kl);
-                    const int sec = a.level - pcl;
-                    okl = !(tw >= 0 && bit_of(pu_l, tw)) && (inl ? sec + 1 <= a.max_sec : pcl + 1 <= a.max_len);
-                    if (okl && a.fk_pc > 0) {
-                        const int pc2 = pcl + (inl ? 0 : 1);
-                        okl = pc2 < a.fk_pc || (pc2 == a.fk_pc && !child_after(pu_l, kl, a.fk_sup, W));
-                    }
-                    const uint32_t g0 = (abi == 1u || sik == 1u) ? 1u : gcd32(abi, sik);
-                    Al = (int32_t)(sik / g0);
-                    Cl = (int32_t)(abi / g0);
-                }
-            }
-            if (okl) ++n_exp;
-            const uint32_t infol = (uint32_t)kl | ((uint32_t)pcl << 12) | (inl ? 1u << 19 : 0u) | (subl ? 1u << 20 : 0u);
-            const uint32_t pl32 = (uint32_t)pl_;
-            // the groups take the valid items of this pass NG at a time, in order
-            unsigned vmask = __ballot_sync(FULL, okl);
-            while (vmask) {
-                if (__any_sync(FULL, fatal)) break;
-                const int src = gi < __popc(vmask) ? (int)__fns(vmask, 0, gi + 1) : -1;
-#pragma unroll
-                for (int t = 0; t < NG; ++t) vmask &= vmask - 1;
-                const int sl = src < 0 ? 0 : src;
-                const bool ok = src >= 0;
-                const uint32_t info_i = __shfl_sync(FULL, infol, sl);
-                const int k = (int)(info_i & 0xFFFu);
-                const int pc = (int)((info_i >> 12) & 0x7Fu);
-                const bool in_u = (info_i >> 19) & 1u;
-                const bool subi = (info_i >> 20) & 1u;  // Eq. 5: flux taken away from k
-                const int32_t A = __shfl_sync(FULL, Al, sl);
-                const int32_t C0 = __shfl_sync(FULL, Cl, sl);
-                const int32_t C = subi ? -C0 : C0;
-                const int64_t p = (int64_t)__shfl_sync(FULL, pl32, sl);
-                const int32_t *prow = a.par.B + (size_t)p * Mpad;
-                const uint64_t *pu = a.par.U + (size_t)p * W;
-                // Prop. 3: a subtractive step must leave k with positive flux
-                // (the flux of column k sits at row M + k)
-                bool zflux = false;
-                if (ok && subi) zflux = (int64_t)A * prow[nv.M + k] - (int64_t)C0 <= 0;
-
-                // --- AND update (Eq. 3 / Eq. 4 in integers), group-parallel ---
-                int32_t t32[EPL];
-                uint32_t fl = 0;  // bit0 nonzero, bit1 some |t| == 1, bit2 some t outside int32
-                const int4 *prow4 = reinterpret_cast<const int4 *>(prow);
-                const int4 *col4 = dcol + (size_t)k * (Mpad >> 2);
-                if (ok) {
-#pragma unroll
-                    for (int i = 0; i < CPL; ++i) {
-                        const int4 v = prow4[gl + G * i];
-                        const int4 w = col4[gl + G * i];
-                        const int32_t pv[4] = {v.x, v.y, v.z, v.w}, cv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) {
-                            const int64_t tt = (int64_t)A * pv[jj] + (int64_t)C * cv[jj];
-                            const int32_t lo = (int32_t)tt;
-                            const bool fits = tt == (int64_t)lo && lo != INT32_MIN;
-                            t32[4 * i + jj] = lo;
-                            // bit0: a balance row (m < M; the rest is flux or padding) is nonzero
-                            const bool brow = 4 * (gl + G * i) + jj < nv.M;
-                            fl |= ((tt != 0 && brow) ? 1u : 0u) | ((lo == 1 || lo == -1) ? 2u : 0u) | (fits ? 0u : 4u);
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < EPL; ++e) t32[e] = 0;
-                }
-                fl = group_or<G>(fl);
-                const bool nz = fl & 1u;
-                // slow path: the gcd is needed (no unit entry), or an entry is
-                // outside int32 (then the raw entries are recomputed in 64 bits)
-                const bool slow = ok && !zflux && nz && ((fl & 6u) != 2u);
-                const bool big = (fl & 4u) != 0u;
-                bool ovf = false;
-                if (__any_sync(FULL, slow)) {
-                    uint64_t gg = 0, amax = 0;
-                    if (slow && !big) {
-#pragma unroll
-                        for (int e = 0; e < EPL; ++e) {
-                            const uint32_t at = (uint32_t)(t32[e] < 0 ? -t32[e] : t32[e]);
-                            if (at != 0) gg = gg == 0 ? at : gcd32((uint32_t)gg, at);
-                        }
-                    } else if (slow) {
-                        const GcdMax gm = raw_gcd_max(prow4, col4, gl, G, CPL, A, C);
-                        gg = gm.g;
-                        amax = gm.m;
-                    }
-#pragma unroll
-                    for (int off = G / 2; off > 0; off >>= 1) {
-                        const uint64_t og = __shfl_xor_sync(FULL, gg, off);
-                        gg = og == 0 ? gg : (gg == 0 ? og : gcd64(gg, og));
-                        const uint64_t y = __shfl_xor_sync(FULL, amax, off);
-                        amax = y > amax ? y : amax;
-                    }
-                    if (slow) {
-                        ovf = big && amax / gg > 2147483647ull;
-                        if (!ovf && gg > 1) {
-                            const bool pow2 = (gg & (gg - 1)) == 0;
-                            const int sh = __ffsll((long long)gg) - 1;
-                            if (!big) {
-#pragma unroll
-                                for (int e = 0; e < EPL; ++e)
-                                    t32[e] = t32[e] == 0 ? 0 : (pow2 ? (t32[e] >> sh) : t32[e] / (int32_t)gg);
-                            } else {
-#pragma unroll
-                                for (int i = 0; i < CPL; ++i) {
-                                    const int4 v = prow4[gl + G * i];
-                                    const int4 w = col4[gl + G * i];
-                                    const int32_t pv[4] = {v.x, v.y, v.z, v.w}, cv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                                    for (int jj = 0; jj < 4; ++jj) {
-                                        const int64_t tt = (int64_t)A * pv[jj] + (int64_t)C * cv[jj];
-                                        t32[4 * i + jj] = (int32_t)(tt / (int64_t)gg);
-                                    }
-                                }
-                            }
-                        }
-                    }
-                }
-                if (zflux && gl == 0) ++n_zero;
-                const bool bal = ok && !zflux && !nz;
-                const bool grown = ok && !zflux && nz && !ovf;
-                if (ovf && !zflux && gl == 0) ++n_ovf;
-                if (bal && gl == 0) {
-                    ++n_bal;  // all metabolites stable: to the arbiter
-                    if (insert_support(a, W, pu, k) < INS_DUP) fatal = true;
-                }
-                fatal = group_or<G>(fatal ? 1u : 0u) != 0;
-                // superset rule: the new column k completes a result accepted
-                // at an earlier level (the group's lanes split its bucket)
-                bool pr = false;
-                if (grown && !in_u) {
-                    const int64_t b1 = a.bptr[k];
-                    const int64_t n = a.bptr[k + 1] - b1;
-                    if (W <= 2 && a.cptr) {
-                        if (gl == 0) pr = pruned_indexed(a, pu, k, W, nv.N);
-                    } else if (W <= 2) {
-                        const uint64_t u0 = child_word(pu, 0, k), u1 = W == 2 ? child_word(pu, 1, k) : 0ull;
-                        bool maybe = n > 0;
-                        if (maybe && a.band) {
-                            const uint64_t i0 = __ldg(a.band + (size_t)k * W), i1 = W == 2 ? __ldg(a.band + (size_t)k * W + 1) : 0ull;
-                            maybe = ((i0 & ~u0) | (i1 & ~u1)) == 0;
-                        }
-                        for (int64_t i = gl; i < n && !pr && maybe; i += G) {
-                            const uint64_t *E = a.bres + (size_t)(b1 + i) * W;
-                            const uint64_t e0 = __ldg(E), e1 = W == 2 ? __ldg(E + 1) : 0ull;
-                            pr = ((e0 & ~u0) | (e1 & ~u1)) == 0;
-                        }
-                    } else {
-                        for (int64_t i = gl; i < n && !pr; i += G) pr = result_inside_wide(a, pu, k, b1 + i);
-                    }
-                }
-                pr = group_or<G>(pr ? 1u : 0u) != 0;
-                if (pr && gl == 0) ++n_pruned;
-                bool norm = grown && !pr;
-                // first-K: the lane masks of the rows the child's support
-                // consumes and produces (the parent's, plus column k's)
-                uint32_t fxc = 0, fxp = 0;
-                if (a.child.fx && norm) {
-                    const size_t fo = (size_t)p * (2 * G);
-                    fxc = a.par.fx[fo + gl] | blg[nv.o_fixc + k * G + gl];
-                    fxp = a.par.fx[fo + G + gl] | blg[nv.o_fixp + k * G + gl];
-                }
-                // first-K at the length cap: the child can only take secondary
-                // steps, which add flux to columns of its support.  A row with a
-                // surplus (deficit) that no column of the support consumes
-                // (produces) keeps its sign under every such step, so the child
-                // never balances; with no secondary step left it cannot move.
-                if (a.cap_dead && __any_sync(FULL, norm && pc + (in_u ? 0 : 1) >= a.max_len)) {
-                    bool dead = false;
-                    const int pcc = pc + (in_u ? 0 : 1);
-                    if (norm && pcc >= a.max_len) {
-                        if (a.level - pcc + 1 >= a.max_sec) {
-                            dead = true;
-                        } else if (a.child.fx) {
-#pragma unroll
-                            for (int i = 0; i < CPL; ++i)
-#pragma unroll
-                                for (int jj = 0; jj < 4; ++jj) {
-                                    const int32_t v = t32[4 * i + jj];
-                                    const uint32_t fix = v > 0 ? fxc : fxp;
-                                    if (v != 0 && 4 * (gl + G * i) + jj < nv.M && !((fix >> (4 * i + jj)) & 1u))
-                                        dead = true;
-                                }
-                        }
-                    }
-                    dead = group_or<G>(dead ? 1u : 0u) != 0;
-                    if (dead && gl == 0) ++n_capdead;
-                    norm = norm && !dead;
-                }
-
-                // first-K one below the cap: the child's results have support U
-                // or U + {c} for one more column c.  Balance needs both signs in
-                // every row a support touches, and a row that U touches with one
-                // sign only (a surplus with no consumer, a deficit with no
-                // producer in U) is a row EF keeps nonzero under secondary
-                // steps.  With such rows, some column c must give each of them
-                // the missing sign and find the opposite sign in U for every
-                // row of its own (twin rule kept); the group tries the columns
-                // able to fix the one-sided row with the shortest fixer list.
-                if (a.cap_dead && a.child.fx && __any_sync(FULL, norm && pc + (in_u ? 0 : 1) == a.max_len - 1)) {
-                    const bool mine = norm && pc + (in_u ? 0 : 1) == a.max_len - 1;
-                    uint32_t dl = 0;            // this lane's one-sided rows, bits as in fxc / fxp
-                    uint32_t pick = 0xFFFFFFFFu;  // list length << 20 | surplus << 19 | row
-                    if (mine) {
-#pragma unroll
-                        for (int i = 0; i < CPL; ++i)
-#pragma unroll
-                            for (int jj = 0; jj < 4; ++jj) {
-                                const int r = 4 * (gl + G * i) + jj;
-                                const int32_t v = t32[4 * i + jj];
-                                const uint32_t fix = v > 0 ? fxc : fxp;
-                                if (v != 0 && r < nv.M && !((fix >> (4 * i + jj)) & 1u)) {
-                                    dl |= 1u << (4 * i + jj);
-                                    const int lp = (v > 0 ? nv.o_consptr : nv.o_prodptr) + r;
-                                    const uint32_t len = min(bl[lp + 1] - bl[lp], 4095u);
-                                    const uint32_t cand = (len << 20) | (v > 0 ? 1u << 19 : 0u) | (uint32_t)r;
-                                    pick = cand < pick ? cand : pick;
-                                }
-                            }
-                    }
-                    const uint32_t nd = group_add<G>((uint32_t)__popc(dl));
-                    pick = group_min<G>(pick);
-                    bool open = mine && nd > 0;  // still looking for a completing column
-                    const int r0 = (int)(pick & 0x7FFFFu);
-                    const bool sur0 = (pick >> 19) & 1u;
-                    const int lp0 = open ? (sur0 ? nv.o_consptr : nv.o_prodptr) + r0 : 0;
-                    const int b0 = open ? (int)bl[lp0] : 0;
-                    const int n0 = open ? (int)bl[lp0 + 1] - b0 : 0;
-                    const int eo0 = sur0 ? nv.o_consent : nv.o_prodent;
-                    bool found = false;
-                    for (int c0 = 0; __any_sync(FULL, open && c0 < n0); c0 += G) {
-                        const bool act = open && c0 < n0;
-                        const int ci = c0 + gl;
-                        int kc = -1;
-                        if (act && ci < n0) kc = ent_index(bl[eo0 + b0 + ci]);
-                        bool ok2 = kc >= 0;
-                        if (ok2) {
-                            const int tw = (int)bl[nv.o_twin + kc];
-                            ok2 = !(tw >= 0 && (tw == k || ((pu[tw >> 6] >> (tw & 63)) & 1ull)));
-                        }
-                        const int cb = ok2 ? (int)blg[nv.o_colptr + kc] : 0;
-                        const int cn = ok2 ? (int)blg[nv.o_colptr + kc + 1] - cb : 0;
-                        const int cmax = (int)__reduce_max_sync(FULL, (unsigned)cn);
-                        uint32_t hit = 0;  // one-sided rows of U the column fixes
-                        for (int q = 0; q < cmax; ++q) {
-                            int r = 0, sg = 0;
-                            if (q < cn) {
-                                const uint32_t ent = blg[nv.o_colent + cb + q];
-                                r = ent_index(ent);
-                                sg = ent_coef(ent) > 0 ? 1 : -1;
-                            }
-                            const int src = lead + ((r >> 2) % G);
-                            const int bit = 4 * ((r >> 2) / G) + (r & 3);
-                            const uint32_t wc = __shfl_sync(FULL, fxc, src);
-                            const uint32_t wp = __shfl_sync(FULL, fxp, src);
-                            const uint32_t wd = __shfl_sync(FULL, dl, src);
-                            if (q < cn) {
-                                // the column produces r: U must consume it, and the reverse
-                                if (!(((sg > 0 ? wc : wp) >> bit) & 1u)) ok2 = false;
-                                hit += (wd >> bit) & 1u;
-                            }
-                        }
-                        ok2 = ok2 && hit == nd;
-                        const bool any2 = group_or<G>(ok2 ? 1u : 0u) != 0;
-                        if (act && any2) {
-                            found = true;
-                            open = false;
-                        }
-                    }
-                    const bool dead = mine && nd > 0 && !found;
-                    if (dead && gl == 0) ++n_capdead;
-                    norm = norm && !dead;
-                }
-
-                // --- pivot key and fingerprint ---
-                uint32_t key = 0xFFFFFFFFu, hlo = 0, hhi = 0;
-                if (norm) {
-#pragma unroll
-                    for (int i = 0; i < CPL; ++i)
-#pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) {
-                            const int m = 4 * (gl + G * i) + jj;
-                            const int32_t v = t32[4 * i + jj];
-                            if (v != 0 && m < nv.M) {
-                                const uint32_t kk = bl[(v > 0 ? nv.o_keypos : nv.o_keyneg) + m];
-                                key = kk < key ? kk : key;
-                            }
-                            hash_entry((uint32_t)m, (uint32_t)v, hlo, hhi);
-                        }
-                    for (int w = gl; w < W; w += G) {
-                        const uint64_t x = mix64(child_word(pu, w, k) ^ (0x2545f4914f6cdd1dull * (uint64_t)(w + 1)));
-                        hlo += (uint32_t)x;
-                        hhi ^= (uint32_t)(x >> 32);
-                    }
-                }
-                key = group_min<G>(key);
-                hlo = group_add<G>(hlo);
-                hhi = group_xor<G>(hhi);
-
-                // --- a reserved row for every surviving child of the round ---
-                const unsigned nm = __ballot_sync(FULL, norm && gl == 0);
-                const int cnt = __popc(nm);
-                if (cnt > 0) {
-                    const int rank = __popc(nm & ((1u << lead) - 1u));
-                    uint64_t fresh = 0;
-                    if (pool_left < cnt) {
-                        if (lane == 0) fresh = atomicAdd(&a.ctr[C_WRITTEN], (unsigned long long)a.blk);
-                        fresh = __shfl_sync(FULL, fresh, 0);
-                    }
-                    const uint64_t idx = rank < pool_left ? pool_next + (uint64_t)rank
-                                                          : fresh + (uint64_t)(rank - pool_left);
-                    if (pool_left < cnt) {
-                        pool_next = fresh + (uint64_t)(cnt - pool_left);
-                        pool_left = a.blk - (cnt - pool_left);
-                    } else {
-                        pool_next += (uint64_t)cnt;
-                        pool_left -= cnt;
-                    }
-                    if (norm) {
-                        if ((int64_t)idx < row_cap) {
-                            int4 *db = reinterpret_cast<int4 *>(a.child.B + (size_t)idx * Mpad);
-#pragma unroll
-                            for (int i = 0; i < CPL; ++i)
-                                db[gl + G * i] = make_int4(t32[4 * i + 0], t32[4 * i + 1], t32[4 * i + 2], t32[4 * i + 3]);
-                            uint64_t *du = a.child.U + (size_t)idx * W;
-                            for (int w = gl; w < W; w += G) du[w] = child_word(pu, w, k);
-                            if (a.child.fx) {
-                                a.child.fx[(size_t)idx * (2 * G) + gl] = fxc;
-                                a.child.fx[(size_t)idx * (2 * G) + G + gl] = fxp;
-                            }
-                            if (gl == 0) a.child.meta[idx] = pack_meta(branch_key(bl, nv, key, a.sub), pc + (in_u ? 0 : 1));
-                        } else if (gl == 0) {
-                            ++n_unwritten;
-                        }
-                        if (gl == 0) {
-                            if ((int64_t)idx < a.fp_cap) {
-                                uint64_t f = ((uint64_t)hhi << 32) | hlo;
-                                if (f == kDeadFp) f = kDeadFp - 1;
-                                a.fp[idx] = f;
-                            } else {
-                                record_diag(a.ctr, ERR_BOUNDS, 7, (long long)idx, a.fp_cap, a.level);
-                                fatal = true;
-                            }
-                        }
-                    }
-                }
-            }
-        }
-        if (__any_sync(FULL, fatal)) break;
-    }
-    // rows reserved but not used: no fingerprint (the dedup pass skips them) and
-    // no branches (the next level reads every row of the arena)
-    for (int x = lane; x < pool_left; x += 32) {
-        if ((int64_t)(pool_next + x) < a.fp_cap) a.fp[pool_next + x] = kDeadFp;
-        if ((int64_t)(pool_next + x) < row_cap) a.child.meta[pool_next + x] = 0u;
-    }
-    if (n_exp) atomicAdd(&a.ctr[C_EXP], n_exp);
-    if (n_ovf) atomicAdd(&a.ctr[C_OVF], n_ovf);
-    if (n_bal) atomicAdd(&a.ctr[C_BAL], n_bal);
-    if (n_pruned) atomicAdd(&a.ctr[C_PRUNED], n_pruned);
-    if (n_unwritten) atomicAdd(&a.ctr[C_UNWRITTEN], n_unwritten);
-    if (n_zero) atomicAdd(&a.ctr[C_ZERO], n_zero);
-    if (n_capdead) atomicAdd(&a.ctr[C_CAPDEAD], n_capdead);
-}
-
-template <int G, int CPL>
-__global__ void __launch_bounds__(kExpandWarps * 32, (CPL <= 2 ? 3 : 2)) generate_kernel(NetView nv, LevelArgs a,
-                                                                                      int staged)
-{
-    extern __shared__ __align__(16) uint32_t smem[];
-    const int wid = threadIdx.x >> 5;
-    // staged: 0 nothing, 1 the whole blob, 2 its sparse tables [o_consptr, o_hbits)
-    const int w0 = staged == 2 ? nv.o_consptr : 0;
-    const int nw = staged == 1 ? nv.blob_words : (staged == 2 ? nv.o_hbits - nv.o_consptr : 0);
-    uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + nw);
-    const uint32_t *bl = nv.blob;
-    if (staged) {
-        const uint32_t *sb = stage_words(nv, smem, mbar, w0, nw, a.ctr);
-        if (sb == nullptr) return;
-        // offsets index the blob: the staged range answers for [w0, w0 + nw)
-        bl = reinterpret_cast<const uint32_t *>(reinterpret_cast<uintptr_t>(sb) - (uintptr_t)w0 * 4u);
-    }
-    generate_range<G, CPL>(nv, a, bl, staged == 2 ? nv.blob : bl, (int64_t)blockIdx.x * kExpandWarps + wid,
-                           (int64_t)gridDim.x * kExpandWarps);
-}
-
-// ---------------------------------------------------------------------------
 // Generate, narrow networks (at most 64 internal rows): incremental state
 // summaries.
 //
@@ -1931,14 +1298,9 @@ template <int G>
 __device__ void generate_narrow(const NetView &nv, const LevelArgs &a, const uint32_t *bl, int64_t worker,
                                 int64_t nworkers)
 {
-    constexpr int CPL = 2;
-    constexpr int NG = 32 / G;
     const int lane = threadIdx.x & 31;
-    const int gi = lane / G;
-    const int gl = lane % G;
     const int W = nv.W;
     const int Mpad = nv.Mpad;
-    const int4 *dcol = reinterpret_cast<const int4 *>(bl + nv.o_dcols);
     const int64_t row_cap = a.child.cap;
 
     unsigned long long n_exp = 0, n_ovf = 0, n_bal = 0, n_pruned = 0, n_unwritten = 0;
@@ -3449,52 +2811,6 @@ int generate_narrow_grid_t(const NetView &nv, int sm_count)
     return sm_count * per_sm;
 }
 
-// the generic kernel stages the whole static network when it fits, else its
-// sparse tables when those fit (the dense columns stay in global memory)
-inline int generic_staging(const NetView &nv)
-{
-    if (nv.blob_words * 4 <= kStageLimitBytes) return 1;
-    if ((nv.o_hbits - nv.o_consptr) * 4 <= kStageSparseLimitBytes && nv.o_consptr % 4 == 0 && nv.o_hbits % 4 == 0)
-        return 2;
-    return 0;
-}
-inline size_t generic_smem(const NetView &nv, int mode)
-{
-    return (size_t)(mode == 1 ? nv.blob_words : (mode == 2 ? nv.o_hbits - nv.o_consptr : 0)) * 4 + 16;
-}
-
-template <int G, int CPL>
-cudaError_t launch_generate_t(const NetView &nv, const LevelArgs &a, int grid, cudaStream_t s)
-{
-    const int mode = generic_staging(nv);
-    const size_t sm = generic_smem(nv, mode);
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaFuncSetAttribute(generate_kernel<G, CPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (kStageLimitBytes > kStageSparseLimitBytes ? kStageLimitBytes : kStageSparseLimitBytes) + 16);
-        attr_set = true;
-    }
-    generate_kernel<G, CPL><<<grid, kExpandWarps * 32, sm, s>>>(nv, a, mode);
-    return cudaGetLastError();
-}
-
-template <int G, int CPL>
-int generate_grid_t(const NetView &nv, int sm_count)
-{
-    const size_t sm = generic_smem(nv, generic_staging(nv));
-    cudaFuncSetAttribute(generate_kernel<G, CPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (kStageLimitBytes > kStageSparseLimitBytes ? kStageLimitBytes : kStageSparseLimitBytes) + 16);
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, generate_kernel<G, CPL>, kExpandWarps * 32, sm) !=
-            cudaSuccess ||
-        per_sm < 1) {
-        cudaGetLastError();
-        per_sm = 1;
-    }
-    return sm_count * per_sm;
-}
-
-
 }  // namespace
 
 #define EFM_EPL_DISPATCH(EPLV, CALL) \
@@ -3516,20 +2832,6 @@ cudaError_t launch_seed(const NetView &nv, const LevelArgs &a, int target, cudaS
 #undef CALL_SEED
 }
 
-// (lanes per child, 16-byte chunks per lane) for each row width Mpad = 32 EPL
-#define EFM_GROUP_DISPATCH(EPLV, CALL) \
-    switch (EPLV) {                    \
-    case 1: return CALL(4, 2);         \
-    case 2: return CALL(8, 2);         \
-    case 4: return CALL(16, 2);        \
-    case 8: return CALL(32, 2);        \
-    case 16: return CALL(32, 4);       \
-    case 28: return CALL(32, 7);       \
-    case 32: return CALL(32, 8);       \
-    default: break;                    \
-    }
-
-
 cudaError_t launch_generate(const NetView &nv, const LevelArgs &a, int grid, cudaStream_t s)
 {
     // narrow networks: incremental summaries (needs the arenas' summary arrays)
@@ -3537,9 +2839,6 @@ cudaError_t launch_generate(const NetView &nv, const LevelArgs &a, int grid, cud
         if (nv.EPL == 1) return launch_generate_narrow_t<4>(nv, a, grid, s);
         if (nv.EPL == 2) return launch_generate_narrow_t<8>(nv, a, grid, s);
     }
-#define CALL_GEN(G, C) launch_generate_t<G, C>(nv, a, grid, s)
-    EFM_GROUP_DISPATCH(nv.EPL, CALL_GEN)
-#undef CALL_GEN
     return cudaErrorInvalidValue;
 }
 
@@ -3547,9 +2846,6 @@ int generate_grid(const NetView &nv, int sm_count)
 {
     if (nv.narrow && nv.EPL == 1) return generate_narrow_grid_t<4>(nv, sm_count);
     if (nv.narrow && nv.EPL == 2) return generate_narrow_grid_t<8>(nv, sm_count);
-#define CALL_GGRID(G, C) generate_grid_t<G, C>(nv, sm_count)
-    EFM_GROUP_DISPATCH(nv.EPL, CALL_GGRID)
-#undef CALL_GGRID
     return sm_count;
 }
 

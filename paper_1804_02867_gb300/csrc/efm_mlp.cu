@@ -174,76 +174,104 @@ __global__ void __launch_bounds__(kFeatWarps * 32) features_kernel(NetView nv, A
     for (int64_t r = (int64_t)blockIdx.x * kFeatWarps + wid; r < n; r += (int64_t)gridDim.x * kFeatWarps) {
         const int64_t pos = first + r * stride;
         const int64_t p = map ? (int64_t)map[pos] : pos;
-        const uint64_t *U = par.U + (size_t)p * W;
-        const int32_t *B = par.B + (size_t)p * nv.Mpad;
-        const uint32_t meta = par.meta[p];
-        int nz = 0;
-        uint32_t amax = 0;
-        for (int m = lane; m < nv.M; m += 32) {
-            const int32_t v = B[m];
-            nz += v != 0;
-            const uint32_t av = (uint32_t)(v < 0 ? -v : v);
-            amax = av > amax ? av : amax;
-        }
+        int nz = 0, pcl = 0, ndep = 0, anydep = 0;
+        uint32_t amax = 0, meta;
+        float colsum = 0.f;
+        float low[4] = {1.f, 1.f, 1.f, 1.f};  // the four lowest columns
         emb[wid][lane] = 0.f;
         emb[wid][lane + 32] = 0.f;
         __syncwarp();
-        float colsum = 0.f;
-        int pcl = 0;
-        for (int w = lane; w < W; w += 32) {
-            uint64_t x = U[w];
-            pcl += __popcll(x);
-            while (x) {
-                const int b = __ffsll((long long)x) - 1;
-                x &= x - 1;
-                const uint32_t k = (uint32_t)(w * 64 + b);
-                const uint32_t h = col_hash(k);
-                atomicAdd(&emb[wid][h & 63u], (h & 64u) ? 1.f : -1.f);
-                colsum += (float)k;
+        auto add_column = [&](uint32_t k) {
+            const uint32_t h = col_hash(k);
+            atomicAdd(&emb[wid][h & 63u], (h & 64u) ? 1.f : -1.f);
+            colsum += (float)k;
+        };
+        if (par.hdr) {
+            // sparse state (layout in efm_sparse.cu): the column list, then
+            // the entries; flux entries (rows past M) are not balance rows
+            const uint4 hd = par.hdr[p];
+            const uint4 *pay = par.pay + hd.x;
+            meta = hd.y;
+            const int n = (int)((meta >> 23) & 0x7Fu);
+            const uint16_t *lst = reinterpret_cast<const uint16_t *>(pay) + 4;
+            const uint64_t *D = dep ? dep + (size_t)(meta & 0x3FFu) * W : nullptr;
+            for (int i = lane; i < n; i += 32) {
+                const int k = lst[i];
+                add_column((uint32_t)k);
+                ++pcl;
+                if (D) ndep += (int)((D[k >> 6] >> (k & 63)) & 1ull);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i < n) low[i] = (float)lst[i] / (float)nv.N;
+            const int2 *ent = reinterpret_cast<const int2 *>(pay + sparse_list_units(n));
+            for (int i = lane; i < (int)(hd.z & 0x7FFu); i += 32) {
+                const int2 e = ent[i];
+                if (e.x >= nv.M) continue;
+                ++nz;
+                const uint32_t av = (uint32_t)(e.y < 0 ? -e.y : e.y);
+                amax = av > amax ? av : amax;
+            }
+            if (D)
+                for (int w = lane; w < W; w += 32) anydep |= D[w] != 0ull;
+        } else {
+            const uint64_t *U = par.U + (size_t)p * W;
+            const int32_t *B = par.B + (size_t)p * nv.Mpad;
+            meta = par.meta[p];
+            for (int m = lane; m < nv.M; m += 32) {
+                const int32_t v = B[m];
+                nz += v != 0;
+                const uint32_t av = (uint32_t)(v < 0 ? -v : v);
+                amax = av > amax ? av : amax;
+            }
+            for (int w = lane; w < W; w += 32) {
+                uint64_t x = U[w];
+                pcl += __popcll(x);
+                while (x) {
+                    const int b = __ffsll((long long)x) - 1;
+                    x &= x - 1;
+                    add_column((uint32_t)(w * 64 + b));
+                }
+            }
+            // lowest words first, one ballot per word
+            int got = 0;
+            for (int w0 = 0; w0 < W && got < 4; w0 += 32) {
+                const uint64_t x = (w0 + lane < W) ? U[w0 + lane] : 0ull;
+                unsigned nzm = __ballot_sync(FULLMASK, x != 0ull);
+                while (nzm && got < 4) {
+                    const int src = __ffs((int)nzm) - 1;
+                    nzm &= nzm - 1;
+                    uint64_t y = __shfl_sync(FULLMASK, x, src);
+                    while (y && got < 4) {
+                        const int b = __ffsll((long long)y) - 1;
+                        y &= y - 1;
+                        low[got++] = (float)((w0 + src) * 64 + b) / (float)nv.N;
+                    }
+                }
+            }
+            // flux-dependent columns of the pivot (tags of dep_out | dep_in) inside U
+            const int piv = (int)(meta & 0x3FFu);
+            if (dep && piv < nv.M) {
+                const uint64_t *D = dep + (size_t)piv * W;
+                for (int w = lane; w < W; w += 32) {
+                    ndep += __popcll(U[w] & D[w]);
+                    anydep |= D[w] != 0ull;
+                }
             }
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             nz += __shfl_xor_sync(FULLMASK, nz, off);
             pcl += __shfl_xor_sync(FULLMASK, pcl, off);
+            ndep += __shfl_xor_sync(FULLMASK, ndep, off);
+            anydep |= __shfl_xor_sync(FULLMASK, anydep, off);
             colsum += __shfl_xor_sync(FULLMASK, colsum, off);
             const uint32_t o = __shfl_xor_sync(FULLMASK, amax, off);
             amax = o > amax ? o : amax;
         }
-        // the four lowest columns: lowest words first, one ballot per word
-        float low[4] = {1.f, 1.f, 1.f, 1.f};
-        int got = 0;
-        for (int w0 = 0; w0 < W && got < 4; w0 += 32) {
-            const uint64_t x = (w0 + lane < W) ? U[w0 + lane] : 0ull;
-            unsigned nzm = __ballot_sync(FULLMASK, x != 0ull);
-            while (nzm && got < 4) {
-                const int src = __ffs((int)nzm) - 1;
-                nzm &= nzm - 1;
-                uint64_t y = __shfl_sync(FULLMASK, x, src);
-                while (y && got < 4) {
-                    const int b = __ffsll((long long)y) - 1;
-                    y &= y - 1;
-                    low[got++] = (float)((w0 + src) * 64 + b) / (float)nv.N;
-                }
-            }
-        }
         __syncwarp();
         const int pc = (int)((meta >> 23) & 0x7Fu);
         const int piv = (int)(meta & 0x3FFu);
-        // flux-dependent columns of the pivot (tags of dep_out | dep_in) inside U
-        int ndep = 0, anydep = 0;
-        if (dep && piv < nv.M) {
-            const uint64_t *D = dep + (size_t)piv * W;
-            for (int w = lane; w < W; w += 32) {
-                ndep += __popcll(U[w] & D[w]);
-                anydep |= D[w] != 0ull;
-            }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                ndep += __shfl_xor_sync(FULLMASK, ndep, off);
-                anydep |= __shfl_xor_sync(FULLMASK, anydep, off);
-            }
-        }
         const int deg = (int)((meta >> 10) & 0x1FFFu);
         const int sec = level - (pc - 1);
         const float inv_sqrt = pcl > 0 ? rsqrtf((float)pcl) : 0.f;
@@ -292,20 +320,33 @@ __global__ void __launch_bounds__(kFeatWarps * 32) features_kernel(NetView nv, A
 
 // Training label of a sampled state: 1 when its support lies inside one of
 // the answer's supports (the state can still reach that answer).
-__global__ void labels_kernel(const uint64_t *Uar, int W, const uint32_t *map, int64_t first, int64_t stride,
+__global__ void labels_kernel(Arena par, int W, const uint32_t *map, int64_t first, int64_t stride,
                               int64_t n, const uint64_t *ans, int64_t n_ans, float *y, int64_t row0)
 {
     const int lane = threadIdx.x & 31;
     for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n;
          r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int64_t pos = first + r * stride;
-        const uint64_t *U = Uar + (size_t)(map ? (int64_t)map[pos] : pos) * W;
+        const int64_t p = map ? (int64_t)map[pos] : pos;
         bool in = false;
-        for (int64_t a = lane; a < n_ans && !in; a += 32) {
-            const uint64_t *A = ans + (size_t)a * W;
-            bool sub = true;
-            for (int w = 0; w < W && sub; ++w) sub = (U[w] & ~A[w]) == 0;
-            in = sub;
+        if (par.hdr) {  // sparse state: its column list
+            const uint4 hd = par.hdr[p];
+            const uint16_t *lst = reinterpret_cast<const uint16_t *>(par.pay + hd.x) + 4;
+            const int m = (int)((hd.y >> 23) & 0x7Fu);
+            for (int64_t a = lane; a < n_ans && !in; a += 32) {
+                const uint64_t *A = ans + (size_t)a * W;
+                bool sub = true;
+                for (int i = 0; i < m && sub; ++i) sub = (A[lst[i] >> 6] >> (lst[i] & 63)) & 1ull;
+                in = sub;
+            }
+        } else {
+            const uint64_t *U = par.U + (size_t)p * W;
+            for (int64_t a = lane; a < n_ans && !in; a += 32) {
+                const uint64_t *A = ans + (size_t)a * W;
+                bool sub = true;
+                for (int w = 0; w < W && sub; ++w) sub = (U[w] & ~A[w]) == 0;
+                in = sub;
+            }
         }
         const bool any = __any_sync(FULLMASK, in);
         if (lane == 0) y[row0 + r] = any ? 1.f : 0.f;
@@ -694,12 +735,12 @@ cudaError_t launch_features(const NetView &nv, const Arena &par, const uint32_t 
     return cudaGetLastError();
 }
 
-cudaError_t launch_labels(const uint64_t *U, int W, const uint32_t *map, int64_t first, int64_t stride, int64_t n,
+cudaError_t launch_labels(const Arena &par, int W, const uint32_t *map, int64_t first, int64_t stride, int64_t n,
                           const uint64_t *ans, int64_t n_ans, float *y, int64_t row0, cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
     const int64_t blocks = std::min<int64_t>((n + 7) / 8, (int64_t)sm_count_cached() * 16);
-    labels_kernel<<<(unsigned)blocks, 256, 0, s>>>(U, W, map, first, stride, n, ans, n_ans, y, row0);
+    labels_kernel<<<(unsigned)blocks, 256, 0, s>>>(par, W, map, first, stride, n, ans, n_ans, y, row0);
     return cudaGetLastError();
 }
 

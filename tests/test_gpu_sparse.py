@@ -1,0 +1,69 @@
+"""Sparse states of the level pass: sizes where the layout's edges lie.
+
+* dense reactions (20-60 metabolites each): a state's entries exceed what the
+  payload pool holds per row, so levels are run again with a larger pool;
+* coefficients whose rows share divisors (the entries are divided);
+* column lists that end at and around a 16-byte unit (4, 12, 20 columns),
+  reached by budgets that stop at different depths.
+
+Supports and every counter must equal the oracle's.
+"""
+import numpy as np
+import pytest
+
+from paper_1804_02867_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def efm():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1804_02867_gb300 import build, efmgraph
+
+    build.build()
+    efmgraph.load_library()
+    return efmgraph
+
+
+def check(oracle_lib, efm, net, targets, max_len, max_sec, budget, **kw):
+    with efm.Network(net) as nw:
+        got = efm.enumerate_targets(nw, targets, max_len, max_sec, 0, budget, **kw)
+    out = []
+    for t, (sup, ctr) in zip(targets, got):
+        osup, octr = oracle_lib.enumerate_pathways(net, t, oracle_lib.Limits(max_len, max_sec, 0, budget))
+        assert np.array_equal(sup, osup), (net.name, t, budget)
+        assert ctr == octr, (net.name, t, budget, ctr, octr)
+        out.append(ctr)
+    return out
+
+
+@pytest.mark.parametrize("size_range,budget", [((20, 60), 1 << 10), ((20, 60), 1 << 13), ((6, 14), 1 << 12)])
+def test_dense_reactions(oracle_lib, efm, size_range, budget):
+    net = synth.generate(n_int=100, n_targets=3, n_hubs=3, n_substrates=2, n_rxn=160, n_rev=40, size_range=size_range,
+                         coef_probs={1: 0.5, 2: 0.3, 3: 0.2}, gamma=None, hub_degree=(5, 20), seed=77,
+                         name=f"dense-{size_range[1]}")
+    out = check(oracle_lib, efm, net, net.targets, 24, 2, budget)
+    assert any(c["frontier_max"] > 100 for c in out)
+
+
+@pytest.mark.parametrize("max_len", [3, 4, 5, 12, 13, 20, 21])
+def test_list_unit_edges(oracle_lib, efm, max_len):
+    """A chain-like network (few branches) whose supports grow to max_len."""
+    net = synth.generate(n_int=70, n_targets=2, n_hubs=2, n_substrates=2, n_rxn=90, n_rev=20, size_range=(2, 3),
+                         coef_probs={1: 0.4, 2: 0.4, 4: 0.2}, gamma=None, hub_degree=(5, 20), seed=91, name="chainlike")
+    check(oracle_lib, efm, net, net.targets + [-1], max_len, 3, 1 << 12)
+
+
+@pytest.mark.parametrize("max_results", [1, 50])
+def test_capped(oracle_lib, efm, max_results):
+    net = synth.generate(n_int=120, n_targets=2, n_hubs=3, n_substrates=2, n_rxn=300, n_rev=60, size_range=(2, 5),
+                         coef_probs=synth.CORE_COEFS, gamma=2.2, hub_degree=(20, 60), seed=5, name="mid-120")
+    with efm.Network(net) as nw:
+        got = efm.enumerate_targets(nw, net.targets, 20, 2, max_results, 1 << 14)
+    for t, (sup, ctr) in zip(net.targets, got):
+        osup, octr = oracle_lib.enumerate_pathways(net, t, oracle_lib.Limits(20, 2, max_results, 1 << 14))
+        assert np.array_equal(sup, osup) and ctr == octr, (t, ctr, octr)
