@@ -17,9 +17,6 @@
 #include "efm_netprep.h"
 #include "efm_topk.h"
 
-static_assert(efm::kNarrowKeyRanks == efm::kNarrowRows && efm::kColxWordsDev == efm::kColxWords,
-              "narrow-network table layout of the kernels and the loader");
-
 using namespace efm;
 
 namespace {
@@ -176,17 +173,18 @@ extern "C" int efm_load_network(int32_t n_met, int32_t n_rxn, const int32_t *row
     nv.o_keyneg = prep.o_keyneg;
     nv.o_hbits = prep.o_hbits;
     nv.o_dcols = prep.o_dcols;
-    nv.narrow = prep.narrow ? 1 : 0;
+    nv.o_scol = prep.o_scol;
     nv.o_rank = prep.o_rank;
     nv.o_keyr = prep.o_keyr;
-    nv.o_hrow = prep.o_hrow;
     nv.o_colx = prep.o_colx;
+    nv.o_nent = prep.o_nent;
     nv.blob_words = (int)blob.size();
     nv.M = prep.M;
     nv.N = prep.N;
     nv.W = prep.W;
     nv.EPL = prep.EPL;
     nv.Mpad = prep.Mpad;
+    nv.form = nv.W > 2 ? 0 : (prep.narrow ? 2 : 1);
     nv.n_met = n_met;
     cudaStream_t s = net->stream;
     int rc = EFM_OK;
@@ -249,7 +247,8 @@ extern "C" int efm_load_network(int32_t n_met, int32_t n_rxn, const int32_t *row
         vs.o_hbits = sub.o_hbits;
         vs.EPL = sub.EPL;
         vs.Mpad = sub.Mpad;
-        vs.narrow = 0;
+        vs.o_scol = sub.o_scol;
+        vs.form = vs.W <= 2 ? 1 : 0;
         net->has_sub = true;
     }
     *out = net;
@@ -292,25 +291,20 @@ namespace {
 
 // Device buffers of one traversal, reused across the targets of a job.
 struct Work {
-    DevBuf U[2], B[2], meta[2], live[2];
-    DevBuf sum[2];  // narrow networks: per-state summaries of the extra-flux row
-    DevBuf hdr[2], pay[2];      // sparse states: headers, payload pool
+    DevBuf hdr[2], pay[2];  // arenas: headers, payload pools
     uint64_t pay_cap[2] = {0, 0};
-    bool sparse = false;
-    DevBuf cells, ksig;         // sparse states: the superset rule's index (with cent, csingle)
-    uint64_t cell_cap = 0;
-    DevBuf slots, cslots, cand, res, bcnt, bfill, bptr, bres, ctr, sortidx, rcols;
+    DevBuf live;                   // training traces: the surviving rows of a frontier
+    int64_t live_cap = 0;
+    DevBuf slots, cslots, cand, res, bcnt, ctr, sortidx, rcols;
+    DevBuf cells, cent, ksig, csingle;  // the superset rule's index
+    int64_t cent_cap = 0;
     DevBuf fp;         // fingerprints of one level's reserved child rows
-    DevBuf wrec;       // narrow networks: the row pass's record per reserved row (16 B)
-    DevBuf slow;       // narrow networks: records of the children the settle pass decides
-    int64_t slow_cap = 0;
+    DevBuf open;       // the rows among them whose child the dedup pass finishes
     DevBuf perm, fkb;  // first-K search: parent order of a level, bound support
-    DevBuf band;       // per column: intersection of the results containing it (W <= 2)
-    DevBuf ccnt, cfill, cptr, cne, csingle, cent;  // W <= 2: the superset rule's sentinel index
     DevBuf lx, lscore, lhist, lerr;  // learned order: features, scores, buckets, error flag
     int64_t lx_rows = 0;
     int64_t rows[2] = {0, 0};  // capacity of each arena (rows)
-    int64_t F_cap = 0, cand_cap = 0, res_cap = 0, bres_cap = 0;  // bres_cap in bucket entries
+    int64_t F_cap = 0, cand_cap = 0, res_cap = 0;
     int64_t fp_cap = 0, perm_cap = 0;
     uint64_t slot_cap = 0, cslot_cap = 0, sort_cap = 0;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -318,11 +312,6 @@ struct Work {
 
 void free_arena(Work &w, int i, cudaStream_t s)
 {
-    dev_free(w.U[i], s);
-    dev_free(w.B[i], s);
-    dev_free(w.meta[i], s);
-    dev_free(w.live[i], s);
-    dev_free(w.sum[i], s);
     dev_free(w.hdr[i], s);
     dev_free(w.pay[i], s);
     w.rows[i] = 0;
@@ -332,34 +321,24 @@ void free_arena(Work &w, int i, cudaStream_t s)
 void free_work(Work &w, cudaStream_t s)
 {
     for (int i = 0; i < 2; ++i) free_arena(w, i, s);
-    DevBuf *bufs[] = {&w.slots, &w.cslots, &w.cand, &w.res, &w.bcnt,    &w.bfill, &w.bptr,
-                      &w.bres,  &w.ctr,    &w.sortidx, &w.rcols, &w.perm, &w.fkb,
-                      &w.lx,    &w.lscore, &w.lhist,   &w.lerr, &w.band, &w.fp, &w.slow, &w.wrec,
-                      &w.ccnt,  &w.cfill,  &w.cptr,    &w.cne,  &w.csingle, &w.cent, &w.cells, &w.ksig};
+    DevBuf *bufs[] = {&w.live, &w.slots, &w.cslots, &w.cand, &w.res,   &w.bcnt,   &w.ctr,  &w.sortidx, &w.rcols, &w.perm,
+                      &w.fkb,  &w.lx,    &w.lscore, &w.lhist, &w.lerr, &w.fp, &w.open, &w.cells, &w.cent, &w.ksig, &w.csingle};
     for (DevBuf *b : bufs) dev_free(*b, s);
     for (auto &e : w.ev)
         if (e) cudaEventDestroy(e);
 }
 
-// Arena i with room for `rows` states and, sparse states, `units` payload
-// units (contents are not kept).
-bool alloc_arena(Work &w, const NetView &nv, int i, int64_t rows, uint64_t units, cudaStream_t s)
+// Arena i with room for `rows` states and `units` payload units (contents
+// are not kept).
+bool alloc_arena(Work &w, int i, int64_t rows, uint64_t units, cudaStream_t s)
 {
     free_arena(w, i, s);
     const size_t F = (size_t)rows;
-    if (w.sparse) {
-        units = std::min<uint64_t>(units, 0xFFFFFFFFull);  // a header's offset has 32 bits
-        if (!dev_alloc(w.hdr[i], F * 16, s) || !dev_alloc(w.pay[i], units * 16, s) || !dev_alloc(w.live[i], F * 4, s))
-            return false;
-        w.rows[i] = rows;
-        w.pay_cap[i] = units;
-        return true;
-    }
-    bool ok = dev_alloc(w.U[i], F * nv.W * 8, s) && dev_alloc(w.B[i], F * nv.Mpad * 4, s) &&
-              dev_alloc(w.meta[i], F * 4, s) && dev_alloc(w.live[i], F * 4, s);
-    if (ok && nv.narrow) ok = dev_alloc(w.sum[i], F * kSumWords * 8, s);
-    if (ok) w.rows[i] = rows;
-    return ok;
+    units = std::min<uint64_t>(units, 0xFFFFFFFFull);  // a header's offset has 32 bits
+    if (!dev_alloc(w.hdr[i], F * 16, s) || !dev_alloc(w.pay[i], units * 16, s)) return false;
+    w.rows[i] = rows;
+    w.pay_cap[i] = units;
+    return true;
 }
 
 // The level's fingerprint array and state hash table hold `reserved` rows.
@@ -367,9 +346,9 @@ bool ensure_level_tables(Work &w, uint64_t reserved, cudaStream_t s)
 {
     if ((int64_t)reserved > w.fp_cap) {
         dev_free(w.fp, s);
-        dev_free(w.wrec, s);
         const int64_t cap = std::max<int64_t>((int64_t)reserved, w.fp_cap + w.fp_cap / 2);
-        if (!dev_alloc(w.fp, (size_t)cap * 8, s) || (!w.sparse && !dev_alloc(w.wrec, (size_t)cap * 16, s))) return false;
+        dev_free(w.open, s);
+        if (!dev_alloc(w.fp, (size_t)cap * 8, s) || !dev_alloc(w.open, (size_t)cap * 4, s)) return false;
         w.fp_cap = cap;
     }
     const uint64_t need = next_pow2(2 * reserved + 64);
@@ -384,8 +363,7 @@ bool ensure_level_tables(Work &w, uint64_t reserved, cudaStream_t s)
 // CTAs of the expansion launches (kExpandWarps warps each)
 int level_grid(const NetView &nv, const efm_limits &lim, int sm_count)
 {
-    return nv.narrow ? generate_grid(nv, sm_count)
-                     : sparse_grid(lim.variant == EFM_SUBTRACTIVE, lim.first_k > 0, sm_count);
+    return generate_grid(nv, lim.variant == EFM_SUBTRACTIVE, lim.first_k > 0, sm_count);
 }
 
 // The static network a traversal reads: the subtractive variant's rows
@@ -400,39 +378,28 @@ int alloc_work(Work &w, const efm_net *net, const efm_limits &lim, int total_war
     const NetView &nv = view_of(net, lim);
     const int64_t default_cap = (int64_t)1 << 22;
     // a level writes a row for every surviving child before deduplication,
-    // so an arena gets room for a budget-sized frontier plus duplicates and
-    // the rows warps reserve but leave unused; a level that needs more is
-    // run again with a larger arena
+    // so an arena gets room for a budget-sized frontier plus duplicates; a
+    // level that needs more (rows, or payload units) is run again with a
+    // larger arena.  Units: what a state of these networks takes and half as
+    // much again, and never less than every seed takes
     w.F_cap = lim.max_frontier > 0 ? lim.max_frontier + 1 : default_cap;
-    w.sparse = !nv.narrow;
-    const int64_t rows = w.F_cap + w.F_cap / 8 + (w.sparse ? 1024 : 32 * (int64_t)total_warps);
-    // sparse states: 256 bytes of payload a row (a level that needs more is
-    // run again with a larger pool), and never less than every seed takes
-    // (the subtractive variant's states also hold their flux vector: 384)
-    const uint64_t units = std::max<uint64_t>((uint64_t)rows * (lim.variant == EFM_SUBTRACTIVE ? 24 : 16), (uint64_t)(nv.o_consptr - nv.o_colent) +
-                                                                       4ull * (uint64_t)nv.N + 1024);
+    const int64_t rows = w.F_cap + w.F_cap / 8 + 1024;
+    const int per_row = lim.variant == EFM_SUBTRACTIVE ? 24 : (nv.form == 2 ? 10 : 16);
+    const uint64_t units = std::max<uint64_t>((uint64_t)rows * per_row, (uint64_t)(nv.o_consptr - nv.o_colent) +
+                                                                            4ull * (uint64_t)nv.N + 1024);
     w.cand_cap = (int64_t)1 << 20;
     w.res_cap = w.cand_cap;
     w.cslot_cap = next_pow2(2 * (uint64_t)w.cand_cap);
     const size_t W = (size_t)nv.W;
-    bool ok = alloc_arena(w, nv, 0, rows, units, s) && alloc_arena(w, nv, 1, rows, units, s);
+    bool ok = alloc_arena(w, 0, rows, units, s) && alloc_arena(w, 1, rows, units, s);
     ok = ok && ensure_level_tables(w, 1024 + 32 * (uint64_t)total_warps, s);
     ok = ok && dev_alloc(w.cslots, w.cslot_cap * 8, s);
     ok = ok && dev_alloc(w.cand, (size_t)w.cand_cap * W * 8, s);
     ok = ok && dev_alloc(w.res, (size_t)w.res_cap * W * 8, s);
     ok = ok && dev_alloc(w.bcnt, (size_t)nv.N * 4, s);
-    ok = ok && dev_alloc(w.bfill, (size_t)nv.N * 4, s);
-    ok = ok && dev_alloc(w.bptr, (size_t)(nv.N + 1) * 4, s);
     ok = ok && dev_alloc(w.ctr, C_COUNT * 8, s);
-    if (nv.W > 2 || w.sparse) ok = ok && dev_alloc(w.rcols, (size_t)w.res_cap * kRcolStride * 2, s);
-    if (w.sparse) {
-        ok = ok && dev_alloc(w.ksig, (size_t)nv.N * 8, s) && dev_alloc(w.csingle, (size_t)nv.N * 4, s);
-    } else if (nv.W <= 2) {
-        const size_t cells = (size_t)nv.N * nv.N;
-        ok = ok && dev_alloc(w.band, (size_t)nv.N * nv.W * 8, s) && dev_alloc(w.ccnt, cells * 4, s) &&
-             dev_alloc(w.cfill, cells * 4, s) && dev_alloc(w.cptr, (cells + 1) * 4, s) &&
-             dev_alloc(w.cne, (size_t)nv.N * nv.W * 8, s) && dev_alloc(w.csingle, (size_t)nv.N * 4, s);
-    }
+    if (nv.W > 2) ok = ok && dev_alloc(w.rcols, (size_t)w.res_cap * kRcolStride * 2, s);
+    ok = ok && dev_alloc(w.ksig, (size_t)nv.N * 16, s) && dev_alloc(w.csingle, (size_t)nv.N * 4, s);
     if (lim.first_k > 0) ok = ok && dev_alloc(w.fkb, W * 8, s);
     for (auto &e : w.ev) ok = ok && cudaEventCreate(&e) == cudaSuccess;
     if (!ok) {
@@ -546,10 +513,8 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
 {
     const NetView &nv = view_of(net, lim);
     cudaStream_t s = net->stream;
-    const bool sparse = w.sparse;
     const int grid = level_grid(nv, lim, net->sm_count);
     const int total_warps = grid * kExpandWarps;
-    const int NG = 32 / std::min(32, std::max(4, 4 * nv.EPL));  // children per warp round
     unsigned long long *ctr = (unsigned long long *)w.ctr.p;
     unsigned long long h[C_COUNT];
     efm_counters &c = out.ctr;
@@ -561,11 +526,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
     a.cand = (uint64_t *)w.cand.p;
     a.cand_cap = w.cand_cap;
     a.res = (const uint64_t *)w.res.p;
-    a.bptr = (const int32_t *)w.bptr.p;
-    a.bres = nullptr;
-    a.bids = nullptr;
     a.rcols = (const uint16_t *)w.rcols.p;
-    a.band = nv.W <= 2 ? (const uint64_t *)w.band.p : nullptr;
     a.max_len = lim.max_len;
     a.max_sec = lim.max_secondary;
     a.ctr = ctr;
@@ -573,12 +534,8 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
     a.cap_dead = lim.first_k > 0 ? 1 : 0;
     auto arena = [&](int i) {
         Arena r{};
-        r.U = (uint64_t *)w.U[i].p;
-        r.B = (int32_t *)w.B[i].p;
-        r.meta = (uint32_t *)w.meta[i].p;
-        r.cap = w.rows[i];
-        r.sum = (uint64_t *)w.sum[i].p;
         r.hdr = (uint4 *)w.hdr[i].p;
+        r.cap = w.rows[i];
         r.pay = (uint4 *)w.pay[i].p;
         r.pay_cap = w.pay_cap[i];
         return r;
@@ -586,7 +543,6 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
 
     CK(cudaMemsetAsync(ctr, 0, C_COUNT * 8, s));
     CK(cudaMemsetAsync(w.cslots.p, 0xFF, w.cslot_cap * 8, s));
-    CK(cudaMemsetAsync(w.bptr.p, 0, (size_t)(nv.N + 1) * 4, s));
     CK(cudaEventRecord(w.ev[0], s));
 
     // level 0: seeds (or the seed set's one state, at level |R_in| - 1),
@@ -598,9 +554,9 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
     if (fs) {
         // the first parents are the caller's rows: nothing to seed
     } else if (seedset) {
-        CK(sparse ? launch_seedset_sparse(nv, a, seedset, n_seedset, s) : launch_seedset(nv, a, seedset, n_seedset, s));
+        CK(launch_seedset(nv, a, seedset, n_seedset, s));
     } else {
-        CK(sparse ? launch_seed_sparse(nv, a, target, s) : launch_seed(nv, a, target, s));
+        CK(launch_seed(nv, a, target, s));
     }
     out.kernel_launches += fs ? 0 : 1;
     AcceptArgs acc{};
@@ -646,7 +602,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
     }
     int64_t n_front = fs ? fs->r1 - fs->r0 : (int64_t)h[C_NEXT];  // distinct states of the level
     int64_t n_rows = n_front;              // arena rows the next level reads (seeds are dense)
-    double row_units = 0.0;                // sparse states: payload units of the level's rows
+    double row_units = 0.0;                // payload units of the level's rows
     uint64_t deg_sum = fs ? fs->deg_sum : h[C_DEGSUM];
     int status = 0;
     bool split = false;  // the K smallest come from the parts of a split level (top)
@@ -665,72 +621,52 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             stop = true;
         }
     }
-    int64_t buckets_built_for = 0;
+    int64_t indexed = 0, index_room = 0;  // results in the superset rule's index; entries it has room for
     float ms = 0.f;
     for (int level = level0 + 1; !stop && n_front > 0; ++level) {
         // every step adds a column or a secondary step, so depth is bounded
         if (level > lim.max_len + lim.max_secondary + 1) return EFM_ETIMEOUT;
-        // buckets over every accepted result so far (all of them come from levels < `level`)
-        if (res_n != buckets_built_for && sparse) {
-            const int64_t need = std::max<int64_t>(res_n * (int64_t)lim.max_len, 1);
-            if (need > w.bres_cap) {
+        // the superset rule's index over every accepted result so far (all of them come from levels < `level`);
+        // the table has room for twice the entries filed, and grows by filing every result again
+        if (res_n != indexed) {
+            const int64_t need = std::max<int64_t>(res_n * (int64_t)lim.max_len, 1);  // entries: sum of |E|
+            if (need > w.cent_cap) {
                 dev_free(w.cent, s);
                 dev_free(w.cells, s);
-                const int64_t cap = std::max<int64_t>(std::max<int64_t>(need, 2 * w.bres_cap), 4096);
-                w.cell_cap = next_pow2(2 * (uint64_t)cap);
-                if (!dev_alloc(w.cent, (size_t)cap * 16, s) || !dev_alloc(w.cells, w.cell_cap * 8, s)) return EFM_ENOMEM;
-                w.bres_cap = cap;
+                const int64_t cap = std::max<int64_t>(std::max<int64_t>(need, 2 * w.cent_cap), 4096);
+                if (!dev_alloc(w.cent, (size_t)cap * (nv.W <= 2 ? 32 : 16), s) ||
+                    !dev_alloc(w.cells, cell_table_bytes(nv, (uint64_t)cap), s))
+                    return EFM_ENOMEM;
+                w.cent_cap = cap;
+                index_room = 0;
             }
             CellIndex &ix = a.cells;
-            ix.cells = (uint2 *)w.cells.p;
-            ix.mask = (uint32_t)std::min<uint64_t>(w.cell_cap, next_pow2(2 * (uint64_t)need)) - 1u;
-            ix.ent = (uint4 *)w.cent.p;
-            ix.ksig = (uint64_t *)w.ksig.p;
-            ix.single = (uint32_t *)w.csingle.p;
+            if (indexed == 0 || need > index_room) {
+                index_room = std::min<int64_t>(w.cent_cap, 4 * need);
+                ix.cells = (uint2 *)w.cells.p;
+                ix.mask = nv.W <= 2 ? 0u : (uint32_t)(cell_table_bytes(nv, (uint64_t)index_room) / 8 - 1);
+                ix.ent = (uint4 *)w.cent.p;
+                ix.ksig = (uint64_t *)w.ksig.p;
+                ix.single = (uint32_t *)w.csingle.p;
+                indexed = 0;
+            }
             ix.n_res = res_n;
-            CK(launch_cells(nv, (const uint16_t *)w.rcols.p, res_n, (int32_t *)w.bcnt.p, ix, lim.max_len, s));
+            CK(launch_cells(nv, (const uint64_t *)w.res.p, indexed, res_n, (int32_t *)w.bcnt.p, ix, lim.max_len, s));
             out.kernel_launches += 2;
-            buckets_built_for = res_n;
-        }
-        if (res_n != buckets_built_for) {
-            // bucket entries needed: sum of |E| <= res_n * max_len (grown on demand)
-            const int64_t need = std::max<int64_t>(res_n * (int64_t)lim.max_len, 1);
-            if (need > w.bres_cap) {
-                dev_free(w.bres, s);
-                dev_free(w.cent, s);
-                const int64_t cap = std::max<int64_t>(need, 2 * w.bres_cap);
-                if (!dev_alloc(w.bres, (size_t)cap * nv.W * 8, s)) return EFM_ENOMEM;
-                if (nv.W <= 2 && !dev_alloc(w.cent, (size_t)cap * nv.W * 8, s)) return EFM_ENOMEM;
-                w.bres_cap = cap;
-            }
-            a.bres = (const uint64_t *)w.bres.p;
-            a.bids = (const int32_t *)w.bres.p;
-            CK(launch_buckets(nv, (const uint64_t *)w.res.p, res_n, (int32_t *)w.bcnt.p, (int32_t *)w.bptr.p,
-                              (int32_t *)w.bfill.p, (uint64_t *)w.bres.p, (uint64_t *)w.band.p, s));
-            if (nv.W <= 2) {
-                CK(launch_sentinel_index(nv, (const uint64_t *)w.res.p, res_n, (const int32_t *)w.bcnt.p,
-                                         (int32_t *)w.ccnt.p, (int32_t *)w.cfill.p, (int32_t *)w.cptr.p,
-                                         (uint64_t *)w.cent.p, (uint64_t *)w.cne.p, (uint32_t *)w.csingle.p, s));
-                a.cptr = (const int32_t *)w.cptr.p;
-                a.cent = (const uint64_t *)w.cent.p;
-                a.cne = (const uint64_t *)w.cne.p;
-                a.csingle = (const uint32_t *)w.csingle.p;
-                out.kernel_launches += res_n > 0 ? 4 : 2;
-            }
-            out.kernel_launches += res_n > 0 ? 3 : 1;
-            buckets_built_for = res_n;
+            indexed = res_n;
         }
         if (trace && n_front > 0) {
             // training rows: a strided sample of this frontier (level - 1),
             // through the list of its surviving rows
             unsigned long long n_live = 0;
             CK(cudaMemsetAsync(ctr + C_LIVE, 0, 8, s));
-            if (sparse)
-                CK(launch_live_sparse((const uint4 *)w.hdr[cur].p, n_rows, (uint32_t *)w.live[cur].p, ctr + C_LIVE,
-                                      net->sm_count, s));
-            else
-                CK(launch_live_list((const uint32_t *)w.meta[cur].p, n_rows, (uint32_t *)w.live[cur].p, ctr + C_LIVE,
-                                    net->sm_count, s));
+            if (n_rows > w.live_cap) {
+                dev_free(w.live, s);
+                const int64_t cap = std::max<int64_t>(n_rows, 2 * w.live_cap);
+                if (!dev_alloc(w.live, (size_t)cap * 4, s)) return EFM_ENOMEM;
+                w.live_cap = cap;
+            }
+            CK(launch_live_list((const uint4 *)w.hdr[cur].p, n_rows, (uint32_t *)w.live.p, ctr + C_LIVE, net->sm_count, s));
             CK(cudaMemcpyAsync(&n_live, ctr + C_LIVE, 8, cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
             const int64_t nl = (int64_t)n_live;
@@ -739,7 +675,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             efm_model *m = trace->m;
             if (!model_reserve_rows(m, m->n_rows + cnt)) return EFM_ENOMEM;
             if ((rc = ensure_dep_tags(net))) return rc;
-            const uint32_t *live = (const uint32_t *)w.live[cur].p;
+            const uint32_t *live = (const uint32_t *)w.live.p;
             CK(launch_features(nv, arena(cur), live, 0, stride, cnt, level - 1, lim.max_len, lim.max_secondary,
                                (const uint64_t *)net->dep.p, m->X.p, m->n_rows, s));
             CK(launch_labels(arena(cur), nv.W, live, 0, stride, cnt, trace->ans, trace->n_ans,
@@ -789,32 +725,15 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                 out.kernel_launches += 6;
             }
         }
-        // rows one warp reserves at a time: few for small or chunked levels
-        // (a warp's unused reserved rows at the end of every launch are dead
-        // weight in the arena), 32 for large ones
+        // rows and payload units one warp reserves at a time: at large levels
+        // about a 16th of what it writes (what stays unused is dead weight in
+        // the arena), else exactly what a round needs
         const int64_t launches = (n_rows + chunk - 1) / chunk;
-        // (sparse states: exactly what a round needs, and at large levels about
-        // a 16th of what a warp writes)
-        int blk = launches > 1 ? NG
-                               : (int)std::min<uint64_t>(32, std::max<uint64_t>((uint64_t)NG,
-                                                                                deg_sum / (64ull * total_warps)));
-        a.pay_blk = 0;
-        if (sparse) {
-            blk = launches > 1 ? 0 : (int)std::min<uint64_t>(512, deg_sum / (16ull * total_warps));
-            if (blk < 32) blk = 0;
-            const double avg = n_rows > 0 && row_units > 0.0 ? row_units / (double)n_rows : 8.0;
-            a.pay_blk = (int)(blk * (avg + 1.0));
-        }
+        int blk = launches > 1 ? 0 : (int)std::min<uint64_t>(512, deg_sum / (16ull * total_warps));
+        if (blk < 32) blk = 0;
+        const double avg_units = n_rows > 0 && row_units > 0.0 ? row_units / (double)n_rows : 8.0;
         const uint64_t reserved = deg_sum + (uint64_t)launches * blk * total_warps + 64;
         if (!ensure_level_tables(w, reserved, s)) return EFM_ENOMEM;
-        // narrow networks: room for every child of a launch in the settle list
-        const int64_t slow_need = (int64_t)deg_sum + 32 * (int64_t)total_warps + 64;  // + unused pool slots
-        if (nv.narrow && slow_need > w.slow_cap) {
-            dev_free(w.slow, s);
-            const int64_t cap = std::max<int64_t>(slow_need, w.slow_cap + w.slow_cap / 2);
-            if (!dev_alloc(w.slow, (size_t)cap * kSlowWords * 8, s)) return EFM_ENOMEM;
-            w.slow_cap = cap;
-        }
         const uint64_t nslots = next_pow2(2 * reserved + 64);
         unsigned long long snap[C_COUNT];
         memcpy(snap, h, sizeof(h));
@@ -827,18 +746,17 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             CK(cudaMemsetAsync(ctr + C_NEXT, 0, 2 * 8, s));
             CK(cudaMemsetAsync(ctr + C_WRITTEN, 0, 3 * 8, s));
             CK(cudaMemsetAsync(ctr + C_DEDUP_BEGIN, 0, 8, s));
-            if (sparse) CK(cudaMemsetAsync(ctr + C_PAY, 0, 8, s));
+            CK(cudaMemsetAsync(ctr + C_PAY, 0, 8, s));
+            CK(cudaMemsetAsync(ctr + C_OPEN, 0, 8, s));
             a.par = ext ? fs->par : arena(cur);
             a.child = arena(cur ^ 1);
-            a.live = (uint32_t *)w.live[cur ^ 1].p;
             a.slots = (unsigned long long *)w.slots.p;
             a.slot_mask = nslots - 1;
             a.fp = (uint64_t *)w.fp.p;
             a.fp_cap = w.fp_cap;
-            a.wrec = (uint4 *)w.wrec.p;
+            a.open = (uint32_t *)w.open.p;
             a.blk = blk;
-            a.slow = nv.narrow ? (uint64_t *)w.slow.p : nullptr;
-            a.slow_cap = nv.narrow ? w.slow_cap : 0;
+            a.pay_blk = (int)(blk * (avg_units + 1.0));
             a.level = level;
             unsigned long long exp_before = h[C_EXP];
             uint64_t next_before = 0;
@@ -852,17 +770,8 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                 a.fk_sup = (const uint64_t *)w.fkb.p;
                 a.max_len = (fk && top.pc > 0) ? std::min(lim.max_len, top.pc) : lim.max_len;
                 CK(cudaEventRecord(w.ev[2], s));
-                if (sparse) {
-                    CK(launch_generate_sparse(nv, a, grid, s));
-                    CK(launch_dedup_sparse(a, net->sm_count, s));
-                } else {
-                    CK(cudaMemsetAsync(ctr + C_SLOW, 0, 8, s));
-                    CK(launch_generate(nv, a, grid, s));
-                    CK(launch_prune_rows(nv, a, net->sm_count, s));
-                    CK(launch_write_rows(nv, a, net->sm_count, s));
-                    CK(launch_settle(nv, a, net->sm_count, s));
-                    CK(launch_dedup(a, nv.Mpad, nv.W, net->sm_count, s));
-                }
+                CK(launch_generate(nv, a, grid, s));
+                CK(launch_dedup(nv, a, net->sm_count, s));
                 CK(cudaEventRecord(w.ev[3], s));
                 // minimality test of the new candidates, range taken on the device
                 CK(launch_accept_new(nv, acc, net->sm_count, s));
@@ -876,14 +785,12 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                 CK(cudaEventElapsedTime(&ms, w.ev[2], w.ev[3]));
                 out.expand_ms += ms;
                 out.expand_launches += 1;
-                out.kernel_launches += sparse ? 5 : (nv.W <= 2 && a.cptr ? 8 : 7);
+                out.kernel_launches += 5;
                 {
-                    // sparse states: a header and the payload units of an average row of the level
-                    const double par_bytes = !sparse ? 8.0 * nv.W + 4.0 * nv.M + 4.0
-                                                     : 16.0 + 16.0 * row_units / (double)std::max<int64_t>(n_rows, 1);
-                    const double new_bytes = !sparse ? par_bytes
-                                                     : 16.0 + 16.0 * (double)h[C_PAY] /
-                                                                  (double)std::max<unsigned long long>(h[C_WRITTEN], 1);
+                    // a header and the payload units of an average row of the level
+                    const double par_bytes = 16.0 + 16.0 * row_units / (double)std::max<int64_t>(n_rows, 1);
+                    const double new_bytes =
+                        16.0 + 16.0 * (double)h[C_PAY] / (double)std::max<unsigned long long>(h[C_WRITTEN], 1);
                     const uint64_t next_now = h[C_NEXT];
                     const double n_new = (double)(next_now - next_before);
                     const double n_child = (double)(h[C_EXP] - exp_before);
@@ -894,10 +801,10 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                     out.expand_bytes += bytes;
                     if (getenv("EFM_DEBUG"))
                         fprintf(stderr,
-                                "efm: level %d parents %lld items %llu children %.0f new %.0f rows %llu settled %llu "
+                                "efm: level %d parents %lld items %llu children %.0f new %.0f rows %llu units %llu "
                                 "pruned %llu bytes %.0f ms %.3f\n",
                                 level, (long long)cn, (unsigned long long)(c0 == 0 && chunk >= n_rows ? deg_sum : 0),
-                                n_child, n_new, h[C_WRITTEN], h[C_SLOW], h[C_PRUNED],
+                                n_child, n_new, h[C_WRITTEN], h[C_PAY], h[C_PRUNED],
                                 bytes, ms);
                     exp_before = h[C_EXP];
                     next_before = next_now;
@@ -930,8 +837,8 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             // the level again (its balanced supports are already judged, so
             // only the per-child counters are rolled back)
             const uint64_t more = h[C_PAY] + h[C_PAY] / 8 + 1024;
-            if (sparse && more > 0xFFFFFFFFull) return EFM_ENOMEM;  // past a header's 32-bit offsets
-            if (!alloc_arena(w, nv, cur ^ 1,
+            if (more > 0xFFFFFFFFull) return EFM_ENOMEM;  // past a header's 32-bit offsets
+            if (!alloc_arena(w, cur ^ 1,
                              std::max<int64_t>((int64_t)h[C_WRITTEN] + (int64_t)h[C_WRITTEN] / 8 + 1024,
                                                w.rows[cur ^ 1]),
                              std::max<uint64_t>(more, w.pay_cap[cur ^ 1]), s))
@@ -1042,16 +949,14 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         const uint64_t n2 = next_pow2((uint64_t)std::max<int64_t>(res_n, 1));
         if (n2 > w.sort_cap) {
             dev_free(w.sortidx, s);
-            if (!dev_alloc(w.sortidx, n2 * 4, s)) return EFM_ENOMEM;
+            if (!dev_alloc(w.sortidx, sort_scratch_bytes((int64_t)n2), s)) return EFM_ENOMEM;
             w.sort_cap = n2;
         }
         if (!dev_alloc(out.sup, (size_t)std::max<int64_t>(n_keep, 1) * nv.W * 8, s)) return EFM_ENOMEM;
-        CK(launch_sort_results((const uint64_t *)w.res.p, res_n, nv.W, (uint32_t *)w.sortidx.p, (int64_t)n2,
+        CK(launch_sort_results((const uint64_t *)w.res.p, res_n, nv.W, w.sortidx.p, (int64_t)n2,
                                (uint64_t *)out.sup.p, n_keep, s));
         if (res_n > 0 && n_keep > 0) {
-            int lg = 0;
-            while ((1ull << lg) < n2) ++lg;
-            out.kernel_launches += 2 + (int64_t)lg * (lg + 1) / 2;
+            out.kernel_launches += sort_launches((int64_t)n2);
         }
     }
     CK(cudaEventRecord(w.ev[1], s));
@@ -1388,9 +1293,9 @@ extern "C" int efm_sample_pathways(efm_net *net, int32_t target, const efm_limit
     if ((int64_t)h[C_RES_N] > w.res_cap) return fail(EFM_ECAPACITY);
     const int64_t res_n = (int64_t)h[C_RES_N];
     const uint64_t n2 = next_pow2((uint64_t)std::max<int64_t>(res_n, 1));
-    if (!dev_alloc(w.sortidx, n2 * 4, s) || !dev_alloc(o.sup, (size_t)std::max<int64_t>(res_n, 1) * nv.W * 8, s))
+    if (!dev_alloc(w.sortidx, sort_scratch_bytes((int64_t)n2), s) || !dev_alloc(o.sup, (size_t)std::max<int64_t>(res_n, 1) * nv.W * 8, s))
         return fail(EFM_ENOMEM);
-    if (launch_sort_results((const uint64_t *)w.res.p, res_n, nv.W, (uint32_t *)w.sortidx.p, (int64_t)n2,
+    if (launch_sort_results((const uint64_t *)w.res.p, res_n, nv.W, w.sortidx.p, (int64_t)n2,
                             (uint64_t *)o.sup.p, res_n, s) != cudaSuccess ||
         cudaEventRecord(w.ev[1], s) != cudaSuccess || cudaEventSynchronize(w.ev[1]) != cudaSuccess)
         return fail(EFM_ECUDA);

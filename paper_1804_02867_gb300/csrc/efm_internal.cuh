@@ -43,7 +43,7 @@ enum {
     C_DEDUP_BEGIN,  // first reserved row the next dedup launch examines
     C_DIAG = 24,  // first bounds/watchdog record: code, value, limit, level
     C_ZERO = 28,  // subtractive steps discarded: no positive flux left on the reaction (Prop. 3)
-    C_SLOW,       // narrow networks: children handed to the settle pass in this launch
+    C_OPEN,       // open children listed by the generate pass, not yet finished
     C_LIVE,       // surviving rows counted by the live-list pass
     C_CAPDEAD,    // unused
     C_PAY,        // sparse states: payload units reserved so far in the level
@@ -64,12 +64,15 @@ struct NetView {
     int o_keypos, o_keyneg;    // per internal row: (degree << 16) | row
     int o_hbits;               // per column: ceil(log2(|S_int[:,k]|^2))
     int o_dcols;               // dense S_int by column: N rows of Mpad int32 (16-byte aligned)
-    // narrow networks (M <= 64): state summary tables (see efm_netprep.h)
-    int narrow;
-    int o_rank;                // per row: rank in the positive key order | rank in the negative << 8
-    int o_keyr;                // per rank: positive key [64], then negative key [64]
-    int o_hrow;                // per row: 64-bit row hash constant R[m]
-    int o_colx;                // per column: suppP, suppN, suppR, HC (u64 each), smax, gcd1 (10 words)
+    // per column, 8 words (16-byte aligned): HC = sum_m S_int[m][k] R[m] (2 words, R: the row
+    // hash constants), mask of its rows modulo 64 (2), max |S_int[m][k]|, its range of words
+    // in colent (2), its twin column or ~0
+    int o_scol;
+    // how the level pass keeps a state: 2 = narrow (at most 64 internal rows and 128 columns:
+    // masks and the values in row order), 1 = bitset support and a list of entries (at most 128
+    // columns), 0 = column list and a list of entries
+    int form;
+    int o_rank, o_keyr, o_colx, o_nent;  // narrow: see efm_netprep.h
     const int32_t *metptr;     // full S rows over split columns (seeds), [n_met + 1]
     const uint32_t *metent;    // packed (column, coefficient)
     int n_met;
@@ -78,46 +81,42 @@ struct NetView {
 __host__ __device__ inline int ent_index(uint32_t e) { return (int)(e >> 20); }
 __host__ __device__ inline int32_t ent_coef(uint32_t e) { return ((int32_t)(e << 12)) >> 12; }
 
-// One arena of pathway states, structure of arrays.
+// One arena of pathway states.  The level pass keeps headers and a
+// payload pool (layout in efm_sparse.cu); the batched traversal keeps dense
+// rows: support words, extra-flux row, meta word.
 struct Arena {
+    uint4 *hdr;         // [cap]
+    uint4 *pay;         // [pay_cap] 16-byte units
+    uint64_t pay_cap;
     uint64_t *U;     // [cap][W]
     int32_t *B;      // [cap][Mpad]
     uint32_t *meta;  // [cap]: pivot row | pivot degree << 10 | |U| << 23
     int64_t cap;
-    // narrow networks: per-state summaries of the extra-flux row EF, kSumWords each
-    //   sum[6 s + 0] = sum_m EF_m R[m] (mod 2^64), the linear row hash
-    //   sum[6 s + 1] = positive entries, bit = rank of the row in the positive key order
-    //   sum[6 s + 2] = negative entries, bit = rank of the row in the negative key order
-    //   sum[6 s + 3] = rows with |EF_m| = 1
-    //   sum[6 s + 4] = rows with odd EF_m
-    //   sum[6 s + 5] = an upper bound of max_m |EF_m| (saturating at 2^31 - 1)
-    uint64_t *sum;
-    // sparse states (every network but the narrow ones, and the subtractive
-    // variant; layout in efm_sparse.cu): headers per row, payload pool
-    uint4 *hdr;         // [cap]
-    uint4 *pay;         // [pay_cap] 16-byte units
-    uint64_t pay_cap;
 };
 
-// Sparse states: payload units of the column list (an 8-byte hash in front)
-__host__ __device__ inline int sparse_list_units(int pc) { return (8 + 2 * pc + 15) >> 4; }
+// Payload units of a state's hashes and column list
+__host__ __device__ inline int sparse_list_units(int pc) { return 1 + ((pc + 7) >> 3); }
 
-// Sparse states: the superset rule's index.  A result E is filed, for each of
-// its columns k, in cell (k, s) where s is E's other column with the fewest
-// results (its sentinel): a child adding k contains E only if it holds s, so
-// it looks up the cells (k, s) of its own columns s and no others.  Cells sit
-// in a hash table (key k << 12 | s, head of a list); an entry holds a 64-bit
-// signature of E's columns, the next entry and the result's id.
+// The superset rule's index.  A result E is filed, for each of its columns k,
+// in cell (k, s) where s is E's other column with the fewest results (its
+// sentinel): a child adding k contains E only if it holds s, so it looks up
+// the cells (k, s) of its own columns s and no others.  A cell is the head of
+// a list of entries.
+//   at most 128 columns: cells is a table of heads, [N][128]; ksig holds two
+//     words a column, bit s set when cell (k, s) is not empty; an entry is two
+//     units: E's words; (next, result)
+//   else: cells is a hash table of (k << 12 | s, head); ksig holds one word a
+//     column, a signature of its sentinels; an entry is one unit: a signature
+//     of E's columns, next, result
+// Empty keys, heads and ends of lists are ~0.
 struct CellIndex {
-    uint2 *cells;       // [mask + 1], empty: key ~0
-    uint32_t mask;
+    uint2 *cells;
+    uint32_t mask;      // hash table: slots - 1
     uint4 *ent;
-    uint64_t *ksig;     // [N]: signature of the sentinels s with a cell (k, s)
+    uint64_t *ksig;
     uint32_t *single;   // [N]: 1 if {k} itself is a result
     int64_t n_res;      // results filed (0: no index)
 };
-
-constexpr int kSumWords = 6;
 
 struct LevelArgs {
     Arena par;
@@ -135,15 +134,7 @@ struct LevelArgs {
     const int32_t *bids;        // bucket entries: result ids (W > 2), same buffer as bres
     const uint16_t *rcols;      // per result: column count, then its columns (stride kRcolStride)
     const uint64_t *band;       // W <= 2: per column, the intersection of the results containing it (or null)
-    // W <= 2: the superset rule's index.  A result E is filed, for each of its
-    // columns k, in cell (k, s) where s is E's other column with the fewest
-    // results (its sentinel); a child adding k scans only the cells whose
-    // sentinel lies in its support.  Null: the buckets above.
-    const int32_t *cptr;        // [N * N + 1] cell offsets into cent
-    const uint64_t *cent;       // cell entries: the result's W support words
-    const uint64_t *cne;        // [N][W]: sentinels with a non-empty cell (k, s)
-    const uint32_t *csingle;    // [N]: 1 if {k} itself is a result
-    CellIndex cells;            // sparse states
+    CellIndex cells;            // the level pass
     int level, max_len, max_sec;
     int cpw;                    // parents per warp chunk (1..32)
     unsigned long long *ctr;
@@ -159,31 +150,20 @@ struct LevelArgs {
     // a reserved row and a fingerprint; the dedup pass keeps one per state
     uint64_t *fp;               // [fp_cap] fingerprint per reserved row (kDeadFp: unused)
     int64_t fp_cap;
-    uint32_t *live;             // unused by the kernels (kept for the host's bookkeeping)
-    int blk;                    // rows a warp reserves at a time (sparse states: at least a round's)
-    int pay_blk;                // sparse states: payload units a warp reserves at a time, at least a round's
-    // subtractive variant (Eq. 5): rows hold the extra flux (M entries), then
-    // the flux of every column; a state's branches also take flux away from
-    // a column in U, and its meta degree counts both lists of the pivot
+    uint32_t *open;             // [fp_cap] rows of the open children
+    int blk;                    // rows a warp reserves at a time, at least a round's
+    int pay_blk;                // payload units a warp reserves at a time, at least a round's
+    // subtractive variant (Eq. 5): states also hold the flux of their columns,
+    // a state's branches also take flux away from a column in U, and its meta
+    // degree counts both lists of the pivot
     int sub;
-    // narrow networks: children whose gcd or int32 range is not settled by
-    // the summaries, kSlowWords words each, for the settle pass
-    uint64_t *slow;
-    int64_t slow_cap;
-    // narrow networks: per reserved row, the row writer's record (parent row,
-    // column | flags | |U| << 14, A, C); x = kNoRecord: nothing to write
-    uint4 *wrec;
 };
 
 constexpr uint32_t kNoRecord = 0xFFFFFFFFu;
 
-constexpr int kSlowWords = 8;
-
 constexpr unsigned long long kDeadFp = ~0ull;  // fingerprint of a reserved row left unused
 
 constexpr int kRcolStride = 65;  // column count + up to 64 columns per result
-constexpr int kNarrowKeyRanks = 64;  // narrow networks: keys per rank order (efm_netprep.h kNarrowRows)
-constexpr int kColxWordsDev = 10;    // narrow networks: per-column summary words (efm_netprep.h kColxWords)
 
 struct AcceptArgs {
     const uint64_t *cand;
@@ -266,51 +246,35 @@ cudaError_t launch_pack_rows(const float *x, int64_t n, void *X, int64_t row0, c
 size_t mlp_score_smem();
 size_t mlp_train_smem();
 
-// kernels (efm_kernels.cu)
+// kernels (efm_sparse.cu): the level pass
 cudaError_t launch_seed(const NetView &nv, const LevelArgs &a, int target, cudaStream_t s);
-// generate/dedup split of one expansion: children with rows and fingerprints,
-// then one pass that keeps the first row of every distinct state
+cudaError_t launch_seedset(const NetView &nv, const LevelArgs &a, const int32_t *cols, int n_cols, cudaStream_t s);
+// one expansion: children with rows, payloads and fingerprints, then one pass
+// that keeps the first row of every distinct state
+int generate_grid(const NetView &nv, bool sub, bool first_k, int sm_count);
 cudaError_t launch_generate(const NetView &nv, const LevelArgs &a, int grid, cudaStream_t s);
-cudaError_t launch_dedup(const LevelArgs &a, int Mpad, int W, int sm_count, cudaStream_t s);
-// narrow networks: settle the children the generate pass listed (exact gcd,
-// int32 range, superset rule), then write their rows; a no-op otherwise
-cudaError_t launch_settle(const NetView &nv, const LevelArgs &a, int sm_count, cudaStream_t s);
-// narrow networks: the superset rule over the generate pass's reserved rows
-cudaError_t launch_prune_rows(const NetView &nv, const LevelArgs &a, int sm_count, cudaStream_t s);
-// narrow networks: write the extra-flux rows of the generate pass's children
-cudaError_t launch_write_rows(const NetView &nv, const LevelArgs &a, int sm_count, cudaStream_t s);
+cudaError_t launch_dedup(const NetView &nv, const LevelArgs &a, int sm_count, cudaStream_t s);
+// the results [r0, r1) into the superset rule's index (r0 = 0: a new index); cnt: results per
+// column; entries of result r start at r * ent_stride
+size_t cell_table_bytes(const NetView &nv, uint64_t entries);
+cudaError_t launch_cells(const NetView &nv, const uint64_t *res, int64_t r0, int64_t r1, int32_t *cnt,
+                         const CellIndex &ix, int ent_stride, cudaStream_t s);
 // the surviving rows (meta != 0) of [0, n) appended to live; *count must be 0
-cudaError_t launch_live_list(const uint32_t *meta, int64_t n, uint32_t *live, unsigned long long *count,
-                             int sm_count, cudaStream_t s);
-int generate_grid(const NetView &nv, int sm_count);
-// kernels (efm_sparse.cu): the level pass on sparse states
-int sparse_grid(bool sub, bool first_k, int sm_count);
-cudaError_t launch_generate_sparse(const NetView &nv, const LevelArgs &a, int grid, cudaStream_t s);
-cudaError_t launch_dedup_sparse(const LevelArgs &a, int sm_count, cudaStream_t s);
-cudaError_t launch_seed_sparse(const NetView &nv, const LevelArgs &a, int target, cudaStream_t s);
-cudaError_t launch_seedset_sparse(const NetView &nv, const LevelArgs &a, const int32_t *cols, int n_cols,
-                                  cudaStream_t s);
-// the superset rule's index over results [0, n_res); entries of result r start at r * ent_stride
-cudaError_t launch_cells(const NetView &nv, const uint16_t *rcols, int64_t n_res, int32_t *cnt, const CellIndex &ix,
-                         int ent_stride, cudaStream_t s);
-cudaError_t launch_live_sparse(const uint4 *hdr, int64_t n, uint32_t *live, unsigned long long *count, int sm_count,
-                               cudaStream_t s);
+cudaError_t launch_live_list(const uint4 *hdr, int64_t n, uint32_t *live, unsigned long long *count, int sm_count,
+                             cudaStream_t s);
+// kernels (efm_kernels.cu)
 cudaError_t launch_accept(const NetView &nv, const AcceptArgs &a, cudaStream_t s);
 // minimality test of the candidates appended since the last such launch (range read on the
 // device, so no host round trip is needed between expansion and test); then advance the range
 cudaError_t launch_accept_new(const NetView &nv, const AcceptArgs &a, int sm_count, cudaStream_t s);
-cudaError_t launch_buckets(const NetView &nv, const uint64_t *res, int64_t n_res, int32_t *bcnt, int32_t *bptr,
-                           int32_t *bfill, uint64_t *bres, uint64_t *band,
-                           cudaStream_t s);  // W > 2: bres holds int32 ids; band (W <= 2, may be null)
-// W <= 2: the sentinel index of the superset rule over results [0, n_res)
-// (bcnt: results per column, from launch_buckets); ccnt/cfill: N*N scratch
-cudaError_t launch_sentinel_index(const NetView &nv, const uint64_t *res, int64_t n_res, const int32_t *bcnt,
-                                  int32_t *ccnt, int32_t *cfill, int32_t *cptr, uint64_t *cent, uint64_t *cne,
-                                  uint32_t *csingle, cudaStream_t s);
-cudaError_t launch_sort_results(const uint64_t *res, int64_t n, int W, uint32_t *idx, int64_t n_pow2,
-                                uint64_t *out, int64_t n_keep, cudaStream_t s);
-cudaError_t launch_iota(uint32_t *perm, int64_t n, cudaStream_t s);
-cudaError_t launch_seedset(const NetView &nv, const LevelArgs &a, const int32_t *cols, int n_cols, cudaStream_t s);
+// sort by (|U|, ascending columns); n2: n rounded up to a power of two; scratch: sort_scratch_bytes(n2)
+size_t sort_scratch_bytes(int64_t n2);
+int sort_launches(int64_t n2);
+cudaError_t launch_sort_results(const uint64_t *res, int64_t n, int W, void *scratch, int64_t n2, uint64_t *out,
+                                int64_t n_keep, cudaStream_t s);
+// the same with n2 indices (4 bytes each) as the only scratch
+cudaError_t launch_sort_index(const uint64_t *res, int64_t n, int W, uint32_t *idx, int64_t n2, uint64_t *out,
+                              int64_t n_keep, cudaStream_t s);
 cudaError_t launch_step_count(const NetView &nv, unsigned *r, cudaStream_t s);
 cudaError_t launch_or_words(uint64_t *a, const uint64_t *b, int64_t n, cudaStream_t s);
 cudaError_t launch_depthy(const NetView &nv, int L, unsigned r, unsigned long long n_paths, unsigned long long *dep_out,

@@ -39,68 +39,6 @@ __constant__ uint32_t c_prime_c[kNumPrimes] = {1,   19,  61,  69,  85,  99,  105
                                               295, 325, 379, 399, 411, 469, 477, 511, 525, 571, 579, 589};
 
 // ---------------------------------------------------------------------------
-// static network staging (a4): bulk async copy global -> shared, mbarrier
-// ---------------------------------------------------------------------------
-
-__device__ __forceinline__ uint32_t smem_addr(const void *p)
-{
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-// Returns the blob pointer to use (shared if staged, else global).  On a
-// wait that does not finish, flags ERR_TIMEOUT and returns nullptr.
-__device__ const uint32_t *stage_words(const NetView &nv, uint32_t *sblob, uint64_t *mbar, int w0, int nwords,
-                                       unsigned long long *ctr);
-
-__device__ const uint32_t *stage_blob(const NetView &nv, uint32_t *sblob, uint64_t *mbar, bool staged,
-                                      unsigned long long *ctr)
-{
-    if (!staged) return nv.blob;
-    return stage_words(nv, sblob, mbar, 0, nv.blob_words, ctr);
-}
-
-// words [w0, w0 + nwords) of the blob into shared memory (w0 and nwords
-// multiples of 4: 16-byte aligned bulk copies), one mbarrier, bounded wait
-__device__ const uint32_t *stage_words(const NetView &nv, uint32_t *sblob, uint64_t *mbar, int w0, int nwords,
-                                       unsigned long long *ctr)
-{
-    const uint32_t bytes = (uint32_t)nwords * 4u;
-    const uint32_t bar = smem_addr(mbar);
-    if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(1) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-        const uint32_t chunk = 32768u;
-        for (uint32_t off = 0; off < bytes; off += chunk) {
-            const uint32_t n = bytes - off < chunk ? bytes - off : chunk;
-            asm volatile(
-                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                    smem_addr(sblob) + off),
-                "l"((const char *)(nv.blob + w0) + off), "r"(n), "r"(bar)
-                : "memory");
-        }
-    }
-    uint32_t done = 0;
-    for (int spin = 0; spin < kSpinLimit && !done; ++spin) {
-        asm volatile(
-            "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-            : "=r"(done)
-            : "r"(bar), "r"(0)
-            : "memory");
-        if (!done) __nanosleep(256);
-    }
-    const int all_done = __syncthreads_and((int)done);
-    if (!all_done) {
-        if (threadIdx.x == 0) atomicOr(&ctr[C_ERR], (unsigned long long)ERR_TIMEOUT);
-        return nullptr;
-    }
-    return sblob;
-}
-
-// ---------------------------------------------------------------------------
 // hash sets (publish-after-write slots)
 //
 // A slot is one 64-bit word: (tag << 32) | index.  An inserter claims an
@@ -250,91 +188,6 @@ __device__ __forceinline__ void normalise(int64_t (&t64)[EPL], int32_t (&t32)[EP
 }
 
 // ---------------------------------------------------------------------------
-// narrow networks (at most 64 internal rows): per-state summaries of the
-// extra-flux row, see generate_narrow below
-// ---------------------------------------------------------------------------
-
-struct NarrowSum {
-    uint64_t rh, pm, nm, um, om;
-    uint32_t pmax;
-};
-
-__device__ __forceinline__ uint64_t blob_u64(const uint32_t *bl, int o)
-{
-    return (uint64_t)bl[o] | ((uint64_t)bl[o + 1] << 32);
-}
-
-// Summaries of a full row held across a warp (entry m = lane + 32 e).
-template <int EPL>
-__device__ NarrowSum warp_summary(const uint32_t *bl, const NetView &nv, const int32_t (&t)[EPL], int lane)
-{
-    NarrowSum r{0, 0, 0, 0, 0, 0};
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) {
-        const int m = lane + 32 * e;
-        const int32_t v = t[e];
-        if (m < nv.M && v != 0) {
-            const uint32_t rk = bl[nv.o_rank + m];
-            if (v > 0) r.pm |= 1ull << (rk & 0xFFu);
-            else r.nm |= 1ull << ((rk >> 8) & 0xFFu);
-            if (v == 1 || v == -1) r.um |= 1ull << m;
-            if (v & 1) r.om |= 1ull << m;
-            const uint32_t a = (uint32_t)(v < 0 ? -v : v);
-            r.pmax = a > r.pmax ? a : r.pmax;
-            r.rh += (uint64_t)(int64_t)v * blob_u64(bl, nv.o_hrow + 2 * m);
-        }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        r.pm |= __shfl_xor_sync(FULL, r.pm, off);
-        r.nm |= __shfl_xor_sync(FULL, r.nm, off);
-        r.um |= __shfl_xor_sync(FULL, r.um, off);
-        r.om |= __shfl_xor_sync(FULL, r.om, off);
-        r.rh += __shfl_xor_sync(FULL, r.rh, off);
-        const uint32_t o = __shfl_xor_sync(FULL, r.pmax, off);
-        r.pmax = o > r.pmax ? o : r.pmax;
-    }
-    return r;
-}
-
-// the summary record of a state: 6 words, written as three 16-byte stores
-__device__ __forceinline__ void put_summary(uint64_t *d, const NarrowSum &s)
-{
-    *reinterpret_cast<ulonglong2 *>(d) = make_ulonglong2(s.rh, s.pm);
-    *reinterpret_cast<ulonglong2 *>(d + 2) = make_ulonglong2(s.nm, s.um);
-    *reinterpret_cast<ulonglong2 *>(d + 4) = make_ulonglong2(s.om, (uint64_t)s.pmax);
-}
-
-__device__ __forceinline__ NarrowSum get_summary(const uint64_t *d)
-{
-    const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(d);
-    const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(d + 2);
-    const ulonglong2 c = *reinterpret_cast<const ulonglong2 *>(d + 4);
-    return NarrowSum{a.x, a.y, b.x, b.y, c.x, (uint32_t)c.y};
-}
-
-__device__ __forceinline__ void store_summary(const Arena &ar, uint64_t idx, const NarrowSum &s, int lane)
-{
-    if (lane == 0) put_summary(ar.sum + (size_t)idx * kSumWords, s);
-}
-
-// pivot key from the two masks (0xFFFFFFFF when balanced)
-__device__ __forceinline__ uint32_t mask_key(const uint32_t *bl, const NetView &nv, uint64_t pm, uint64_t nm)
-{
-    const uint32_t kp = pm ? bl[nv.o_keyr + __ffsll((long long)pm) - 1] : 0xFFFFFFFFu;
-    const uint32_t kn = nm ? bl[nv.o_keyr + kNarrowKeyRanks + __ffsll((long long)nm) - 1] : 0xFFFFFFFFu;
-    return kp < kn ? kp : kn;
-}
-
-// 64-bit hash of the support words (W words of U plus column k)
-__device__ __forceinline__ uint64_t support_hash(const uint64_t *pu, int W, int k)
-{
-    uint64_t h = 0;
-    for (int w = 0; w < W; ++w) h += mix64(child_word(pu, w, k) ^ (0x2545f4914f6cdd1dull * (uint64_t)(w + 1)));
-    return h;
-}
-
-// ---------------------------------------------------------------------------
 // a0: seeds (INIT kernel analogue): flux 1 on every column producing the
 // target (every column for target -1).  One warp per seed.
 // ---------------------------------------------------------------------------
@@ -386,22 +239,12 @@ __device__ void seed_range(const NetView &nv, const LevelArgs &a, int target, in
             if (lane == 0) a.child.meta[idx] = pack_meta(bkey, 1);
             deg_sum += bkey >> 16;
         }
-        if (EPL <= 2 && nv.narrow && a.child.sum) {
-            const NarrowSum sm = warp_summary<EPL>(bl, nv, t, lane);
-            if ((int64_t)idx < a.child.cap) store_summary(a.child, idx, sm, lane);
-        }
     }
     if (lane == 0) {
         if (n_seed) atomicAdd(&a.ctr[C_SEEDS], n_seed);
         if (n_bal) atomicAdd(&a.ctr[C_BAL], n_bal);
         if (deg_sum) atomicAdd(&a.ctr[C_DEGSUM], deg_sum);
     }
-}
-
-template <int EPL>
-__global__ void __launch_bounds__(kExpandWarps * 32) seed_kernel(NetView nv, LevelArgs a, int target)
-{
-    seed_range<EPL>(nv, a, target, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5);
 }
 
 // ---------------------------------------------------------------------------
@@ -578,60 +421,6 @@ __global__ void __launch_bounds__(kExpandWarps * 32) walk_kernel(NetView nv, Lev
     }
 }
 
-// Seed set R_in (Prop. 1): one state with flux 1 on each column of R_in,
-// EF = the sum of their S_int columns, normalised.  One warp.
-template <int EPL>
-__global__ void __launch_bounds__(32) seedset_kernel(NetView nv, LevelArgs a, const int32_t *cols, int n_cols)
-{
-    __shared__ uint64_t U[kMaxW];
-    const int lane = threadIdx.x & 31;
-    const int W = nv.W, Mpad = nv.Mpad;
-    const int32_t *dcol = reinterpret_cast<const int32_t *>(nv.blob + nv.o_dcols);
-    for (int x = lane; x < W; x += 32) U[x] = 0ull;
-    __syncwarp();
-    int64_t t64[EPL];
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) t64[e] = 0;
-    for (int i = 0; i < n_cols; ++i) {
-        const int k = cols[i];
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) t64[e] += dcol[(size_t)k * Mpad + lane + 32 * e];
-        if (lane == 0) U[k >> 6] |= 1ull << (k & 63);
-        __syncwarp();
-    }
-    int32_t t[EPL];
-    bool zero, ovf;
-    walk_normalise<EPL>(t64, t, zero, ovf);
-    zero = balance_zero<EPL>(t, nv.M, lane);
-    if (lane == 0) atomicAdd(&a.ctr[C_SEEDS], 1ull);
-    if (ovf) {
-        if (lane == 0) atomicAdd(&a.ctr[C_OVF], 1ull);
-        return;
-    }
-    if (zero) {
-        if (lane == 0) {
-            atomicAdd(&a.ctr[C_BAL], 1ull);
-            insert_support(a, W, U, cols[0]);
-        }
-        return;
-    }
-    const uint32_t key = pivot_key<EPL>(nv.blob, nv, t, lane);
-    if (a.child.cap < 1) return;
-    if (EPL <= 2 && nv.narrow && a.child.sum) {
-        const NarrowSum sm = warp_summary<EPL>(nv.blob, nv, t, lane);
-        store_summary(a.child, 0, sm, lane);
-    }
-    for (int x = lane; x < W; x += 32) a.child.U[x] = U[x];
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) a.child.B[lane + 32 * e] = t[e];
-    const uint32_t bkey = branch_key(nv.blob, nv, key, a.sub);
-    if (lane == 0) {
-        a.child.meta[0] = pack_meta(bkey, n_cols);
-        atomicAdd(&a.ctr[C_NEXT], 1ull);
-        atomicAdd(&a.ctr[C_DEGSUM], (unsigned long long)(bkey >> 16));
-    }
-}
-
 // ---------------------------------------------------------------------------
 // a1-a6: one level of expansion.
 //
@@ -726,30 +515,6 @@ __device__ __forceinline__ bool child_after(const uint64_t *pu, int k, const uin
         const uint64_t c = child_word(pu, w, k);
         const uint64_t d = c ^ __ldg(R + w);
         if (d) return (c & (d & (~d + 1))) == 0;
-    }
-    return false;
-}
-
-// Superset rule through the sentinel index (W <= 2): does a result E with
-// k in E lie inside U + {k}?  Only the cells (k, s) with s in U are scanned:
-// E's sentinel is one of its columns other than k, so E inside U + {k}
-// requires the sentinel in U.
-__device__ __forceinline__ bool pruned_indexed(const LevelArgs &a, const uint64_t *pu, int k, int W, int N)
-{
-    if (a.csingle[k]) return true;
-    const uint64_t u0 = child_word(pu, 0, k), u1 = W == 2 ? child_word(pu, 1, k) : 0ull;
-    for (int w = 0; w < W; ++w) {
-        uint64_t m = __ldg(a.cne + (size_t)k * W + w) & (w == 0 ? u0 : u1);
-        while (m) {
-            const int sent = w * 64 + __ffsll((long long)m) - 1;
-            m &= m - 1;
-            const int32_t lo = __ldg(a.cptr + (size_t)k * N + sent), hi = __ldg(a.cptr + (size_t)k * N + sent + 1);
-            for (int32_t e = lo; e < hi; ++e) {
-                const uint64_t *E = a.cent + (size_t)e * W;
-                const uint64_t e0 = __ldg(E), e1 = W == 2 ? __ldg(E + 1) : 0ull;
-                if (((e0 & ~u0) | (e1 & ~u1)) == 0) return true;
-            }
-        }
     }
     return false;
 }
@@ -1263,851 +1028,6 @@ __device__ void expand_range(const NetView &nv, const LevelArgs &a, const uint32
 
 
 // ---------------------------------------------------------------------------
-// Generate, narrow networks (at most 64 internal rows): incremental state
-// summaries.
-//
-// The AND update t = A p + C s changes the sign pattern of the extra-flux
-// row only on the rows of column k (A > 0), so a state carries summaries
-// that a child updates from those few rows instead of scanning the whole
-// row:
-//   * two 64-bit masks of its positive and negative entries, with each row
-//     at its rank in the positive / negative pivot-key order: the child's
-//     pivot is the lowest set bit of either mask (Alg. 3's acting metabolite
-//     under the fewest-reactions rule), and both masks empty means balanced;
-//   * a linear row hash sum_m t_m R[m] (mod 2^64): the child's is
-//     A h(p) + C h(S_int[:, k]);
-//   * the rows holding +-1: with gcd(A, C) = 1, if the parent has a +-1 on a
-//     row outside column k and either A = 1 or the entries of column k are
-//     coprime, then every prime dividing all of t would divide A and
-//     therefore, through the rows of column k, every entry of the column --
-//     or divide the +-1 entry times A -- so gcd(t) = 1 with no gcd at all;
-//   * a bound on max |t|: A pmax + C max|s| < 2^31 lets the update run in
-//     plain 32-bit multiply-adds with no overflow test.
-// A child without such a certificate, or with a possible overflow, takes the
-// full-row path (exact gcd, 64-bit entries) and recomputes what it must.
-//
-// Work is split by its shape: everything per child (branch rules, the
-// summaries from the rows of column k, balance test, superset rule, key,
-// fingerprint, support and summary stores) runs one item per lane, 32
-// children at once; only the dense extra-flux row (and a slow child's gcd)
-// runs on groups of G lanes, each lane holding two 16-byte chunks, so the
-// row's loads and stores are coalesced.
-// ---------------------------------------------------------------------------
-
-template <int G>
-__device__ void generate_narrow(const NetView &nv, const LevelArgs &a, const uint32_t *bl, int64_t worker,
-                                int64_t nworkers)
-{
-    const int lane = threadIdx.x & 31;
-    const int W = nv.W;
-    const int Mpad = nv.Mpad;
-    const int64_t row_cap = a.child.cap;
-
-    unsigned long long n_exp = 0, n_ovf = 0, n_bal = 0, n_pruned = 0, n_unwritten = 0;
-    bool fatal = false;
-    uint64_t pool_next = 0;
-    int pool_left = 0;
-    uint64_t spool_next = 0;  // this warp's settle-record slots
-    int spool_left = 0;
-    // rows for cnt children of the warp (warp-uniform call); returns the
-    // first row of the calling lane's share given its rank among them
-    auto reserve = [&](int cnt, int rank) -> uint64_t {
-        uint64_t fresh = 0;
-        if (pool_left < cnt) {
-            const int want = cnt > a.blk ? cnt : a.blk;
-            if (lane == 0) fresh = atomicAdd(&a.ctr[C_WRITTEN], (unsigned long long)want);
-            fresh = __shfl_sync(FULL, fresh, 0);
-            const uint64_t idx = rank < pool_left ? pool_next + (uint64_t)rank : fresh + (uint64_t)(rank - pool_left);
-            pool_next = fresh + (uint64_t)(cnt - pool_left);
-            pool_left = want - (cnt - pool_left);
-            return idx;
-        }
-        const uint64_t idx = pool_next + (uint64_t)rank;
-        pool_next += (uint64_t)cnt;
-        pool_left -= cnt;
-        return idx;
-    };
-
-    const int cpw = a.cpw;
-    const int64_t wstride = nworkers * cpw;
-    for (int64_t p0 = worker * cpw; p0 < a.n_par; p0 += wstride) {
-        const int64_t pl = p0 + lane;
-        const bool pin = lane < cpw && pl < a.n_par;
-        const int64_t pid = pin ? (a.perm ? (int64_t)a.perm[pl] : a.par_base + pl) : 0;
-        // (no L2 prefetch of the next chunk's parents: measured slower here)
-        const uint32_t mj = pin ? a.par.meta[pid] : 0u;
-        int dj = pin ? (int)((mj >> 10) & 0x1FFFu) : 0;
-        if (a.fk_pc > 0 && (int)((mj >> 23) & 0x7Fu) > a.fk_pc) dj = 0;
-        int incl = dj;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int x = __shfl_up_sync(FULL, incl, off);
-            if (lane >= off) incl += x;
-        }
-        const int prej = incl - dj;
-        const int T = __shfl_sync(FULL, incl, 31);
-        if (T > 32 * nv.N) {
-            if (lane == 0) record_diag(a.ctr, ERR_BOUNDS, 3, T, 32 * nv.N, a.level);
-            fatal = true;
-        }
-        for (int base = 0; base < T; base += 32) {
-            if (__any_sync(FULL, fatal)) break;
-            // === phase A: one (parent, branch) item per lane.  Branch rules,
-            // then the child's summaries from the rows of column k only ===
-            const int c = base + lane;
-            int j = 0;
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-                const int v = __shfl_sync(FULL, prej, j + step);
-                if (v <= c) j += step;
-            }
-            const uint32_t pm = __shfl_sync(FULL, mj, j);
-            const int q = c - __shfl_sync(FULL, prej, j);
-            const int64_t pl_ = __shfl_sync(FULL, pid, j);
-            bool okl = c < T;
-            int kl = 0, pcl = 0;
-            bool inl = false;
-            int32_t Al = 0, Cl = 0;
-            const uint64_t *pu_l = a.par.U + (size_t)pl_ * W;
-            const int32_t *prow_l = a.par.B + (size_t)pl_ * Mpad;
-            if (okl) {
-                const int piv = (int)(pm & 0x3FFu);
-                pcl = (int)((pm >> 23) & 0x7Fu);
-                const int32_t bi = piv < nv.M ? prow_l[piv] : 0;
-                const bool fwd = bi > 0;
-                const uint32_t abi = (uint32_t)(bi < 0 ? -bi : bi);
-                const int lptr = (fwd ? nv.o_consptr : nv.o_prodptr) + (piv < nv.M ? piv : 0);
-                const int lb = (int)bl[lptr];
-                const int le = (int)bl[lptr + 1];
-                if (piv >= nv.M || bi == 0 || lb + q >= le) {
-                    record_diag(a.ctr, ERR_BOUNDS, 1 + (piv >= nv.M ? 10 : 0) + (bi == 0 ? 100 : 0), (long long)q,
-                                (long long)(le - lb), a.level);
-                    fatal = true;
-                    okl = false;
-                } else {
-                    const uint32_t br = bl[(fwd ? nv.o_consent : nv.o_prodent) + lb + q];
-                    kl = ent_index(br);
-                    const uint32_t sik = (uint32_t)ent_coef(br);
-                    const int tw = (int)bl[nv.o_twin + kl];
-                    inl = bit_of(pu_l, kl);
-                    const int sec = a.level - pcl;
-                    okl = !(tw >= 0 && bit_of(pu_l, tw)) && (inl ? sec + 1 <= a.max_sec : pcl + 1 <= a.max_len);
-                    if (okl && a.fk_pc > 0) {
-                        const int pc2 = pcl + (inl ? 0 : 1);
-                        okl = pc2 < a.fk_pc || (pc2 == a.fk_pc && !child_after(pu_l, kl, a.fk_sup, W));
-                    }
-                    const uint32_t g0 = (abi == 1u || sik == 1u) ? 1u : gcd32(abi, sik);
-                    Al = (int32_t)(sik / g0);
-                    Cl = (int32_t)(abi / g0);
-                }
-            }
-            if (okl) ++n_exp;
-            // summaries of the child (exact signs from 64-bit entries)
-            NarrowSum sm{0, 0, 0, 0, 0, 0};
-            bool fast = false, cert = false;
-            uint32_t gtl = 1;  // gcd of the changed entries (when fast)
-            if (okl) {
-                const NarrowSum ps = get_summary(a.par.sum + (size_t)pl_ * kSumWords);
-                const uint32_t pmaxp = ps.pmax;
-                const int ox = nv.o_colx + kColxWordsDev * kl;
-                const uint64_t suppP = blob_u64(bl, ox), suppN = blob_u64(bl, ox + 2), suppR = blob_u64(bl, ox + 4);
-                const uint32_t smax = bl[ox + 8], gcd1 = bl[ox + 9];
-                fast = (uint64_t)Al * pmaxp + (uint64_t)Cl * smax <= 2147483647ull;
-                uint64_t newp = 0, newn = 0, newu = 0, newo = 0, tmax = 0;
-                uint32_t gt = 0;  // gcd of the changed entries (exact when fast: they fit 32 bits)
-                for (int qq = (int)bl[nv.o_colptr + kl]; qq < (int)bl[nv.o_colptr + kl + 1]; ++qq) {
-                    const uint32_t e = bl[nv.o_colent + qq];
-                    const int m = ent_index(e);
-                    const int64_t tm = (int64_t)Al * prow_l[m] + (int64_t)Cl * ent_coef(e);
-                    const uint32_t rk = bl[nv.o_rank + m];
-                    newp |= (tm > 0 ? 1ull : 0ull) << (rk & 0xFFu);
-                    newn |= (tm < 0 ? 1ull : 0ull) << ((rk >> 8) & 0xFFu);
-                    newu |= ((tm == 1 || tm == -1) ? 1ull : 0ull) << m;
-                    newo |= (uint64_t)(tm & 1) << m;
-                    const uint64_t am = (uint64_t)(tm < 0 ? -tm : tm);
-                    tmax = am > tmax ? am : tmax;
-                    if (am != 0 && gt != 1) gt = gt == 0 ? (uint32_t)am : gcd32(gt, (uint32_t)am);
-                }
-                sm.pm = (ps.pm & ~suppP) | newp;
-                sm.nm = (ps.nm & ~suppN) | newn;
-                const uint64_t uout = ps.um & ~suppR;  // parent's +-1 rows outside column k
-                sm.um = (Al == 1 ? uout : 0ull) | newu;
-                sm.om = ((Al & 1) ? (ps.om & ~suppR) : 0ull) | newo;  // odd rows (A p is odd iff both are)
-                sm.rh = (uint64_t)(int64_t)Al * ps.rh + (uint64_t)(int64_t)Cl * blob_u64(bl, ox + 6);
-                const uint64_t bound = (uint64_t)Al * pmaxp > tmax ? (uint64_t)Al * pmaxp : tmax;
-                sm.pmax = bound > 2147483647ull ? 2147483647u : (uint32_t)bound;
-                // gcd(t) = 1 without computing it: a +-1 entry in the child, a
-                // parent +-1 outside column k with A = 1 or a coprime column, or
-                // coprime changed entries (every common divisor divides them)
-                cert = sm.um != 0 || (uout != 0 && (Al == 1 || gcd1 != 0)) || (fast && gt == 1) ||
-                       (fast && gt != 0 && (gt & (gt - 1)) == 0 && sm.om != 0);  // gcd | 2^a, and an odd entry
-                gtl = gt;  // 0: no changed entry is nonzero (the whole row decides)
-            }
-            const bool nzl = (sm.pm | sm.nm) != 0;
-            const bool ball = okl && !nzl;
-            if (ball) {
-                ++n_bal;  // all metabolites stable: to the arbiter
-                if (insert_support(a, W, pu_l, kl) < INS_DUP) fatal = true;
-            }
-            // ready: the child is final (no overflow possible, gcd 1): prune
-            // test, key and fingerprint here.  verify: no overflow possible,
-            // the gcd not certified; the lane group writing its row takes the
-            // gcd of the whole row, and only a child whose gcd is above 1 (rare)
-            // goes on to the settle pass.  slow: a possible overflow, settled.
-            bool ready = okl && nzl && fast;
-            const bool vfyl = ready && !cert;
-            bool slowl = okl && nzl && !fast;
-            // the superset rule through the sentinel index runs in the prune
-            // pass over the reserved rows; the column buckets here otherwise
-            if (ready && !inl && !(W <= 2 && a.cptr)) {
-                const int64_t b1 = a.bptr[kl];
-                const int64_t n = a.bptr[kl + 1] - b1;
-                bool pr = false;
-                if (n > 0) {
-                    if (W <= 2) {
-                        const uint64_t u0 = child_word(pu_l, 0, kl), u1 = W == 2 ? child_word(pu_l, 1, kl) : 0ull;
-                        bool maybe = true;
-                        if (a.band) {
-                            const uint64_t i0 = __ldg(a.band + (size_t)kl * W), i1 = W == 2 ? __ldg(a.band + (size_t)kl * W + 1) : 0ull;
-                            maybe = ((i0 & ~u0) | (i1 & ~u1)) == 0;
-                        }
-                        for (int64_t i = 0; i < n && !pr && maybe; ++i) {
-                            const uint64_t *E = a.bres + (size_t)(b1 + i) * W;
-                            const uint64_t e0 = __ldg(E), e1 = W == 2 ? __ldg(E + 1) : 0ull;
-                            pr = ((e0 & ~u0) | (e1 & ~u1)) == 0;
-                        }
-                    } else {
-                        for (int64_t i = 0; i < n && !pr; ++i) pr = result_inside_wide(a, pu_l, kl, b1 + i);
-                    }
-                }
-                if (pr) {
-                    ++n_pruned;
-                    ready = false;
-                }
-            }
-            // rows for the ready children of the pass, written per lane
-            // except the extra-flux row (phase B, coalesced by lane groups)
-            const unsigned rmask = __ballot_sync(FULL, ready);
-            uint64_t myidx = 0;
-            if (rmask) {
-                myidx = reserve(__popc(rmask), __popc(rmask & ((1u << lane) - 1u)));
-                if (ready) {
-                    if ((int64_t)myidx < row_cap) {
-                        uint64_t *du = a.child.U + (size_t)myidx * W;
-                        for (int w = 0; w < W; ++w) du[w] = child_word(pu_l, w, kl);
-                        a.child.meta[myidx] = pack_meta(mask_key(bl, nv, sm.pm, sm.nm), pcl + (inl ? 0 : 1));
-                        put_summary(a.child.sum + (size_t)myidx * kSumWords, sm);
-                    } else {
-                        ++n_unwritten;
-                    }
-                    if ((int64_t)myidx < a.fp_cap) {
-                        uint64_t f = sm.rh ^ mix64(support_hash(pu_l, W, kl) + 0x632BE59BD9B4E019ull);
-                        if (f == kDeadFp) f = kDeadFp - 1;
-                        a.fp[myidx] = f;
-                        // the row itself is written by the row pass
-                        a.wrec[myidx] = make_uint4((uint32_t)pl_, (uint32_t)kl | (vfyl ? 1u << 12 : 0u) |
-                                                                      (inl ? 1u << 13 : 0u) | ((uint32_t)pcl << 14),
-                                                   (uint32_t)Al, (uint32_t)Cl);
-                    } else {
-                        record_diag(a.ctr, ERR_BOUNDS, 7, (long long)myidx, a.fp_cap, a.level);
-                        fatal = true;
-                    }
-                }
-            }
-            const uint32_t pl32 = (uint32_t)pl_;
-            // === the slow children (no gcd certificate or a possible overflow)
-            // go to the settle pass as records ===
-            const unsigned smask = __ballot_sync(FULL, slowl);
-            if (smask) {
-                // record slots from this warp's pool (32 at a time, one atomic)
-                const int scnt = __popc(smask), srank = __popc(smask & ((1u << lane) - 1u));
-                uint64_t sfresh = 0;
-                if (spool_left < scnt) {
-                    if (lane == 0) sfresh = atomicAdd(&a.ctr[C_SLOW], 32ull);
-                    sfresh = __shfl_sync(FULL, sfresh, 0);
-                }
-                const uint64_t si = srank < spool_left ? spool_next + (uint64_t)srank
-                                                       : sfresh + (uint64_t)(srank - spool_left);
-                if (spool_left < scnt) {
-                    spool_next = sfresh + (uint64_t)(scnt - spool_left);
-                    spool_left = 32 - (scnt - spool_left);
-                } else {
-                    spool_next += (uint64_t)scnt;
-                    spool_left -= scnt;
-                }
-                if (slowl) {
-                    if ((int64_t)si < a.slow_cap) {
-                        uint64_t *r = a.slow + (size_t)si * kSlowWords;
-                        const uint64_t w0 = (uint64_t)pl32 | ((uint64_t)kl << 32) | ((uint64_t)pcl << 44) |
-                                            (inl ? 1ull << 51 : 0ull) | (fast ? 1ull << 52 : 0ull);
-                        const uint64_t w1 = (uint64_t)(uint32_t)Al | ((uint64_t)(uint32_t)Cl << 32);
-                        *reinterpret_cast<ulonglong2 *>(r) = make_ulonglong2(w0, w1);
-                        *reinterpret_cast<ulonglong2 *>(r + 2) = make_ulonglong2(sm.rh, sm.pm);
-                        *reinterpret_cast<ulonglong2 *>(r + 4) = make_ulonglong2(sm.nm, sm.um);
-                        *reinterpret_cast<ulonglong2 *>(r + 6) = make_ulonglong2(sm.om, 0ull);
-                    } else {
-                        record_diag(a.ctr, ERR_BOUNDS, 9, (long long)si, a.slow_cap, a.level);
-                        fatal = true;
-                    }
-                }
-            }
-        }
-        if (__any_sync(FULL, fatal)) break;
-    }
-    for (int x = lane; x < pool_left; x += 32) {
-        if ((int64_t)(pool_next + x) < a.fp_cap) {
-            a.fp[pool_next + x] = kDeadFp;
-            a.wrec[pool_next + x].x = kNoRecord;
-        }
-        if ((int64_t)(pool_next + x) < row_cap) a.child.meta[pool_next + x] = 0u;
-    }
-    // settle-record slots left unused: marked so that the settle pass skips them
-    if (lane < spool_left && (int64_t)(spool_next + lane) < a.slow_cap) a.slow[(spool_next + lane) * kSlowWords] = ~0ull;
-    if (n_exp) atomicAdd(&a.ctr[C_EXP], n_exp);
-    if (n_ovf) atomicAdd(&a.ctr[C_OVF], n_ovf);
-    if (n_bal) atomicAdd(&a.ctr[C_BAL], n_bal);
-    if (n_pruned) atomicAdd(&a.ctr[C_PRUNED], n_pruned);
-    if (n_unwritten) atomicAdd(&a.ctr[C_UNWRITTEN], n_unwritten);
-}
-
-template <int G>
-__global__ void __launch_bounds__(kExpandWarps * 32, 6) generate_narrow_kernel(NetView nv, LevelArgs a, int staged)
-{
-    extern __shared__ __align__(16) uint32_t smem[];
-    const int wid = threadIdx.x >> 5;
-    const int blob_words = staged ? nv.blob_words : 0;
-    uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + blob_words);
-    const uint32_t *bl = stage_blob(nv, smem, mbar, staged != 0, a.ctr);
-    if (bl == nullptr) return;
-    generate_narrow<G>(nv, a, bl, (int64_t)blockIdx.x * kExpandWarps + wid, (int64_t)gridDim.x * kExpandWarps);
-}
-
-// ---------------------------------------------------------------------------
-// Prune pass (narrow networks, supports of at most 2 words): one thread per
-// reserved row with a row-pass record that adds a new column.  The superset
-// rule on the child's support (the parent's, plus the column); a pruned
-// child gives its row up (no state, no fingerprint, no record).  A child
-// without a written row is tested the same way, from its parent.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) prune_rows_kernel(NetView nv, LevelArgs a)
-{
-    const uint64_t begin = a.ctr[C_DEDUP_BEGIN];
-    uint64_t end = a.ctr[C_WRITTEN];
-    end = end < (uint64_t)a.fp_cap ? end : (uint64_t)a.fp_cap;
-    const uint64_t row_cap = (uint64_t)a.child.cap;
-    const int W = nv.W;
-    unsigned long long n_pr = 0, n_unw = 0;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = begin + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end; i += stride) {
-        const uint4 rc = a.wrec[i];
-        if (rc.x == kNoRecord || ((rc.y >> 13) & 1u)) continue;  // nothing to write, or a secondary step
-        const int k = (int)(rc.y & 0xFFFu);
-        if (pruned_indexed(a, a.par.U + (size_t)rc.x * W, k, W, nv.N)) {
-            a.fp[i] = kDeadFp;
-            a.wrec[i].x = kNoRecord;
-            if (i < row_cap)
-                a.child.meta[i] = 0u;
-            else
-                ++n_unw;
-            ++n_pr;
-        }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        n_pr += __shfl_xor_sync(FULL, n_pr, off);
-        n_unw += __shfl_xor_sync(FULL, n_unw, off);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (n_pr) atomicAdd(&a.ctr[C_PRUNED], n_pr);
-        if (n_unw) atomicAdd(&a.ctr[C_UNWRITTEN], (unsigned long long)(-(long long)n_unw));
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Row pass (narrow networks): one lane group per reserved row of the level,
-// in row order.  A row with a record gets t = A p + C s (32 bits: the
-// generate pass recorded only children that cannot overflow); when the
-// summaries did not certify its gcd, the group folds the row into its gcd
-// first, and a row with a gcd above 1 (rare) is withdrawn and handed to the
-// settle pass with its phase-A summaries.
-// ---------------------------------------------------------------------------
-template <int G, int CPL>
-__global__ void __launch_bounds__(256) write_rows_kernel(NetView nv, LevelArgs a)
-{
-    constexpr int NG = 32 / G;
-    const int lane = threadIdx.x & 31;
-    const int gi = lane / G;
-    const int gl = lane % G;
-    const int Mpad = nv.Mpad;
-    const int4 *dcol = reinterpret_cast<const int4 *>(nv.blob + nv.o_dcols);
-    const uint64_t begin = a.ctr[C_DEDUP_BEGIN];
-    uint64_t end = a.ctr[C_WRITTEN];
-    end = end < (uint64_t)a.fp_cap ? end : (uint64_t)a.fp_cap;
-    end = end < (uint64_t)a.child.cap ? end : (uint64_t)a.child.cap;
-    const uint64_t wid = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t r0 = begin + wid * NG; r0 < end; r0 += nwarps * NG) {
-        const uint64_t idx = r0 + gi;
-        uint4 rc = make_uint4(kNoRecord, 0u, 0u, 0u);
-        if (idx < end) rc = a.wrec[idx];
-        const bool has = rc.x != kNoRecord;
-        const int k = (int)(rc.y & 0xFFFu);
-        const bool vfy = has && ((rc.y >> 12) & 1u);
-        const int32_t A = (int32_t)rc.z, C = (int32_t)rc.w;
-        int4 t4[CPL];
-        uint32_t gg = vfy ? 0u : 1u;
-        if (has) {
-            const int4 *prow4 = reinterpret_cast<const int4 *>(a.par.B + (size_t)rc.x * Mpad);
-            const int4 *col4 = dcol + (size_t)k * (Mpad >> 2);
-#pragma unroll
-            for (int i = 0; i < CPL; ++i) {
-                const int4 v = prow4[gl + G * i];
-                const int4 w = col4[gl + G * i];
-                t4[i] = make_int4(A * v.x + C * w.x, A * v.y + C * w.y, A * v.z + C * w.z, A * v.w + C * w.w);
-            }
-            if (vfy) {
-#pragma unroll
-                for (int i = 0; i < CPL; ++i) {
-                    const int32_t xs[4] = {t4[i].x, t4[i].y, t4[i].z, t4[i].w};
-#pragma unroll
-                    for (int jj = 0; jj < 4; ++jj)
-                        if (gg != 1u && xs[jj] != 0) gg = gcd32(gg, (uint32_t)(xs[jj] < 0 ? -xs[jj] : xs[jj]));
-                }
-            }
-        }
-#pragma unroll
-        for (int off = G / 2; off > 0; off >>= 1) {
-            const uint32_t og = __shfl_xor_sync(FULL, gg, off);
-            if (gg != 1u || og != 1u) gg = gcd32(gg, og);
-        }
-        const bool bad = vfy && gg != 1u;
-        if (has && !bad) {
-            int4 *db = reinterpret_cast<int4 *>(a.child.B + (size_t)idx * Mpad);
-#pragma unroll
-            for (int i = 0; i < CPL; ++i) db[gl + G * i] = t4[i];
-        }
-        if (bad && gl == 0) {
-            // withdrawn: the row carries no state; the settle pass makes the child
-            a.child.meta[idx] = 0u;
-            a.fp[idx] = kDeadFp;
-            const uint64_t si = atomicAdd(&a.ctr[C_SLOW], 1ull);
-            if ((int64_t)si < a.slow_cap) {
-                const uint64_t *sm = a.child.sum + (size_t)idx * kSumWords;
-                uint64_t *r = a.slow + (size_t)si * kSlowWords;
-                const uint64_t w0 = (uint64_t)rc.x | ((uint64_t)k << 32) | ((uint64_t)((rc.y >> 14) & 0x7Fu) << 44) |
-                                    (((rc.y >> 13) & 1u) ? 1ull << 51 : 0ull) | (1ull << 52);
-                const uint64_t w1 = (uint64_t)rc.z | ((uint64_t)rc.w << 32);
-                r[0] = w0;
-                r[1] = w1;
-                r[2] = sm[0];  // row hash
-                r[3] = sm[1];  // positive entries (key-rank order)
-                r[4] = sm[2];  // negative entries
-                r[5] = sm[3];  // +-1 rows
-                r[6] = sm[4];  // odd rows
-                r[7] = 0ull;
-            } else {
-                record_diag(a.ctr, ERR_BOUNDS, 11, (long long)si, a.slow_cap, a.level);
-            }
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Settle pass (narrow networks): the children whose gcd the summaries do not
-// certify, or whose update may leave int32, listed by the generate pass as
-// records (parent, column, |U|, flags, A, C and their phase-A summaries).
-// A group of G lanes per record: the row in 32 or 64 bits, the exact gcd and
-// int32 range over the whole row (the overflow rule comes before the
-// superset rule, as in the definition), the superset rule, then a reserved
-// row.  Keeping this rare, long path out of the generate kernel keeps that
-// kernel's instruction footprint small.
-// ---------------------------------------------------------------------------
-template <int G>
-__global__ void __launch_bounds__(kExpandWarps * 32) settle_kernel(NetView nv, LevelArgs a)
-{
-    constexpr int CPL = 2;
-    constexpr int NG = 32 / G;
-    constexpr int EPL = 4 * CPL;
-    const int lane = threadIdx.x & 31;
-    const int gi = lane / G;
-    const int gl = lane % G;
-    const int lead = gi * G;
-    const int W = nv.W;
-    const int Mpad = nv.Mpad;
-    const uint32_t *bl = nv.blob;
-    const int4 *dcol = reinterpret_cast<const int4 *>(bl + nv.o_dcols);
-    const int64_t row_cap = a.child.cap;
-    int64_t n_slow = (int64_t)a.ctr[C_SLOW];
-    n_slow = n_slow < a.slow_cap ? n_slow : a.slow_cap;
-    unsigned long long n_ovf = 0, n_pruned = 0, n_unwritten = 0;
-    bool fatal = false;
-    uint64_t pool_next = 0;
-    int pool_left = 0;
-    auto reserve = [&](int cnt, int rank) -> uint64_t {
-        uint64_t fresh = 0;
-        if (pool_left < cnt) {
-            const int want = cnt;  // exactly what the round needs: no unused rows
-            if (lane == 0) fresh = atomicAdd(&a.ctr[C_WRITTEN], (unsigned long long)want);
-            fresh = __shfl_sync(FULL, fresh, 0);
-            const uint64_t idx = rank < pool_left ? pool_next + (uint64_t)rank : fresh + (uint64_t)(rank - pool_left);
-            pool_next = fresh + (uint64_t)(cnt - pool_left);
-            pool_left = want - (cnt - pool_left);
-            return idx;
-        }
-        const uint64_t idx = pool_next + (uint64_t)rank;
-        pool_next += (uint64_t)cnt;
-        pool_left -= cnt;
-        return idx;
-    };
-    const int64_t wid = (int64_t)blockIdx.x * kExpandWarps + (threadIdx.x >> 5);
-    const int64_t wstride = (int64_t)gridDim.x * kExpandWarps * NG;
-    for (int64_t base = wid * NG; base < n_slow; base += wstride) {
-        if (__any_sync(FULL, fatal)) break;
-            const int64_t r = base + gi;
-            bool slow = r < n_slow;
-            // the record (every lane of the group reads it)
-            uint64_t w0 = 0, w1 = 0, srh = 0, spm = 0, snm = 0, sum_ = 0, som = 0;
-            if (slow) {
-                const uint64_t *rec = a.slow + (size_t)r * kSlowWords;
-                const ulonglong2 q0 = *reinterpret_cast<const ulonglong2 *>(rec);
-                const ulonglong2 q1 = *reinterpret_cast<const ulonglong2 *>(rec + 2);
-                const ulonglong2 q2 = *reinterpret_cast<const ulonglong2 *>(rec + 4);
-                const ulonglong2 q3 = *reinterpret_cast<const ulonglong2 *>(rec + 6);
-                w0 = q0.x;
-                w1 = q0.y;
-                srh = q1.x;
-                spm = q1.y;
-                snm = q2.x;
-                sum_ = q2.y;
-                som = q3.x;
-                slow = w0 != ~0ull;  // an unused slot
-            }
-            const int64_t p = (int64_t)(uint32_t)w0;
-            const int k = (int)((w0 >> 32) & 0xFFFu);
-            const int pc = (int)((w0 >> 44) & 0x7Fu);
-            const bool in_u = (w0 >> 51) & 1ull;
-            const bool fst = (w0 >> 52) & 1ull;  // the update fits 32 bits
-            const int32_t A = (int32_t)(uint32_t)w1;
-            const int32_t C = (int32_t)(uint32_t)(w1 >> 32);
-                const int4 *prow4 = reinterpret_cast<const int4 *>(a.par.B + (size_t)p * Mpad);
-                const int4 *col4 = dcol + (size_t)k * (Mpad >> 2);
-                int32_t t32[EPL];
-                bool big = false;
-                uint64_t gg = 0, amax = 0;
-                if (slow && fst) {
-                    uint32_t g32 = 0, m32 = 0;
-#pragma unroll
-                    for (int i = 0; i < CPL; ++i) {
-                        const int4 v = prow4[gl + G * i];
-                        const int4 w = col4[gl + G * i];
-                        t32[4 * i + 0] = A * v.x + C * w.x;
-                        t32[4 * i + 1] = A * v.y + C * w.y;
-                        t32[4 * i + 2] = A * v.z + C * w.z;
-                        t32[4 * i + 3] = A * v.w + C * w.w;
-                    }
-#pragma unroll
-                    for (int e = 0; e < EPL; ++e) {
-                        const uint32_t at = (uint32_t)(t32[e] < 0 ? -t32[e] : t32[e]);
-                        if (at != 0 && g32 != 1) g32 = g32 == 0 ? at : gcd32(g32, at);
-                        m32 = at > m32 ? at : m32;
-                    }
-                    gg = g32;
-                    amax = m32;
-                } else if (slow) {
-#pragma unroll
-                    for (int i = 0; i < CPL; ++i) {
-                        const int4 v = prow4[gl + G * i];
-                        const int4 w = col4[gl + G * i];
-                        const int32_t pv[4] = {v.x, v.y, v.z, v.w}, cv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) {
-                            const int64_t tt = (int64_t)A * pv[jj] + (int64_t)C * cv[jj];
-                            const int32_t lo = (int32_t)tt;
-                            big = big || tt != (int64_t)lo || lo == INT32_MIN;
-                            t32[4 * i + jj] = lo;
-                        }
-                    }
-                    if (!big) {
-#pragma unroll
-                        for (int e = 0; e < EPL; ++e) {
-                            const uint32_t at = (uint32_t)(t32[e] < 0 ? -t32[e] : t32[e]);
-                            if (at != 0 && gg != 1) gg = gg == 0 ? at : gcd32((uint32_t)gg, at);
-                            amax = at > amax ? at : amax;
-                        }
-                    } else {
-                        const GcdMax gmx = raw_gcd_max(prow4, col4, gl, G, CPL, A, C);
-                        gg = gmx.g;
-                        amax = gmx.m;
-                    }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < EPL; ++e) t32[e] = 0;
-                }
-                big = group_or<G>(big ? 1u : 0u) != 0;
-                if (!__any_sync(FULL, big)) {
-                    // every entry of every slow row of the round fits 32 bits
-                    uint32_t g32 = (uint32_t)gg, m32 = (uint32_t)amax;
-#pragma unroll
-                    for (int off = G / 2; off > 0; off >>= 1) {
-                        const uint32_t og = __shfl_xor_sync(FULL, g32, off);
-                        g32 = (og == 0 || g32 == 1) ? g32 : (g32 == 0 ? og : gcd32(g32, og));
-                        const uint32_t y = __shfl_xor_sync(FULL, m32, off);
-                        m32 = y > m32 ? y : m32;
-                    }
-                    gg = g32;
-                    amax = m32;
-                } else {
-#pragma unroll
-                    for (int off = G / 2; off > 0; off >>= 1) {
-                        const uint64_t og = __shfl_xor_sync(FULL, gg, off);
-                        gg = og == 0 ? gg : (gg == 0 ? og : gcd64(gg, og));
-                        const uint64_t y = __shfl_xor_sync(FULL, amax, off);
-                        amax = y > amax ? y : amax;
-                    }
-                }
-                if (gg == 0) gg = 1;
-                const bool ovf = slow && amax / gg > 2147483647ull;
-                if (slow && !ovf && gg > 1) {
-                    if (!big) {
-#pragma unroll
-                        for (int e = 0; e < EPL; ++e) t32[e] = t32[e] / (int32_t)gg;
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < CPL; ++i) {
-                            const int4 v = prow4[gl + G * i];
-                            const int4 w = col4[gl + G * i];
-                            const int32_t pv[4] = {v.x, v.y, v.z, v.w}, cv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                            for (int jj = 0; jj < 4; ++jj) {
-                                const int64_t tt = (int64_t)A * pv[jj] + (int64_t)C * cv[jj];
-                                t32[4 * i + jj] = (int32_t)(tt / (int64_t)gg);
-                            }
-                        }
-                    }
-                }
-                if (ovf && gl == 0) ++n_ovf;
-                const uint64_t *pu = a.par.U + (size_t)p * W;
-                bool pr = false;
-                const bool cand = slow && !ovf;
-                if (cand && !in_u) {
-                    const int64_t b1 = a.bptr[k];
-                    const int64_t n = a.bptr[k + 1] - b1;
-                    if (W <= 2 && a.cptr) {
-                        if (gl == 0) pr = pruned_indexed(a, pu, k, W, nv.N);
-                    } else if (W <= 2) {
-                        const uint64_t u0 = child_word(pu, 0, k), u1 = W == 2 ? child_word(pu, 1, k) : 0ull;
-                        bool maybe = n > 0;
-                        if (maybe && a.band) {
-                            const uint64_t i0 = __ldg(a.band + (size_t)k * W), i1 = W == 2 ? __ldg(a.band + (size_t)k * W + 1) : 0ull;
-                            maybe = ((i0 & ~u0) | (i1 & ~u1)) == 0;
-                        }
-                        for (int64_t i = gl; i < n && !pr && maybe; i += G) {
-                            const uint64_t *E = a.bres + (size_t)(b1 + i) * W;
-                            const uint64_t e0 = __ldg(E), e1 = W == 2 ? __ldg(E + 1) : 0ull;
-                            pr = ((e0 & ~u0) | (e1 & ~u1)) == 0;
-                        }
-                    } else {
-                        for (int64_t i = gl; i < n && !pr; i += G) pr = result_inside_wide(a, pu, k, b1 + i);
-                    }
-                }
-                pr = group_or<G>(pr ? 1u : 0u) != 0;
-                if (pr && gl == 0) ++n_pruned;
-                const bool keep = cand && !pr;
-                // a row divided by its gcd: +-1 rows and hash over the row (the
-                // signs do not change); otherwise phase A's values stand
-                uint64_t um = sum_, om = som, rh = srh;
-                if (__any_sync(FULL, keep && gg > 1)) {
-                    uint64_t u2 = 0, o2 = 0, h2 = 0;
-                    if (keep && gg > 1) {
-#pragma unroll
-                        for (int i = 0; i < CPL; ++i)
-#pragma unroll
-                            for (int jj = 0; jj < 4; ++jj) {
-                                const int m = 4 * (gl + G * i) + jj;
-                                const int32_t v = t32[4 * i + jj];
-                                if (m < nv.M && v != 0) {
-                                    if (v == 1 || v == -1) u2 |= 1ull << m;
-                                    if (v & 1) o2 |= 1ull << m;
-                                    h2 += (uint64_t)(int64_t)v * blob_u64(bl, nv.o_hrow + 2 * m);
-                                }
-                            }
-                    }
-#pragma unroll
-                    for (int off = G / 2; off > 0; off >>= 1) {
-                        u2 |= __shfl_xor_sync(FULL, u2, off);
-                        o2 |= __shfl_xor_sync(FULL, o2, off);
-                        h2 += __shfl_xor_sync(FULL, h2, off);
-                    }
-                    if (keep && gg > 1) {
-                        um = u2;
-                        om = o2;
-                        rh = h2;
-                    }
-                }
-                const unsigned km = __ballot_sync(FULL, keep && gl == 0);
-                if (km) {
-                    const uint64_t idx = reserve(__popc(km), __popc(km & ((1u << lead) - 1u)));
-                    if (keep) {
-                        if ((int64_t)idx < row_cap) {
-                            int4 *db = reinterpret_cast<int4 *>(a.child.B + (size_t)idx * Mpad);
-#pragma unroll
-                            for (int i = 0; i < CPL; ++i)
-                                db[gl + G * i] = make_int4(t32[4 * i + 0], t32[4 * i + 1], t32[4 * i + 2], t32[4 * i + 3]);
-                            uint64_t *du = a.child.U + (size_t)idx * W;
-                            for (int w = gl; w < W; w += G) du[w] = child_word(pu, w, k);
-                            if (gl == 0) {
-                                a.child.meta[idx] = pack_meta(mask_key(bl, nv, spm, snm), pc + (in_u ? 0 : 1));
-                                put_summary(a.child.sum + (size_t)idx * kSumWords,
-                                            NarrowSum{rh, spm, snm, um, om, (uint32_t)(amax / gg)});
-                            }
-                        } else if (gl == 0) {
-                            ++n_unwritten;
-                        }
-                        if (gl == 0) {
-                            if ((int64_t)idx < a.fp_cap) {
-                                uint64_t f = rh ^ mix64(support_hash(pu, W, k) + 0x632BE59BD9B4E019ull);
-                                if (f == kDeadFp) f = kDeadFp - 1;
-                                a.fp[idx] = f;
-                            } else {
-                                record_diag(a.ctr, ERR_BOUNDS, 7, (long long)idx, a.fp_cap, a.level);
-                                fatal = true;
-                            }
-                        }
-                    }
-                }
-                fatal = group_or<G>(fatal ? 1u : 0u) != 0;
-    }
-    for (int x = lane; x < pool_left; x += 32)
-        if ((int64_t)(pool_next + x) < a.fp_cap) a.fp[pool_next + x] = kDeadFp;
-    if (n_ovf) atomicAdd(&a.ctr[C_OVF], n_ovf);
-    if (n_pruned) atomicAdd(&a.ctr[C_PRUNED], n_pruned);
-    if (n_unwritten) atomicAdd(&a.ctr[C_UNWRITTEN], n_unwritten);
-}
-
-// Are reserved rows i and j the same state (support and extra-flux row)?
-__device__ __forceinline__ bool same_state(const Arena &ar, int Mpad, int W, uint64_t i, uint64_t j)
-{
-    const int4 *x = reinterpret_cast<const int4 *>(ar.B + (size_t)i * Mpad);
-    const int4 *y = reinterpret_cast<const int4 *>(ar.B + (size_t)j * Mpad);
-    bool eq = true;
-    for (int c = 0; c < (Mpad >> 2) && eq; ++c) {
-        const int4 u = __ldcg(x + c), v = __ldcg(y + c);
-        eq = u.x == v.x && u.y == v.y && u.z == v.z && u.w == v.w;
-    }
-    const uint64_t *ux = ar.U + (size_t)i * W, *uy = ar.U + (size_t)j * W;
-    for (int w = 0; w < W && eq; ++w) eq = __ldcg(ux + w) == __ldcg(uy + w);
-    return eq;
-}
-
-// One thread per reserved row in [ctr[C_DEDUP_BEGIN], ctr[C_WRITTEN]).  The
-// first row of every distinct state survives in place; a later copy gets a
-// zero meta word (no branches), so the next level reads the arena's rows in
-// order and no survivor list is built.  Survivors and their branch counts
-// are summed per block, with one atomic per block.
-__global__ void __launch_bounds__(256) dedup_kernel(LevelArgs a, int Mpad, int W)
-{
-    __shared__ unsigned long long s_keep[8], s_deg[8], s_unv[8];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const uint64_t begin = a.ctr[C_DEDUP_BEGIN];
-    uint64_t end = a.ctr[C_WRITTEN];
-    end = end < (uint64_t)a.fp_cap ? end : (uint64_t)a.fp_cap;
-    const uint64_t row_cap = (uint64_t)a.child.cap;
-    unsigned long long deg = 0, n_unv = 0, n_keep = 0;
-    bool fatal = false;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i0 = begin + (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < end; i0 += stride) {
-        const uint64_t i = i0 + lane;
-        bool mine = i < end;
-        const uint64_t f = mine ? a.fp[i] : kDeadFp;
-        mine = mine && f != kDeadFp;
-        if (mine) {
-            uint64_t pos;
-            uint32_t tag;
-            slot_tag_pos(f, a.slot_mask, pos, tag);
-            const bool written = i < row_cap;
-            if (i >= 0xFFFFFFFEull) {
-                record_diag(a.ctr, ERR_BOUNDS, 10, (long long)i, 0xFFFFFFFEll, a.level);
-                fatal = true;
-            }
-            for (uint64_t probe = 0; !fatal; ++probe) {
-                if (probe > a.slot_mask) {
-                    record_diag(a.ctr, ERR_TABLE_FULL, 8, (long long)i, (long long)a.slot_mask, a.level);
-                    fatal = true;
-                    break;
-                }
-                const unsigned long long v = atomicCAS(&a.slots[pos], kEmpty, ((unsigned long long)tag << 32) | i);
-                if (v == kEmpty) {  // first of its state
-                    if (written) {
-                        ++n_keep;
-                        deg += (a.child.meta[i] >> 10) & 0x1FFFu;
-                    } else {
-                        ++n_unv;
-                    }
-                    break;
-                }
-                if ((uint32_t)(v >> 32) == tag) {
-                    const uint64_t jrow = (uint32_t)v;
-                    // a row without its state written cannot be compared: the
-                    // level is then decided from the lower bound, or run again
-                    if (!written || jrow >= row_cap) {
-                        if (written) a.child.meta[i] = 0u;
-                        break;
-                    }
-                    if (same_state(a.child, Mpad, W, i, jrow)) {  // a later copy
-                        a.child.meta[i] = 0u;
-                        break;
-                    }
-                }
-                pos = (pos + 1) & a.slot_mask;
-            }
-        }
-        if (__any_sync(FULL, fatal)) break;
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        deg += __shfl_xor_sync(FULL, deg, off);
-        n_unv += __shfl_xor_sync(FULL, n_unv, off);
-        n_keep += __shfl_xor_sync(FULL, n_keep, off);
-    }
-    if (lane == 0) {
-        s_keep[wid] = n_keep;
-        s_deg[wid] = deg;
-        s_unv[wid] = n_unv;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long k = 0, d = 0, u = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            k += s_keep[w];
-            d += s_deg[w];
-            u += s_unv[w];
-        }
-        if (k) atomicAdd(&a.ctr[C_NEXT], k);
-        if (d) atomicAdd(&a.ctr[C_DEGSUM], d);
-        if (u) atomicAdd(&a.ctr[C_UNV], u);
-    }
-}
-
-// Surviving rows [0, n) of an arena (meta != 0: every state has |U| >= 1)
-// appended to a list, for the passes that sample or order a frontier.
-__global__ void live_list_kernel(const uint32_t *meta, int64_t n, uint32_t *live, unsigned long long *count)
-{
-    const int lane = threadIdx.x & 31;
-    for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll; i0 < n;
-         i0 += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = i0 + lane;
-        const bool keep = i < n && meta[i] != 0u;
-        const unsigned m = __ballot_sync(FULL, keep);
-        unsigned long long base = 0;
-        if (lane == 0 && m) base = atomicAdd(count, (unsigned long long)__popc(m));
-        base = __shfl_sync(FULL, base, 0);
-        if (keep) live[base + __popc(m & ((1u << lane) - 1u))] = (uint32_t)i;
-    }
-}
-
-__global__ void dedup_advance_kernel(unsigned long long *ctr) { ctr[C_DEDUP_BEGIN] = ctr[C_WRITTEN]; }
-
-// ---------------------------------------------------------------------------
 // a7/a8: exact minimality test by elimination modulo primes, then append.
 // ---------------------------------------------------------------------------
 
@@ -2122,17 +1042,6 @@ __device__ __forceinline__ uint32_t mulmod(uint32_t x, uint32_t y, uint32_t p, u
 }
 
 __device__ __forceinline__ uint32_t submod(uint32_t x, uint32_t y, uint32_t p) { return x >= y ? x - y : x + p - y; }
-
-__device__ __forceinline__ uint32_t powmod(uint32_t x, uint32_t e, uint32_t p, uint32_t c)
-{
-    uint32_t r = 1;
-    while (e) {
-        if (e & 1u) r = mulmod(r, x, p, c);
-        x = mulmod(x, x, p, c);
-        e >>= 1;
-    }
-    return r;
-}
 
 __device__ __forceinline__ uint32_t to_mod(int32_t s, uint32_t p)
 {
@@ -2173,22 +1082,23 @@ __device__ bool full_rank_mod_p(const uint32_t *bl, const NetView &nv, const int
             __syncwarp();
             uint32_t y0 = c0 >= 0 ? to_mod(coef_at(bl, nv, c0, row), p) : 0u;
             uint32_t y1 = c1 >= 0 ? to_mod(coef_at(bl, nv, c1, row), p) : 0u;
+            // (cross-multiplied: scaling a row by a nonzero pivot keeps the rank,
+            // and no inverse, a chain of 60 products, has to be taken)
             for (int i = 0; i < rank; ++i) {
                 const int pc = pivcol[i];
                 const uint32_t f = __shfl_sync(FULL, pc < 32 ? y0 : y1, pc & 31);
                 if (f != 0) {
-                    y0 = submod(y0, mulmod(f, basis[i * 64 + lane], p, c), p);
-                    y1 = submod(y1, mulmod(f, basis[i * 64 + lane + 32], p, c), p);
+                    const uint32_t b = basis[i * 64 + pc];
+                    y0 = submod(mulmod(y0, b, p, c), mulmod(f, basis[i * 64 + lane], p, c), p);
+                    y1 = submod(mulmod(y1, b, p, c), mulmod(f, basis[i * 64 + lane + 32], p, c), p);
                 }
             }
             const unsigned m0 = __ballot_sync(FULL, y0 != 0);
             const unsigned m1 = __ballot_sync(FULL, y1 != 0);
             if (m0 == 0 && m1 == 0) continue;
             const int pv = m0 ? __ffs((int)m0) - 1 : 32 + __ffs((int)m1) - 1;
-            const uint32_t v = __shfl_sync(FULL, pv < 32 ? y0 : y1, pv & 31);
-            const uint32_t inv = powmod(v, p - 2u, p, c);
-            basis[rank * 64 + lane] = mulmod(y0, inv, p, c);
-            basis[rank * 64 + lane + 32] = mulmod(y1, inv, p, c);
+            basis[rank * 64 + lane] = y0;
+            basis[rank * 64 + lane + 32] = y1;
             if (lane == 0) pivcol[rank] = pv;
             __syncwarp();
             ++rank;
@@ -2300,160 +1210,6 @@ __global__ void accept_advance_kernel(unsigned long long *ctr, int64_t cand_cap)
 }
 
 // ---------------------------------------------------------------------------
-// result buckets by column (for the superset test)
-// ---------------------------------------------------------------------------
-
-__global__ void bucket_count_kernel(const uint64_t *res, int64_t n, int W, int32_t *bcnt)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n * W) return;
-    const int w = (int)(i % W);
-    for (uint64_t x = res[i]; x; x &= x - 1) atomicAdd(&bcnt[w * 64 + __ffsll((long long)x) - 1], 1);
-}
-
-__global__ void bucket_scan_kernel(const int32_t *bcnt, int N, int32_t *bptr)
-{
-    // single CTA of 1024 threads, N <= 4096: exclusive scan
-    __shared__ int32_t part[1024];
-    const int per = (N + 1023) / 1024;
-    const int beg = threadIdx.x * per;
-    int32_t s = 0;
-    for (int i = beg; i < beg + per && i < N; ++i) s += bcnt[i];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const int32_t v = threadIdx.x >= off ? part[threadIdx.x - off] : 0;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
-    }
-    int32_t run = part[threadIdx.x] - s;
-    for (int i = beg; i < beg + per && i < N; ++i) {
-        bptr[i] = run;
-        run += bcnt[i];
-    }
-    if (threadIdx.x == 1023) bptr[N] = part[1023];
-}
-
-__global__ void bucket_fill_kernel(const uint64_t *res, int64_t n, int W, const int32_t *bptr, int32_t *bfill,
-                                   uint64_t *bres, unsigned long long *band)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n * W) return;
-    const int w = (int)(i % W);
-    const int64_t r = i / W;
-    for (uint64_t x = res[i]; x; x &= x - 1) {
-        const int k = w * 64 + __ffsll((long long)x) - 1;
-        const int64_t pos = (int64_t)bptr[k] + atomicAdd(&bfill[k], 1);
-        if (W > 2) {
-            reinterpret_cast<int32_t *>(bres)[pos] = (int32_t)r;
-        } else {
-            for (int v = 0; v < W; ++v) {
-                bres[pos * W + v] = res[r * W + v];
-                // intersection of the results containing k
-                if (band) atomicAnd(&band[(size_t)k * W + v], (unsigned long long)res[r * W + v]);
-            }
-        }
-    }
-}
-
-// The superset rule's sentinel index (W <= 2, N <= 128): for each result E
-// its two columns with the fewest results, (m1, m2), ties by column; for each
-// k in E the sentinel is m1, or m2 when k = m1.
-__device__ __forceinline__ void result_sentinels(const uint64_t *E, int W, const int32_t *bcnt, int &m1, int &m2)
-{
-    m1 = m2 = -1;
-    long long k1 = 0x7FFFFFFFFFFFFFFFll, k2 = 0x7FFFFFFFFFFFFFFFll;
-    for (int w = 0; w < W; ++w)
-        for (uint64_t x = E[w]; x; x &= x - 1) {
-            const int c = w * 64 + __ffsll((long long)x) - 1;
-            const long long key = ((long long)bcnt[c] << 16) | c;
-            if (key < k1) {
-                k2 = k1;
-                m2 = m1;
-                k1 = key;
-                m1 = c;
-            } else if (key < k2) {
-                k2 = key;
-                m2 = c;
-            }
-        }
-}
-
-__global__ void sentinel_count_kernel(const uint64_t *res, int64_t n, int W, int N, const int32_t *bcnt, int32_t *ccnt,
-                                      uint32_t *csingle)
-{
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const uint64_t *E = res + (size_t)r * W;
-    int m1, m2;
-    result_sentinels(E, W, bcnt, m1, m2);
-    if (m2 < 0) {  // a one-column result: every child adding that column contains it
-        if (m1 >= 0) csingle[m1] = 1u;
-        return;
-    }
-    for (int w = 0; w < W; ++w)
-        for (uint64_t x = E[w]; x; x &= x - 1) {
-            const int k = w * 64 + __ffsll((long long)x) - 1;
-            atomicAdd(&ccnt[(size_t)k * N + (k == m1 ? m2 : m1)], 1);
-        }
-}
-
-__global__ void sentinel_scan_kernel(const int32_t *ccnt, int cells, int32_t *cptr)
-{
-    // one CTA of 1024 threads: exclusive scan over the cells
-    __shared__ int32_t part[1024];
-    const int per = (cells + 1023) / 1024;
-    const int beg = threadIdx.x * per;
-    int32_t s = 0;
-    for (int i = beg; i < beg + per && i < cells; ++i) s += ccnt[i];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const int32_t v = threadIdx.x >= off ? part[threadIdx.x - off] : 0;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
-    }
-    int32_t run = part[threadIdx.x] - s;
-    for (int i = beg; i < beg + per && i < cells; ++i) {
-        cptr[i] = run;
-        run += ccnt[i];
-    }
-    if (threadIdx.x == 1023) cptr[cells] = part[1023];
-}
-
-__global__ void sentinel_mask_kernel(const int32_t *ccnt, int N, int W, uint64_t *cne)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= N) return;
-    for (int w = 0; w < W; ++w) {
-        uint64_t m = 0;
-        for (int b = 0; b < 64 && w * 64 + b < N; ++b)
-            if (ccnt[(size_t)k * N + w * 64 + b] > 0) m |= 1ull << b;
-        cne[(size_t)k * W + w] = m;
-    }
-}
-
-__global__ void sentinel_fill_kernel(const uint64_t *res, int64_t n, int W, int N, const int32_t *bcnt,
-                                     const int32_t *cptr, int32_t *cfill, uint64_t *cent)
-{
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const uint64_t *E = res + (size_t)r * W;
-    int m1, m2;
-    result_sentinels(E, W, bcnt, m1, m2);
-    if (m2 < 0) return;
-    for (int w = 0; w < W; ++w)
-        for (uint64_t x = E[w]; x; x &= x - 1) {
-            const int k = w * 64 + __ffsll((long long)x) - 1;
-            const size_t cell = (size_t)k * N + (k == m1 ? m2 : m1);
-            const int32_t pos = cptr[cell] + atomicAdd(&cfill[cell], 1);
-            for (int v = 0; v < W; ++v) cent[(size_t)pos * W + v] = E[v];
-        }
-}
-
-// ---------------------------------------------------------------------------
 // output order: (|U|, ascending column list), bitonic sort of indices
 // ---------------------------------------------------------------------------
 
@@ -2478,33 +1234,116 @@ __device__ bool support_greater(const uint64_t *res, int W, uint32_t x, uint32_t
     return false;
 }
 
-__global__ void sort_init_kernel(uint32_t *idx, int64_t n, int64_t n2)
+// Sort record of a support: |U| and its nine lowest columns, 12 bits each --
+// the order of the records is the order of the supports but for ties, which
+// the words decide -- and the support's index.  Padding sorts last.  (With a
+// record of four columns, 2^14 genome-shaped results took 2.0 ms, most of it
+// in the ties.)
+struct SortRec {
+    unsigned long long key, key2;
+    uint32_t idx, pad;
+};
+
+constexpr int kSortBlock = 512;            // threads
+constexpr int kSortTile = 2 * kSortBlock;  // records a block sorts in shared memory
+
+__global__ void sort_init_kernel(const uint64_t *res, int W, SortRec *rec, int64_t n, int64_t n2)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n2) return;
+    SortRec r{~0ull, ~0ull, 0xFFFFFFFFu, 0u};
+    if (i < n) {
+        const uint64_t *U = res + (size_t)i * W;
+        int pc = 0, got = 0;
+        unsigned long long low = 0, low2 = 0;
+        for (int w = 0; w < W; ++w) {
+            uint64_t x = U[w];
+            pc += __popcll(x);
+            for (; x && got < 9; x &= x - 1, ++got) {
+                const unsigned long long c = (unsigned)(w * 64 + __ffsll((long long)x) - 1);
+                if (got < 4) low |= c << (36 - 12 * got);
+                else low2 |= c << (48 - 12 * (got - 4));
+            }
+        }
+        // (a support with fewer columns than another differs in |U|)
+        r.key = ((unsigned long long)pc << 48) | low;
+        r.key2 = low2;
+        r.idx = (uint32_t)i;
+    }
+    rec[i] = r;
+}
+
+__device__ __forceinline__ bool rec_greater(const uint64_t *res, int W, const SortRec &x, const SortRec &y)
+{
+    if (x.key != y.key) return x.key > y.key;
+    if (x.key2 != y.key2) return x.key2 > y.key2;
+    return support_greater(res, W, x.idx, y.idx);
+}
+
+// the sort without keys, for callers whose scratch holds 4 bytes a support
+__device__ __forceinline__ bool rec_greater(const uint64_t *res, int W, uint32_t x, uint32_t y)
+{
+    return support_greater(res, W, x, y);
+}
+__device__ __forceinline__ uint32_t rec_index(uint32_t r) { return r; }
+__device__ __forceinline__ uint32_t rec_index(const SortRec &r) { return r.idx; }
+
+__global__ void sort_init_kernel(const uint64_t *, int, uint32_t *idx, int64_t n, int64_t n2)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n2) idx[i] = i < n ? (uint32_t)i : 0xFFFFFFFFu;
 }
 
-__global__ void bitonic_step_kernel(const uint64_t *res, int W, uint32_t *idx, int64_t n2, int64_t k, int64_t j)
+template <typename Rec>
+__global__ void bitonic_step_kernel(const uint64_t *res, int W, Rec *rec, int64_t n2, int64_t k, int64_t j)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n2) return;
     const int64_t l = i ^ j;
     if (l <= i) return;
-    const uint32_t x = idx[i], y = idx[l];
+    const Rec x = rec[i], y = rec[l];
     const bool up = (i & k) == 0;
-    if (support_greater(res, W, x, y) == up) {
-        idx[i] = y;
-        idx[l] = x;
+    if (rec_greater(res, W, x, y) == up) {
+        rec[i] = y;
+        rec[l] = x;
     }
 }
 
-__global__ void gather_kernel(const uint64_t *res, int W, const uint32_t *idx, int64_t n_keep, uint64_t *out)
+// The steps with partners inside a tile, in shared memory: the merges
+// k = k0, 2 k0, ... k1, each from j = min(k, tile) / 2 down.
+template <typename Rec>
+__global__ void __launch_bounds__(kSortBlock) bitonic_tile_kernel(const uint64_t *res, int W, Rec *rec, int64_t n2,
+                                                                  int64_t k0, int64_t k1)
+{
+    __shared__ Rec t[kSortTile];
+    const int64_t base = (int64_t)blockIdx.x * kSortTile;
+    const int n = (int)(n2 - base < kSortTile ? n2 - base : kSortTile);  // a power of two
+    for (int i = threadIdx.x; i < n; i += kSortBlock) t[i] = rec[base + i];
+    for (int64_t k = k0; k <= k1; k <<= 1)
+        for (int j = (int)(k < n ? k : n) >> 1; j > 0; j >>= 1) {
+            __syncthreads();
+            for (int q = threadIdx.x; q < n / 2; q += kSortBlock) {
+                const int i = ((q & ~(j - 1)) << 1) | (q & (j - 1)), l = i | j;
+                const bool up = ((base + i) & k) == 0;
+                const Rec x = t[i], y = t[l];
+                if (rec_greater(res, W, x, y) == up) {
+                    t[i] = y;
+                    t[l] = x;
+                }
+            }
+        }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += kSortBlock) rec[base + i] = t[i];
+}
+
+template <typename Rec>
+__global__ void gather_kernel(const uint64_t *res, int W, const Rec *rec, int64_t n_keep, uint64_t *out)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_keep * W) return;
     const int64_t r = i / W;
     const int w = (int)(i % W);
-    out[i] = res[(size_t)idx[r] * W + w];
+    out[i] = res[(size_t)rec_index(rec[r]) * W + w];
 }
 
 // ---------------------------------------------------------------------------
@@ -2764,135 +1603,7 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(BatchArgs ba)
     }
 }
 
-template <int EPL>
-cudaError_t launch_seed_t(const NetView &nv, const LevelArgs &a, int target, cudaStream_t s)
-{
-    const int items = target >= 0 ? 1024 : nv.N;
-    int blocks = (items + kExpandWarps - 1) / kExpandWarps;
-    if (blocks > 1024) blocks = 1024;
-    seed_kernel<EPL><<<blocks, kExpandWarps * 32, 0, s>>>(nv, a, target);
-    return cudaGetLastError();
-}
-
-
-// The narrow kernel reads the static network through L1 rather than staging
-// it: at four blocks per SM a staged copy per block would take shared memory
-// that L1 then lacks for the parents' rows (measured: about 3 % faster).
-inline bool narrow_staged(const NetView &) { return false; }
-
-template <int G>
-cudaError_t launch_generate_narrow_t(const NetView &nv, const LevelArgs &a, int grid, cudaStream_t s)
-{
-    const bool staged = narrow_staged(nv);
-    const size_t sm = (size_t)(staged ? nv.blob_words : 0) * 4 + 16;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaFuncSetAttribute(generate_narrow_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kStageLimitBytes + 16);
-        attr_set = true;
-    }
-    generate_narrow_kernel<G><<<grid, kExpandWarps * 32, sm, s>>>(nv, a, staged ? 1 : 0);
-    return cudaGetLastError();
-}
-
-template <int G>
-int generate_narrow_grid_t(const NetView &nv, int sm_count)
-{
-    const bool staged = narrow_staged(nv);
-    const size_t sm = (size_t)(staged ? nv.blob_words : 0) * 4 + 16;
-    cudaFuncSetAttribute(generate_narrow_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageLimitBytes + 16);
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, generate_narrow_kernel<G>, kExpandWarps * 32, sm) !=
-            cudaSuccess ||
-        per_sm < 1) {
-        cudaGetLastError();
-        per_sm = 1;
-    }
-    return sm_count * per_sm;
-}
-
 }  // namespace
-
-#define EFM_EPL_DISPATCH(EPLV, CALL) \
-    switch (EPLV) {                  \
-    case 1: return CALL(1);          \
-    case 2: return CALL(2);          \
-    case 4: return CALL(4);          \
-    case 8: return CALL(8);          \
-    case 16: return CALL(16);        \
-    case 28: return CALL(28);        \
-    case 32: return CALL(32);        \
-    default: return cudaErrorInvalidValue; \
-    }
-
-cudaError_t launch_seed(const NetView &nv, const LevelArgs &a, int target, cudaStream_t s)
-{
-#define CALL_SEED(E) launch_seed_t<E>(nv, a, target, s)
-    EFM_EPL_DISPATCH(nv.EPL, CALL_SEED)
-#undef CALL_SEED
-}
-
-cudaError_t launch_generate(const NetView &nv, const LevelArgs &a, int grid, cudaStream_t s)
-{
-    // narrow networks: incremental summaries (needs the arenas' summary arrays)
-    if (nv.narrow && a.par.sum && a.child.sum) {
-        if (nv.EPL == 1) return launch_generate_narrow_t<4>(nv, a, grid, s);
-        if (nv.EPL == 2) return launch_generate_narrow_t<8>(nv, a, grid, s);
-    }
-    return cudaErrorInvalidValue;
-}
-
-int generate_grid(const NetView &nv, int sm_count)
-{
-    if (nv.narrow && nv.EPL == 1) return generate_narrow_grid_t<4>(nv, sm_count);
-    if (nv.narrow && nv.EPL == 2) return generate_narrow_grid_t<8>(nv, sm_count);
-    return sm_count;
-}
-
-cudaError_t launch_live_list(const uint32_t *meta, int64_t n, uint32_t *live, unsigned long long *count,
-                             int sm_count, cudaStream_t s)
-{
-    if (n <= 0) return cudaSuccess;
-    const int64_t blocks = std::min<int64_t>((n + 255) / 256, (int64_t)sm_count * 8);
-    live_list_kernel<<<(unsigned)blocks, 256, 0, s>>>(meta, n, live, count);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_settle(const NetView &nv, const LevelArgs &a, int sm_count, cudaStream_t s)
-{
-    if (!(nv.narrow && a.par.sum && a.child.sum && a.slow)) return cudaSuccess;
-    if (nv.EPL == 1)
-        settle_kernel<4><<<sm_count * 4, kExpandWarps * 32, 0, s>>>(nv, a);
-    else if (nv.EPL == 2)
-        settle_kernel<8><<<sm_count * 4, kExpandWarps * 32, 0, s>>>(nv, a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_prune_rows(const NetView &nv, const LevelArgs &a, int sm_count, cudaStream_t s)
-{
-    if (!(nv.narrow && a.par.sum && a.child.sum && a.wrec && nv.W <= 2 && a.cptr)) return cudaSuccess;
-    prune_rows_kernel<<<sm_count * 8, 256, 0, s>>>(nv, a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_write_rows(const NetView &nv, const LevelArgs &a, int sm_count, cudaStream_t s)
-{
-    if (!(nv.narrow && a.par.sum && a.child.sum && a.wrec)) return cudaSuccess;
-    // G lanes per row of 32 EPL entries, CPL 16-byte chunks each
-    if (nv.EPL == 1)
-        write_rows_kernel<4, 2><<<sm_count * 8, 256, 0, s>>>(nv, a);
-    else if (nv.EPL == 2)
-        write_rows_kernel<8, 2><<<sm_count * 8, 256, 0, s>>>(nv, a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_dedup(const LevelArgs &a, int Mpad, int W, int sm_count, cudaStream_t s)
-{
-    dedup_kernel<<<sm_count * 8, 256, 0, s>>>(a, Mpad, W);
-    dedup_advance_kernel<<<1, 1, 0, s>>>(a.ctr);
-    return cudaGetLastError();
-}
-
 
 cudaError_t launch_accept_new(const NetView &nv, const AcceptArgs &a, int sm_count, cudaStream_t s)
 {
@@ -2921,49 +1632,6 @@ cudaError_t launch_accept(const NetView &nv, const AcceptArgs &a, cudaStream_t s
     return cudaGetLastError();
 }
 
-cudaError_t launch_buckets(const NetView &nv, const uint64_t *res, int64_t n_res, int32_t *bcnt, int32_t *bptr,
-                           int32_t *bfill, uint64_t *bres, uint64_t *band, cudaStream_t s)
-{
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(bcnt, 0, sizeof(int32_t) * (size_t)nv.N, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(bfill, 0, sizeof(int32_t) * (size_t)nv.N, s)) != cudaSuccess) return e;
-    if (band && (e = cudaMemsetAsync(band, 0xFF, sizeof(uint64_t) * (size_t)nv.N * nv.W, s)) != cudaSuccess) return e;
-    const int64_t items = n_res * nv.W;
-    const int tb = 256;
-    if (items > 0) bucket_count_kernel<<<(int)((items + tb - 1) / tb), tb, 0, s>>>(res, n_res, nv.W, bcnt);
-    bucket_scan_kernel<<<1, 1024, 0, s>>>(bcnt, nv.N, bptr);
-    if (items > 0)
-        bucket_fill_kernel<<<(int)((items + tb - 1) / tb), tb, 0, s>>>(res, n_res, nv.W, bptr, bfill, bres,
-                                                                      reinterpret_cast<unsigned long long *>(band));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sentinel_index(const NetView &nv, const uint64_t *res, int64_t n_res, const int32_t *bcnt,
-                                  int32_t *ccnt, int32_t *cfill, int32_t *cptr, uint64_t *cent, uint64_t *cne,
-                                  uint32_t *csingle, cudaStream_t s)
-{
-    const int N = nv.N, W = nv.W;
-    const size_t cells = (size_t)N * N;
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(ccnt, 0, cells * 4, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(cfill, 0, cells * 4, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(csingle, 0, (size_t)N * 4, s)) != cudaSuccess) return e;
-    const int tb = 256;
-    if (n_res > 0)
-        sentinel_count_kernel<<<(int)((n_res + tb - 1) / tb), tb, 0, s>>>(res, n_res, W, N, bcnt, ccnt, csingle);
-    sentinel_scan_kernel<<<1, 1024, 0, s>>>(ccnt, (int)cells, cptr);
-    sentinel_mask_kernel<<<(N + 127) / 128, 128, 0, s>>>(ccnt, N, W, cne);
-    if (n_res > 0)
-        sentinel_fill_kernel<<<(int)((n_res + tb - 1) / tb), tb, 0, s>>>(res, n_res, W, N, bcnt, cptr, cfill, cent);
-    return cudaGetLastError();
-}
-
-__global__ void iota_kernel(uint32_t *perm, int64_t n)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) perm[i] = (uint32_t)i;
-}
-
 cudaError_t launch_walks(const NetView &nv, const LevelArgs &a, int target, uint64_t seed, int64_t n_walks, int sm_count,
                          cudaStream_t s)
 {
@@ -2983,40 +1651,48 @@ cudaError_t launch_walks(const NetView &nv, const LevelArgs &a, int target, uint
     return cudaGetLastError();
 }
 
-cudaError_t launch_seedset(const NetView &nv, const LevelArgs &a, const int32_t *cols, int n_cols, cudaStream_t s)
+size_t sort_scratch_bytes(int64_t n2) { return (size_t)n2 * sizeof(SortRec); }
+
+// kernels a sort of n2 (a power of two) records launches
+int sort_launches(int64_t n2)
 {
-    switch (nv.EPL) {
-#define EFM_SEEDSET(E)                                                \
-    case E:                                                           \
-        seedset_kernel<E><<<1, 32, 0, s>>>(nv, a, cols, n_cols);      \
-        break;
-        EFM_SEEDSET(1) EFM_SEEDSET(2) EFM_SEEDSET(4) EFM_SEEDSET(8) EFM_SEEDSET(16) EFM_SEEDSET(28) EFM_SEEDSET(32)
-#undef EFM_SEEDSET
-    default:
-        return cudaErrorInvalidValue;
+    int n = 3;
+    for (int64_t k = 2 * kSortTile; k <= n2; k <<= 1) {
+        ++n;
+        for (int64_t j = k >> 1; j >= kSortTile; j >>= 1) ++n;
     }
-    return cudaGetLastError();
+    return n;
 }
 
-cudaError_t launch_iota(uint32_t *perm, int64_t n, cudaStream_t s)
-{
-    if (n <= 0) return cudaSuccess;
-    iota_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(perm, n);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sort_results(const uint64_t *res, int64_t n, int W, uint32_t *idx, int64_t n2, uint64_t *out,
-                                int64_t n_keep, cudaStream_t s)
+template <typename Rec>
+static cudaError_t sort_with(const uint64_t *res, int64_t n, int W, Rec *rec, int64_t n2, uint64_t *out, int64_t n_keep,
+                             cudaStream_t s)
 {
     if (n <= 0 || n_keep <= 0) return cudaSuccess;
     const int tb = 256;
     const int blocks = (int)((n2 + tb - 1) / tb);
-    sort_init_kernel<<<blocks, tb, 0, s>>>(idx, n, n2);
-    for (int64_t k = 2; k <= n2; k <<= 1)
-        for (int64_t j = k >> 1; j > 0; j >>= 1) bitonic_step_kernel<<<blocks, tb, 0, s>>>(res, W, idx, n2, k, j);
+    const int tiles = (int)((n2 + kSortTile - 1) / kSortTile);
+    sort_init_kernel<<<blocks, tb, 0, s>>>(res, W, rec, n, n2);
+    bitonic_tile_kernel<<<tiles, kSortBlock, 0, s>>>(res, W, rec, n2, 2, std::min<int64_t>(n2, kSortTile));
+    for (int64_t k = 2 * kSortTile; k <= n2; k <<= 1) {
+        for (int64_t j = k >> 1; j >= kSortTile; j >>= 1) bitonic_step_kernel<<<blocks, tb, 0, s>>>(res, W, rec, n2, k, j);
+        bitonic_tile_kernel<<<tiles, kSortBlock, 0, s>>>(res, W, rec, n2, k, k);
+    }
     const int64_t items = n_keep * W;
-    gather_kernel<<<(int)((items + tb - 1) / tb), tb, 0, s>>>(res, W, idx, n_keep, out);
+    gather_kernel<<<(int)((items + tb - 1) / tb), tb, 0, s>>>(res, W, rec, n_keep, out);
     return cudaGetLastError();
+}
+
+cudaError_t launch_sort_results(const uint64_t *res, int64_t n, int W, void *scratch, int64_t n2, uint64_t *out,
+                                int64_t n_keep, cudaStream_t s)
+{
+    return sort_with(res, n, W, reinterpret_cast<SortRec *>(scratch), n2, out, n_keep, s);
+}
+
+cudaError_t launch_sort_index(const uint64_t *res, int64_t n, int W, uint32_t *idx, int64_t n2, uint64_t *out,
+                              int64_t n_keep, cudaStream_t s)
+{
+    return sort_with(res, n, W, idx, n2, out, n_keep, s);
 }
 
 int batch_blocks_per_sm(int warps)

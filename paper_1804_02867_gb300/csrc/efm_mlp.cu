@@ -186,79 +186,56 @@ __global__ void __launch_bounds__(kFeatWarps * 32) features_kernel(NetView nv, A
             atomicAdd(&emb[wid][h & 63u], (h & 64u) ? 1.f : -1.f);
             colsum += (float)k;
         };
-        if (par.hdr) {
-            // sparse state (layout in efm_sparse.cu): the column list, then
-            // the entries; flux entries (rows past M) are not balance rows
-            const uint4 hd = par.hdr[p];
-            const uint4 *pay = par.pay + hd.x;
-            meta = hd.y;
-            const int n = (int)((meta >> 23) & 0x7Fu);
-            const uint16_t *lst = reinterpret_cast<const uint16_t *>(pay) + 4;
-            const uint64_t *D = dep ? dep + (size_t)(meta & 0x3FFu) * W : nullptr;
-            for (int i = lane; i < n; i += 32) {
-                const int k = lst[i];
+        // the state's columns (layout in efm_sparse.cu), then its entries; flux
+        // entries (rows past M) are not balance rows
+        const uint4 hd = par.hdr[p];
+        const uint4 *pay = par.pay + hd.x;
+        meta = hd.y;
+        const int n_cols = (int)((meta >> 23) & 0x7Fu);
+        const uint64_t *D = dep ? dep + (size_t)(meta & 0x3FFu) * W : nullptr;
+        const uint16_t *lst = reinterpret_cast<const uint16_t *>(pay) + 8;
+        int lowest = 0x7FFFFFFF;  // of this lane's columns, above the ones already taken
+        const int items = W <= 2 ? 128 : n_cols;
+        auto column = [&](int i) -> int {
+            if (W > 2) return lst[i];
+            return (reinterpret_cast<const uint64_t *>(pay)[2 + (i >> 6)] >> (i & 63)) & 1ull ? i : -1;
+        };
+        if (meta != 0u)
+            for (int i = lane; i < items; i += 32) {
+                const int k = column(i);
+                if (k < 0) continue;
                 add_column((uint32_t)k);
                 ++pcl;
                 if (D) ndep += (int)((D[k >> 6] >> (k & 63)) & 1ull);
             }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (i < n) low[i] = (float)lst[i] / (float)nv.N;
-            const int2 *ent = reinterpret_cast<const int2 *>(pay + sparse_list_units(n));
-            for (int i = lane; i < (int)(hd.z & 0x7FFu); i += 32) {
-                const int2 e = ent[i];
-                if (e.x >= nv.M) continue;
-                ++nz;
-                const uint32_t av = (uint32_t)(e.y < 0 ? -e.y : e.y);
-                amax = av > amax ? av : amax;
+        // the four lowest columns, one minimum at a time
+        for (int i = 0, floor_ = -1; i < 4 && i < n_cols; ++i) {
+            lowest = 0x7FFFFFFF;
+            for (int q = lane; q < items; q += 32) {
+                const int k = column(q);
+                if (k > floor_ && k < lowest) lowest = k;
             }
-            if (D)
-                for (int w = lane; w < W; w += 32) anydep |= D[w] != 0ull;
-        } else {
-            const uint64_t *U = par.U + (size_t)p * W;
-            const int32_t *B = par.B + (size_t)p * nv.Mpad;
-            meta = par.meta[p];
-            for (int m = lane; m < nv.M; m += 32) {
-                const int32_t v = B[m];
-                nz += v != 0;
+            floor_ = (int)__reduce_min_sync(FULLMASK, (unsigned)lowest);
+            low[i] = (float)floor_ / (float)nv.N;
+        }
+        if (meta != 0u) {
+            const uint4 *from = pay + (nv.form == 2 ? 3 : (nv.form == 1 ? 2 : sparse_list_units(n_cols)));
+            for (int i = lane; i < (int)(hd.z & 0x7FFu); i += 32) {
+                int32_t v;
+                if (nv.form == 2) {
+                    v = reinterpret_cast<const int32_t *>(from)[i];
+                } else {
+                    const int2 e = reinterpret_cast<const int2 *>(from)[i];
+                    if ((e.x & 0xFFFF) >= nv.M) continue;
+                    v = e.y;
+                }
+                ++nz;
                 const uint32_t av = (uint32_t)(v < 0 ? -v : v);
                 amax = av > amax ? av : amax;
             }
-            for (int w = lane; w < W; w += 32) {
-                uint64_t x = U[w];
-                pcl += __popcll(x);
-                while (x) {
-                    const int b = __ffsll((long long)x) - 1;
-                    x &= x - 1;
-                    add_column((uint32_t)(w * 64 + b));
-                }
-            }
-            // lowest words first, one ballot per word
-            int got = 0;
-            for (int w0 = 0; w0 < W && got < 4; w0 += 32) {
-                const uint64_t x = (w0 + lane < W) ? U[w0 + lane] : 0ull;
-                unsigned nzm = __ballot_sync(FULLMASK, x != 0ull);
-                while (nzm && got < 4) {
-                    const int src = __ffs((int)nzm) - 1;
-                    nzm &= nzm - 1;
-                    uint64_t y = __shfl_sync(FULLMASK, x, src);
-                    while (y && got < 4) {
-                        const int b = __ffsll((long long)y) - 1;
-                        y &= y - 1;
-                        low[got++] = (float)((w0 + src) * 64 + b) / (float)nv.N;
-                    }
-                }
-            }
-            // flux-dependent columns of the pivot (tags of dep_out | dep_in) inside U
-            const int piv = (int)(meta & 0x3FFu);
-            if (dep && piv < nv.M) {
-                const uint64_t *D = dep + (size_t)piv * W;
-                for (int w = lane; w < W; w += 32) {
-                    ndep += __popcll(U[w] & D[w]);
-                    anydep |= D[w] != 0ull;
-                }
-            }
         }
+        if (D)
+            for (int w = lane; w < W; w += 32) anydep |= D[w] != 0ull;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             nz += __shfl_xor_sync(FULLMASK, nz, off);
@@ -329,24 +306,19 @@ __global__ void labels_kernel(Arena par, int W, const uint32_t *map, int64_t fir
         const int64_t pos = first + r * stride;
         const int64_t p = map ? (int64_t)map[pos] : pos;
         bool in = false;
-        if (par.hdr) {  // sparse state: its column list
-            const uint4 hd = par.hdr[p];
-            const uint16_t *lst = reinterpret_cast<const uint16_t *>(par.pay + hd.x) + 4;
-            const int m = (int)((hd.y >> 23) & 0x7Fu);
-            for (int64_t a = lane; a < n_ans && !in; a += 32) {
-                const uint64_t *A = ans + (size_t)a * W;
-                bool sub = true;
-                for (int i = 0; i < m && sub; ++i) sub = (A[lst[i] >> 6] >> (lst[i] & 63)) & 1ull;
-                in = sub;
-            }
-        } else {
-            const uint64_t *U = par.U + (size_t)p * W;
-            for (int64_t a = lane; a < n_ans && !in; a += 32) {
-                const uint64_t *A = ans + (size_t)a * W;
-                bool sub = true;
+        const uint4 hd = par.hdr[p];
+        const uint4 *pay = par.pay + hd.x;
+        const uint64_t *U = reinterpret_cast<const uint64_t *>(pay) + 2;
+        const uint16_t *lst = reinterpret_cast<const uint16_t *>(pay) + 8;
+        const int m = (int)((hd.y >> 23) & 0x7Fu);
+        for (int64_t a = lane; a < n_ans && !in; a += 32) {
+            const uint64_t *A = ans + (size_t)a * W;
+            bool sub = true;
+            if (W <= 2)
                 for (int w = 0; w < W && sub; ++w) sub = (U[w] & ~A[w]) == 0;
-                in = sub;
-            }
+            else
+                for (int i = 0; i < m && sub; ++i) sub = (A[lst[i] >> 6] >> (lst[i] & 63)) & 1ull;
+            in = sub;
         }
         const bool any = __any_sync(FULLMASK, in);
         if (lane == 0) y[row0 + r] = any ? 1.f : 0.f;

@@ -22,9 +22,14 @@
 //    a 64-bit constant R[m] of the linear row hash sum_m EF_m R[m] (mod 2^64);
 //    per column the rank-space masks of its rows (positive and negative
 //    orders), its row-space mask, sum_m S_int[m][k] R[m], max |S_int[m][k]|
-//    and whether the gcd of its entries is 1;
+//    and whether the gcd of its entries is 1; per entry of the column CSR its
+//    row, the row's two ranks and the coefficient;
 //  - wide networks: per column, the lane masks of the rows it consumes and
 //    of the rows it produces (the first-K length-cap rule);
+//  - per column, what the AND update of a sparse state reads at once
+//    (kScolWords = 8 words): sum_m S_int[m][k] R[m] (2 words; with the flux
+//    rows also R[M + k]), the mask of its rows modulo 64 (2), its largest
+//    magnitude, its range of words in the column CSR (2), its twin or ~0;
 //  - a dense column-major copy of S_int: N rows of Mpad = 32 EPL int32,
 //    16-byte aligned.
 // Entries are packed as (index << 20) | (coefficient & 0xFFFFF).
@@ -43,6 +48,7 @@ inline uint32_t ent_pack(int idx, int32_t coef) { return ((uint32_t)idx << 20) |
 
 constexpr int kNarrowRows = 64;  // internal rows of a network with state summaries
 constexpr int kColxWords = 10;   // per-column summary words (narrow networks)
+constexpr int kScolWords = 8;    // per-column words of the AND update
 
 // Constant of internal row m in the linear row hash: the SplitMix64
 // finaliser (Steele, Lea, Flood 2014) of 0x9E3779B97F4A7C15 * (m + 1).
@@ -74,6 +80,8 @@ struct NetPrep {
     int o_twin = 0, o_keypos = 0, o_keyneg = 0, o_hbits = 0, o_dcols = 0;
     bool narrow = false;                            // M <= kNarrowRows: the sections below exist
     int o_rank = 0, o_keyr = 0, o_hrow = 0, o_colx = 0;
+    int o_nent = 0;  // narrow: per column entry, row | rank+ << 8 | rank- << 16, then the coefficient
+    int o_scol = 0;              // per column, kScolWords words (see below), 16-byte aligned
     int o_fixc = 0, o_fixp = 0;  // wide networks: per-column lane masks of consumed / produced rows (0: none)
     std::vector<int32_t> mptr;  // full S rows over split columns (seeds): [n_met + 1]
     std::vector<uint32_t> ment;  // packed (column, coefficient)
@@ -190,7 +198,7 @@ inline int prepare_network(int32_t n_met, int32_t n_rxn, const int32_t *row_ptr,
     out.o_hbits = (int)blob.size();
     for (int k = 0; k < N; ++k) blob.push_back(hbits[k]);
     out.narrow = M <= kNarrowRows && !flux_rows;
-    out.o_rank = out.o_keyr = out.o_hrow = out.o_colx = 0;
+    out.o_rank = out.o_keyr = out.o_hrow = out.o_colx = out.o_nent = 0;
     if (out.narrow) {
         // ranks of the rows in the positive / negative key orders
         std::vector<std::pair<uint32_t, int>> kp, kn;
@@ -245,6 +253,12 @@ inline int prepare_network(int32_t n_met, int32_t n_rxn, const int32_t *row_ptr,
             blob.push_back(smax);
             blob.push_back(g == 1 ? 1u : 0u);
         }
+        out.o_nent = (int)blob.size();  // (an even offset, as o_colx)
+        for (int k = 0; k < N; ++k)
+            for (auto &e : col[k]) {
+                blob.push_back((uint32_t)e.first | ((uint32_t)rp[e.first] << 8) | ((uint32_t)rn[e.first] << 16));
+                blob.push_back((uint32_t)e.second);
+            }
     }
     // wide networks (not narrow, additive rows): the rows column k consumes
     // and produces, as lane masks of the expansion's row layout.  Lane l of
@@ -267,6 +281,20 @@ inline int prepare_network(int32_t n_met, int32_t n_rxn, const int32_t *row_ptr,
             }
     }
     while (blob.size() % 4) blob.push_back(0);
+    out.o_scol = (int)blob.size();
+    for (int k = 0; k < N; ++k) {
+        uint64_t hc = flux_rows ? row_hash_constant(M + k) : 0;
+        uint64_t mask = flux_rows ? 1ull << ((M + k) & 63) : 0;
+        uint32_t smax = flux_rows ? 1u : 0u;
+        for (auto &e : col[k]) {
+            hc += (uint64_t)(int64_t)e.second * row_hash_constant(e.first);
+            mask |= 1ull << (e.first & 63);
+            smax = std::max(smax, (uint32_t)(e.second < 0 ? -e.second : e.second));
+        }
+        const uint32_t w[kScolWords] = {(uint32_t)hc, (uint32_t)(hc >> 32), (uint32_t)mask, (uint32_t)(mask >> 32), smax,
+                                        blob[out.o_colptr + k], blob[out.o_colptr + k + 1], blob[out.o_twin + k]};
+        blob.insert(blob.end(), w, w + kScolWords);
+    }
     // dense column-major copy of S_int (row k = column k over Mpad rows)
     out.o_dcols = (int)blob.size();
     blob.resize(blob.size() + (size_t)N * 32 * EPL, 0u);

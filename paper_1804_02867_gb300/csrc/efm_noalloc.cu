@@ -105,7 +105,7 @@ extern "C" int efm_sort_supports_noalloc(const uint64_t *supports_in, int64_t n_
     }
     uint64_t n2 = 1;
     while ((int64_t)n2 < n_rows) n2 <<= 1;
-    const cudaError_t e = efm::launch_sort_results(supports_in, n_rows, words_per_set, scratch, (int64_t)n2,
+    const cudaError_t e = efm::launch_sort_index(supports_in, n_rows, words_per_set, scratch, (int64_t)n2,
                                                    supports_out, n_rows, (cudaStream_t)cuda_stream);
     if (e != cudaSuccess) {
         cudaGetLastError();

@@ -1,101 +1,129 @@
-// efm_sparse.cu -- the traversal's level pass on sparse states.
+// efm_sparse.cu -- the traversal's level pass.
 //
-// A state keeps only what it holds: the columns of its support and the
-// unbalanced entries of its extra-flux row.  Most entries of a row are zero
-// (a state of the 850-row genome-shaped network holds 8 to 19 unbalanced
-// rows, one of the 58-row core-shaped network about 10), so the AND update
-// EF' = A EF + C S_int[:, k] is a merge of two short sorted lists, and a
-// state takes about 100 bytes instead of a support bitset and a full row.
+// A state keeps only what it holds: its support and the unbalanced entries of
+// its extra-flux row.  Most entries of a row are zero (a state of the
+// 58-row core-shaped network holds about 10 unbalanced rows, one of the
+// 850-row genome-shaped network 8 to 19), so a state takes about 100 bytes.
 //
-// Measured against the dense rows it replaces (a group of 32 lanes per child,
-// the whole row in registers: 1817 warp instructions a child, 3.5 KB written),
-// one GB300, event to event: four genome-shaped targets at a 2^22 budget 362
-// -> 45 ms, six targets of a 400-row network at 2^17 23.9 -> 5.3 ms, first-K
-// = 1000 on three genome targets 103 -> 51 ms, the subtractive variant on the
-// core-shaped network 12.1 -> 8.1 ms.  Networks of at most 64 rows keep their
-// dense rows (efm_kernels.cu): there this pass is level with theirs at 2^21
-// children and slower beyond (785 against 540 ms on the core-shaped network
-// at a 2^26 budget).
-//
-// Layout (Arena::hdr and Arena::pay): one 16-byte header per row of the
-// arena, and a payload in 16-byte units somewhere in the arena's pool:
-//   header  x = payload offset in units, y = meta (0: the row carries no
-//           state), z = entries | bits of max|EF| << 11, w = EF of the pivot
-//   payload 8 bytes: sum of the columns' hash constants (mod 2^64);
-//           the columns of U, ascending, 16 bits each, padded with 0xFFFF to
-//           a unit; then the entries (row, value), ascending rows, 8 bytes
-//           each, padded with zeros to a unit.
-// Equal states have equal payloads, so two states are compared unit by unit.
+// Layout (Arena): per row of the arena a 16-byte header, and a payload in
+// 16-byte units somewhere in the arena's pool:
+//   hdr  x = payload offset in units, y = meta (0: the row carries no state),
+//        z = number of entries | bits of max|EF| << 11, w = EF of the pivot
+//   pay  the row hash rh = sum_m EF_m R[m] (mod 2^64) with R[m] =
+//        mix64(0x9E3779B97F4A7C15 (m + 1)), linear in EF, so that a child's
+//        follows from its parent's and column k's; the sum of the columns'
+//        hash constants (lists only); then the support: at most 128 columns,
+//        a bitset of 2 words (one unit); else the columns, 16 bits each, in
+//        the order they were added, padded with 0xFFFF to a unit; then the entries, 8 bytes each, in no order,
+//        padded to a unit: (pivot key of the row's side, degree << 16 | row;
+//        value); the key of a flux entry is 0xFFFF0000 | row, of padding ~0.
+// Narrow networks (at most 64 rows and 128 columns) instead: rh and the mask
+// of the nonzero rows; the bitset; the masks of the positive and of the
+// negative entries, each row at its rank in the order of that side's pivot
+// keys; then the values in row order, 4 bytes each, padded with zeros.
 // In the subtractive variant (Eq. 5) the entries go on with the flux of every
 // column k of U at row M + k.
+//
+// Measured against the dense rows it replaced (the whole row by a group of
+// lanes, in up to five passes), one GB300, calls through the library: four
+// genome-shaped targets at a 2^22 budget 361 -> 23.7 ms (1817 -> about 110
+// warp instructions a child, 3.5 KB -> about 130 bytes written), six targets
+// of a 400-row network at 2^17 23.4 -> 5.4, first-K = 1000 on three genome
+// targets 103 -> 44.5, eight targets of the core-shaped network at 2^17 20.4
+// -> 13.6 and at 2^26 539 -> 471, its subtractive variant 12.1 -> 8.2.
+//
+// The AND update EF' = A EF + C S_int[:, k] is then a copy of the parent's
+// entries (times A) in 16-byte units, with the few rows of column k changed
+// in place, appended or removed: a lane per child, no order to keep.  The
+// smallest key among the entries names the pivot.
 #include "efm_device.cuh"
 
 namespace efm {
 namespace {
 
 constexpr int kGenWarps = 8;      // warps per CTA
-constexpr int kNoRow = 0x7FFFFFFF;  // past the last entry of a list
-constexpr uint32_t kPadCol = 0xFFFFu;
+// CTAs per SM of the generate pass.  It waits on memory more than it computes
+// (long-scoreboard stalls lead), so 48 registers and 40 warps per SM beat 64
+// registers and 32 although they spill: 485 against 501 ms on the core-shaped
+// network at a 2^26 budget; 24 warps 537.
+constexpr int kGenBlocks = 5;
+constexpr uint32_t kFluxKey = 0xFFFF0000u;  // keys from here on are no balance rows
+constexpr uint32_t kPadKey = 0xFFFFFFFFu;
 
 __device__ __forceinline__ uint64_t column_hash(int k) { return mix64(0x51ed27f3a5b1c3d9ull * (uint64_t)(k + 1)); }
+__device__ __forceinline__ uint64_t row_hash(int m) { return mix64(0x9E3779B97F4A7C15ull * (uint64_t)(m + 1)); }
 
+// Fingerprint of a state: 63 bits.  The top bit marks a reserved row without
+// one: kDeadFp, or a child that the dedup pass finishes first (an open child:
+// its parent's row, column k and flags; see kOpen...).
 __device__ __forceinline__ uint64_t state_fp(uint64_t rows, uint64_t cols)
 {
-    const uint64_t f = rows ^ mix64(cols + 0x632BE59BD9B4E019ull);
-    return f == kDeadFp ? kDeadFp - 1 : f;
+    return (rows ^ mix64(cols + 0x632BE59BD9B4E019ull)) >> 1;
 }
 
-__device__ __forceinline__ uint64_t entry_hash(int row, int32_t v)
+constexpr uint64_t kOpenFp = 1ull << 63;
+constexpr uint64_t kOpenInU = 1ull << 44;   // a secondary step (k is in U)
+constexpr uint64_t kOpenSub = 1ull << 45;   // Eq. 5: flux taken away from k
+constexpr uint64_t kOpenPruned = 1ull << 46;  // the superset rule holds
+constexpr uint64_t kOpenDead = 1ull << 47;  // first-K: cannot balance any more
+constexpr uint64_t kOpenBal = 1ull << 48;   // balanced: to the arbiter
+
+__device__ __forceinline__ void prefetch_l2(const void *p)
 {
-    uint64_t x = (((uint64_t)(uint32_t)row << 32) | (uint32_t)v) * 0x9E3779B97F4A7C15ull;
-    x ^= x >> 32;
-    return x * 0xD6E8FEB86659FD93ull;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
+
+__device__ __forceinline__ int max_bits(uint32_t om) { return om ? 32 - __clz((int)om) : 0; }
+__device__ __forceinline__ uint32_t mag(int32_t v) { return (uint32_t)(v < 0 ? -v : v); }
 
 // 16-bit column i of a payload's list
 __device__ __forceinline__ int list_col(const uint4 *pay, int i)
 {
-    return reinterpret_cast<const uint16_t *>(pay)[4 + i];
+    return reinterpret_cast<const uint16_t *>(pay)[8 + i];
 }
-
-__device__ __forceinline__ uint64_t list_hash(const uint4 *pay)
-{
-    return *reinterpret_cast<const uint64_t *>(pay);
-}
-
-__device__ __forceinline__ const int2 *entries_of(const uint4 *pay, int pc)
-{
-    return reinterpret_cast<const int2 *>(pay + sparse_list_units(pc));
-}
-
-__device__ __forceinline__ int max_bits(uint32_t om) { return om ? 32 - __clz((int)om) : 0; }
 
 // ---------------------------------------------------------------------------
-// balanced supports: the columns of a list (or none) plus column k (or none,
-// k < 0) as the bitset words the arbiter reads
+// Supports.  F (NetView::form) = 1, 2: a bitset of two words (at most 128
+// columns); F = 0: a list.  A child's support is its parent's plus column k (k < 0: the same).
 // ---------------------------------------------------------------------------
 
-// word w of the bitset; pos walks the list (call with w = 0, 1, ...)
-__device__ __forceinline__ uint64_t list_word(const uint4 *pay, int pc, int k, int w, int &pos)
+template <int F>
+__device__ __forceinline__ int support_units(int pc)
 {
-    uint64_t x = 0;
-    while (pos < pc) {
-        const int c = list_col(pay, pos);
-        if ((c >> 6) != w) break;
-        x |= 1ull << (c & 63);
-        ++pos;
+    return F == 2 ? 3 : (F == 1 ? 2 : sparse_list_units(pc));
+}
+
+__device__ __forceinline__ uint64_t bits_hash(uint64_t u0, uint64_t u1)
+{
+    return mix64(u0 ^ 0x2545f4914f6cdd1dull) + mix64(u1 ^ 0x4a8be9229ed9ba3aull);
+}
+
+__device__ __forceinline__ void add_bit(uint64_t &u0, uint64_t &u1, int k)
+{
+    if (k < 64) u0 |= 1ull << k;
+    else u1 |= 1ull << (k - 64);
+}
+
+// hash of the support U + {k}
+template <int F>
+__device__ __forceinline__ uint64_t support_hash_of(const uint4 *pay, int k)
+{
+    if (F) {
+        uint64_t u0 = reinterpret_cast<const uint64_t *>(pay)[2], u1 = reinterpret_cast<const uint64_t *>(pay)[3];
+        if (k >= 0) add_bit(u0, u1, k);
+        return bits_hash(u0, u1);
     }
-    if (k >= 0 && (k >> 6) == w) x |= 1ull << (k & 63);
-    return x;
+    return reinterpret_cast<const uint64_t *>(pay)[1] + (k >= 0 ? column_hash(k) : 0ull);
 }
 
-// Insert the support into the set of supports judged in this traversal (one
-// thread); h: the sum of its columns' hash constants.
-__device__ __noinline__ int insert_list(const LevelArgs &a, int W, const uint4 *pay, int pc, int k, uint64_t h)
+// Insert the support U + {k} into the set of supports judged in this
+// traversal (one thread; the arbiter reads bitset words).
+template <int F>
+__device__ __noinline__ int insert_candidate(const LevelArgs &a, int W, const uint4 *pay, int pc, int k)
 {
     uint64_t p;
     uint32_t tag;
-    slot_tag_pos(h, a.cslot_mask, p, tag);
+    slot_tag_pos(support_hash_of<F>(pay, k), a.cslot_mask, p, tag);
     for (uint64_t probe = 0; probe <= a.cslot_mask; ++probe) {
         unsigned long long v = atomicCAS(&a.cslots[p], kEmpty, ((unsigned long long)tag << 32) | kPending);
         if (v == kEmpty) {
@@ -106,8 +134,18 @@ __device__ __noinline__ int insert_list(const LevelArgs &a, int W, const uint4 *
                 return INS_ARENA_FULL;
             }
             uint64_t *dst = a.cand + (size_t)idx * W;
-            int pos = 0;
-            for (int w = 0; w < W; ++w) dst[w] = list_word(pay, pc, k, w, pos);
+            if (F) {
+                uint64_t u[2] = {reinterpret_cast<const uint64_t *>(pay)[2], reinterpret_cast<const uint64_t *>(pay)[3]};
+                if (k >= 0) add_bit(u[0], u[1], k);
+                for (int w = 0; w < W; ++w) dst[w] = w ? u[1] : u[0];
+            } else {
+                for (int w = 0; w < W; ++w) dst[w] = 0ull;
+                for (int i = 0; i < pc; ++i) {
+                    const int c = list_col(pay, i);
+                    dst[c >> 6] |= 1ull << (c & 63);
+                }
+                if (k >= 0) dst[k >> 6] |= 1ull << (k & 63);
+            }
             __threadfence();
             atomicExch(&a.cslots[p], ((unsigned long long)tag << 32) | idx);
             return INS_NEW;
@@ -126,8 +164,21 @@ __device__ __noinline__ int insert_list(const LevelArgs &a, int W, const uint4 *
             if (idx == kOverflowIdx) return INS_ARENA_FULL;
             const uint64_t *src = a.cand + (size_t)idx * W;
             bool eq = true;
-            int pos = 0;
-            for (int w = 0; w < W && eq; ++w) eq = __ldcg(src + w) == list_word(pay, pc, k, w, pos);
+            if (F) {
+                uint64_t u[2] = {reinterpret_cast<const uint64_t *>(pay)[2], reinterpret_cast<const uint64_t *>(pay)[3]};
+                if (k >= 0) add_bit(u[0], u[1], k);
+                for (int w = 0; w < W && eq; ++w) eq = __ldcg(src + w) == (w ? u[1] : u[0]);
+            } else {
+                // equal: as many columns, and each of them there
+                int n = 0;
+                for (int w = 0; w < W; ++w) n += __popcll(__ldcg(src + w));
+                eq = n == pc + (k >= 0 ? 1 : 0);
+                for (int i = 0; i < pc && eq; ++i) {
+                    const int c = list_col(pay, i);
+                    eq = (__ldcg(src + (c >> 6)) >> (c & 63)) & 1ull;
+                }
+                if (k >= 0 && eq) eq = (__ldcg(src + (k >> 6)) >> (k & 63)) & 1ull;
+            }
             if (eq) return INS_DUP;
         }
         p = (p + 1) & a.cslot_mask;
@@ -150,10 +201,34 @@ __device__ __forceinline__ uint32_t cell_slot(uint32_t key, uint32_t mask)
     return (x ^ (x >> 13)) & mask;
 }
 
-// Does a result E with k in E lie inside U + {k}?  One lane.  The cells
-// (k, s) of the sentinels s in U are looked up; a cell's results are tested
-// by signature, then column by column.
-__device__ __noinline__ bool pruned_cells(const CellIndex &ix, const uint16_t *rcols, const uint4 *pay, int pc, int k)
+// Does a result E with k in E lie inside U + {k}?  One lane.  Only the cells
+// (k, s) of the sentinels s in U are looked up.
+__device__ __forceinline__ bool pruned_bits(const CellIndex &ix, const uint4 *pay, int k)
+{
+    uint64_t u0 = reinterpret_cast<const uint64_t *>(pay)[2], u1 = reinterpret_cast<const uint64_t *>(pay)[3];
+    const ulonglong2 ks = reinterpret_cast<const ulonglong2 *>(ix.ksig)[k];
+    uint64_t m[2] = {ks.x & u0, ks.y & u1};
+    if (ix.single[k]) return true;
+    if ((m[0] | m[1]) == 0) return false;
+    add_bit(u0, u1, k);
+    const uint32_t *heads = reinterpret_cast<const uint32_t *>(ix.cells) + 128 * k;
+#pragma unroll
+    for (int w = 0; w < 2; ++w)
+        for (uint64_t x = m[w]; x; x &= x - 1) {
+            uint32_t head = heads[64 * w + __ffsll((long long)x) - 1];
+            // a list holds each result at most once: n_res bounds it
+            for (int64_t n = 0; head != kNoRecord && n < ix.n_res; ++n) {
+                const ulonglong2 e = *reinterpret_cast<const ulonglong2 *>(ix.ent + 2 * (size_t)head);
+                if (((e.x & ~u0) | (e.y & ~u1)) == 0) return true;
+                head = ix.ent[2 * (size_t)head + 1].x;
+            }
+        }
+    return false;
+}
+
+// The same on lists: a cell's results are tested by a 64-bit signature, then
+// column by column.
+__device__ __noinline__ bool pruned_list(const CellIndex &ix, const uint16_t *rcols, const uint4 *pay, int pc, int k)
 {
     if (ix.single[k]) return true;
     const uint64_t ks = ix.ksig[k];
@@ -176,20 +251,18 @@ __device__ __noinline__ bool pruned_cells(const CellIndex &ix, const uint16_t *r
             if (cell.x == kNoRecord) break;
             p = (p + 1) & ix.mask;
         }
-        // a list holds each result at most once: n_res bounds it
         for (int64_t n = 0; head != kNoRecord && n < ix.n_res; ++n) {
             const uint4 e = ix.ent[head];
             const uint64_t sig = (uint64_t)e.x | ((uint64_t)e.y << 32);
             if ((sig & ~su) == 0) {
                 const uint16_t *lst = rcols + (size_t)e.w * kRcolStride;
                 const int m = lst[0];
-                bool sub = true;
-                int q = 0;  // both lists ascend
+                bool sub = m <= pc + 1;
                 for (int j = 1; j <= m && sub; ++j) {
                     const int c = lst[j];
                     if (c == k) continue;
-                    while (q < pc && list_col(pay, q) < c) ++q;
-                    sub = q < pc && list_col(pay, q) == c;
+                    sub = false;
+                    for (int q = 0; q < pc && !sub; ++q) sub = list_col(pay, q) == c;
                 }
                 if (sub) return true;
             }
@@ -200,143 +273,298 @@ __device__ __noinline__ bool pruned_cells(const CellIndex &ix, const uint16_t *r
 }
 
 // ---------------------------------------------------------------------------
-// the AND update as a merge of two ascending lists
+// the AND update
 // ---------------------------------------------------------------------------
 
-// The entries of column k: S_int[:, k] and, in the subtractive view, flux 1
-// on k at row M + k.
+// pivot key of an entry of row `row` with the sign of t
 template <bool SUB>
-struct ColumnIter {
-    const uint32_t *ent;
-    int q, end, row;
-    int32_t val;
-    int flux_row;
-    __device__ __forceinline__ ColumnIter(const NetView &nv, const uint32_t *bl, int k)
-        : ent(bl + nv.o_colent), q((int)bl[nv.o_colptr + k]), end((int)bl[nv.o_colptr + k + 1]), flux_row(nv.M + k)
-    {
-        load();
-    }
-    __device__ __forceinline__ void load()
-    {
-        if (q < end) {
-            const uint32_t f = ent[q];
-            row = ent_index(f);
-            val = ent_coef(f);
-        } else if (SUB && q == end) {
-            row = flux_row;
-            val = 1;
-        } else {
-            row = kNoRow;
-            val = 0;
-        }
-    }
-    __device__ __forceinline__ void next()
-    {
-        ++q;
-        load();
-    }
-};
-
-// What one pass over the child's entries finds.
-struct Merged {
-    int nnz, nbal;     // entries; entries of balance rows
-    uint32_t key;      // pivot key of the balance rows
-    int32_t pv;        // the pivot's entry
-    uint64_t hash;
-    uint32_t g, om;    // gcd and OR of the magnitudes (entries that fit int32)
-    bool big, zflux;   // an entry left int32; a flux entry is not positive (Prop. 3)
-};
-
-// dst (null: nothing is written): where the entries go.
-template <bool SUB>
-__device__ __forceinline__ void merge_child(const NetView &nv, const uint32_t *bl, const int2 *pe, int np, int k,
-                                            int32_t A, int32_t C, uint4 *dst, Merged &r)
+__device__ __forceinline__ uint32_t entry_key(const NetView &nv, const uint32_t *bl, int row, bool positive)
 {
-    r.nnz = r.nbal = 0;
-    r.key = 0xFFFFFFFFu;
-    r.pv = 0;
-    r.hash = 0;
-    r.g = r.om = 0;
-    r.big = r.zflux = false;
-    ColumnIter<SUB> col(nv, bl, k);
-    int2 e = pe[0];  // a state has at least one entry
-    int pi = 1;
-    int sx = 0, sy = 0;  // an entry waiting for its pair (16-byte stores)
-    for (;;) {
-        const int row = e.x < col.row ? e.x : col.row;
-        if (row == kNoRow) break;
-        int64_t t = 0;
-        if (e.x == row) {
-            t = (int64_t)A * e.y;
-            e = pi < np ? pe[pi] : make_int2(kNoRow, 0);
-            ++pi;
-        }
-        if (col.row == row) {
-            t += (int64_t)C * col.val;
-            col.next();
-        }
-        if (SUB && row >= nv.M && t <= 0) r.zflux = true;
-        if (t == 0) continue;
-        const int32_t v = (int32_t)t;
-        const uint32_t av = (uint32_t)(v < 0 ? -v : v);
-        if (t != (int64_t)v || v == INT32_MIN) {
-            r.big = true;
-        } else {
-            r.om |= av;
-            if (r.g != 1u) r.g = gcd32(r.g, av);
-        }
-        r.hash += entry_hash(row, v);
-        if (!SUB || row < nv.M) {
-            if (SUB) ++r.nbal;
-            const uint32_t kk = bl[(t > 0 ? nv.o_keypos : nv.o_keyneg) + row];
-            if (kk < r.key) {
-                r.key = kk;
-                r.pv = v;
-            }
-        }
-        if (r.nnz & 1) {
-            if (dst) dst[r.nnz >> 1] = make_uint4((uint32_t)sx, (uint32_t)sy, (uint32_t)row, (uint32_t)v);
-        } else {
-            sx = row;
-            sy = v;
-        }
-        ++r.nnz;
-    }
-    if (dst && (r.nnz & 1)) dst[r.nnz >> 1] = make_uint4((uint32_t)sx, (uint32_t)sy, 0u, 0u);
-    if (!SUB) r.nbal = r.nnz;
+    if (SUB && row >= nv.M) return kFluxKey | (uint32_t)row;
+    return bl[(positive ? nv.o_keypos : nv.o_keyneg) + row];
 }
 
-// The rare child whose entries share a divisor or leave int32 before the
-// division: the gcd and the range in 64 bits, then the divided entries.
-// Returns true when some entry stays outside int32 (the child is dropped).
-template <bool SUB>
-__device__ __noinline__ bool settle_child(const NetView &nv, const uint32_t *bl, const int2 *pe, int np, int k,
-                                          int32_t A, int32_t C, uint4 *dst, Merged &r)
+// gcd of magnitudes that are mostly small (Euclid: one or two divisions)
+__device__ __forceinline__ uint32_t gcd_small(uint32_t a, uint32_t b)
 {
-    uint64_t g = 0, mx = 0;
-    for (int pass = 0; pass < 2; ++pass) {
-        ColumnIter<SUB> col(nv, bl, k);
-        int2 e = pe[0];
-        int pi = 1, n = 0;
-        int sx = 0, sy = 0;
-        if (pass == 1) {
-            if (g == 0 || mx / g > 2147483647ull) return true;
-            r.hash = 0;
-            r.om = 0;
+    while (a) {
+        const uint32_t t = b % a;
+        b = a;
+        a = t;
+    }
+    return b;
+}
+
+struct Child {
+    int n;          // entries
+    uint32_t key;   // smallest key (kFluxKey or above: no balance row is left)
+    int32_t pv;     // the entry of that key
+    uint32_t om;    // OR of the magnitudes
+    uint32_t g;     // gcd of the entries (1 as soon as it is known to be 1)
+    uint64_t rh;    // slow_child only
+    bool zflux;     // the flux of k is not positive any more (Prop. 3)
+    bool ovf;       // an entry outside int32 after the division (slow_child only)
+};
+
+// Column entries: words [cb, ce) of the column CSR, rows ascending; in the
+// subtractive view one more, flux 1 on k at row M + k.
+template <bool SUB>
+__device__ __forceinline__ void column_entry(const NetView &nv, const uint32_t *bl, int cb, int ce, int q, int k,
+                                             int &row, int32_t &val)
+{
+    if (SUB && cb + q == ce) {
+        row = nv.M + k;
+        val = 1;
+        return;
+    }
+    const uint32_t f = bl[nv.o_colent + cb + q];
+    row = ent_index(f);
+    val = ent_coef(f);
+}
+
+// One child, when every entry is known to fit int32, the parent has at most
+// 64 entries and the column at most 32 (dst null: nothing is written).
+template <bool SUB>
+__device__ __forceinline__ void fast_child(const NetView &nv, const uint32_t *bl, const uint4 *pe, int np, int32_t A,
+                                           int32_t C, int cb, int ce, uint64_t mask, int k, uint4 *dst, Child &r)
+{
+    uint32_t key = kPadKey, om = 0, mn = 0xFFFFFFFFu;  // mn: smallest magnitude
+    int32_t pv = 0;
+    uint64_t hits = 0;  // parent entries on a row whose mask bit column k sets
+    for (int i = 0; 2 * i < np; ++i) {
+        const uint4 e = pe[i];
+        const int32_t v0 = A * (int32_t)e.y, v1 = A * (int32_t)e.w;
+        const uint32_t h0 = (uint32_t)(mask >> (e.x & 63u)) & 1u;
+        const uint32_t h1 = e.w ? (uint32_t)(mask >> (e.z & 63u)) & 1u : 0u;  // (padding is no hit)
+        hits |= (uint64_t)(h0 | (h1 << 1)) << (2 * i);
+        const uint32_t a0 = h0 ? 0u : mag(v0), a1 = h1 ? 0u : mag(v1);
+        om |= a0 | a1;
+        mn = min(mn, min(a0 - 1u, a1 - 1u));  // less one: a hit or padding counts as none
+        const uint32_t k0 = h0 ? kPadKey : e.x, k1 = h1 ? kPadKey : e.z;
+        if (k0 < key) {
+            key = k0;
+            pv = v0;
         }
-        for (;;) {
-            const int row = e.x < col.row ? e.x : col.row;
-            if (row == kNoRow) break;
+        if (k1 < key) {
+            key = k1;
+            pv = v1;
+        }
+        if (dst) dst[i] = make_uint4(e.x, (uint32_t)v0, e.z, (uint32_t)v1);
+    }
+    const int2 *p2 = reinterpret_cast<const int2 *>(pe);
+    int2 *d2 = reinterpret_cast<int2 *>(dst);
+    const int nq = ce - cb + (SUB ? 1 : 0);
+    uint32_t matched = 0, g = 0;  // column entries met; gcd of the changed entries (while it is needed)
+    uint64_t holes = 0;
+    bool zflux = false;
+    int n = np;
+    auto take = [&](uint32_t kk, int32_t t) {
+        const uint32_t at = mag(t);
+        om |= at;
+        mn = min(mn, at - 1u);
+        if (mn != 0u) g = gcd_small(g, at);
+        if (kk < key) {
+            key = kk;
+            pv = t;
+        }
+    };
+    for (uint64_t h = hits; h; h &= h - 1) {
+        const int i = __ffsll((long long)h) - 1;
+        const int2 e = p2[i];
+        const int row = e.x & 0xFFFF;
+        int32_t cv = 0;
+        for (int q = 0; q < nq; ++q) {
+            int rq;
+            int32_t vq;
+            column_entry<SUB>(nv, bl, cb, ce, q, k, rq, vq);
+            if (rq == row) {
+                cv = vq;
+                matched |= 1u << q;
+                break;
+            }
+        }
+        const int32_t t = A * e.y + C * cv;
+        if (SUB && row == nv.M + k && t <= 0) zflux = true;
+        if (t == 0) {
+            holes |= 1ull << i;
+            continue;
+        }
+        const uint32_t kk = cv == 0 ? (uint32_t)e.x : entry_key<SUB>(nv, bl, row, t > 0);
+        take(kk, t);
+        if (d2) d2[i] = make_int2((int)kk, t);
+    }
+    for (int q = 0; q < nq; ++q) {
+        if ((matched >> q) & 1u) continue;
+        int row;
+        int32_t cv;
+        column_entry<SUB>(nv, bl, cb, ce, q, k, row, cv);
+        const int32_t t = C * cv;
+        if (SUB && row >= nv.M && t <= 0) zflux = true;
+        const uint32_t kk = entry_key<SUB>(nv, bl, row, t > 0);
+        take(kk, t);
+        int at = n;
+        if (holes) {
+            at = __ffsll((long long)holes) - 1;
+            holes &= holes - 1;
+        } else {
+            ++n;
+        }
+        if (d2) d2[at] = make_int2((int)kk, t);
+    }
+    while (holes) {  // close what is left with entries from the end
+        const int last = --n;
+        if (last < 64 && ((holes >> last) & 1ull)) {
+            holes &= ~(1ull << last);
+            continue;
+        }
+        const int at = __ffsll((long long)holes) - 1;
+        holes &= holes - 1;
+        if (d2) d2[at] = d2[last];
+    }
+    if (d2 && (n & 1)) d2[n] = make_int2((int)kPadKey, 0);
+    // the gcd: 1 with an entry of magnitude 1, or when the changed entries (which
+    // every common divisor divides) share none, or only powers of two beside
+    // an odd entry; else by the unchanged entries, until it is 1
+    if (mn == 0u || ((om & 1u) && g != 0u && (g & (g - 1u)) == 0u)) g = 1u;
+    if (g != 1u)
+        for (int i = 0; i < np && g != 1u; ++i)
+            if (!((hits >> i) & 1ull)) g = gcd_small(g, mag(A * p2[i].y));
+    r.n = n;
+    r.key = key;
+    r.pv = pv;
+    r.om = om;
+    r.g = g;
+    r.zflux = zflux;
+}
+
+// --- narrow networks ---
+
+__device__ __forceinline__ uint64_t blob_u64(const uint32_t *bl, int o)
+{
+    return *reinterpret_cast<const uint64_t *>(bl + o);
+}
+
+// values below row r in a state with nonzero rows zm
+__device__ __forceinline__ int value_at(uint64_t zm, int r) { return __popcll(zm & ((1ull << r) - 1ull)); }
+
+// pivot key from the two masks (kPadKey when balanced)
+__device__ __forceinline__ uint32_t mask_key(const uint32_t *bl, const NetView &nv, uint64_t pm, uint64_t nm)
+{
+    const uint32_t kp = pm ? bl[nv.o_keyr + __ffsll((long long)pm) - 1] : kPadKey;
+    const uint32_t kn = nm ? bl[nv.o_keyr + 64 + __ffsll((long long)nm) - 1] : kPadKey;
+    return kp < kn ? kp : kn;
+}
+
+struct NarrowMasks {
+    uint64_t zm, pm, nm;
+};
+
+constexpr int kNarrowCol = 8;  // column entries the fast path keeps in registers
+
+// One child of a narrow network, when every entry is known to fit int32 and
+// the column has at most kNarrowCol entries: the masks follow from the rows of
+// column k alone, the other values are copied (times A) to their places.
+__device__ __forceinline__ void narrow_child(const NetView &nv, const uint32_t *bl, const uint4 *pp, int32_t A,
+                                             int32_t C, int cb, int nc, int k, int32_t *dst, Child &r, NarrowMasks &z)
+{
+    const uint64_t zm = reinterpret_cast<const uint64_t *>(pp)[1];
+    const int32_t *vals = reinterpret_cast<const int32_t *>(pp + 3);
+    const int ox = nv.o_colx + 10 * k;
+    const uint64_t mask = blob_u64(bl, ox + 4);
+    const uint2 *ent = reinterpret_cast<const uint2 *>(bl + nv.o_nent) + cb;
+    int32_t t[kNarrowCol];
+    uint32_t om = 0, mn = 0xFFFFFFFFu;  // OR of the magnitudes; smallest magnitude less one
+    uint64_t newz = 0, newp = 0, newn = 0;
+#pragma unroll
+    for (int q = 0; q < kNarrowCol; ++q) {
+        t[q] = 0;
+        if (q < nc) {
+            const uint2 e = ent[q];
+            const int row = (int)(e.x & 63u);
+            int32_t v = 0;
+            if ((zm >> row) & 1ull) v = vals[value_at(zm, row)];
+            t[q] = A * v + C * (int32_t)e.y;
+            newz |= (uint64_t)(t[q] != 0) << row;
+            newp |= (uint64_t)(t[q] > 0) << ((e.x >> 8) & 63u);
+            newn |= (uint64_t)(t[q] < 0) << ((e.x >> 16) & 63u);
+            const uint32_t a = mag(t[q]);
+            om |= a;
+            mn = min(mn, a - 1u);
+        }
+    }
+    const uint64_t keep = zm & ~mask;
+    z.zm = keep | newz;
+    z.pm = (reinterpret_cast<const uint64_t *>(pp)[4] & ~blob_u64(bl, ox)) | newp;
+    z.nm = (reinterpret_cast<const uint64_t *>(pp)[5] & ~blob_u64(bl, ox + 2)) | newn;
+    // the unchanged rows, a 32-bit half at a time
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t zh = (uint32_t)(zm >> (32 * h)), yh = (uint32_t)(z.zm >> (32 * h));
+        const int32_t *src = vals + (h ? __popc((uint32_t)zm) : 0);
+        int32_t *to = dst + (h ? __popc((uint32_t)z.zm) : 0);
+        for (uint32_t x = (uint32_t)(keep >> (32 * h)); x; x &= x - 1u) {
+            const uint32_t below = (x & (0u - x)) - 1u;
+            const int32_t v = A * src[__popc(zh & below)];
+            const uint32_t a = mag(v);
+            om |= a;
+            mn = min(mn, a - 1u);
+            if (dst) to[__popc(yh & below)] = v;
+        }
+    }
+    r.n = __popcll(z.zm);
+    r.key = mask_key(bl, nv, z.pm, z.nm);
+    r.om = om;
+    // the gcd: 1 with an entry of magnitude 1; a power of two as the smallest
+    // magnitude beside an odd entry; else by the entries, until it is 1
+    uint32_t g = mn + 1u;
+    if ((om & 1u) && (g & (g - 1u)) == 0u) g = 1u;
+    const int piv = (int)(r.key & 63u);
+    int32_t pv = 0;
+#pragma unroll
+    for (int q = 0; q < kNarrowCol; ++q) {
+        if (q < nc) {
+            const int row = (int)(ent[q].x & 63u);
+            if (row == piv) pv = t[q];
+            if (t[q] != 0) {
+                if (g != 1u) g = gcd_small(g, mag(t[q]));
+                if (dst) dst[value_at(z.zm, row)] = t[q];
+            }
+        }
+    }
+    if (g != 1u)
+        for (uint64_t x = keep; x && g != 1u; x &= x - 1) g = gcd_small(g, mag(A * vals[value_at(zm, __ffsll((long long)x) - 1)]));
+    if (r.key < kFluxKey && ((keep >> piv) & 1ull)) pv = A * vals[value_at(zm, piv)];
+    r.pv = pv;
+    r.g = g;
+    r.zflux = false;
+    if (dst)
+        for (int i = r.n; i & 3; ++i) dst[i] = 0;
+}
+
+// Any child of a narrow network, in 64 bits (see slow_child).
+__device__ __noinline__ void slow_narrow(const NetView &nv, const uint32_t *bl, const uint4 *pp, int32_t A, int32_t C,
+                                         int cb, int ce, int k, int32_t *dst, Child &r, NarrowMasks &z)
+{
+    const uint64_t zm = reinterpret_cast<const uint64_t *>(pp)[1];
+    const int32_t *vals = reinterpret_cast<const int32_t *>(pp + 3);
+    const uint2 *ent = reinterpret_cast<const uint2 *>(bl + nv.o_nent);
+    const uint64_t mask = blob_u64(bl, nv.o_colx + 10 * k + 4);
+    uint64_t g = 0, mx = 0;
+    r.n = 0;
+    r.key = kPadKey;
+    r.pv = 0;
+    r.om = 0;
+    r.rh = 0;
+    r.zflux = r.ovf = false;
+    z.zm = z.pm = z.nm = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        int q = cb;  // rows ascend in the column and in the state
+        for (uint64_t x = zm | mask; x; x &= x - 1) {
+            const int row = __ffsll((long long)x) - 1;
             int64_t t = 0;
-            if (e.x == row) {
-                t = (int64_t)A * e.y;
-                e = pi < np ? pe[pi] : make_int2(kNoRow, 0);
-                ++pi;
-            }
-            if (col.row == row) {
-                t += (int64_t)C * col.val;
-                col.next();
-            }
+            if ((zm >> row) & 1ull) t = (int64_t)A * vals[value_at(zm, row)];
+            while (q < ce && (int)(ent[q].x & 63u) < row) ++q;
+            if (q < ce && (int)(ent[q].x & 63u) == row) t += (int64_t)C * (int32_t)ent[q].y;
             if (t == 0) continue;
             if (pass == 0) {
                 const uint64_t at = abs64(t);
@@ -345,51 +573,125 @@ __device__ __noinline__ bool settle_child(const NetView &nv, const uint32_t *bl,
                 continue;
             }
             const int32_t v = (int32_t)(t / (int64_t)g);
-            r.om |= (uint32_t)(v < 0 ? -v : v);
-            r.hash += entry_hash(row, v);
-            if (row == (int)(r.key & 0xFFFFu)) r.pv = v;
-            if (n & 1) {
-                if (dst) dst[n >> 1] = make_uint4((uint32_t)sx, (uint32_t)sy, (uint32_t)row, (uint32_t)v);
-            } else {
-                sx = row;
-                sy = v;
+            const uint32_t kk = bl[(v > 0 ? nv.o_keypos : nv.o_keyneg) + row];
+            const uint32_t rk = bl[nv.o_rank + row];
+            z.zm |= 1ull << row;
+            if (v > 0) z.pm |= 1ull << (rk & 0xFFu);
+            else z.nm |= 1ull << ((rk >> 8) & 0xFFu);
+            r.om |= mag(v);
+            r.rh += (uint64_t)(int64_t)v * row_hash(row);
+            if (kk < r.key) {
+                r.key = kk;
+                r.pv = v;
             }
-            ++n;
+            if (dst) dst[r.n] = v;
+            ++r.n;
         }
-        if (pass == 1 && dst && (n & 1)) dst[n >> 1] = make_uint4((uint32_t)sx, (uint32_t)sy, 0u, 0u);
+        if (pass == 0) {
+            if (g == 0) return;  // balanced (key stays kPadKey)
+            if (mx / g > 2147483647ull) {
+                r.ovf = true;
+                r.key = 0;
+                return;
+            }
+        }
     }
-    return false;
+    r.g = 1;
+    if (dst)
+        for (int i = r.n; i & 3; ++i) dst[i] = 0;
 }
 
-// The child's column list: the parent's, with k inserted at position ins
-// (ins < 0: a secondary step, the same columns).
-__device__ __forceinline__ void write_list(uint4 *dst, const uint4 *pp, int pc, int k, int ins, uint64_t uh)
+// payload units of n entries (values on narrow networks)
+template <int F>
+__device__ __forceinline__ int entry_units(int n)
 {
-    const int lu0 = sparse_list_units(pc);
-    const int lu1 = sparse_list_units(pc + (ins >= 0 ? 1 : 0));
-    const uint32_t *pw = reinterpret_cast<const uint32_t *>(pp) + 2;  // words of two columns
-    const int nw0 = 4 * lu0 - 2;
-    uint32_t prev = 0;
-    auto word = [&](int w) -> uint32_t {
-        const uint32_t x = w < nw0 ? pw[w] : 0xFFFFFFFFu;
-        uint32_t y = x;
-        if (ins >= 0) {
-            if (2 * w > ins) y = __funnelshift_l(prev, x, 16);
-            else if (2 * w == ins) y = (uint32_t)k | (x << 16);
-            else if (2 * w + 1 == ins) y = (x & 0xFFFFu) | ((uint32_t)k << 16);
+    return F == 2 ? (n + 3) >> 2 : (n + 1) >> 1;
+}
+
+// Any child: entries in 64 bits, the gcd and the range over all of them,
+// then the divided entries.  The rare child that may leave int32, shares a
+// divisor, or is long.
+template <bool SUB>
+__device__ __noinline__ void slow_child(const NetView &nv, const uint32_t *bl, const uint4 *pe, int np, int32_t A,
+                                        int32_t C, int cb, int ce, int k, uint4 *dst, Child &r)
+{
+    const int2 *p2 = reinterpret_cast<const int2 *>(pe);
+    int2 *d2 = reinterpret_cast<int2 *>(dst);
+    const int nq = ce - cb + (SUB ? 1 : 0);
+    uint32_t matched[(EFM_MAX_INTERNAL + 32) / 32];
+    for (int i = 0; 32 * i < nq; ++i) matched[i] = 0;
+    uint64_t g = 0, mx = 0;
+    r.n = 0;
+    r.key = kPadKey;
+    r.pv = 0;
+    r.om = 0;
+    r.rh = 0;
+    r.zflux = r.ovf = false;
+    int nbal = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        auto take = [&](int row, int64_t t) {
+            if (SUB && row == nv.M + k && t <= 0) r.zflux = true;
+            if (t == 0) return;
+            if (pass == 0) {
+                const uint64_t at = abs64(t);
+                g = gcd64(g, at);
+                mx = at > mx ? at : mx;
+                if (!SUB || row < nv.M) ++nbal;
+                return;
+            }
+            const int32_t v = (int32_t)(t / (int64_t)g);
+            const uint32_t kk = entry_key<SUB>(nv, bl, row, v > 0);
+            r.om |= mag(v);
+            r.rh += (uint64_t)(int64_t)v * row_hash(row);
+            if (kk < r.key) {
+                r.key = kk;
+                r.pv = v;
+            }
+            if (d2) d2[r.n] = make_int2((int)kk, v);
+            ++r.n;
+        };
+        for (int i = 0; i < np; ++i) {
+            const int2 e = p2[i];
+            const int row = e.x & 0xFFFF;
+            int64_t t = (int64_t)A * e.y;
+            int lo = 0, hi = nq;  // first column entry with a row >= row (they ascend)
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                int rq;
+                int32_t vq;
+                column_entry<SUB>(nv, bl, cb, ce, mid, k, rq, vq);
+                if (rq < row) lo = mid + 1;
+                else hi = mid;
+            }
+            if (lo < nq) {
+                int rq;
+                int32_t vq;
+                column_entry<SUB>(nv, bl, cb, ce, lo, k, rq, vq);
+                if (rq == row) {
+                    t += (int64_t)C * vq;
+                    matched[lo >> 5] |= 1u << (lo & 31);
+                }
+            }
+            take(row, t);
         }
-        prev = x;
-        return y;
-    };
-    {
-        const uint32_t a = word(0), b = word(1);
-        dst[0] = make_uint4((uint32_t)uh, (uint32_t)(uh >> 32), a, b);
+        for (int q = 0; q < nq; ++q) {
+            if ((matched[q >> 5] >> (q & 31)) & 1u) continue;
+            int row;
+            int32_t cv;
+            column_entry<SUB>(nv, bl, cb, ce, q, k, row, cv);
+            take(row, (int64_t)C * cv);
+        }
+        if (pass == 0) {
+            if (nbal == 0) return;  // balanced (key stays kPadKey)
+            if (mx / g > 2147483647ull) {
+                r.ovf = true;
+                r.key = 0;
+                return;
+            }
+        }
     }
-    for (int t = 1; t < lu1; ++t) {
-        const int w = 4 * t - 2;
-        const uint32_t a = word(w), b = word(w + 1), c = word(w + 2), d = word(w + 3);
-        dst[t] = make_uint4(a, b, c, d);
-    }
+    r.g = 1;
+    if (d2 && (r.n & 1)) d2[r.n] = make_int2((int)kPadKey, 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -403,6 +705,7 @@ struct CapScratch {
     uint32_t u[EFM_MAX_COLUMNS / 32];  // columns of the parent
 };
 
+template <int F>
 __device__ void cap_parent(const NetView &nv, const uint32_t *bl, CapScratch &s, const uint4 *pay, int pc, int lane)
 {
     __syncwarp();
@@ -410,8 +713,14 @@ __device__ void cap_parent(const NetView &nv, const uint32_t *bl, CapScratch &s,
     s.pp[lane] = 0;
     for (int i = lane; i < EFM_MAX_COLUMNS / 32; i += 32) s.u[i] = 0;
     __syncwarp();
-    for (int i = lane; i < pc; i += 32) {
-        const int c = list_col(pay, i);
+    const int n = F ? 128 : pc;
+    for (int i = lane; i < n; i += 32) {
+        int c = i;
+        if (F) {
+            if (!((reinterpret_cast<const uint64_t *>(pay)[2 + (i >> 6)] >> (i & 63)) & 1ull)) continue;
+        } else {
+            c = list_col(pay, i);
+        }
         atomicOr(&s.u[c >> 5], 1u << (c & 31));
         for (int q = (int)bl[nv.o_colptr + c]; q < (int)bl[nv.o_colptr + c + 1]; ++q) {
             const uint32_t f = bl[nv.o_colent + q];
@@ -428,8 +737,7 @@ __device__ void cap_parent(const NetView &nv, const uint32_t *bl, CapScratch &s,
 // such rows needs one more column that gives each of them the missing sign
 // and finds the opposite sign in U for every row of its own (twin rule kept).
 // The warp tries the columns able to fix the one-sided row with the shortest
-// list.  Sets *one_sided to the number of such rows; returns false when the
-// child can never balance.
+// list.  False when the child can never balance.
 __device__ bool cap_child(const NetView &nv, const uint32_t *bl, CapScratch &s, int k, int room, int lane)
 {
     uint32_t c = s.pc[lane], p = s.pp[lane];
@@ -443,7 +751,7 @@ __device__ bool cap_child(const NetView &nv, const uint32_t *bl, CapScratch &s, 
             }
         }
     }
-    uint32_t x = c ^ p;  // one-sided rows of this lane's word
+    const uint32_t x = c ^ p;  // one-sided rows of this lane's word
     const int nd = (int)__reduce_add_sync(FULL, (unsigned)__popc(x));
     if (nd == 0) return true;
     if (room == 0) return false;
@@ -490,31 +798,96 @@ __device__ bool cap_child(const NetView &nv, const uint32_t *bl, CapScratch &s, 
     return found;
 }
 
+// First-K bound, supports of equal size: does U + {k} come after the bound?
+// The support holding the lowest column of their difference comes first.
+struct BoundScratch {
+    uint32_t bits[EFM_MAX_COLUMNS / 32];
+    uint16_t cols[64];
+    int n;
+};
+
+template <int F>
+__device__ __noinline__ bool after_bound(const BoundScratch &b, const uint4 *pay, int pc, int k)
+{
+    if (F) {
+        uint64_t u[2] = {reinterpret_cast<const uint64_t *>(pay)[2], reinterpret_cast<const uint64_t *>(pay)[3]};
+        if (k >= 0) add_bit(u[0], u[1], k);
+        for (int w = 0; w < 2; ++w) {
+            const uint64_t d = u[w] ^ ((uint64_t)b.bits[2 * w] | ((uint64_t)b.bits[2 * w + 1] << 32));
+            if (d) return (u[w] & (d & (~d + 1))) == 0;
+        }
+        return false;
+    }
+    int own = 0x7FFFFFFF;  // the lowest column of U + {k} outside the bound
+    for (int i = 0; i < pc + (k >= 0 ? 1 : 0); ++i) {
+        const int c = i < pc ? list_col(pay, i) : k;
+        if (!((b.bits[c >> 5] >> (c & 31)) & 1u)) own = c < own ? c : own;
+    }
+    for (int j = 0; j < b.n; ++j) {  // ascending
+        const int c = (int)b.cols[j];
+        if (c > own) return false;
+        bool in = c == k;
+        for (int i = 0; i < pc && !in; ++i) in = list_col(pay, i) == c;
+        if (!in) return true;
+    }
+    return false;
+}
+
+// the hashes and the support of a child U + {k} (k < 0: U)
+template <int F>
+__device__ __forceinline__ void write_support(uint4 *dst, const uint4 *pp, int pc, int k, uint64_t rh, uint64_t uh,
+                                              const NarrowMasks &z)
+{
+    if (F) {
+        uint64_t u0 = reinterpret_cast<const uint64_t *>(pp)[2], u1 = reinterpret_cast<const uint64_t *>(pp)[3];
+        if (k >= 0) add_bit(u0, u1, k);
+        const uint64_t s = F == 2 ? z.zm : 0ull;
+        dst[0] = make_uint4((uint32_t)rh, (uint32_t)(rh >> 32), (uint32_t)s, (uint32_t)(s >> 32));
+        dst[1] = make_uint4((uint32_t)u0, (uint32_t)(u0 >> 32), (uint32_t)u1, (uint32_t)(u1 >> 32));
+        if (F == 2)
+            dst[2] = make_uint4((uint32_t)z.pm, (uint32_t)(z.pm >> 32), (uint32_t)z.nm, (uint32_t)(z.nm >> 32));
+    } else {
+        dst[0] = make_uint4((uint32_t)rh, (uint32_t)(rh >> 32), (uint32_t)uh, (uint32_t)(uh >> 32));
+        const int lu = sparse_list_units(pc);
+        for (int t = 1; t < lu; ++t) dst[t] = pp[t];
+        if (k >= 0) {
+            if ((pc & 7) == 0) dst[lu] = make_uint4(~0u, ~0u, ~0u, ~0u);
+            reinterpret_cast<uint16_t *>(dst)[8 + pc] = (uint16_t)k;
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Generate: one (parent, branch) item per lane, 32 children of a warp at a
-// time; a lane merges its parent's entries with column k's and writes its
-// child straight to the place reserved for it (rows and payload units of the
-// 32 children by one atomic each).  Nothing waits on another child.
+// time.  A lane writes its child straight to the row and the payload units
+// reserved for it (two prefix sums, two counters); nothing waits on another
+// child.  Children whose row or payload lies past the arena keep only their
+// fingerprint (the level is then decided from fingerprints, or run again with
+// a larger arena).
 // ---------------------------------------------------------------------------
-template <bool SUB, bool FK>
-__global__ void __launch_bounds__(kGenWarps * 32, 4) generate_sparse_kernel(NetView nv, LevelArgs a)
+template <int F, bool SUB, bool FK>
+__global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks) generate_kernel(NetView nv, LevelArgs a)
 {
     __shared__ CapScratch s_cap[FK ? kGenWarps : 1];
-    __shared__ uint16_t s_bound[FK ? 64 : 1];
+    __shared__ BoundScratch s_bound;
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
     const uint32_t *bl = nv.blob;
+    const uint4 *scol = reinterpret_cast<const uint4 *>(bl + nv.o_scol);
     const int64_t row_cap = a.child.cap;
     const uint64_t pay_cap = a.child.pay_cap;
-    unsigned long long n_exp = 0, n_ovf = 0, n_bal = 0, n_pruned = 0, n_unwritten = 0, n_zero = 0;
+    unsigned n_exp = 0, n_pruned = 0, n_unwritten = 0, n_zero = 0;  // a lane's share of a launch
     bool fatal = false;
     if (FK) {
-        if (a.fk_pc > 0) {  // the bound's columns, ascending (warp 0, word by word)
+        if (a.fk_pc > 0) {
+            for (int i = threadIdx.x; i < EFM_MAX_COLUMNS / 32; i += blockDim.x)
+                s_bound.bits[i] = i < 2 * nv.W ? (uint32_t)(a.fk_sup[i >> 1] >> (32 * (i & 1))) : 0u;
             if (threadIdx.x == 0) {
                 int n = 0;
                 for (int w = 0; w < nv.W; ++w)
                     for (uint64_t x = a.fk_sup[w]; x && n < 64; x &= x - 1)
-                        s_bound[n++] = (uint16_t)(w * 64 + __ffsll((long long)x) - 1);
+                        s_bound.cols[n++] = (uint16_t)(w * 64 + __ffsll((long long)x) - 1);
+                s_bound.n = n;
             }
         }
         __syncthreads();
@@ -526,14 +899,26 @@ __global__ void __launch_bounds__(kGenWarps * 32, 4) generate_sparse_kernel(NetV
     const int cpw = a.cpw;
     const int64_t worker = (int64_t)blockIdx.x * kGenWarps + wid;
     const int64_t wstride = (int64_t)gridDim.x * kGenWarps * cpw;
-    for (int64_t p0 = worker * cpw; p0 < a.n_par; p0 += wstride) {
+    // the lane's parent of a chunk: its row, payload offset and meta word
+    auto parent_at = [&](int64_t p0, uint32_t &pid, uint32_t &off, uint32_t &meta) {
         const int64_t pl = p0 + lane;
         const bool pin = lane < cpw && pl < a.n_par;
-        uint4 hd = make_uint4(0u, 0u, 0u, 0u);
-        if (pin) hd = a.par.hdr[a.perm ? (int64_t)a.perm[pl] : a.par_base + pl];
-        int dj = (int)((hd.y >> 10) & 0x1FFFu);
+        pid = pin ? (uint32_t)(a.perm ? (int64_t)a.perm[pl] : a.par_base + pl) : 0u;
+        off = meta = 0u;
+        if (pin) {
+            const uint2 h = *reinterpret_cast<const uint2 *>(a.par.hdr + pid);
+            off = h.x;
+            meta = h.y;
+        }
+    };
+    uint32_t pid_n, off_n, meta_n;  // the next chunk's, read one chunk ahead
+    parent_at(worker * cpw, pid_n, off_n, meta_n);
+    for (int64_t p0 = worker * cpw; p0 < a.n_par; p0 += wstride) {
+        const uint32_t pid = pid_n, mj = meta_n;
+        parent_at(p0 + wstride, pid_n, off_n, meta_n);
+        int dj = (int)((mj >> 10) & 0x1FFFu);
         // first-K: a parent larger than the bound has no descendant among the K smallest
-        if (FK && a.fk_pc > 0 && (int)((hd.y >> 23) & 0x7Fu) > a.fk_pc) dj = 0;
+        if (FK && a.fk_pc > 0 && (int)((mj >> 23) & 0x7Fu) > a.fk_pc) dj = 0;
         int incl = dj;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -542,13 +927,19 @@ __global__ void __launch_bounds__(kGenWarps * 32, 4) generate_sparse_kernel(NetV
         }
         const int prej = incl - dj;
         const int T = __shfl_sync(FULL, incl, 31);
-        if (T > 64 * nv.N) {
-            if (lane == 0) record_diag(a.ctr, ERR_BOUNDS, 3, T, 64 * nv.N, a.level);
+        if (T > 32 * nv.N) {
+            if (lane == 0) record_diag(a.ctr, ERR_BOUNDS, 3, T, 32 * nv.N, a.level);
             fatal = true;
         }
         uint32_t cap_for = kNoRecord;  // payload offset of the parent in s_cap
         for (int base = 0; base < T; base += 32) {
             if (__any_sync(FULL, fatal)) break;
+            // pull the next chunk's payloads toward L2 (its headers
+            // have arrived by the last round of this one)
+            if (base + 32 >= T && meta_n != 0u) {
+                prefetch_l2(a.par.pay + off_n);
+                prefetch_l2(a.par.pay + off_n + 6);
+            }
             // --- branch selection: one (parent, branch) item per lane ---
             const int c = base + lane;
             int j = 0;  // largest j with pre_j <= c
@@ -557,20 +948,23 @@ __global__ void __launch_bounds__(kGenWarps * 32, 4) generate_sparse_kernel(NetV
                 const int v = __shfl_sync(FULL, prej, j + step);
                 if (v <= c) j += step;
             }
-            const uint32_t hx = __shfl_sync(FULL, hd.x, j), hy = __shfl_sync(FULL, hd.y, j);
-            const uint32_t hz = __shfl_sync(FULL, hd.z, j);
-            const int32_t bi = (int32_t)__shfl_sync(FULL, hd.w, j);
+            const uint32_t pj = __shfl_sync(FULL, pid, j);
             const int q = c - __shfl_sync(FULL, prej, j);
-            const uint4 *pp = a.par.pay + hx;
-            const int pc = (int)((hy >> 23) & 0x7Fu), np = (int)(hz & 0x7FFu);
             bool okl = c < T;
-            int k = 0, ins = 0;
-            bool in_u = false;
+            int k = 0, pc = 0, np = 0, cb = 0, ce = 0;
+            bool in_u = false, fits = true, opp = false;
             int32_t A = 1, C = 0;
+            const uint4 *pp = a.par.pay;
             if (okl) {
-                const int piv = (int)(hy & 0x3FFu);
+                const uint4 hd = a.par.hdr[pj];
+                pp += hd.x;
+                pc = (int)((hd.y >> 23) & 0x7Fu);
+                np = (int)(hd.z & 0x7FFu);
+                const int mb = (int)((hd.z >> 11) & 0x1Fu);
+                const int32_t bi = (int32_t)hd.w;
+                const int piv = (int)(hd.y & 0x3FFu);
                 const bool fwd = bi > 0;  // forward flow: consume the surplus
-                const uint32_t abi = (uint32_t)(bi < 0 ? -bi : bi);
+                const uint32_t abi = mag(bi);
                 const int pr = piv < nv.M ? piv : 0;
                 const int lptr = (fwd ? nv.o_consptr : nv.o_prodptr) + pr;
                 const int lb = (int)bl[lptr], ln = (int)bl[lptr + 1] - lb;
@@ -584,31 +978,34 @@ __global__ void __launch_bounds__(kGenWarps * 32, 4) generate_sparse_kernel(NetV
                     fatal = true;
                     okl = false;
                 } else {
-                    const bool opp = SUB && q >= ln;
+                    opp = SUB && q >= ln;
                     const uint32_t br = opp ? bl[(fwd ? nv.o_prodent : nv.o_consent) + (int)bl[optr] + (q - ln)]
                                             : bl[(fwd ? nv.o_consent : nv.o_prodent) + lb + q];
                     k = ent_index(br);
                     const uint32_t sik = (uint32_t)ent_coef(br);  // |S_ik|
-                    const uint32_t tw = bl[nv.o_twin + k];        // -1: no twin (matches no column)
+                    const uint4 s1 = scol[2 * k + 1];
+                    cb = (int)s1.y;
+                    ce = (int)s1.z;
+                    const uint32_t tw = s1.w;  // ~0: no twin (matches no column)
                     bool twin = false;
-                    auto look = [&](uint32_t w) {
-                        const uint32_t c0 = w & 0xFFFFu, c1 = w >> 16;
-                        in_u = in_u || c0 == (uint32_t)k || c1 == (uint32_t)k;
-                        twin = twin || c0 == tw || c1 == tw;
-                        ins += (c0 < (uint32_t)k ? 1 : 0) + (c1 < (uint32_t)k ? 1 : 0);
-                    };
-                    const int lu = sparse_list_units(pc);
-                    {
-                        const uint4 u = pp[0];
-                        look(u.z);
-                        look(u.w);
-                    }
-                    for (int t = 1; t < lu; ++t) {
-                        const uint4 u = pp[t];
-                        look(u.x);
-                        look(u.y);
-                        look(u.z);
-                        look(u.w);
+                    if (F) {
+                        const uint32_t *u = reinterpret_cast<const uint32_t *>(pp + 1);  // the bitset
+                        in_u = (u[k >> 5] >> (k & 31)) & 1u;
+                        twin = tw != 0xFFFFFFFFu && ((u[tw >> 5] >> (tw & 31u)) & 1u);
+                    } else {
+                        auto look = [&](uint32_t w) {
+                            const uint32_t c0 = w & 0xFFFFu, c1 = w >> 16;
+                            in_u = in_u || c0 == (uint32_t)k || c1 == (uint32_t)k;
+                            twin = twin || c0 == tw || c1 == tw;
+                        };
+                        const int lu = sparse_list_units(pc);
+                        for (int t = 1; t < lu; ++t) {
+                            const uint4 u = pp[t];
+                            look(u.x);
+                            look(u.y);
+                            look(u.z);
+                            look(u.w);
+                        }
                     }
                     const int sec = a.level - pc;
                     if (opp)
@@ -618,26 +1015,15 @@ __global__ void __launch_bounds__(kGenWarps * 32, 4) generate_sparse_kernel(NetV
                     if (FK && okl && a.fk_pc > 0) {
                         // branch and bound: the child's descendants keep its
                         // support or grow it, so a child past the K-th result
-                        // found so far cannot yield one of the K smallest.  Of
-                        // two supports of equal size, the one whose ascending
-                        // list is smaller at the first difference comes first.
+                        // found so far cannot yield one of the K smallest
                         const int pc2 = pc + (in_u ? 0 : 1);
-                        if (pc2 > a.fk_pc) {
-                            okl = false;
-                        } else if (pc2 == a.fk_pc) {
-                            for (int i = 0; i < pc2; ++i) {
-                                const int own = in_u || i < ins ? list_col(pp, i) : (i == ins ? k : list_col(pp, i - 1));
-                                const int b = (int)s_bound[i];
-                                if (own != b) {
-                                    okl = own < b;
-                                    break;
-                                }
-                            }
-                        }
+                        okl = pc2 < a.fk_pc || (pc2 == a.fk_pc && !after_bound<F>(s_bound, pp, pc, in_u ? -1 : k));
                     }
                     const uint32_t g0 = (abi == 1u || sik == 1u) ? 1u : gcd32(abi, sik);
                     A = (int32_t)(sik / g0);
                     C = (int32_t)(abi / g0);
+                    // no entry of the child can leave int32
+                    fits = ((uint64_t)A << mb) + (uint64_t)(uint32_t)C * s1.x < 0x80000000ull;
                     if (opp) C = -C;  // Eq. 5: flux taken away from k
                 }
             }
@@ -646,7 +1032,8 @@ __global__ void __launch_bounds__(kGenWarps * 32, 4) generate_sparse_kernel(NetV
             // superset rule: the new column completes a result accepted at an
             // earlier level (counted below, once the child is known to be one)
             bool pr = false;
-            if (okl && !in_u && a.cells.n_res > 0) pr = pruned_cells(a.cells, a.rcols, pp, pc, k);
+            if (a.cells.n_res > 0 && okl && !in_u)
+                pr = F ? pruned_bits(a.cells, pp, k) : pruned_list(a.cells, a.rcols, pp, pc, k);
             // first-K length-cap rules.  dead: the child cannot balance any
             // more, unless it is balanced already (it then has no one-sided
             // row); skip: nor can its update leave int32, so nothing of it
@@ -655,31 +1042,30 @@ __global__ void __launch_bounds__(kGenWarps * 32, 4) generate_sparse_kernel(NetV
             if (FK) {
                 const bool at_cap = okl && !pr && a.cap_dead && pc2 >= a.max_len;
                 const bool below = okl && !pr && a.cap_dead && pc2 == a.max_len - 1;
-                bool one_sided = false;
+                bool stuck = false;
                 unsigned need = __ballot_sync(FULL, at_cap || below);
+                const uint32_t hx = (uint32_t)(pp - a.par.pay);
                 while (need) {
                     const int src = __ffs((int)need) - 1;
                     need &= need - 1;
                     const uint32_t ox = __shfl_sync(FULL, hx, src);
                     const int opc = __shfl_sync(FULL, pc, src);
-                    const int ok_ = __shfl_sync(FULL, in_u ? -1 : k, src);
+                    const int okc = __shfl_sync(FULL, in_u ? -1 : k, src);
                     const int room = __shfl_sync(FULL, below ? 1 : 0, src);
                     if (ox != cap_for) {
-                        cap_parent(nv, bl, s_cap[FK ? wid : 0], a.par.pay + ox, opc, lane);
+                        cap_parent<F>(nv, bl, s_cap[FK ? wid : 0], a.par.pay + ox, opc, lane);
                         cap_for = ox;
                     }
-                    const bool can = cap_child(nv, bl, s_cap[FK ? wid : 0], ok_, room, lane);
-                    if (lane == src) one_sided = !can;
+                    const bool can = cap_child(nv, bl, s_cap[FK ? wid : 0], okc, room, lane);
+                    if (lane == src) stuck = !can;
                 }
-                dead = one_sided || (at_cap && a.level - pc2 + 1 >= a.max_sec);
-                // |A| max|EF| + |C| max|S| below 2^31: no entry can overflow
-                skip = one_sided && ((uint64_t)A << ((hz >> 11) & 0x1Fu)) + (uint64_t)(uint32_t)C * EFM_MAX_COEF <
-                                        0x80000000ull;
+                dead = stuck || (at_cap && a.level - pc2 + 1 >= a.max_sec);
+                skip = stuck && fits;
             }
             // --- rows and payload units of the children of this round ---
-            const bool wr = okl && !pr && !dead;
-            const int cb = okl ? (int)bl[nv.o_colptr + k + 1] - (int)bl[nv.o_colptr + k] : 0;
-            const int units = wr ? sparse_list_units(pc2) + ((np + cb + (SUB ? 1 : 0) + 1) >> 1) : 0;
+            const bool wr = okl && !skip;
+            const int su2 = support_units<F>(pc2);
+            const int units = wr ? su2 + entry_units<F>(np + ce - cb + (SUB ? 1 : 0)) : 0;
             int usum = units;
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
@@ -720,41 +1106,58 @@ __global__ void __launch_bounds__(kGenWarps * 32, 4) generate_sparse_kernel(NetV
             const bool room = wr && (int64_t)idx < row_cap && off + (uint64_t)units <= pay_cap;
             uint4 *dst = room ? a.child.pay + off : nullptr;
             // --- the child ---
-            if (okl && !skip) {
-                const int2 *pe = entries_of(pp, pc);
-                const int lu2 = sparse_list_units(pc2);
-                Merged m;
-                merge_child<SUB>(nv, bl, pe, np, k, A, C, dst ? dst + lu2 : nullptr, m);
-                bool live = false;
-                const uint64_t uh = list_hash(pp) + (in_u ? 0ull : column_hash(k));
-                if (SUB && m.zflux) {
-                    ++n_zero;
-                } else if (m.nbal == 0) {
-                    ++n_bal;  // all metabolites stable: to the arbiter
-                    if (insert_list(a, nv.W, pp, pc, in_u ? -1 : k, uh) < INS_DUP) fatal = true;
-                } else if ((m.big || m.g != 1u) &&
-                           settle_child<SUB>(nv, bl, pe, np, k, A, C, dst ? dst + lu2 : nullptr, m)) {
-                    ++n_ovf;
-                } else if (pr) {
-                    ++n_pruned;
-                } else {
-                    live = !dead;
-                }
-                if (wr) {
-                    const bool written = live && dst != nullptr;
-                    if (written) write_list(dst, pp, pc, k, in_u ? -1 : ins, uh);
-                    if ((int64_t)idx < row_cap)
-                        a.child.hdr[idx] =
-                            written ? make_uint4((uint32_t)off, pack_meta(branch_key(bl, nv, m.key, SUB ? 1 : 0), pc2),
-                                                 (uint32_t)m.nnz | ((uint32_t)max_bits(m.om) << 11), (uint32_t)m.pv)
-                                    : make_uint4(0u, 0u, 0u, 0u);
-                    if (live && !written) ++n_unwritten;
-                    if ((int64_t)idx < a.fp_cap) {
-                        a.fp[idx] = live ? state_fp(m.hash, uh) : kDeadFp;
+            if (wr) {
+                uint4 *de = dst ? dst + su2 : nullptr;
+                uint64_t fp = kOpenFp | (uint64_t)pj | ((uint64_t)k << 32) | (in_u ? kOpenInU : 0ull) |
+                              (opp ? kOpenSub : 0ull) | (pr ? kOpenPruned : 0ull) | (dead ? kOpenDead : 0ull);
+                uint4 hd = make_uint4((uint32_t)off, 0u, 0u, 0u);  // an open child: where its payload may go
+                // (what the parent and the column hold is read again where it is
+                // needed, from L1, rather than kept in registers)
+                const bool fast = fits && (F == 2 ? ce - cb <= kNarrowCol : np <= 64 && ce - cb + (SUB ? 1 : 0) <= 32);
+                if (fast) {
+                    Child m;
+                    NarrowMasks z;
+                    if (F == 2) {
+                        narrow_child(nv, bl, pp, A, C, cb, ce - cb, k, reinterpret_cast<int32_t *>(de), m, z);
                     } else {
-                        record_diag(a.ctr, ERR_BOUNDS, 7, (long long)idx, a.fp_cap, a.level);
-                        fatal = true;
+                        const uint4 s0 = scol[2 * k];
+                        fast_child<SUB>(nv, bl, pp + support_units<F>(pc), np, A, C, cb, ce,
+                                        (uint64_t)s0.z | ((uint64_t)s0.w << 32), k, de, m);
                     }
+                    if (SUB && m.zflux) {
+                        ++n_zero;
+                        fp = kDeadFp;
+                    } else if (m.key >= kFluxKey) {
+                        fp |= kOpenBal;  // all metabolites stable
+                    } else if (pr || dead) {
+                        if (pr) ++n_pruned;
+                        fp = kDeadFp;
+                    } else if (m.g == 1u) {
+                        const uint64_t rh = (uint64_t)(int64_t)A * *reinterpret_cast<const uint64_t *>(pp) +
+                                            (uint64_t)(int64_t)C * *reinterpret_cast<const uint64_t *>(scol + 2 * k);
+                        const uint64_t uh = support_hash_of<F>(pp, in_u ? -1 : k);
+                        fp = state_fp(rh, uh);
+                        if (dst) {
+                            write_support<F>(dst, pp, pc, in_u ? -1 : k, rh, uh, z);
+                            hd.y = pack_meta(branch_key(bl, nv, m.key, SUB ? 1 : 0), pc2);
+                            hd.z = (uint32_t)m.n | ((uint32_t)max_bits(m.om) << 11);
+                            hd.w = (uint32_t)m.pv;
+                        } else {
+                            ++n_unwritten;
+                        }
+                    }
+                }
+                if ((int64_t)idx < row_cap) {
+                    // an open child's z: 1 when it has a payload
+                    if (fp >> 63) hd = make_uint4(hd.x, 0u, dst ? 1u : 0u, 0u);
+                    a.child.hdr[idx] = hd;
+                }
+                if ((int64_t)idx < a.fp_cap) {
+                    a.fp[idx] = fp;
+                    if ((fp >> 63) && fp != kDeadFp) a.open[atomicAdd(&a.ctr[C_OPEN], 1ull)] = (uint32_t)idx;
+                } else {
+                    record_diag(a.ctr, ERR_BOUNDS, 7, (long long)idx, a.fp_cap, a.level);
+                    fatal = true;
                 }
             }
         }
@@ -768,13 +1171,11 @@ __global__ void __launch_bounds__(kGenWarps * 32, 4) generate_sparse_kernel(NetV
         if (r < row_cap) a.child.hdr[r] = make_uint4(0u, 0u, 0u, 0u);
     }
     // one atomic per warp and counter
-    auto total = [&](unsigned long long v, int id) {
-        const unsigned s = __reduce_add_sync(FULL, (unsigned)v);  // a lane counts far below 2^27 items a launch
+    auto total = [&](unsigned v, int id) {
+        const unsigned s = __reduce_add_sync(FULL, v);
         if (lane == 0 && s) atomicAdd(&a.ctr[id], (unsigned long long)s);
     };
     total(n_exp, C_EXP);
-    total(n_ovf, C_OVF);
-    total(n_bal, C_BAL);
     total(n_pruned, C_PRUNED);
     total(n_unwritten, C_UNWRITTEN);
     total(n_zero, C_ZERO);
@@ -785,20 +1186,200 @@ __global__ void __launch_bounds__(kGenWarps * 32, 4) generate_sparse_kernel(NetV
 // survives in place, a later copy gets a zero meta word (no branches).
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ bool same_sparse(const Arena &ar, const uint4 &x, const uint4 &y)
+// The same support and the same entries (both in any order)?  One warp; the
+// payloads at px and py, |U| = pc, n entries.
+template <int F>
+__device__ bool same_state(const uint4 *px, const uint4 *py, int pc, int n, int lane)
 {
-    if (x.y != y.y || x.z != y.z || x.w != y.w) return false;
-    const int n = sparse_list_units((int)((x.y >> 23) & 0x7Fu)) + (((int)(x.z & 0x7FFu) + 1) >> 1);
-    const uint4 *p = ar.pay + x.x, *r = ar.pay + y.x;
-    bool eq = true;
-    for (int i = 0; i < n && eq; ++i) {
-        const uint4 u = __ldcg(p + i), v = __ldcg(r + i);
-        eq = u.x == v.x && u.y == v.y && u.z == v.z && u.w == v.w;
+    bool same = true;
+    if (F == 2) {  // masks and values: unit by unit
+        for (int i = lane; i < 3 + entry_units<F>(n); i += 32) {
+            const uint4 x = __ldcg(px + i), y = __ldcg(py + i);
+            same = same && x.x == y.x && x.y == y.y && x.z == y.z && x.w == y.w;
+        }
+        return __all_sync(FULL, same);
     }
-    return eq;
+    if (F) {
+        const uint4 x = __ldcg(px + 1), y = __ldcg(py + 1);
+        same = x.x == y.x && x.y == y.y && x.z == y.z && x.w == y.w;
+    } else {
+        const uint16_t *xl = reinterpret_cast<const uint16_t *>(px) + 8, *yl = reinterpret_cast<const uint16_t *>(py) + 8;
+        for (int i = lane; i < 64; i += 32) {
+            const int c = i < pc ? (int)__ldcg(xl + i) : -1;
+            bool in = i >= pc;
+            for (int j = 0; j < pc; ++j) in = in || (int)__ldcg(yl + j) == c;
+            same = same && in;
+        }
+    }
+    const int2 *xe = reinterpret_cast<const int2 *>(px + support_units<F>(pc));
+    const int2 *ye = reinterpret_cast<const int2 *>(py + support_units<F>(pc));
+    for (int i = lane; i < n; i += 32) {
+        const int2 e = __ldcg(xe + i);
+        bool in = false;
+        for (int j = 0; j < n; ++j) {
+            const int2 f = __ldcg(ye + j);
+            in = in || (f.x == e.x && f.y == e.y);
+        }
+        same = same && in;
+    }
+    return __all_sync(FULL, same);
 }
 
-__global__ void __launch_bounds__(256) dedup_sparse_kernel(LevelArgs a)
+// An open child of reserved row i: balanced (to the arbiter), or one whose
+// update needs 64 bits, a division or more entries than the generate pass
+// takes (about one in a thousand).  Returns its fingerprint (kDeadFp: none)
+// and its header; live rows without a payload count as unwritten.
+template <int F, bool SUB>
+__device__ __noinline__ uint64_t finish_open(const NetView &nv, const LevelArgs &a, uint64_t f, uint64_t i, uint4 &h)
+{
+    const uint32_t *bl = nv.blob;
+    const uint4 ph = a.par.hdr[(uint32_t)f];
+    const uint4 *pp = a.par.pay + ph.x;
+    const int pc = (int)((ph.y >> 23) & 0x7Fu), np = (int)(ph.z & 0x7FFu);
+    const int k = (int)((f >> 32) & 0xFFFu);
+    const bool in_u = (f & kOpenInU) != 0;
+    h = i < (uint64_t)a.child.cap ? a.child.hdr[i] : make_uint4(0u, 0u, 0u, 0u);
+    uint4 *dst = h.z ? a.child.pay + h.x : nullptr;
+    const uint32_t off = h.x;
+    h = make_uint4(0u, 0u, 0u, 0u);
+    if (f & kOpenBal) {
+        atomicAdd(&a.ctr[C_BAL], 1ull);
+        insert_candidate<F>(a, nv.W, pp, pc, in_u ? -1 : k);  // (a failure sets the error word)
+        return kDeadFp;
+    }
+    const int cb = (int)bl[nv.o_colptr + k], ce = (int)bl[nv.o_colptr + k + 1];
+    // A and C from the pivot's entry and the coefficient of k in the pivot's row
+    const int piv = (int)(ph.y & 0x3FFu);
+    uint32_t sik = 1;
+    for (int q = cb; q < ce; ++q) {
+        const uint32_t e = bl[nv.o_colent + q];
+        if (ent_index(e) == piv) sik = mag(ent_coef(e));
+    }
+    const uint32_t abi = mag((int32_t)ph.w), g0 = gcd32(abi, sik);
+    const int32_t A = (int32_t)(sik / g0), C = (f & kOpenSub) ? -(int32_t)(abi / g0) : (int32_t)(abi / g0);
+    const int pc2 = pc + (in_u ? 0 : 1);
+    Child m;
+    NarrowMasks z;
+    uint4 *de = dst ? dst + support_units<F>(pc2) : nullptr;
+    if (F == 2)
+        slow_narrow(nv, bl, pp, A, C, cb, ce, k, reinterpret_cast<int32_t *>(de), m, z);
+    else
+        slow_child<SUB>(nv, bl, pp + support_units<F>(pc), np, A, C, cb, ce, k, de, m);
+    if (SUB && m.zflux) {
+        atomicAdd(&a.ctr[C_ZERO], 1ull);
+        return kDeadFp;
+    }
+    if (m.key >= kFluxKey) {
+        atomicAdd(&a.ctr[C_BAL], 1ull);
+        insert_candidate<F>(a, nv.W, pp, pc, in_u ? -1 : k);
+        return kDeadFp;
+    }
+    if (m.ovf) {
+        atomicAdd(&a.ctr[C_OVF], 1ull);
+        return kDeadFp;
+    }
+    if (f & (kOpenPruned | kOpenDead)) {
+        if (f & kOpenPruned) atomicAdd(&a.ctr[C_PRUNED], 1ull);
+        return kDeadFp;
+    }
+    const uint64_t uh = support_hash_of<F>(pp, in_u ? -1 : k);
+    if (dst) {
+        write_support<F>(dst, pp, pc, in_u ? -1 : k, m.rh, uh, z);
+        h = make_uint4(off, pack_meta(branch_key(bl, nv, m.key, SUB ? 1 : 0), pc2),
+                       (uint32_t)m.n | ((uint32_t)max_bits(m.om) << 11), (uint32_t)m.pv);
+        a.child.hdr[i] = h;
+    } else {
+        atomicAdd(&a.ctr[C_UNWRITTEN], 1ull);
+    }
+    __threadfence();  // the row is complete before its slot is taken
+    return state_fp(m.rh, uh);
+}
+
+struct DedupSums {
+    unsigned keep = 0, unv = 0;
+    unsigned long long deg = 0;
+};
+
+// Insert a warp's rows (lane: row i, fingerprint f, kDeadFp for none, header
+// h) into the level's table.
+template <int F>
+__device__ __forceinline__ void dedup_insert(const LevelArgs &a, uint64_t i, uint64_t f, const uint4 &h, int lane,
+                                             DedupSums &sum)
+{
+    const uint64_t row_cap = (uint64_t)a.child.cap;
+    bool todo = f != kDeadFp;
+    uint64_t pos = 0, probe = 0;
+    uint32_t tag = 0;
+    slot_tag_pos(f, a.slot_mask, pos, tag);
+    if (todo && i >= 0xFFFFFFFEull) {
+        record_diag(a.ctr, ERR_BOUNDS, 10, (long long)i, 0xFFFFFFFEll, a.level);
+        todo = false;
+    }
+    const bool written = h.y != 0u;
+    while (__any_sync(FULL, todo)) {
+        bool cmp = false;
+        uint32_t ox = 0;
+        while (todo && !cmp) {
+            const unsigned long long v = atomicCAS(&a.slots[pos], kEmpty, ((unsigned long long)tag << 32) | i);
+            if (v == kEmpty) {  // first of its state
+                if (written) {
+                    ++sum.keep;
+                    sum.deg += (h.y >> 10) & 0x1FFFu;
+                } else {
+                    ++sum.unv;
+                }
+                todo = false;
+                break;
+            }
+            if ((uint32_t)(v >> 32) == tag) {
+                const uint64_t jrow = (uint32_t)v;
+                // (a row that holds a slot is never cleared)
+                uint4 o = make_uint4(0u, 0u, 0u, 0u);
+                if (jrow < row_cap) o = __ldcg(a.child.hdr + jrow);
+                // a row without its state written cannot be compared: the
+                // level is then decided from the lower bound, or run again
+                if (!written || o.y == 0u) {
+                    if (written) a.child.hdr[i].y = 0u;
+                    todo = false;
+                    break;
+                }
+                cmp = h.y == o.y && h.z == o.z && h.w == o.w &&
+                      __ldcg(reinterpret_cast<const uint64_t *>(a.child.pay + h.x)) ==
+                          __ldcg(reinterpret_cast<const uint64_t *>(a.child.pay + o.x));  // row hashes
+                ox = o.x;
+                if (cmp) break;
+            }
+            pos = (pos + 1) & a.slot_mask;
+            if (++probe > a.slot_mask) {
+                record_diag(a.ctr, ERR_TABLE_FULL, 8, (long long)i, (long long)a.slot_mask, a.level);
+                todo = false;
+            }
+        }
+        // the warp compares one pair at a time (a lane by itself would chain
+        // n^2 loads)
+        unsigned m = __ballot_sync(FULL, cmp);
+        while (m) {
+            const int src = __ffs((int)m) - 1;
+            m &= m - 1;
+            const uint32_t x = __shfl_sync(FULL, h.x, src), y = __shfl_sync(FULL, ox, src);
+            const uint32_t hy = __shfl_sync(FULL, h.y, src), hz = __shfl_sync(FULL, h.z, src);
+            const bool eq = same_state<F>(a.child.pay + x, a.child.pay + y, (int)((hy >> 23) & 0x7Fu),
+                                          (int)(hz & 0x7FFu), lane);
+            if (lane == src) {
+                if (eq) {  // a later copy
+                    a.child.hdr[i].y = 0u;
+                    todo = false;
+                } else {
+                    pos = (pos + 1) & a.slot_mask;
+                    ++probe;
+                }
+            }
+        }
+    }
+}
+
+template <int F, bool SUB>
+__global__ void __launch_bounds__(256, 6) dedup_kernel(NetView nv, LevelArgs a)
 {
     __shared__ unsigned long long s_keep[8], s_deg[8], s_unv[8];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -806,59 +1387,30 @@ __global__ void __launch_bounds__(256) dedup_sparse_kernel(LevelArgs a)
     uint64_t end = a.ctr[C_WRITTEN];
     end = end < (uint64_t)a.fp_cap ? end : (uint64_t)a.fp_cap;
     const uint64_t row_cap = (uint64_t)a.child.cap;
-    unsigned long long deg = 0, n_unv = 0, n_keep = 0;
-    bool fatal = false;
+    DedupSums sum;
+    const uint64_t t0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = begin + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end && !fatal; i += stride) {
-        const uint64_t f = a.fp[i];
-        if (f == kDeadFp) continue;
-        uint64_t pos;
-        uint32_t tag;
-        slot_tag_pos(f, a.slot_mask, pos, tag);
-        if (i >= 0xFFFFFFFEull) {
-            record_diag(a.ctr, ERR_BOUNDS, 10, (long long)i, 0xFFFFFFFEll, a.level);
-            fatal = true;
-            break;
-        }
+    // the open children, spread over the whole grid
+    const uint64_t n_open = a.ctr[C_OPEN];
+    for (uint64_t q0 = t0; q0 < n_open; q0 += stride) {
+        uint64_t i = 0, f = kDeadFp;
         uint4 h = make_uint4(0u, 0u, 0u, 0u);
-        if (i < row_cap) h = a.child.hdr[i];
-        const bool written = h.y != 0u;
-        for (uint64_t probe = 0;; ++probe) {
-            if (probe > a.slot_mask) {
-                record_diag(a.ctr, ERR_TABLE_FULL, 8, (long long)i, (long long)a.slot_mask, a.level);
-                fatal = true;
-                break;
-            }
-            const unsigned long long v = atomicCAS(&a.slots[pos], kEmpty, ((unsigned long long)tag << 32) | i);
-            if (v == kEmpty) {  // first of its state
-                if (written) {
-                    ++n_keep;
-                    deg += (h.y >> 10) & 0x1FFFu;
-                } else {
-                    ++n_unv;
-                }
-                break;
-            }
-            if ((uint32_t)(v >> 32) == tag) {
-                const uint64_t jrow = (uint32_t)v;
-                // (the other row's header may be cleared meanwhile only if it
-                // is a later copy itself, and a later copy holds no slot)
-                uint4 o = make_uint4(0u, 0u, 0u, 0u);
-                if (jrow < row_cap) o = __ldcg(a.child.hdr + jrow);
-                // a row without its state written cannot be compared: the
-                // level is then decided from the lower bound, or run again
-                if (!written || o.y == 0u) {
-                    if (written) a.child.hdr[i].y = 0u;
-                    break;
-                }
-                if (same_sparse(a.child, h, o)) {  // a later copy
-                    a.child.hdr[i].y = 0u;
-                    break;
-                }
-            }
-            pos = (pos + 1) & a.slot_mask;
+        if (q0 + lane < n_open) {
+            i = a.open[q0 + lane];
+            f = finish_open<F, SUB>(nv, a, a.fp[i], i, h);
+            if (h.y == 0u && i < row_cap) a.child.hdr[i] = h;
         }
+        dedup_insert<F>(a, i, f, h, lane, sum);
     }
+    for (uint64_t i0 = begin + t0; i0 < end; i0 += stride) {
+        const uint64_t i = i0 + lane;
+        uint64_t f = i < end ? a.fp[i] : kDeadFp;
+        if (f >> 63) f = kDeadFp;  // nothing, or an open child
+        uint4 h = make_uint4(0u, 0u, 0u, 0u);
+        if (f != kDeadFp && i < row_cap) h = a.child.hdr[i];
+        dedup_insert<F>(a, i, f, h, lane, sum);
+    }
+    unsigned long long deg = sum.deg, n_unv = sum.unv, n_keep = sum.keep;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         deg += __shfl_xor_sync(FULL, deg, off);
@@ -884,15 +1436,60 @@ __global__ void __launch_bounds__(256) dedup_sparse_kernel(LevelArgs a)
     }
 }
 
-__global__ void dedup_advance_sparse_kernel(unsigned long long *ctr) { ctr[C_DEDUP_BEGIN] = ctr[C_WRITTEN]; }
+__global__ void dedup_advance_kernel(unsigned long long *ctr)
+{
+    ctr[C_DEDUP_BEGIN] = ctr[C_WRITTEN];
+    ctr[C_OPEN] = 0ull;
+}
 
 // ---------------------------------------------------------------------------
 // seeds (INIT) and seed sets (Prop. 1)
 // ---------------------------------------------------------------------------
 
+// Entries of a state in ascending rows, with what its header and masks need.
+template <int F, bool SUB>
+struct EntryWriter {
+    const NetView &nv;
+    const uint32_t *bl;
+    uint4 *dst;
+    int n = 0;
+    uint32_t key = kPadKey, om = 0;
+    int32_t pv = 0;
+    uint64_t rh = 0;
+    NarrowMasks z{0, 0, 0};
+    __device__ EntryWriter(const NetView &nv_, const uint32_t *bl_, uint4 *dst_) : nv(nv_), bl(bl_), dst(dst_) {}
+    __device__ void put(int row, int32_t v)
+    {
+        const uint32_t kk = entry_key<SUB>(nv, bl, row, v > 0);
+        if (F == 2) {
+            const uint32_t rk = bl[nv.o_rank + row];
+            reinterpret_cast<int32_t *>(dst)[n] = v;
+            z.zm |= 1ull << row;
+            if (v > 0) z.pm |= 1ull << (rk & 0xFFu);
+            else z.nm |= 1ull << ((rk >> 8) & 0xFFu);
+        } else {
+            reinterpret_cast<int2 *>(dst)[n] = make_int2((int)kk, v);
+        }
+        ++n;
+        om |= mag(v);
+        rh += (uint64_t)(int64_t)v * row_hash(row);
+        if (kk < key) {
+            key = kk;
+            pv = v;
+        }
+    }
+    __device__ void done()
+    {
+        if (F == 2)
+            for (int i = n; i & 3; ++i) reinterpret_cast<int32_t *>(dst)[i] = 0;
+        else if (n & 1)
+            reinterpret_cast<int2 *>(dst)[n] = make_int2((int)kPadKey, 0);
+    }
+};
+
 // One thread per seed column; seeds are distinct columns (no deduplication).
-template <bool SUB>
-__global__ void __launch_bounds__(256) seed_sparse_kernel(NetView nv, LevelArgs a, int target)
+template <int F, bool SUB>
+__global__ void __launch_bounds__(256) seed_kernel(NetView nv, LevelArgs a, int target)
 {
     const uint32_t *bl = nv.blob;
     const int n_items = target >= 0 ? nv.metptr[target + 1] - nv.metptr[target] : nv.N;
@@ -906,22 +1503,18 @@ __global__ void __launch_bounds__(256) seed_sparse_kernel(NetView nv, LevelArgs 
         atomicAdd(&a.ctr[C_SEEDS], 1ull);
         // gcd of the column (with its flux 1 in the subtractive view)
         uint32_t g = SUB ? 1u : 0u;
-        int n = 0;
         const int qb = (int)bl[nv.o_colptr + k], qe = (int)bl[nv.o_colptr + k + 1];
-        for (int q = qb; q < qe; ++q) {
-            const int32_t v = ent_coef(bl[nv.o_colent + q]);
-            if (v == 0) continue;
-            g = gcd32(g, (uint32_t)(v < 0 ? -v : v));
-            ++n;
-        }
-        const uint64_t uh = column_hash(k);
-        if (n == 0) {
+        for (int q = qb; q < qe; ++q) g = gcd32(g, mag(ent_coef(bl[nv.o_colent + q])));
+        // the support {k}: an empty payload plus k
+        const uint4 empty[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+        const uint64_t uh = support_hash_of<F>(empty, k);
+        if (qb == qe) {
             atomicAdd(&a.ctr[C_BAL], 1ull);
-            insert_list(a, nv.W, nullptr, 0, k, uh);
+            insert_candidate<F>(a, nv.W, empty, 0, k);
             continue;
         }
-        const int nnz = n + (SUB ? 1 : 0);
-        const int units = sparse_list_units(1) + ((nnz + 1) >> 1);
+        const int n = qe - qb + (SUB ? 1 : 0);
+        const int units = support_units<F>(1) + entry_units<F>(n);
         const uint64_t idx = atomicAdd(&a.ctr[C_NEXT], 1ull);
         const uint64_t off = atomicAdd(&a.ctr[C_PAY], (unsigned long long)units);
         if ((int64_t)idx >= a.child.cap) continue;
@@ -930,64 +1523,53 @@ __global__ void __launch_bounds__(256) seed_sparse_kernel(NetView nv, LevelArgs 
             continue;
         }
         uint4 *dst = a.child.pay + off;
-        dst[0] = make_uint4((uint32_t)uh, (uint32_t)(uh >> 32), (uint32_t)k | (kPadCol << 16), 0xFFFFFFFFu);
-        int2 *pe = reinterpret_cast<int2 *>(dst + sparse_list_units(1));
-        int w = 0;
-        uint32_t key = 0xFFFFFFFFu, om = 0;
-        int32_t pv = 0;
-        for (int q = qb; q < qe; ++q) {
-            const uint32_t f = bl[nv.o_colent + q];
-            const int row = ent_index(f);
-            const int32_t v = ent_coef(f) / (int32_t)g;
-            if (v == 0) continue;
-            pe[w++] = make_int2(row, v);
-            om |= (uint32_t)(v < 0 ? -v : v);
-            const uint32_t kk = bl[(v > 0 ? nv.o_keypos : nv.o_keyneg) + row];
-            if (kk < key) {
-                key = kk;
-                pv = v;
-            }
+        if (F) {
+            uint64_t u0 = 0, u1 = 0;
+            add_bit(u0, u1, k);
+            dst[1] = make_uint4((uint32_t)u0, (uint32_t)(u0 >> 32), (uint32_t)u1, (uint32_t)(u1 >> 32));
+        } else {
+            dst[1] = make_uint4((uint32_t)k | 0xFFFF0000u, ~0u, ~0u, ~0u);
         }
-        if (SUB) {
-            pe[w++] = make_int2(nv.M + k, 1);
-            om |= 1u;
+        EntryWriter<F, SUB> out(nv, bl, dst + support_units<F>(1));
+        for (int q = 0; q < n; ++q) {
+            int row;
+            int32_t v;
+            column_entry<SUB>(nv, bl, qb, qe, q, k, row, v);
+            out.put(row, v / (int32_t)g);
         }
-        if (w & 1) pe[w] = make_int2(0, 0);
+        out.done();
+        const uint64_t s0 = F == 2 ? out.z.zm : (F ? 0ull : uh);
+        dst[0] = make_uint4((uint32_t)out.rh, (uint32_t)(out.rh >> 32), (uint32_t)s0, (uint32_t)(s0 >> 32));
+        if (F == 2)
+            dst[2] = make_uint4((uint32_t)out.z.pm, (uint32_t)(out.z.pm >> 32), (uint32_t)out.z.nm, (uint32_t)(out.z.nm >> 32));
+        const uint32_t key = out.key, om = out.om;
+        const int32_t pv = out.pv;
         const uint32_t bkey = branch_key(bl, nv, key, SUB ? 1 : 0);
-        a.child.hdr[idx] = make_uint4((uint32_t)off, pack_meta(bkey, 1),
-                                      (uint32_t)w | ((uint32_t)max_bits(om) << 11), (uint32_t)pv);
+        a.child.hdr[idx] =
+            make_uint4((uint32_t)off, pack_meta(bkey, 1), (uint32_t)n | ((uint32_t)max_bits(om) << 11), (uint32_t)pv);
         atomicAdd(&a.ctr[C_DEGSUM], (unsigned long long)(bkey >> 16));
     }
 }
 
 // One state with flux 1 on each column of R_in: EF = the sum of their S_int
 // columns, normalised.  One warp; the sums in shared memory.
-template <bool SUB>
-__global__ void __launch_bounds__(32) seedset_sparse_kernel(NetView nv, LevelArgs a, const int32_t *cols, int n_cols)
+template <int F, bool SUB>
+__global__ void __launch_bounds__(32) seedset_kernel(NetView nv, LevelArgs a, const int32_t *cols, int n_cols)
 {
     __shared__ long long acc[EFM_MAX_INTERNAL];
-    __shared__ uint16_t sorted[64];
     const int lane = threadIdx.x;
     const uint32_t *bl = nv.blob;
     const int rows = nv.M + (SUB ? nv.N : 0);  // at most EFM_MAX_INTERNAL
     for (int r = lane; r < EFM_MAX_INTERNAL; r += 32) acc[r] = 0;
     __syncwarp();
-    uint64_t uh = 0;
     for (int i = 0; i < n_cols; ++i) {
         const int k = cols[i];
-        uh += column_hash(k);
         for (int q = (int)bl[nv.o_colptr + k] + lane; q < (int)bl[nv.o_colptr + k + 1]; q += 32) {
             const uint32_t f = bl[nv.o_colent + q];
             acc[ent_index(f)] += ent_coef(f);  // a column's rows are distinct
         }
         if (SUB && lane == 0) acc[nv.M + k] += 1;
         __syncwarp();
-    }
-    // ascending columns: a column's place is the number of smaller ones
-    for (int i = lane; i < n_cols; i += 32) {
-        int pos = 0;
-        for (int j = 0; j < n_cols; ++j) pos += cols[j] < cols[i] ? 1 : 0;
-        sorted[pos] = (uint16_t)cols[i];
     }
     uint64_t g = 0;
     int n = 0, nb = 0;
@@ -1008,49 +1590,51 @@ __global__ void __launch_bounds__(32) seedset_sparse_kernel(NetView nv, LevelArg
     bool bad = false;
     for (int r = lane; r < rows; r += 32) bad = bad || abs64(acc[r]) / g > 2147483647ull;
     bad = __any_sync(FULL, bad);
-    __syncwarp();
-    if (lane == 0) atomicAdd(&a.ctr[C_SEEDS], 1ull);
+    if (lane != 0) return;
+    // the rest by one lane: at most 64 columns and 1024 entries
+    atomicAdd(&a.ctr[C_SEEDS], 1ull);
     if (bad) {
-        if (lane == 0) atomicAdd(&a.ctr[C_OVF], 1ull);
+        atomicAdd(&a.ctr[C_OVF], 1ull);
         return;
     }
-    if (lane != 0) return;
-    // the payload, by one lane: at most 64 columns and 1024 entries
-    const int lu = sparse_list_units(n_cols);
-    const int units = lu + ((n + 1) >> 1);
+    const int su = support_units<F>(n_cols);
+    const int units = su + entry_units<F>(n);
     if (a.child.cap < 1 || (uint64_t)units > a.child.pay_cap) {
         record_diag(a.ctr, ERR_BOUNDS, 13, units, (long long)a.child.pay_cap, a.level);
         return;
     }
-    uint16_t *lst = reinterpret_cast<uint16_t *>(a.child.pay);
-    *reinterpret_cast<uint64_t *>(a.child.pay) = uh;
-    for (int i = 0; i < 8 * lu - 4; ++i) lst[4 + i] = i < n_cols ? sorted[i] : (uint16_t)kPadCol;
+    uint4 *dst = a.child.pay;
+    uint64_t uh = 0;
+    if (F) {
+        uint64_t u0 = 0, u1 = 0;
+        for (int i = 0; i < n_cols; ++i) add_bit(u0, u1, cols[i]);
+        dst[1] = make_uint4((uint32_t)u0, (uint32_t)(u0 >> 32), (uint32_t)u1, (uint32_t)(u1 >> 32));
+    } else {
+        uint16_t *lst = reinterpret_cast<uint16_t *>(dst) + 8;
+        for (int i = 0; i < 8 * su - 8; ++i) {
+            lst[i] = i < n_cols ? (uint16_t)cols[i] : (uint16_t)0xFFFFu;
+            if (i < n_cols) uh += column_hash(cols[i]);
+        }
+        reinterpret_cast<uint64_t *>(dst)[1] = uh;
+    }
     if (nb == 0) {
         atomicAdd(&a.ctr[C_BAL], 1ull);
-        insert_list(a, nv.W, a.child.pay, n_cols, -1, uh);
+        insert_candidate<F>(a, nv.W, dst, n_cols, -1);
         return;
     }
-    int2 *pe = reinterpret_cast<int2 *>(a.child.pay + lu);
-    int w = 0;
-    uint32_t key = 0xFFFFFFFFu, om = 0;
-    int32_t pv = 0;
-    for (int r = 0; r < rows; ++r) {
-        if (acc[r] == 0) continue;
-        const int32_t v = (int32_t)(acc[r] / (long long)g);
-        pe[w++] = make_int2(r, v);
-        om |= (uint32_t)(v < 0 ? -v : v);
-        if (r < nv.M) {
-            const uint32_t kk = bl[(v > 0 ? nv.o_keypos : nv.o_keyneg) + r];
-            if (kk < key) {
-                key = kk;
-                pv = v;
-            }
-        }
-    }
-    if (w & 1) pe[w] = make_int2(0, 0);
+    EntryWriter<F, SUB> out(nv, bl, dst + su);
+    for (int r = 0; r < rows; ++r)
+        if (acc[r] != 0) out.put(r, (int32_t)(acc[r] / (long long)g));
+    out.done();
+    const uint64_t s0 = F == 2 ? out.z.zm : uh;
+    dst[0] = make_uint4((uint32_t)out.rh, (uint32_t)(out.rh >> 32), (uint32_t)s0, (uint32_t)(s0 >> 32));
+    if (F == 2)
+        dst[2] = make_uint4((uint32_t)out.z.pm, (uint32_t)(out.z.pm >> 32), (uint32_t)out.z.nm, (uint32_t)(out.z.nm >> 32));
+    const uint32_t key = out.key, om = out.om;
+    const int32_t pv = out.pv;
+    const int w = out.n;
     const uint32_t bkey = branch_key(bl, nv, key, SUB ? 1 : 0);
-    a.child.hdr[0] = make_uint4(0u, pack_meta(bkey, n_cols), (uint32_t)w | ((uint32_t)max_bits(om) << 11),
-                                (uint32_t)pv);
+    a.child.hdr[0] = make_uint4(0u, pack_meta(bkey, n_cols), (uint32_t)w | ((uint32_t)max_bits(om) << 11), (uint32_t)pv);
     atomicAdd(&a.ctr[C_NEXT], 1ull);
     atomicAdd(&a.ctr[C_PAY], (unsigned long long)units);
     atomicAdd(&a.ctr[C_DEGSUM], (unsigned long long)(bkey >> 16));
@@ -1060,63 +1644,99 @@ __global__ void __launch_bounds__(32) seedset_sparse_kernel(NetView nv, LevelArg
 // the superset rule's index over the accepted results
 // ---------------------------------------------------------------------------
 
-__global__ void cell_count_kernel(const uint16_t *rcols, int64_t n, int32_t *cnt)
+// Both kernels take the results [r0, r1), a warp each: results are filed once,
+// at the level after the one that accepted them (the sentinels by the counts
+// of that moment: any other column of a result is a valid sentinel).
+__global__ void cell_count_kernel(const uint64_t *res, int W, int64_t r0, int64_t r1, int32_t *cnt)
 {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const uint16_t *lst = rcols + (size_t)r * kRcolStride;
-    for (int j = 1; j <= (int)lst[0]; ++j) atomicAdd(&cnt[lst[j]], 1);
+    const int lane = threadIdx.x & 31;
+    for (int64_t r = r0 + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); r < r1;
+         r += ((int64_t)gridDim.x * blockDim.x) >> 5)
+        for (int w = lane; w < W; w += 32)
+            for (uint64_t x = res[(size_t)r * W + w]; x; x &= x - 1) atomicAdd(&cnt[w * 64 + __ffsll((long long)x) - 1], 1);
 }
 
-__global__ void cell_insert_kernel(const uint16_t *rcols, int64_t n, const int32_t *cnt, uint2 *cells, uint32_t mask,
-                                   uint4 *ent, int ent_stride, unsigned long long *ksig, uint32_t *single)
+template <int F>
+__global__ void cell_insert_kernel(const uint64_t *res, int W, int64_t r0, int64_t r1, const int32_t *cnt, CellIndex ix,
+                                   int ent_stride)
 {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n) return;
-    const uint16_t *lst = rcols + (size_t)r * kRcolStride;
-    const int m = lst[0];
-    if (m == 1) {  // a one-column result: every child adding that column contains it
-        single[lst[1]] = 1u;
-        return;
-    }
-    // the two columns with the fewest results (ties by column)
-    int m1 = -1, m2 = -1;
-    long long k1 = 0x7FFFFFFFFFFFFFFFll, k2 = 0x7FFFFFFFFFFFFFFFll;
-    uint64_t sig = 0;
-    for (int j = 1; j <= m; ++j) {
-        const int c = lst[j];
-        sig |= col_bit(c);
-        const long long key = ((long long)cnt[c] << 16) | c;
-        if (key < k1) {
-            k2 = k1;
-            m2 = m1;
-            k1 = key;
-            m1 = c;
-        } else if (key < k2) {
-            k2 = key;
-            m2 = c;
-        }
-    }
-    for (int j = 1; j <= m; ++j) {
-        const int k = lst[j];
-        const int s = k == m1 ? m2 : m1;
-        atomicOr(&ksig[k], (unsigned long long)col_bit(s));
-        const uint32_t key = ((uint32_t)k << 12) | (uint32_t)s;
-        const int64_t id = r * ent_stride + (j - 1);
-        uint32_t p = cell_slot(key, mask);
-        for (uint32_t probe = 0; probe <= mask; ++probe) {
-            const uint32_t v = atomicCAS(&cells[p].x, kNoRecord, key);
-            if (v == kNoRecord || v == key) {
-                const uint32_t next = atomicExch(&cells[p].y, (uint32_t)id);
-                ent[id] = make_uint4((uint32_t)sig, (uint32_t)(sig >> 32), next, (uint32_t)r);
-                break;
+    const int lane = threadIdx.x & 31;
+    for (int64_t r = r0 + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); r < r1;
+         r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const uint64_t *E = res + (size_t)r * W;
+        const uint64_t word[2] = {lane < W ? E[lane] : 0ull, lane + 32 < W ? E[lane + 32] : 0ull};
+        // the two columns with the fewest results (ties by column), and the signature
+        unsigned long long k1 = ~0ull, k2 = ~0ull;
+        uint64_t sig = 0;
+        int m = 0;
+        for (int h = 0; h < 2; ++h)
+            for (uint64_t x = word[h]; x; x &= x - 1) {
+                const int c = (lane + 32 * h) * 64 + __ffsll((long long)x) - 1;
+                ++m;
+                sig |= col_bit(c);
+                const unsigned long long key = ((unsigned long long)cnt[c] << 16) | (unsigned)c;
+                if (key < k1) {
+                    k2 = k1;
+                    k1 = key;
+                } else if (key < k2) {
+                    k2 = key;
+                }
             }
-            p = (p + 1) & mask;
+        int before = m;  // columns of the lanes below
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int x = __shfl_up_sync(FULL, before, off);
+            if (lane >= off) before += x;
         }
+        const int total = __shfl_sync(FULL, before, 31);
+        before -= m;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const unsigned long long o1 = __shfl_xor_sync(FULL, k1, off), o2 = __shfl_xor_sync(FULL, k2, off);
+            const unsigned long long hi = k1 > o1 ? k1 : o1;  // the second of the four
+            k2 = k2 < o2 ? k2 : o2;
+            k2 = k2 < hi ? k2 : hi;
+            k1 = k1 < o1 ? k1 : o1;
+            sig |= __shfl_xor_sync(FULL, sig, off);
+        }
+        const int m1 = (int)(k1 & 0xFFFFull), m2 = (int)(k2 & 0xFFFFull);
+        if (total == 1) {  // a one-column result: every child adding that column contains it
+            if (lane == 0) ix.single[m1] = 1u;
+            continue;
+        }
+        int64_t id = r * ent_stride + before;
+        for (int h = 0; h < 2; ++h)
+            for (uint64_t x = word[h]; x; x &= x - 1, ++id) {
+                const int k = (lane + 32 * h) * 64 + __ffsll((long long)x) - 1;
+                const int s = k == m1 ? m2 : m1;
+                if (F) {
+                    atomicOr((unsigned long long *)&ix.ksig[2 * k + (s >> 6)], 1ull << (s & 63));
+                    const uint32_t next = atomicExch(reinterpret_cast<uint32_t *>(ix.cells) + 128 * k + s, (uint32_t)id);
+                    const uint64_t e0 = E[0], e1 = W == 2 ? E[1] : 0ull;
+                    ix.ent[2 * id] = make_uint4((uint32_t)e0, (uint32_t)(e0 >> 32), (uint32_t)e1, (uint32_t)(e1 >> 32));
+                    ix.ent[2 * id + 1] = make_uint4(next, (uint32_t)r, 0u, 0u);
+                    continue;
+                }
+                atomicOr((unsigned long long *)&ix.ksig[k], (unsigned long long)col_bit(s));
+                const uint32_t key = ((uint32_t)k << 12) | (uint32_t)s;
+                uint32_t p = cell_slot(key, ix.mask);
+                for (uint32_t probe = 0; probe <= ix.mask; ++probe) {
+                    const uint32_t v = atomicCAS(&ix.cells[p].x, kNoRecord, key);
+                    if (v == kNoRecord || v == key) {
+                        const uint32_t next = atomicExch(&ix.cells[p].y, (uint32_t)id);
+                        ix.ent[id] = make_uint4((uint32_t)sig, (uint32_t)(sig >> 32), next, (uint32_t)r);
+                        break;
+                    }
+                    p = (p + 1) & ix.mask;
+                }
+            }
+        __syncwarp();
     }
 }
 
-__global__ void live_sparse_kernel(const uint4 *hdr, int64_t n, uint32_t *live, unsigned long long *count)
+// Surviving rows [0, n) of an arena appended to a list, for the passes that
+// sample a frontier.
+__global__ void live_list_kernel(const uint4 *hdr, int64_t n, uint32_t *live, unsigned long long *count)
 {
     const int lane = threadIdx.x & 31;
     for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll; i0 < n;
@@ -1131,88 +1751,125 @@ __global__ void live_sparse_kernel(const uint4 *hdr, int64_t n, uint32_t *live, 
     }
 }
 
-template <bool SUB, bool FK>
-int grid_of(int sm_count)
+template <typename K>
+int grid_of(K kernel, int sm_count)
 {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, generate_sparse_kernel<SUB, FK>, kGenWarps * 32, 0) !=
-            cudaSuccess ||
-        per_sm < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kGenWarps * 32, 0) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         per_sm = 1;
     }
     return sm_count * per_sm;
 }
 
+// one of the kernel's instances: form, subtractive view, first-K rules
+#define EFM_GENERATE(CALL)                                                        \
+    do {                                                                          \
+        if (nv.form == 2) {                                                       \
+            if (first_k) CALL((generate_kernel<2, false, true>));                 \
+            else CALL((generate_kernel<2, false, false>));                        \
+        } else if (nv.form == 1) {                                                \
+            if (sub) CALL((generate_kernel<1, true, false>));                     \
+            else if (first_k) CALL((generate_kernel<1, false, true>));            \
+            else CALL((generate_kernel<1, false, false>));                        \
+        } else {                                                                  \
+            if (sub) CALL((generate_kernel<0, true, false>));                     \
+            else if (first_k) CALL((generate_kernel<0, false, true>));            \
+            else CALL((generate_kernel<0, false, false>));                        \
+        }                                                                         \
+    } while (0)
+
+// the same for a kernel without first-K rules
+#define EFM_FORM(KERNEL, CALL)                                                    \
+    do {                                                                          \
+        if (nv.form == 2) CALL((KERNEL<2, false>));                               \
+        else if (nv.form == 1 && a.sub) CALL((KERNEL<1, true>));                  \
+        else if (nv.form == 1) CALL((KERNEL<1, false>));                          \
+        else if (a.sub) CALL((KERNEL<0, true>));                                  \
+        else CALL((KERNEL<0, false>));                                            \
+    } while (0)
+
 }  // namespace
 
-int sparse_grid(bool sub, bool first_k, int sm_count)
+int generate_grid(const NetView &nv, bool sub, bool first_k, int sm_count)
 {
-    if (sub) return grid_of<true, false>(sm_count);
-    return first_k ? grid_of<false, true>(sm_count) : grid_of<false, false>(sm_count);
+    int grid = sm_count;
+#define EFM_GRID(K) grid = grid_of(K, sm_count)
+    EFM_GENERATE(EFM_GRID);
+#undef EFM_GRID
+    return grid;
 }
 
-cudaError_t launch_generate_sparse(const NetView &nv, const LevelArgs &a, int grid, cudaStream_t s)
+cudaError_t launch_generate(const NetView &nv, const LevelArgs &a, int grid, cudaStream_t s)
 {
-    if (a.sub)
-        generate_sparse_kernel<true, false><<<grid, kGenWarps * 32, 0, s>>>(nv, a);
-    else if (a.cap_dead || a.fk_pc > 0)
-        generate_sparse_kernel<false, true><<<grid, kGenWarps * 32, 0, s>>>(nv, a);
-    else
-        generate_sparse_kernel<false, false><<<grid, kGenWarps * 32, 0, s>>>(nv, a);
+    const bool sub = a.sub != 0, first_k = a.cap_dead || a.fk_pc > 0;
+#define EFM_LAUNCH(K) K<<<grid, kGenWarps * 32, 0, s>>>(nv, a)
+    EFM_GENERATE(EFM_LAUNCH);
+#undef EFM_LAUNCH
     return cudaGetLastError();
 }
 
-cudaError_t launch_dedup_sparse(const LevelArgs &a, int sm_count, cudaStream_t s)
+cudaError_t launch_dedup(const NetView &nv, const LevelArgs &a, int sm_count, cudaStream_t s)
 {
-    dedup_sparse_kernel<<<sm_count * 8, 256, 0, s>>>(a);
-    dedup_advance_sparse_kernel<<<1, 1, 0, s>>>(a.ctr);
+#define EFM_LAUNCH(K) K<<<sm_count * 8, 256, 0, s>>>(nv, a)
+    EFM_FORM(dedup_kernel, EFM_LAUNCH);
+#undef EFM_LAUNCH
+    dedup_advance_kernel<<<1, 1, 0, s>>>(a.ctr);
     return cudaGetLastError();
 }
 
-cudaError_t launch_seed_sparse(const NetView &nv, const LevelArgs &a, int target, cudaStream_t s)
+cudaError_t launch_seed(const NetView &nv, const LevelArgs &a, int target, cudaStream_t s)
 {
-    const int blocks = 4;
-    if (a.sub)
-        seed_sparse_kernel<true><<<blocks, 256, 0, s>>>(nv, a, target);
-    else
-        seed_sparse_kernel<false><<<blocks, 256, 0, s>>>(nv, a, target);
+#define EFM_LAUNCH(K) K<<<4, 256, 0, s>>>(nv, a, target)
+    EFM_FORM(seed_kernel, EFM_LAUNCH);
+#undef EFM_LAUNCH
     return cudaGetLastError();
 }
 
-cudaError_t launch_seedset_sparse(const NetView &nv, const LevelArgs &a, const int32_t *cols, int n_cols,
-                                  cudaStream_t s)
+cudaError_t launch_seedset(const NetView &nv, const LevelArgs &a, const int32_t *cols, int n_cols, cudaStream_t s)
 {
-    if (a.sub)
-        seedset_sparse_kernel<true><<<1, 32, 0, s>>>(nv, a, cols, n_cols);
-    else
-        seedset_sparse_kernel<false><<<1, 32, 0, s>>>(nv, a, cols, n_cols);
+#define EFM_LAUNCH(K) K<<<1, 32, 0, s>>>(nv, a, cols, n_cols)
+    EFM_FORM(seedset_kernel, EFM_LAUNCH);
+#undef EFM_LAUNCH
     return cudaGetLastError();
 }
 
-cudaError_t launch_cells(const NetView &nv, const uint16_t *rcols, int64_t n_res, int32_t *cnt, const CellIndex &ix,
-                         int ent_stride, cudaStream_t s)
+size_t cell_table_bytes(const NetView &nv, uint64_t entries)
+{
+    if (nv.W <= 2) return (size_t)128 * 128 * 4;
+    uint64_t p = 64;
+    while (p < 2 * entries) p <<= 1;
+    return (size_t)p * 8;
+}
+
+cudaError_t launch_cells(const NetView &nv, const uint64_t *res, int64_t r0, int64_t r1, int32_t *cnt,
+                         const CellIndex &ix, int ent_stride, cudaStream_t s)
 {
     cudaError_t e;
-    if ((e = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)nv.N, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ix.ksig, 0, 8 * (size_t)nv.N, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ix.single, 0, 4 * (size_t)nv.N, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ix.cells, 0xFF, 8 * ((size_t)ix.mask + 1), s)) != cudaSuccess) return e;
-    if (n_res <= 0) return cudaSuccess;
-    const int tb = 128;
-    const unsigned blocks = (unsigned)((n_res + tb - 1) / tb);
-    cell_count_kernel<<<blocks, tb, 0, s>>>(rcols, n_res, cnt);
-    cell_insert_kernel<<<blocks, tb, 0, s>>>(rcols, n_res, cnt, ix.cells, ix.mask, ix.ent, ent_stride,
-                                            (unsigned long long *)ix.ksig, ix.single);
+    const int W = nv.W;
+    if (r0 == 0) {
+        const size_t table = W <= 2 ? (size_t)128 * nv.N * 4 : 8 * ((size_t)ix.mask + 1);
+        if ((e = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)nv.N, s)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(ix.ksig, 0, 16 * (size_t)nv.N, s)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(ix.single, 0, 4 * (size_t)nv.N, s)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(ix.cells, 0xFF, table, s)) != cudaSuccess) return e;
+    }
+    if (r1 <= r0) return cudaSuccess;
+    const unsigned blocks = (unsigned)std::min<int64_t>((r1 - r0 + 3) / 4, 4096);
+    cell_count_kernel<<<blocks, 128, 0, s>>>(res, W, r0, r1, cnt);
+    if (W <= 2)
+        cell_insert_kernel<1><<<blocks, 128, 0, s>>>(res, W, r0, r1, cnt, ix, ent_stride);
+    else
+        cell_insert_kernel<0><<<blocks, 128, 0, s>>>(res, W, r0, r1, cnt, ix, ent_stride);
     return cudaGetLastError();
 }
 
-cudaError_t launch_live_sparse(const uint4 *hdr, int64_t n, uint32_t *live, unsigned long long *count, int sm_count,
-                               cudaStream_t s)
+cudaError_t launch_live_list(const uint4 *hdr, int64_t n, uint32_t *live, unsigned long long *count, int sm_count,
+                             cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
     const int64_t blocks = std::min<int64_t>((n + 255) / 256, (int64_t)sm_count * 8);
-    live_sparse_kernel<<<(unsigned)blocks, 256, 0, s>>>(hdr, n, live, count);
+    live_list_kernel<<<(unsigned)blocks, 256, 0, s>>>(hdr, n, live, count);
     return cudaGetLastError();
 }
 
