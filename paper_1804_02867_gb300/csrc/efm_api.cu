@@ -392,12 +392,13 @@ int alloc_work(Work &w, const efm_net *net, const efm_limits &lim, int total_war
     w.cslot_cap = next_pow2(2 * (uint64_t)w.cand_cap);
     const size_t W = (size_t)nv.W;
     bool ok = alloc_arena(w, 0, rows, units, s) && alloc_arena(w, 1, rows, units, s);
-    ok = ok && ensure_level_tables(w, 1024 + 32 * (uint64_t)total_warps, s);
+    // (a start: a level that needs more makes them grow)
+    ok = ok && ensure_level_tables(w, std::min<uint64_t>(2 * (uint64_t)rows, 1u << 19), s);
     ok = ok && dev_alloc(w.cslots, w.cslot_cap * 8, s);
     ok = ok && dev_alloc(w.cand, (size_t)w.cand_cap * W * 8, s);
     ok = ok && dev_alloc(w.res, (size_t)w.res_cap * W * 8, s);
     ok = ok && dev_alloc(w.bcnt, (size_t)nv.N * 4, s);
-    ok = ok && dev_alloc(w.ctr, C_COUNT * 8, s);
+    ok = ok && dev_alloc(w.ctr, (C_COUNT + S_COUNT) * 8, s);
     if (nv.W > 2) ok = ok && dev_alloc(w.rcols, (size_t)w.res_cap * kRcolStride * 2, s);
     ok = ok && dev_alloc(w.ksig, (size_t)nv.N * 16, s) && dev_alloc(w.csingle, (size_t)nv.N * 4, s);
     if (lim.first_k > 0) ok = ok && dev_alloc(w.fkb, W * 8, s);
@@ -513,14 +514,19 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
 {
     const NetView &nv = view_of(net, lim);
     cudaStream_t s = net->stream;
-    const int grid = level_grid(nv, lim, net->sm_count);
-    const int total_warps = grid * kExpandWarps;
-    unsigned long long *ctr = (unsigned long long *)w.ctr.p;
-    unsigned long long h[C_COUNT];
+    const int full_grid = level_grid(nv, lim, net->sm_count);
+    unsigned long long *ctr = (unsigned long long *)w.ctr.p, *st = ctr + C_COUNT;
+    unsigned long long h[C_COUNT + S_COUNT];
+    const unsigned long long *hs = h + C_COUNT;
     efm_counters &c = out.ctr;
     memset(&c, 0, sizeof(c));
+    const bool fk = lim.first_k > 0;
+    const bool manual = fk || trace;  // the host looks at every level
+    const int level0 = fs ? fs->level : (seedset ? n_seedset - 1 : 0);
 
     LevelArgs a{};
+    a.st = st;
+    a.manual = manual ? 1 : 0;
     a.cslots = (unsigned long long *)w.cslots.p;
     a.cslot_mask = w.cslot_cap - 1;
     a.cand = (uint64_t *)w.cand.p;
@@ -531,7 +537,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
     a.max_sec = lim.max_secondary;
     a.ctr = ctr;
     a.sub = lim.variant == EFM_SUBTRACTIVE ? 1 : 0;
-    a.cap_dead = lim.first_k > 0 ? 1 : 0;
+    a.cap_dead = fk ? 1 : 0;
     auto arena = [&](int i) {
         Arena r{};
         r.hdr = (uint4 *)w.hdr[i].p;
@@ -540,25 +546,6 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         r.pay_cap = w.pay_cap[i];
         return r;
     };
-
-    CK(cudaMemsetAsync(ctr, 0, C_COUNT * 8, s));
-    CK(cudaMemsetAsync(w.cslots.p, 0xFF, w.cslot_cap * 8, s));
-    CK(cudaEventRecord(w.ev[0], s));
-
-    // level 0: seeds (or the seed set's one state, at level |R_in| - 1),
-    // written densely: the first level reads its parents in arena order
-    int cur = 0;
-    const int level0 = fs ? fs->level : (seedset ? n_seedset - 1 : 0);
-    a.level = level0;
-    a.child = arena(cur);
-    if (fs) {
-        // the first parents are the caller's rows: nothing to seed
-    } else if (seedset) {
-        CK(launch_seedset(nv, a, seedset, n_seedset, s));
-    } else {
-        CK(launch_seed(nv, a, target, s));
-    }
-    out.kernel_launches += fs ? 0 : 1;
     AcceptArgs acc{};
     acc.cand = (const uint64_t *)w.cand.p;
     acc.res = (uint64_t *)w.res.p;
@@ -566,6 +553,47 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
     acc.rcols = (uint16_t *)w.rcols.p;
     acc.ctr = ctr;
     acc.cand_cap = w.cand_cap;
+    acc.st = st;
+    acc.level0 = level0;
+    acc.max_level = lim.max_len + lim.max_secondary + 1;
+    acc.max_frontier = lim.max_frontier;
+    acc.max_results = lim.max_results;
+
+    // the superset rule's index, with room for `results` results (filed ones: the first n)
+    auto build_index = [&](int64_t results, int64_t n) -> int {
+        const int64_t need = results * (int64_t)lim.max_len;
+        if (need > w.cent_cap) {
+            dev_free(w.cent, s);
+            dev_free(w.cells, s);
+            w.cent_cap = 0;
+            if (!dev_alloc(w.cent, (size_t)need * (nv.W <= 2 ? 32 : 16), s) ||
+                !dev_alloc(w.cells, cell_table_bytes(nv, (uint64_t)need), s))
+                return EFM_ENOMEM;
+            w.cent_cap = need;
+        }
+        CellIndex &ix = a.cells;
+        ix.cells = (uint2 *)w.cells.p;
+        ix.mask = nv.W <= 2 ? 0u : (uint32_t)(cell_table_bytes(nv, (uint64_t)need) / 8 - 1);
+        ix.ent = (uint4 *)w.cent.p;
+        ix.ksig = (uint64_t *)w.ksig.p;
+        ix.single = (uint32_t *)w.csingle.p;
+        ix.cnt = (int32_t *)w.bcnt.p;
+        ix.ent_stride = lim.max_len;
+        ix.room = results;
+        acc.ix = ix;
+        CK(launch_index(nv, ix, (const uint64_t *)w.res.p, n, s));
+        out.kernel_launches += n > 0 ? 1 : 0;
+        return EFM_OK;
+    };
+    auto set_tables = [&]() {
+        a.slots = (unsigned long long *)w.slots.p;
+        a.fp = (uint64_t *)w.fp.p;
+        a.fp_cap = w.fp_cap;
+        a.open = (uint32_t *)w.open.p;
+        acc.fp_cap = w.fp_cap;
+        acc.slot_cap = w.slot_cap;
+    };
+    // the counters and the level state
     auto read_ctr = [&]() -> int {
         if (cudaMemcpyAsync(h, ctr, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) {
@@ -573,91 +601,181 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             return EFM_ECUDA;
         }
         const int e = err_from_bits(h[C_ERR]);
-        if (e != EFM_OK && getenv("EFM_DEBUG"))
-            fprintf(stderr, "efm: device error bits %llx diag code %llu value %lld limit %lld level %lld\n",
-                    h[C_ERR], h[C_DIAG], (long long)h[C_DIAG + 1], (long long)h[C_DIAG + 2],
-                    (long long)h[C_DIAG + 3]);
+        if (getenv("EFM_DEBUG"))
+            fprintf(stderr, "efm: level %llu stop %llu rows %llu states %llu branches %llu children so far %llu results %llu "
+                    "error bits %llx (code %llu value %lld limit %lld level %lld)\n",
+                    hs[S_LEVEL], hs[S_STOP], hs[S_NROWS], hs[S_NFRONT], hs[S_DEG], h[C_EXP], h[C_RES_N], h[C_ERR],
+                    h[C_DIAG], (long long)h[C_DIAG + 1], (long long)h[C_DIAG + 2], (long long)h[C_DIAG + 3]);
         return e;
     };
-    const bool fk = lim.first_k > 0;
+    auto put_state = [&](int i, unsigned long long v) -> int {
+        h[C_COUNT + i] = v;
+        CK(cudaMemcpyAsync(st + i, &h[C_COUNT + i], 8, cudaMemcpyHostToDevice, s));
+        CK(cudaStreamSynchronize(s));
+        return EFM_OK;
+    };
+    // CTAs of a generate launch over a level with `deg` branches: all, or at
+    // small levels one per SM (a launch's cost grows with its CTAs)
+    auto grid_for = [&](uint64_t deg) { return deg <= (uint64_t)net->sm_count * 64 ? std::min(net->sm_count, full_grid) : full_grid; };
+    // one expansion and the minimality test of its balanced supports
+    auto launch_level = [&](int level, int grid, int advance) -> int {
+        a.level = acc.level = level;
+        acc.advance = advance;
+        a.warps = grid * kExpandWarps;
+        acc.warps = full_grid * kExpandWarps;
+        acc.child_rows = a.child.cap;
+        CK(launch_generate(nv, a, grid, s));
+        CK(launch_dedup(nv, a, grid < full_grid ? (net->sm_count + 7) / 8 : net->sm_count, s));
+        CK(launch_accept_new(nv, acc, net->sm_count, s));
+        out.kernel_launches += 3;
+        return EFM_OK;
+    };
+
+    CK(cudaMemsetAsync(ctr, 0, sizeof(h), s));
+    CK(cudaMemsetAsync(w.cslots.p, 0xFF, w.cslot_cap * 8, s));
+    int rc = build_index(std::max<int64_t>(2048, w.cent_cap / std::max(lim.max_len, 1)), 0);
+    if (rc) return rc;
+    set_tables();
+    CK(cudaEventRecord(w.ev[0], s));
+
+    // level 0: seeds (or the seed set's one state, at level |R_in| - 1),
+    // written densely: the first level reads its parents in arena order
+    int cur = 0;
+    a.level = level0;
+    a.child = arena(cur);
+    int64_t res_n = 0;
     std::vector<uint64_t> window(fk ? (size_t)kResultWindow * nv.W : 0);
     TopK top;
     top.K = lim.first_k;
     top.W = nv.W;
-    CK(launch_accept_new(nv, acc, net->sm_count, s));
-    out.kernel_launches += 2;
-    int rc = read_ctr();
-    if (rc) return rc;
-    int64_t res_n = (int64_t)std::min<unsigned long long>(h[C_RES_N], (unsigned long long)w.res_cap);
-    if (fk && res_n > 0) {
-        std::vector<uint64_t> fresh((size_t)res_n * nv.W);
-        CK(cudaMemcpyAsync(fresh.data(), w.res.p, fresh.size() * 8, cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        top.add(fresh.data(), res_n);
-        if (top.pc > 0) CK(cudaMemcpyAsync(w.fkb.p, top.kth.data(), (size_t)nv.W * 8, cudaMemcpyHostToDevice, s));
-    }
-    if (fk && seed_top && !seed_top->empty()) {
-        top.add(seed_top->data(), (int64_t)(seed_top->size() / nv.W));
-        if (top.pc > 0) CK(cudaMemcpyAsync(w.fkb.p, top.kth.data(), (size_t)nv.W * 8, cudaMemcpyHostToDevice, s));
-    }
-    int64_t n_front = fs ? fs->r1 - fs->r0 : (int64_t)h[C_NEXT];  // distinct states of the level
-    int64_t n_rows = n_front;              // arena rows the next level reads (seeds are dense)
-    double row_units = 0.0;                // payload units of the level's rows
-    uint64_t deg_sum = fs ? fs->deg_sum : h[C_DEGSUM];
     int status = 0;
     bool split = false;  // the K smallest come from the parts of a split level (top)
-    c.levels = 1;
     bool stop = false;
-    if (lim.max_frontier > 0 && n_front > lim.max_frontier) {
-        status |= EFM_TRUNCATED;
-        stop = true;
-    } else if (!fs && n_front > w.rows[cur]) {
-        return EFM_ECAPACITY;
+    if (fs) {
+        // the first parents are the caller's rows: nothing to seed
+        const int64_t n = fs->r1 - fs->r0;
+        memset(h, 0, sizeof(h));
+        unsigned long long *x = h + C_COUNT;
+        x[S_LEVEL] = (unsigned long long)level0;
+        x[S_NROWS] = x[S_NFRONT] = (unsigned long long)n;
+        x[S_DEG] = fs->deg_sum;
+        x[S_RESERVED] = fs->deg_sum + 64;
+        x[S_SLOTS] = next_pow2(2 * x[S_RESERVED] + 64);
+        if (lim.max_frontier > 0 && n > lim.max_frontier) {
+            x[S_STOP] = STOP_TRUNCATED;
+        } else {
+            x[S_FRONTIER] = x[S_FRONTIER_MAX] = (unsigned long long)n;
+            if ((int64_t)x[S_RESERVED] > w.fp_cap || x[S_SLOTS] > w.slot_cap) x[S_STOP] = STOP_TABLES;
+        }
+        CK(cudaMemcpyAsync(ctr, h, sizeof(h), cudaMemcpyHostToDevice, s));
+        CK(cudaStreamSynchronize(s));
     } else {
-        c.frontier += n_front;
-        c.frontier_max = std::max<int64_t>(c.frontier_max, n_front);
-        if (lim.max_results > 0 && (int64_t)h[C_RES] >= lim.max_results) {
-            status |= EFM_CAPPED;
-            stop = true;
-        }
+        if (seedset)
+            CK(launch_seedset(nv, a, seedset, n_seedset, s));
+        else
+            CK(launch_seed(nv, a, target, s));
+        acc.level = level0;
+        acc.advance = 3;
+        acc.child_rows = a.child.cap;
+        acc.warps = full_grid * kExpandWarps;
+        CK(launch_accept_new(nv, acc, net->sm_count, s));
+        out.kernel_launches += 2;
+        if (manual && (rc = read_ctr())) return rc;
     }
-    int64_t indexed = 0, index_room = 0;  // results in the superset rule's index; entries it has room for
-    float ms = 0.f;
-    for (int level = level0 + 1; !stop && n_front > 0; ++level) {
-        // every step adds a column or a secondary step, so depth is bounded
-        if (level > lim.max_len + lim.max_secondary + 1) return EFM_ETIMEOUT;
-        // the superset rule's index over every accepted result so far (all of them come from levels < `level`);
-        // the table has room for twice the entries filed, and grows by filing every result again
-        if (res_n != indexed) {
-            const int64_t need = std::max<int64_t>(res_n * (int64_t)lim.max_len, 1);  // entries: sum of |E|
-            if (need > w.cent_cap) {
-                dev_free(w.cent, s);
-                dev_free(w.cells, s);
-                const int64_t cap = std::max<int64_t>(std::max<int64_t>(need, 2 * w.cent_cap), 4096);
-                if (!dev_alloc(w.cent, (size_t)cap * (nv.W <= 2 ? 32 : 16), s) ||
-                    !dev_alloc(w.cells, cell_table_bytes(nv, (uint64_t)cap), s))
-                    return EFM_ENOMEM;
-                w.cent_cap = cap;
-                index_room = 0;
-            }
-            CellIndex &ix = a.cells;
-            if (indexed == 0 || need > index_room) {
-                index_room = std::min<int64_t>(w.cent_cap, 4 * need);
-                ix.cells = (uint2 *)w.cells.p;
-                ix.mask = nv.W <= 2 ? 0u : (uint32_t)(cell_table_bytes(nv, (uint64_t)index_room) / 8 - 1);
-                ix.ent = (uint4 *)w.cent.p;
-                ix.ksig = (uint64_t *)w.ksig.p;
-                ix.single = (uint32_t *)w.csingle.p;
-                indexed = 0;
-            }
-            ix.n_res = res_n;
-            CK(launch_cells(nv, (const uint64_t *)w.res.p, indexed, res_n, (int32_t *)w.bcnt.p, ix, lim.max_len, s));
-            out.kernel_launches += 2;
-            indexed = res_n;
+    if (fk) {
+        res_n = (int64_t)std::min<unsigned long long>(h[C_RES_N], (unsigned long long)w.res_cap);
+        if (res_n > 0) {
+            std::vector<uint64_t> fresh((size_t)res_n * nv.W);
+            CK(cudaMemcpyAsync(fresh.data(), w.res.p, fresh.size() * 8, cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+            top.add(fresh.data(), res_n);
         }
-        if (trace && n_front > 0) {
-            // training rows: a strided sample of this frontier (level - 1),
-            // through the list of its surviving rows
+        if (seed_top && !seed_top->empty()) top.add(seed_top->data(), (int64_t)(seed_top->size() / nv.W));
+        if (top.pc > 0) CK(cudaMemcpyAsync(w.fkb.p, top.kth.data(), (size_t)nv.W * 8, cudaMemcpyHostToDevice, s));
+    }
+    float ms = 0.f;
+    int level = level0;  // last completed level (as far as the host knows)
+    int reruns = 0;
+    bool known = manual || fs;  // h holds the state
+    while (!stop) {
+        if (known && hs[S_STOP] != STOP_NONE) {
+            switch (hs[S_STOP]) {
+            case STOP_DONE: stop = true; break;
+            case STOP_CAPPED: status |= EFM_CAPPED; stop = true; break;
+            case STOP_TRUNCATED: status |= EFM_TRUNCATED; stop = true; break;
+            case STOP_TABLES:
+                if (!ensure_level_tables(w, hs[S_RESERVED], s)) return EFM_ENOMEM;
+                set_tables();
+                if ((rc = put_state(S_STOP, STOP_NONE))) return rc;
+                break;
+            case STOP_INDEX:
+                res_n = (int64_t)std::min<unsigned long long>(h[C_RES_N], (unsigned long long)w.res_cap);
+                if ((int64_t)h[C_RES_N] > w.res_cap) return EFM_ECAPACITY;
+                if ((rc = build_index(4 * res_n, res_n))) return rc;
+                // (the tables may have to grow as well)
+                if (!ensure_level_tables(w, hs[S_RESERVED], s)) return EFM_ENOMEM;
+                set_tables();
+                if ((rc = put_state(S_STOP, STOP_NONE))) return rc;
+                break;
+            case STOP_RERUN: {
+                // some children found no row, and the distinct fingerprints and
+                // rows, a lower bound of |F_l|, do not decide the level: grow the
+                // child arena to every reserved row and run the level again (only
+                // the per-child counters are rolled back; nothing was judged)
+                if (++reruns > 4) return EFM_ECAPACITY;
+                const uint64_t more = h[C_PAY] + h[C_PAY] / 8 + 1024;
+                if (more > 0xFFFFFFFFull) return EFM_ENOMEM;  // past a header's 32-bit offsets
+                if (!alloc_arena(w, cur ^ 1,
+                                 std::max<int64_t>((int64_t)h[C_WRITTEN] + (int64_t)h[C_WRITTEN] / 8 + 1024,
+                                                   w.rows[cur ^ 1]),
+                                 std::max<uint64_t>(more, w.pay_cap[cur ^ 1]), s))
+                    return EFM_ENOMEM;
+                const int back[] = {C_EXP, C_OVF, C_BAL, C_PRUNED, C_ZERO};
+                for (int i = 0; i < 5; ++i) h[back[i]] = hs[S_SNAP + i];
+                const int clear[] = {C_NEXT, C_DEGSUM, C_WRITTEN, C_UNWRITTEN, C_UNV, C_PAY, C_DEDUP_BEGIN, C_OPEN};
+                for (int i : clear) h[i] = 0;
+                h[C_COUNT + S_STOP] = STOP_NONE;
+                CK(cudaMemcpyAsync(ctr, h, sizeof(h), cudaMemcpyHostToDevice, s));
+                CK(cudaStreamSynchronize(s));
+                break;
+            }
+            default: return EFM_ECUDA;  // STOP_ERROR comes with an error bit
+            }
+            if (stop) break;
+        }
+        if (!manual) {
+            // several levels at a time while they are small: a level's launches
+            // return at once when an earlier one has stopped the search
+            const uint64_t deg = known ? hs[S_DEG] : 64;
+            const int n = deg <= 65536 ? 4 : (deg <= (1u << 20) ? 2 : 1);
+            CK(cudaEventRecord(w.ev[2], s));
+            for (int i = 0; i < n; ++i) {
+                const int lv = level + 1 + i;
+                const bool ext = fs && lv == level0 + 1;
+                a.par = ext ? fs->par : arena(cur ^ (i & 1));
+                a.child = arena(cur ^ (i & 1) ^ 1);
+                // the level's state table: cleared by the launch itself, or, at a
+                // large level whose size the host knows, by a memset
+                a.first = n > 1 || !known;
+                if (!a.first) CK(cudaMemsetAsync(w.slots.p, 0xFF, hs[S_SLOTS] * 8, s));
+                if ((rc = launch_level(lv, grid_for(deg << (2 * i)), 2))) return rc;
+            }
+            CK(cudaEventRecord(w.ev[3], s));
+            if ((rc = read_ctr())) return rc;
+            CK(cudaEventElapsedTime(&ms, w.ev[2], w.ev[3]));
+            out.expand_ms += ms;
+            const int done = (int)hs[S_LEVEL] - level;
+            if (done > 0) reruns = 0;
+            cur ^= done & 1;
+            level += done;
+            known = true;
+            continue;
+        }
+        const int64_t n_rows = (int64_t)hs[S_NROWS];
+        const uint64_t par_deg = hs[S_DEG];
+        if (trace) {
+            // training rows: a strided sample of this frontier, through the
+            // list of its surviving rows
             unsigned long long n_live = 0;
             CK(cudaMemsetAsync(ctr + C_LIVE, 0, 8, s));
             if (n_rows > w.live_cap) {
@@ -676,7 +794,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             if (!model_reserve_rows(m, m->n_rows + cnt)) return EFM_ENOMEM;
             if ((rc = ensure_dep_tags(net))) return rc;
             const uint32_t *live = (const uint32_t *)w.live.p;
-            CK(launch_features(nv, arena(cur), live, 0, stride, cnt, level - 1, lim.max_len, lim.max_secondary,
+            CK(launch_features(nv, arena(cur), live, 0, stride, cnt, level, lim.max_len, lim.max_secondary,
                                (const uint64_t *)net->dep.p, m->X.p, m->n_rows, s));
             CK(launch_labels(arena(cur), nv.W, live, 0, stride, cnt, trace->ans, trace->n_ans,
                              (float *)m->y.p, m->n_rows, s));
@@ -685,9 +803,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         // first-K: the level's parents in proposal order (positions -> arena
         // rows), expanded in chunks with the bound refreshed between them
         // (rows of later copies have no branches: they cost a meta read)
-        const int64_t par_rows = n_rows;    // this level's parents
-        const uint64_t par_deg = deg_sum;
-        const bool ext = fs && level == level0 + 1;  // parents in the caller's arena
+        const bool ext = fs && level == level0;  // parents in the caller's arena
         int64_t chunk = n_rows;
         const uint32_t *order = nullptr;
         if (fk) {
@@ -715,7 +831,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                     CK(cudaMemsetAsync(w.lerr.p, 0, 4, s));
                 }
                 if ((rc = ensure_dep_tags(net))) return rc;
-                CK(launch_features(nv, arena(cur), nullptr, 0, 1, n_rows, level - 1, lim.max_len, lim.max_secondary,
+                CK(launch_features(nv, arena(cur), nullptr, 0, 1, n_rows, level, lim.max_len, lim.max_secondary,
                                    (const uint64_t *)net->dep.p, w.lx.p, 0, s));
                 CK(launch_mlp_score(w.lx.p, n_rows, model->wb.p, (const float *)model->params.p,
                                     (float *)w.lscore.p, (unsigned *)w.lerr.p, s));
@@ -725,147 +841,58 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                 out.kernel_launches += 6;
             }
         }
-        // rows and payload units one warp reserves at a time: at large levels
-        // about a 16th of what it writes (what stays unused is dead weight in
-        // the arena), else exactly what a round needs
-        const int64_t launches = (n_rows + chunk - 1) / chunk;
-        int blk = launches > 1 ? 0 : (int)std::min<uint64_t>(512, deg_sum / (16ull * total_warps));
-        if (blk < 32) blk = 0;
-        const double avg_units = n_rows > 0 && row_units > 0.0 ? row_units / (double)n_rows : 8.0;
-        const uint64_t reserved = deg_sum + (uint64_t)launches * blk * total_warps + 64;
-        if (!ensure_level_tables(w, reserved, s)) return EFM_ENOMEM;
-        const uint64_t nslots = next_pow2(2 * reserved + 64);
-        unsigned long long snap[C_COUNT];
-        memcpy(snap, h, sizeof(h));
-        const int64_t n_front_level = n_front;  // distinct parents of this level
-        // the level, run again with a larger child arena if some children
-        // found no row and the fingerprints alone cannot show a truncation
-        for (int attempt = 0;; ++attempt) {
-            if (attempt > 4) return EFM_ECAPACITY;
-            CK(cudaMemsetAsync(w.slots.p, 0xFF, nslots * 8, s));
-            CK(cudaMemsetAsync(ctr + C_NEXT, 0, 2 * 8, s));
-            CK(cudaMemsetAsync(ctr + C_WRITTEN, 0, 3 * 8, s));
-            CK(cudaMemsetAsync(ctr + C_DEDUP_BEGIN, 0, 8, s));
-            CK(cudaMemsetAsync(ctr + C_PAY, 0, 8, s));
-            CK(cudaMemsetAsync(ctr + C_OPEN, 0, 8, s));
-            a.par = ext ? fs->par : arena(cur);
-            a.child = arena(cur ^ 1);
-            a.slots = (unsigned long long *)w.slots.p;
-            a.slot_mask = nslots - 1;
-            a.fp = (uint64_t *)w.fp.p;
-            a.fp_cap = w.fp_cap;
-            a.open = (uint32_t *)w.open.p;
-            a.blk = blk;
-            a.pay_blk = (int)(blk * (avg_units + 1.0));
-            a.level = level;
-            unsigned long long exp_before = h[C_EXP];
-            uint64_t next_before = 0;
-            for (int64_t c0 = 0; c0 < n_rows; c0 += chunk) {
-                const int64_t cn = std::min<int64_t>(chunk, n_rows - c0);
-                a.n_par = cn;
-                a.perm = order ? order + c0 : nullptr;
-                a.par_base = order ? 0 : c0 + (ext ? fs->r0 : 0);
-                a.cpw = (int)std::min<int64_t>(32, std::max<int64_t>(1, (cn + total_warps - 1) / total_warps));
-                a.fk_pc = fk ? top.pc : 0;
-                a.fk_sup = (const uint64_t *)w.fkb.p;
-                a.max_len = (fk && top.pc > 0) ? std::min(lim.max_len, top.pc) : lim.max_len;
-                CK(cudaEventRecord(w.ev[2], s));
-                CK(launch_generate(nv, a, grid, s));
-                CK(launch_dedup(nv, a, net->sm_count, s));
-                CK(cudaEventRecord(w.ev[3], s));
-                // minimality test of the new candidates, range taken on the device
-                CK(launch_accept_new(nv, acc, net->sm_count, s));
-                // one round trip per chunk: the counters and, in a first-K search, a
-                // window of the results that follow the ones already seen
-                const int64_t win = fk ? std::min<int64_t>(kResultWindow, w.res_cap - res_n) : 0;
-                if (win > 0)
-                    CK(cudaMemcpyAsync(window.data(), (const uint64_t *)w.res.p + (size_t)res_n * nv.W,
-                                       (size_t)win * nv.W * 8, cudaMemcpyDeviceToHost, s));
-                if ((rc = read_ctr())) return rc;
-                CK(cudaEventElapsedTime(&ms, w.ev[2], w.ev[3]));
-                out.expand_ms += ms;
-                out.expand_launches += 1;
-                out.kernel_launches += 5;
-                {
-                    // a header and the payload units of an average row of the level
-                    const double par_bytes = 16.0 + 16.0 * row_units / (double)std::max<int64_t>(n_rows, 1);
-                    const double new_bytes =
-                        16.0 + 16.0 * (double)h[C_PAY] / (double)std::max<unsigned long long>(h[C_WRITTEN], 1);
-                    const uint64_t next_now = h[C_NEXT];
-                    const double n_new = (double)(next_now - next_before);
-                    const double n_child = (double)(h[C_EXP] - exp_before);
-                    // distinct parents of the chunk (its rows include later copies
-                    // and unused rows, which carry no state)
-                    const double n_par = (double)cn * (double)n_front_level / (double)std::max<int64_t>(n_rows, 1);
-                    const double bytes = par_bytes * n_par + new_bytes * n_new + 16.0 * n_child;
-                    out.expand_bytes += bytes;
-                    if (getenv("EFM_DEBUG"))
-                        fprintf(stderr,
-                                "efm: level %d parents %lld items %llu children %.0f new %.0f rows %llu units %llu "
-                                "pruned %llu bytes %.0f ms %.3f\n",
-                                level, (long long)cn, (unsigned long long)(c0 == 0 && chunk >= n_rows ? deg_sum : 0),
-                                n_child, n_new, h[C_WRITTEN], h[C_PAY], h[C_PRUNED],
-                                bytes, ms);
-                    exp_before = h[C_EXP];
-                    next_before = next_now;
+        a.par = ext ? fs->par : arena(cur);
+        a.child = arena(cur ^ 1);
+        for (int64_t c0 = 0; c0 < n_rows; c0 += chunk) {
+            const int64_t cn = std::min<int64_t>(chunk, n_rows - c0);
+            a.first = c0 == 0 ? 1 : 0;
+            a.n_par = cn;
+            a.perm = order ? order + c0 : nullptr;
+            a.par_base = order ? 0 : c0 + (ext ? fs->r0 : 0);
+            a.fk_pc = fk ? top.pc : 0;
+            a.fk_sup = (const uint64_t *)w.fkb.p;
+            a.max_len = (fk && top.pc > 0) ? std::min(lim.max_len, top.pc) : lim.max_len;
+            CK(cudaEventRecord(w.ev[2], s));
+            if ((rc = launch_level(level + 1, grid_for(par_deg), c0 + cn < n_rows ? 1 : 2))) return rc;
+            CK(cudaEventRecord(w.ev[3], s));
+            // one round trip per chunk: the counters and, in a first-K search, a
+            // window of the results that follow the ones already seen
+            const int64_t win = fk ? std::min<int64_t>(kResultWindow, w.res_cap - res_n) : 0;
+            if (win > 0)
+                CK(cudaMemcpyAsync(window.data(), (const uint64_t *)w.res.p + (size_t)res_n * nv.W,
+                                   (size_t)win * nv.W * 8, cudaMemcpyDeviceToHost, s));
+            if ((rc = read_ctr())) return rc;
+            CK(cudaEventElapsedTime(&ms, w.ev[2], w.ev[3]));
+            out.expand_ms += ms;
+            const int64_t res_now = (int64_t)std::min<unsigned long long>(h[C_RES_N], (unsigned long long)w.res_cap);
+            if (fk && res_now > res_n) {
+                // the new results (beyond the window: fetched now) tighten the bound
+                const uint64_t *fresh = window.data();
+                std::vector<uint64_t> more;
+                if (res_now - res_n > win) {
+                    more.resize((size_t)(res_now - res_n) * nv.W);
+                    CK(cudaMemcpyAsync(more.data(), (const uint64_t *)w.res.p + (size_t)res_n * nv.W,
+                                       more.size() * 8, cudaMemcpyDeviceToHost, s));
+                    CK(cudaStreamSynchronize(s));
+                    fresh = more.data();
                 }
-                const int64_t res_now = (int64_t)std::min<unsigned long long>(h[C_RES_N], (unsigned long long)w.res_cap);
-                if (fk && res_now > res_n) {
-                    // the new results (beyond the window: fetched now) tighten the bound
-                    const uint64_t *fresh = window.data();
-                    std::vector<uint64_t> more;
-                    if (res_now - res_n > win) {
-                        more.resize((size_t)(res_now - res_n) * nv.W);
-                        CK(cudaMemcpyAsync(more.data(), (const uint64_t *)w.res.p + (size_t)res_n * nv.W,
-                                           more.size() * 8, cudaMemcpyDeviceToHost, s));
-                        CK(cudaStreamSynchronize(s));
-                        fresh = more.data();
-                    }
-                    const int pc_before = top.pc;
-                    const std::vector<uint64_t> kth_before = top.kth;
-                    top.add(fresh, res_now - res_n);
-                    if (top.pc > 0 && (top.pc != pc_before || top.kth != kth_before))
-                        CK(cudaMemcpyAsync(w.fkb.p, top.kth.data(), (size_t)nv.W * 8, cudaMemcpyHostToDevice, s));
-                }
+                const int pc_before = top.pc;
+                const std::vector<uint64_t> kth_before = top.kth;
+                top.add(fresh, res_now - res_n);
+                if (top.pc > 0 && (top.pc != pc_before || top.kth != kth_before))
+                    CK(cudaMemcpyAsync(w.fkb.p, top.kth.data(), (size_t)nv.W * 8, cudaMemcpyHostToDevice, s));
                 res_n = res_now;
             }
-            if (h[C_UNWRITTEN] == 0) break;  // every child has its row: the level is exact
-            // some children found no row: their distinct fingerprints and the
-            // distinct written rows bound |F_l| from below
-            if (lim.max_frontier > 0 && (int64_t)(h[C_NEXT] + h[C_UNV]) > lim.max_frontier) break;
-            // not decided: grow the child arena to every reserved row and run
-            // the level again (its balanced supports are already judged, so
-            // only the per-child counters are rolled back)
-            const uint64_t more = h[C_PAY] + h[C_PAY] / 8 + 1024;
-            if (more > 0xFFFFFFFFull) return EFM_ENOMEM;  // past a header's 32-bit offsets
-            if (!alloc_arena(w, cur ^ 1,
-                             std::max<int64_t>((int64_t)h[C_WRITTEN] + (int64_t)h[C_WRITTEN] / 8 + 1024,
-                                               w.rows[cur ^ 1]),
-                             std::max<uint64_t>(more, w.pay_cap[cur ^ 1]), s))
-                return EFM_ENOMEM;
-            const int back[] = {C_EXP, C_OVF, C_BAL, C_PRUNED, C_ZERO};
-            for (int i : back) {
-                h[i] = snap[i];
-                CK(cudaMemcpyAsync(ctr + i, &snap[i], 8, cudaMemcpyHostToDevice, s));
-            }
-            CK(cudaStreamSynchronize(s));
         }
-        const bool unwritten = h[C_UNWRITTEN] != 0;
-        n_front = unwritten ? (int64_t)(h[C_NEXT] + h[C_UNV]) : (int64_t)h[C_NEXT];
-        n_rows = (int64_t)std::min<unsigned long long>(h[C_WRITTEN], (unsigned long long)w.rows[cur ^ 1]);
-        deg_sum = h[C_DEGSUM];
-        row_units = (double)h[C_PAY];
-        c.levels = level - level0 + 1;
+        if (hs[S_STOP] == STOP_RERUN) continue;
+        reruns = 0;
+        level += 1;
         cur ^= 1;
-        if (lim.max_frontier > 0 && n_front > lim.max_frontier) {
-            if (!(fk && split_depth > 0 && par_rows > 1)) {
-                status |= EFM_TRUNCATED;
-                break;
-            }
+        if (hs[S_STOP] == STOP_TRUNCATED && fk && split_depth > 0 && n_rows > 1) {
             // first-K: the level's parents in parts of about half the
             // budget's worth of children, each run to the end
             Work w2;
-            int rc2 = alloc_work(w2, net, lim, total_warps, s);
+            int rc2 = alloc_work(w2, net, lim, full_grid * kExpandWarps, s);
             if (rc2 == EFM_ENOMEM) {
                 // no room for a second work area: the answer stays uncertified
                 free_work(w2, s);
@@ -873,19 +900,21 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                 status |= EFM_TRUNCATED;
                 break;
             }
+            const int64_t n_front = (int64_t)hs[S_NFRONT];
             const int64_t parts = std::min<int64_t>(
-                par_rows, std::max<int64_t>(2, (2 * n_front + lim.max_frontier - 1) / lim.max_frontier));
+                n_rows, std::max<int64_t>(2, (2 * n_front + lim.max_frontier - 1) / lim.max_frontier));
             // the level's parents: this search's arena, or the caller's rows
             // when the level is a part's first
             const Arena par_arena = ext ? fs->par : arena(cur ^ 1);
             const int64_t par0 = ext ? fs->r0 : 0;
             for (int64_t p = 0; rc2 == EFM_OK && p < parts; ++p) {
-                FrontierStart sub{par_arena, par0 + par_rows * p / parts, par0 + par_rows * (p + 1) / parts, level - 1,
+                FrontierStart sub{par_arena, par0 + n_rows * p / parts, par0 + n_rows * (p + 1) / parts, level - 1,
                                   par_deg};
                 if (sub.r1 <= sub.r0) continue;
                 TargetOut so;
-                const std::vector<uint64_t> known = top.rows;
-                rc2 = run_target(net, w2, lim, target, so, nullptr, nullptr, nullptr, 0, &sub, &known, split_depth - 1);
+                const std::vector<uint64_t> known_top = top.rows;
+                rc2 = run_target(net, w2, lim, target, so, nullptr, nullptr, nullptr, 0, &sub, &known_top,
+                                 split_depth - 1);
                 if (rc2 == EFM_OK) {
                     status |= so.status;
                     if (so.n > 0) {
@@ -922,14 +951,13 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             split = true;
             break;
         }
-        if (unwritten) return EFM_ECAPACITY;  // unreachable: the loop above runs such a level again
-        c.frontier += n_front;
-        c.frontier_max = std::max<int64_t>(c.frontier_max, n_front);
-        if (lim.max_results > 0 && (int64_t)h[C_RES] >= lim.max_results) {
-            status |= EFM_CAPPED;
-            break;
-        }
     }
+    res_n = (int64_t)std::min<unsigned long long>(h[C_RES_N], (unsigned long long)w.res_cap);
+    c.levels = std::max<int64_t>(c.levels, (int64_t)hs[S_LEVEL] - level0 + 1);
+    c.frontier += (int64_t)hs[S_FRONTIER];
+    c.frontier_max = std::max<int64_t>(c.frontier_max, (int64_t)hs[S_FRONTIER_MAX]);
+    out.expand_launches += (int64_t)hs[S_EXPANDS];
+    out.expand_bytes += (double)hs[S_BYTES];
     if ((int64_t)h[C_RES_N] > w.res_cap) return EFM_ECAPACITY;
     if (w.lerr.p) {
         unsigned e = 0;

@@ -50,6 +50,40 @@ enum {
     C_COUNT = 40
 };
 
+// Level state of a traversal, kept on the device behind its counter block
+// (unsigned long long each): the last CTA of a level's minimality test decides
+// whether the search goes on and sets the next level's parameters, so that
+// the host can launch several levels without a round trip between them.
+enum {
+    S_STOP = 0,   // STOP_*: later launches return at once
+    S_LEVEL,      // last completed level
+    S_NROWS,      // its arena rows (the next level's parents)
+    S_NFRONT,     // its distinct states
+    S_DEG,        // sum of their branch counts
+    S_UNITS,      // payload units of its rows
+    S_SLOTS,      // next level: slots of the state table (a power of two)
+    S_RESERVED,   // next level: rows that may be reserved
+    S_BLK,        // next level: rows a warp reserves at a time
+    S_PAY_BLK,    // next level: payload units a warp reserves at a time
+    S_FRONTIER,   // sum and largest of the levels' distinct states
+    S_FRONTIER_MAX,
+    S_BYTES,      // algorithmic bytes of the expansions so far
+    S_EXPANDS,    // levels expanded
+    S_TICKET,     // CTAs of the running minimality launch that are done
+    S_SNAP,       // C_EXP, C_OVF, C_BAL, C_PRUNED, C_ZERO when the running level began
+    S_COUNT = S_SNAP + 8
+};
+enum : unsigned long long {
+    STOP_NONE = 0,
+    STOP_DONE,       // the frontier is empty
+    STOP_TRUNCATED,  // it exceeds the budget
+    STOP_CAPPED,     // max_results reached
+    STOP_RERUN,      // children without a row: the level again, with a larger arena
+    STOP_TABLES,     // the next level needs larger tables
+    STOP_INDEX,      // the superset rule's index is full
+    STOP_ERROR       // an error bit, or too many levels
+};
+
 // Static network, packed into one 16-byte aligned word array (the "blob").
 // Packed entry: (index << 20) | (coefficient & 0xFFFFF), index < 4096,
 // coefficient a signed 20-bit value.
@@ -115,10 +149,16 @@ struct CellIndex {
     uint4 *ent;
     uint64_t *ksig;
     uint32_t *single;   // [N]: 1 if {k} itself is a result
-    int64_t n_res;      // results filed (0: no index)
+    int64_t room;       // results it has room for (0: no index)
+    int32_t *cnt;       // [N]: filed results per column
+    int ent_stride;     // entries of result r start at r * ent_stride
 };
 
 struct LevelArgs {
+    unsigned long long *st;     // level state
+    int manual;                 // 1: the parents are n_par, par_base and perm below; 0: all rows of the last level
+    int first;                  // first launch of its level: clear the state table
+    int warps;                  // warps of the generate launch
     Arena par;
     int64_t n_par;
     Arena child;
@@ -136,7 +176,7 @@ struct LevelArgs {
     const uint64_t *band;       // W <= 2: per column, the intersection of the results containing it (or null)
     CellIndex cells;            // the level pass
     int level, max_len, max_sec;
-    int cpw;                    // parents per warp chunk (1..32)
+    int cpw;                    // parents per warp chunk (1..32; batched traversal)
     unsigned long long *ctr;
     // first-K search (zero / null otherwise)
     const uint32_t *perm;       // parent order: position -> arena index (null: arena rows par_base + position)
@@ -151,8 +191,6 @@ struct LevelArgs {
     uint64_t *fp;               // [fp_cap] fingerprint per reserved row (kDeadFp: unused)
     int64_t fp_cap;
     uint32_t *open;             // [fp_cap] rows of the open children
-    int blk;                    // rows a warp reserves at a time, at least a round's
-    int pay_blk;                // payload units a warp reserves at a time, at least a round's
     // subtractive variant (Eq. 5): states also hold the flux of their columns,
     // a state's branches also take flux away from a column in U, and its meta
     // degree counts both lists of the pivot
@@ -167,13 +205,21 @@ constexpr int kRcolStride = 65;  // column count + up to 64 columns per result
 
 struct AcceptArgs {
     const uint64_t *cand;
-    int64_t cand_begin, cand_end;  // ignored when dev_range: [ctr[C_ACC_BEGIN], ctr[C_CAND_N]) instead
-    int dev_range;
+    int64_t cand_begin, cand_end;  // ignored with advance: [ctr[C_ACC_BEGIN], ctr[C_CAND_N]) instead
     int64_t cand_cap;
     uint64_t *res;
     uint16_t *rcols;            // written on accept when non-null
     int64_t res_cap;
     unsigned long long *ctr;
+    // single-job traversal
+    CellIndex ix;               // accepted results are filed here
+    unsigned long long *st;
+    int advance;                // what the last CTA does: 0 nothing, 1 a chunk of a level ends, 2 a level, 3 the seeds
+    int level, level0, max_level;
+    int64_t max_frontier, max_results;
+    int64_t fp_cap, child_rows;
+    uint64_t slot_cap;
+    int warps;                  // warps of the next generate launch
 };
 
 // Batched traversal: per-CTA scratch slice layout (byte offsets)
@@ -254,18 +300,16 @@ cudaError_t launch_seedset(const NetView &nv, const LevelArgs &a, const int32_t 
 int generate_grid(const NetView &nv, bool sub, bool first_k, int sm_count);
 cudaError_t launch_generate(const NetView &nv, const LevelArgs &a, int grid, cudaStream_t s);
 cudaError_t launch_dedup(const NetView &nv, const LevelArgs &a, int sm_count, cudaStream_t s);
-// the results [r0, r1) into the superset rule's index (r0 = 0: a new index); cnt: results per
-// column; entries of result r start at r * ent_stride
+// an empty superset index, then the results [0, n) filed in it
 size_t cell_table_bytes(const NetView &nv, uint64_t entries);
-cudaError_t launch_cells(const NetView &nv, const uint64_t *res, int64_t r0, int64_t r1, int32_t *cnt,
-                         const CellIndex &ix, int ent_stride, cudaStream_t s);
+cudaError_t launch_index(const NetView &nv, const CellIndex &ix, const uint64_t *res, int64_t n, cudaStream_t s);
 // the surviving rows (meta != 0) of [0, n) appended to live; *count must be 0
 cudaError_t launch_live_list(const uint4 *hdr, int64_t n, uint32_t *live, unsigned long long *count, int sm_count,
                              cudaStream_t s);
 // kernels (efm_kernels.cu)
 cudaError_t launch_accept(const NetView &nv, const AcceptArgs &a, cudaStream_t s);
 // minimality test of the candidates appended since the last such launch (range read on the
-// device, so no host round trip is needed between expansion and test); then advance the range
+// device); accepted results are filed in the index; then the level state moves on
 cudaError_t launch_accept_new(const NetView &nv, const AcceptArgs &a, int sm_count, cudaStream_t s);
 // sort by (|U|, ascending columns); n2: n rounded up to a power of two; scratch: sort_scratch_bytes(n2)
 size_t sort_scratch_bytes(int64_t n2);

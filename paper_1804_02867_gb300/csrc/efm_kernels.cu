@@ -1127,27 +1127,11 @@ __device__ void accept_range(const NetView &nv, const AcceptArgs &a, uint32_t *w
         const uint64_t *U = a.cand + (size_t)ci * W;
         const uint64_t u0 = lane < W ? U[lane] : 0ull;
         const uint64_t u1 = lane + 32 < W ? U[lane + 32] : 0ull;
-        // ascending column list: words 0..31 (lanes, slot 0), then 32..63
-        const int n0 = __popcll(u0), n1 = __popcll(u1);
-        int s0 = n0, s1 = n1;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int x0 = __shfl_up_sync(FULL, s0, off), x1 = __shfl_up_sync(FULL, s1, off);
-            if (lane >= off) {
-                s0 += x0;
-                s1 += x1;
-            }
-        }
-        const int tot0 = __shfl_sync(FULL, s0, 31);
-        const int n = tot0 + __shfl_sync(FULL, s1, 31);
+        const int n = support_columns(u0, u1, cols);
         if (n > 64) {
             if (lane == 0) atomicOr(&a.ctr[C_ERR], (unsigned long long)ERR_LEN);
             continue;
         }
-        int pos0 = s0 - n0, pos1 = tot0 + s1 - n1;
-        for (uint64_t x = u0; x; x &= x - 1) cols[pos0++] = lane * 64 + __ffsll((long long)x) - 1;
-        for (uint64_t x = u1; x; x &= x - 1) cols[pos1++] = (lane + 32) * 64 + __ffsll((long long)x) - 1;
-        __syncwarp();
         // Drop one column: the kept nn = n - 1 columns must be independent.
         // (The balanced flux ray is positive on every column of U, so the
         // dropped column is a combination of the others.)
@@ -1179,6 +1163,8 @@ __device__ void accept_range(const NetView &nv, const AcceptArgs &a, uint32_t *w
                     for (int j = lane; j < n; j += 32) lst[1 + j] = (uint16_t)cols[j];
                     if (lane == 0) lst[0] = (uint16_t)n;
                 }
+                if ((int64_t)idx < a.ix.room)
+                    file_result(a.ix, W, (int64_t)idx, cols, n, __shfl_sync(FULL, u0, 0), __shfl_sync(FULL, u0, 1));
             } else if (lane == 0) {
                 atomicOr(&a.ctr[C_ERR], (unsigned long long)ERR_RES_CAP);
             }
@@ -1189,24 +1175,129 @@ __device__ void accept_range(const NetView &nv, const AcceptArgs &a, uint32_t *w
     if (lane == 0 && n_acc) atomicAdd(&a.ctr[C_RES], n_acc);
 }
 
+__device__ __forceinline__ uint64_t next_pow2_dev(uint64_t x)
+{
+    uint64_t p = 1;
+    while (p < x) p <<= 1;
+    return p;
+}
+
+// Levels without a host round trip.  With one launch list and one counter copy
+// per level (15 calls, 60-90 us a level at small frontiers) the small searches
+// waited on the host: the last CTA of the minimality test now decides the
+// level and sets the next one's parameters, and the host launches up to four
+// levels (three kernels each) ahead.  One GB300, calls through the library:
+// the smallest query 1.28 -> 0.87 ms, one core query 3.1 -> 2.4, eight core
+// targets at 2^17 13.6 -> 9.3, a 400-row network 5.4 -> 4.1.
+
+// The end of a level (one thread, after every CTA of its last launch is done):
+// the decisions on it, and the next level's parameters.  v: the counters and
+// the state as they stand.
+__device__ void advance_level(const AcceptArgs &a, const unsigned long long *v)
+{
+    unsigned long long *c = a.ctr, *st = a.st;
+    const unsigned long long *sv = v + C_COUNT;
+    auto get = [&](int i) { return v[i]; };
+    if (a.advance == 1) return;
+    const bool seeds = a.advance == 3;
+    const uint64_t next = get(C_NEXT), unv = get(C_UNV), written = seeds ? next : get(C_WRITTEN);
+    const uint64_t deg = get(C_DEGSUM), units = get(C_PAY), unwritten = get(C_UNWRITTEN);
+    const uint64_t front = next + (unwritten ? unv : 0ull);
+    unsigned long long stop = STOP_NONE;
+    if (get(C_ERR)) {
+        stop = STOP_ERROR;
+    } else if (a.max_frontier > 0 && (int64_t)front > a.max_frontier) {
+        stop = STOP_TRUNCATED;
+    } else if (seeds && (int64_t)next > a.child_rows) {  // more seeds than rows
+        atomicOr(&c[C_ERR], (unsigned long long)ERR_TABLE_FULL);
+        stop = STOP_ERROR;
+    } else if (unwritten) {
+        st[S_STOP] = STOP_RERUN;  // the counters stay as they are for the host
+        return;
+    }
+    if (!seeds) {
+        // algorithmic bytes: a header and the payload units of an average row,
+        // per distinct parent and new state; 16 bytes of slot traffic per child
+        const uint64_t prow = sv[S_NROWS], pfront = sv[S_NFRONT];
+        st[S_BYTES] = sv[S_BYTES] + 16 * (pfront + next) + (prow ? 16 * (uint64_t)((double)sv[S_UNITS] * pfront / prow) : 0ull) +
+                       (written ? 16 * (uint64_t)((double)units * next / written) : 0ull) +
+                       16 * (get(C_EXP) - sv[S_SNAP]);
+        st[S_EXPANDS] = sv[S_EXPANDS] + 1;
+    }
+    st[S_LEVEL] = (unsigned long long)a.level;
+    st[S_NROWS] = written < (uint64_t)a.child_rows ? written : (uint64_t)a.child_rows;
+    st[S_NFRONT] = front;
+    st[S_DEG] = deg;
+    st[S_UNITS] = units;
+    if (stop == STOP_NONE) {
+        st[S_FRONTIER] = sv[S_FRONTIER] + front;
+        if (front > sv[S_FRONTIER_MAX]) st[S_FRONTIER_MAX] = front;
+        if (a.max_results > 0 && (int64_t)get(C_RES) >= a.max_results) stop = STOP_CAPPED;
+        else if (front == 0) stop = STOP_DONE;
+        else if (a.level + 1 > a.max_level) {  // every step adds a column or a secondary step: unreachable
+            atomicOr(&c[C_ERR], (unsigned long long)ERR_WATCHDOG);
+            stop = STOP_ERROR;
+        }
+    }
+    // rows and payload units one warp reserves at a time: at large levels about
+    // a 16th of what it writes (what stays unused is dead weight in the arena),
+    // else exactly what a round needs
+    uint64_t blk = deg / (16ull * (uint64_t)a.warps);
+    blk = blk > 512 ? 512 : (blk < 32 ? 0 : blk);
+    const uint64_t avg = written ? units / written : 8;
+    const uint64_t reserved = deg + blk * (uint64_t)a.warps + 64;
+    const uint64_t slots = next_pow2_dev(2 * reserved + 64);
+    st[S_BLK] = blk;
+    st[S_PAY_BLK] = blk * (avg + 2);
+    st[S_RESERVED] = reserved;
+    st[S_SLOTS] = slots;
+    const int snap[] = {C_EXP, C_OVF, C_BAL, C_PRUNED, C_ZERO};
+    for (int i = 0; i < 5; ++i) st[S_SNAP + i] = get(snap[i]);
+    if (stop == STOP_NONE && (int64_t)get(C_RES_N) > a.ix.room) stop = STOP_INDEX;
+    if (stop == STOP_NONE && ((int64_t)reserved > a.fp_cap || slots > a.slot_cap)) stop = STOP_TABLES;
+    const int clear[] = {C_NEXT, C_DEGSUM, C_WRITTEN, C_UNWRITTEN, C_UNV, C_PAY, C_DEDUP_BEGIN};
+    if (stop == STOP_NONE || stop == STOP_INDEX || stop == STOP_TABLES)
+        for (int i = 0; i < 7; ++i) c[clear[i]] = 0ull;
+    st[S_STOP] = stop;
+}
+
 __global__ void __launch_bounds__(kAcceptWarps * 32) accept_kernel(NetView nv, AcceptArgs a)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     const int wid = threadIdx.x >> 5;
-    if (a.dev_range) {
+    if (a.advance) {
+        if (a.st[S_STOP] != STOP_NONE) return;
+        // a level that will run again is judged then: nothing may be filed before
+        const uint64_t front = a.ctr[C_NEXT] + a.ctr[C_UNV];
+        const bool rerun = a.advance == 2 && a.ctr[C_UNWRITTEN] != 0ull &&
+                           !(a.max_frontier > 0 && (int64_t)front > a.max_frontier);
         // the expansion launches before this one have finished: the range is stable
         a.cand_begin = (int64_t)a.ctr[C_ACC_BEGIN];
         const int64_t n = (int64_t)a.ctr[C_CAND_N];
-        a.cand_end = n < a.cand_cap ? n : a.cand_cap;
+        a.cand_end = rerun ? a.cand_begin : (n < a.cand_cap ? n : a.cand_cap);
     }
+    const int64_t cand_end = a.cand_end;
     accept_range(nv, a, smem + wid * kAcceptWarpWords, (int64_t)blockIdx.x * kAcceptWarps + wid,
                  (int64_t)gridDim.x * kAcceptWarps);
-}
-
-__global__ void accept_advance_kernel(unsigned long long *ctr, int64_t cand_cap)
-{
-    const unsigned long long n = ctr[C_CAND_N];
-    ctr[C_ACC_BEGIN] = n < (unsigned long long)cand_cap ? n : (unsigned long long)cand_cap;
+    if (!a.advance) return;
+    // the last CTA moves the level state on
+    __shared__ int s_last;
+    __shared__ unsigned long long s_ctr[C_COUNT + S_COUNT];
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&a.st[S_TICKET], 1ull) == (unsigned long long)gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (int i = threadIdx.x; i < C_COUNT + S_COUNT; i += blockDim.x) s_ctr[i] = __ldcg(&a.ctr[i]);  // (the state follows)
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        a.st[S_TICKET] = 0ull;
+        a.ctr[C_ACC_BEGIN] = (unsigned long long)cand_end;
+        a.ctr[C_DEDUP_BEGIN] = s_ctr[C_WRITTEN];  // (a chunk; a level clears it)
+        a.ctr[C_OPEN] = 0ull;
+        advance_level(a, s_ctr);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1353,13 +1444,6 @@ __global__ void gather_kernel(const uint64_t *res, int W, const Rec *rec, int64_
 // barriers between the steps, in its own slice of a scratch pool.  The level
 // decisions (truncation, cap, counters) are those of the single-job host loop.
 // ---------------------------------------------------------------------------
-
-__device__ __forceinline__ uint64_t next_pow2_dev(uint64_t x)
-{
-    uint64_t p = 1;
-    while (p < x) p <<= 1;
-    return p;
-}
 
 // CTA-level bucket rebuild over results [0, n_res)
 __device__ void cta_buckets(const NetView &nv, const uint64_t *res, int64_t n_res, int32_t *bcnt, int32_t *bptr,
@@ -1609,10 +1693,7 @@ cudaError_t launch_accept_new(const NetView &nv, const AcceptArgs &a, int sm_cou
 {
     const size_t sm = (size_t)kAcceptWarps * kAcceptWarpWords * 4;
     cudaFuncSetAttribute(accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    AcceptArgs d = a;
-    d.dev_range = 1;
-    accept_kernel<<<sm_count * 2, kAcceptWarps * 32, sm, s>>>(nv, d);
-    accept_advance_kernel<<<1, 1, 0, s>>>(a.ctr, a.cand_cap);
+    accept_kernel<<<sm_count, kAcceptWarps * 32, sm, s>>>(nv, a);
     return cudaGetLastError();
 }
 

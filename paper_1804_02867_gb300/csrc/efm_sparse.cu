@@ -48,7 +48,6 @@ constexpr int kGenWarps = 8;      // warps per CTA
 // network at a 2^26 budget; 24 warps 537.
 constexpr int kGenBlocks = 5;
 constexpr uint32_t kFluxKey = 0xFFFF0000u;  // keys from here on are no balance rows
-constexpr uint32_t kPadKey = 0xFFFFFFFFu;
 
 __device__ __forceinline__ uint64_t column_hash(int k) { return mix64(0x51ed27f3a5b1c3d9ull * (uint64_t)(k + 1)); }
 __device__ __forceinline__ uint64_t row_hash(int m) { return mix64(0x9E3779B97F4A7C15ull * (uint64_t)(m + 1)); }
@@ -74,7 +73,6 @@ __device__ __forceinline__ void prefetch_l2(const void *p)
 }
 
 __device__ __forceinline__ int max_bits(uint32_t om) { return om ? 32 - __clz((int)om) : 0; }
-__device__ __forceinline__ uint32_t mag(int32_t v) { return (uint32_t)(v < 0 ? -v : v); }
 
 // 16-bit column i of a payload's list
 __device__ __forceinline__ int list_col(const uint4 *pay, int i)
@@ -191,16 +189,6 @@ __device__ __noinline__ int insert_candidate(const LevelArgs &a, int W, const ui
 // the superset rule (see CellIndex in efm_internal.cuh)
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ uint64_t col_bit(int c) { return 1ull << ((uint32_t)(c * 0x9E3779B1u) >> 26); }
-
-__device__ __forceinline__ uint32_t cell_slot(uint32_t key, uint32_t mask)
-{
-    uint32_t x = key * 0x85EBCA6Bu;
-    x ^= x >> 15;
-    x *= 0xC2B2AE35u;
-    return (x ^ (x >> 13)) & mask;
-}
-
 // Does a result E with k in E lie inside U + {k}?  One lane.  Only the cells
 // (k, s) of the sentinels s in U are looked up.
 __device__ __forceinline__ bool pruned_bits(const CellIndex &ix, const uint4 *pay, int k)
@@ -216,8 +204,8 @@ __device__ __forceinline__ bool pruned_bits(const CellIndex &ix, const uint4 *pa
     for (int w = 0; w < 2; ++w)
         for (uint64_t x = m[w]; x; x &= x - 1) {
             uint32_t head = heads[64 * w + __ffsll((long long)x) - 1];
-            // a list holds each result at most once: n_res bounds it
-            for (int64_t n = 0; head != kNoRecord && n < ix.n_res; ++n) {
+            // a list holds each result at most once
+            for (int64_t n = 0; head != kNoRecord && n < ix.room; ++n) {
                 const ulonglong2 e = *reinterpret_cast<const ulonglong2 *>(ix.ent + 2 * (size_t)head);
                 if (((e.x & ~u0) | (e.y & ~u1)) == 0) return true;
                 head = ix.ent[2 * (size_t)head + 1].x;
@@ -251,7 +239,7 @@ __device__ __noinline__ bool pruned_list(const CellIndex &ix, const uint16_t *rc
             if (cell.x == kNoRecord) break;
             p = (p + 1) & ix.mask;
         }
-        for (int64_t n = 0; head != kNoRecord && n < ix.n_res; ++n) {
+        for (int64_t n = 0; head != kNoRecord && n < ix.room; ++n) {
             const uint4 e = ix.ent[head];
             const uint64_t sig = (uint64_t)e.x | ((uint64_t)e.y << 32);
             if ((sig & ~su) == 0) {
@@ -282,17 +270,6 @@ __device__ __forceinline__ uint32_t entry_key(const NetView &nv, const uint32_t 
 {
     if (SUB && row >= nv.M) return kFluxKey | (uint32_t)row;
     return bl[(positive ? nv.o_keypos : nv.o_keyneg) + row];
-}
-
-// gcd of magnitudes that are mostly small (Euclid: one or two divisions)
-__device__ __forceinline__ uint32_t gcd_small(uint32_t a, uint32_t b)
-{
-    while (a) {
-        const uint32_t t = b % a;
-        b = a;
-        a = t;
-    }
-    return b;
 }
 
 struct Child {
@@ -439,21 +416,8 @@ __device__ __forceinline__ void fast_child(const NetView &nv, const uint32_t *bl
 
 // --- narrow networks ---
 
-__device__ __forceinline__ uint64_t blob_u64(const uint32_t *bl, int o)
-{
-    return *reinterpret_cast<const uint64_t *>(bl + o);
-}
-
 // values below row r in a state with nonzero rows zm
 __device__ __forceinline__ int value_at(uint64_t zm, int r) { return __popcll(zm & ((1ull << r) - 1ull)); }
-
-// pivot key from the two masks (kPadKey when balanced)
-__device__ __forceinline__ uint32_t mask_key(const uint32_t *bl, const NetView &nv, uint64_t pm, uint64_t nm)
-{
-    const uint32_t kp = pm ? bl[nv.o_keyr + __ffsll((long long)pm) - 1] : kPadKey;
-    const uint32_t kn = nm ? bl[nv.o_keyr + 64 + __ffsll((long long)nm) - 1] : kPadKey;
-    return kp < kn ? kp : kn;
-}
 
 struct NarrowMasks {
     uint64_t zm, pm, nm;
@@ -866,12 +830,25 @@ __device__ __forceinline__ void write_support(uint4 *dst, const uint4 *pp, int p
 // a larger arena).
 // ---------------------------------------------------------------------------
 template <int F, bool SUB, bool FK>
-__global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks) generate_kernel(NetView nv, LevelArgs a)
+__global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks) generate_kernel(const __grid_constant__ NetView nv,
+                                                                         const __grid_constant__ LevelArgs a)
 {
     __shared__ CapScratch s_cap[FK ? kGenWarps : 1];
     __shared__ BoundScratch s_bound;
+    if (a.st[S_STOP] != STOP_NONE) return;
     const int lane = threadIdx.x & 31;
     const int wid = threadIdx.x >> 5;
+    if (a.first) {  // the level's state table, cleared for the dedup pass
+        const uint64_t n = a.st[S_SLOTS] / 2;  // (at least 64 slots, two a store)
+        uint4 *t = reinterpret_cast<uint4 *>(a.slots);
+        for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
+            t[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    }
+    const int64_t n_par = a.manual ? a.n_par : (int64_t)a.st[S_NROWS];
+    // (a level in several launches reserves exactly what a round needs: the
+    // tables have room for one launch's unused rows)
+    const int blk = a.manual ? 0 : (int)a.st[S_BLK], pay_blk = a.manual ? 0 : (int)a.st[S_PAY_BLK];
+    const bool any_result = a.ctr[C_RES_N] != 0ull;  // (none is accepted while this kernel runs)
     const uint32_t *bl = nv.blob;
     const uint4 *scol = reinterpret_cast<const uint4 *>(bl + nv.o_scol);
     const int64_t row_cap = a.child.cap;
@@ -896,13 +873,15 @@ __global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks) generate_kernel(Ne
     // rounds' worth at a time, so that the two counters are not the limit)
     uint64_t row_next = 0, pay_next = 0;
     int row_left = 0, pay_left = 0;
-    const int cpw = a.cpw;
+    // parents per warp and chunk: fewer at small levels, so that their items
+    // spread over all warps
+    const int cpw = (int)min((int64_t)32, max((int64_t)1, (n_par + a.warps - 1) / a.warps));
     const int64_t worker = (int64_t)blockIdx.x * kGenWarps + wid;
     const int64_t wstride = (int64_t)gridDim.x * kGenWarps * cpw;
     // the lane's parent of a chunk: its row, payload offset and meta word
     auto parent_at = [&](int64_t p0, uint32_t &pid, uint32_t &off, uint32_t &meta) {
         const int64_t pl = p0 + lane;
-        const bool pin = lane < cpw && pl < a.n_par;
+        const bool pin = lane < cpw && pl < n_par;
         pid = pin ? (uint32_t)(a.perm ? (int64_t)a.perm[pl] : a.par_base + pl) : 0u;
         off = meta = 0u;
         if (pin) {
@@ -913,7 +892,7 @@ __global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks) generate_kernel(Ne
     };
     uint32_t pid_n, off_n, meta_n;  // the next chunk's, read one chunk ahead
     parent_at(worker * cpw, pid_n, off_n, meta_n);
-    for (int64_t p0 = worker * cpw; p0 < a.n_par; p0 += wstride) {
+    for (int64_t p0 = worker * cpw; p0 < n_par; p0 += wstride) {
         const uint32_t pid = pid_n, mj = meta_n;
         parent_at(p0 + wstride, pid_n, off_n, meta_n);
         int dj = (int)((mj >> 10) & 0x1FFFu);
@@ -1032,7 +1011,7 @@ __global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks) generate_kernel(Ne
             // superset rule: the new column completes a result accepted at an
             // earlier level (counted below, once the child is known to be one)
             bool pr = false;
-            if (a.cells.n_res > 0 && okl && !in_u)
+            if (any_result && okl && !in_u)
                 pr = F ? pruned_bits(a.cells, pp, k) : pruned_list(a.cells, a.rcols, pp, pc, k);
             // first-K length-cap rules.  dead: the child cannot balance any
             // more, unless it is balanced already (it then has no one-sided
@@ -1079,8 +1058,8 @@ __global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks) generate_kernel(Ne
             uint64_t fresh = 0;
             int want_r = 0;
             if (row_left < rows || pay_left < utot) {  // warp-uniform
-                want_r = row_left < rows ? max(rows - row_left, a.blk) : 0;
-                const int want_p = pay_left < utot ? max(utot, a.pay_blk) : 0;
+                want_r = row_left < rows ? max(rows - row_left, blk) : 0;
+                const int want_p = pay_left < utot ? max(utot, pay_blk) : 0;
                 unsigned long long got = 0;
                 if (lane == 0 && want_r) got = atomicAdd(&a.ctr[C_WRITTEN], (unsigned long long)want_r);
                 if (lane == 1 && want_p) got = atomicAdd(&a.ctr[C_PAY], (unsigned long long)want_p);
@@ -1303,14 +1282,14 @@ struct DedupSums {
 // Insert a warp's rows (lane: row i, fingerprint f, kDeadFp for none, header
 // h) into the level's table.
 template <int F>
-__device__ __forceinline__ void dedup_insert(const LevelArgs &a, uint64_t i, uint64_t f, const uint4 &h, int lane,
-                                             DedupSums &sum)
+__device__ __forceinline__ void dedup_insert(const LevelArgs &a, uint64_t mask, uint64_t i, uint64_t f, const uint4 &h,
+                                             int lane, DedupSums &sum)
 {
     const uint64_t row_cap = (uint64_t)a.child.cap;
     bool todo = f != kDeadFp;
     uint64_t pos = 0, probe = 0;
     uint32_t tag = 0;
-    slot_tag_pos(f, a.slot_mask, pos, tag);
+    slot_tag_pos(f, mask, pos, tag);
     if (todo && i >= 0xFFFFFFFEull) {
         record_diag(a.ctr, ERR_BOUNDS, 10, (long long)i, 0xFFFFFFFEll, a.level);
         todo = false;
@@ -1349,9 +1328,9 @@ __device__ __forceinline__ void dedup_insert(const LevelArgs &a, uint64_t i, uin
                 ox = o.x;
                 if (cmp) break;
             }
-            pos = (pos + 1) & a.slot_mask;
-            if (++probe > a.slot_mask) {
-                record_diag(a.ctr, ERR_TABLE_FULL, 8, (long long)i, (long long)a.slot_mask, a.level);
+            pos = (pos + 1) & mask;
+            if (++probe > mask) {
+                record_diag(a.ctr, ERR_TABLE_FULL, 8, (long long)i, (long long)mask, a.level);
                 todo = false;
             }
         }
@@ -1370,7 +1349,7 @@ __device__ __forceinline__ void dedup_insert(const LevelArgs &a, uint64_t i, uin
                     a.child.hdr[i].y = 0u;
                     todo = false;
                 } else {
-                    pos = (pos + 1) & a.slot_mask;
+                    pos = (pos + 1) & mask;
                     ++probe;
                 }
             }
@@ -1379,9 +1358,12 @@ __device__ __forceinline__ void dedup_insert(const LevelArgs &a, uint64_t i, uin
 }
 
 template <int F, bool SUB>
-__global__ void __launch_bounds__(256, 6) dedup_kernel(NetView nv, LevelArgs a)
+__global__ void __launch_bounds__(256, 6) dedup_kernel(const __grid_constant__ NetView nv,
+                                                       const __grid_constant__ LevelArgs a)
 {
     __shared__ unsigned long long s_keep[8], s_deg[8], s_unv[8];
+    if (a.st[S_STOP] != STOP_NONE) return;
+    const uint64_t mask = a.st[S_SLOTS] - 1;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint64_t begin = a.ctr[C_DEDUP_BEGIN];
     uint64_t end = a.ctr[C_WRITTEN];
@@ -1391,8 +1373,9 @@ __global__ void __launch_bounds__(256, 6) dedup_kernel(NetView nv, LevelArgs a)
     const uint64_t t0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     // the open children, spread over the whole grid
+    // (from its end: at a small level other CTAs than those with its rows)
     const uint64_t n_open = a.ctr[C_OPEN];
-    for (uint64_t q0 = t0; q0 < n_open; q0 += stride) {
+    for (uint64_t q0 = stride - blockDim.x - (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); q0 < n_open; q0 += stride) {
         uint64_t i = 0, f = kDeadFp;
         uint4 h = make_uint4(0u, 0u, 0u, 0u);
         if (q0 + lane < n_open) {
@@ -1400,7 +1383,7 @@ __global__ void __launch_bounds__(256, 6) dedup_kernel(NetView nv, LevelArgs a)
             f = finish_open<F, SUB>(nv, a, a.fp[i], i, h);
             if (h.y == 0u && i < row_cap) a.child.hdr[i] = h;
         }
-        dedup_insert<F>(a, i, f, h, lane, sum);
+        dedup_insert<F>(a, mask, i, f, h, lane, sum);
     }
     for (uint64_t i0 = begin + t0; i0 < end; i0 += stride) {
         const uint64_t i = i0 + lane;
@@ -1408,7 +1391,7 @@ __global__ void __launch_bounds__(256, 6) dedup_kernel(NetView nv, LevelArgs a)
         if (f >> 63) f = kDeadFp;  // nothing, or an open child
         uint4 h = make_uint4(0u, 0u, 0u, 0u);
         if (f != kDeadFp && i < row_cap) h = a.child.hdr[i];
-        dedup_insert<F>(a, i, f, h, lane, sum);
+        dedup_insert<F>(a, mask, i, f, h, lane, sum);
     }
     unsigned long long deg = sum.deg, n_unv = sum.unv, n_keep = sum.keep;
 #pragma unroll
@@ -1434,12 +1417,6 @@ __global__ void __launch_bounds__(256, 6) dedup_kernel(NetView nv, LevelArgs a)
         if (d) atomicAdd(&a.ctr[C_DEGSUM], d);
         if (u) atomicAdd(&a.ctr[C_UNV], u);
     }
-}
-
-__global__ void dedup_advance_kernel(unsigned long long *ctr)
-{
-    ctr[C_DEDUP_BEGIN] = ctr[C_WRITTEN];
-    ctr[C_OPEN] = 0ull;
 }
 
 // ---------------------------------------------------------------------------
@@ -1640,96 +1617,18 @@ __global__ void __launch_bounds__(32) seedset_kernel(NetView nv, LevelArgs a, co
     atomicAdd(&a.ctr[C_DEGSUM], (unsigned long long)(bkey >> 16));
 }
 
-// ---------------------------------------------------------------------------
-// the superset rule's index over the accepted results
-// ---------------------------------------------------------------------------
-
-// Both kernels take the results [r0, r1), a warp each: results are filed once,
-// at the level after the one that accepted them (the sentinels by the counts
-// of that moment: any other column of a result is a valid sentinel).
-__global__ void cell_count_kernel(const uint64_t *res, int W, int64_t r0, int64_t r1, int32_t *cnt)
+// results [0, n) into an empty index, a warp each (the minimality test files
+// what it accepts; this is for an index that has to grow)
+__global__ void __launch_bounds__(128) index_kernel(CellIndex ix, const uint64_t *res, int W, int64_t n)
 {
-    const int lane = threadIdx.x & 31;
-    for (int64_t r = r0 + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); r < r1;
-         r += ((int64_t)gridDim.x * blockDim.x) >> 5)
-        for (int w = lane; w < W; w += 32)
-            for (uint64_t x = res[(size_t)r * W + w]; x; x &= x - 1) atomicAdd(&cnt[w * 64 + __ffsll((long long)x) - 1], 1);
-}
-
-template <int F>
-__global__ void cell_insert_kernel(const uint64_t *res, int W, int64_t r0, int64_t r1, const int32_t *cnt, CellIndex ix,
-                                   int ent_stride)
-{
-    const int lane = threadIdx.x & 31;
-    for (int64_t r = r0 + (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5); r < r1;
+    __shared__ int cols[4][64];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n;
          r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const uint64_t *E = res + (size_t)r * W;
-        const uint64_t word[2] = {lane < W ? E[lane] : 0ull, lane + 32 < W ? E[lane + 32] : 0ull};
-        // the two columns with the fewest results (ties by column), and the signature
-        unsigned long long k1 = ~0ull, k2 = ~0ull;
-        uint64_t sig = 0;
-        int m = 0;
-        for (int h = 0; h < 2; ++h)
-            for (uint64_t x = word[h]; x; x &= x - 1) {
-                const int c = (lane + 32 * h) * 64 + __ffsll((long long)x) - 1;
-                ++m;
-                sig |= col_bit(c);
-                const unsigned long long key = ((unsigned long long)cnt[c] << 16) | (unsigned)c;
-                if (key < k1) {
-                    k2 = k1;
-                    k1 = key;
-                } else if (key < k2) {
-                    k2 = key;
-                }
-            }
-        int before = m;  // columns of the lanes below
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int x = __shfl_up_sync(FULL, before, off);
-            if (lane >= off) before += x;
-        }
-        const int total = __shfl_sync(FULL, before, 31);
-        before -= m;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const unsigned long long o1 = __shfl_xor_sync(FULL, k1, off), o2 = __shfl_xor_sync(FULL, k2, off);
-            const unsigned long long hi = k1 > o1 ? k1 : o1;  // the second of the four
-            k2 = k2 < o2 ? k2 : o2;
-            k2 = k2 < hi ? k2 : hi;
-            k1 = k1 < o1 ? k1 : o1;
-            sig |= __shfl_xor_sync(FULL, sig, off);
-        }
-        const int m1 = (int)(k1 & 0xFFFFull), m2 = (int)(k2 & 0xFFFFull);
-        if (total == 1) {  // a one-column result: every child adding that column contains it
-            if (lane == 0) ix.single[m1] = 1u;
-            continue;
-        }
-        int64_t id = r * ent_stride + before;
-        for (int h = 0; h < 2; ++h)
-            for (uint64_t x = word[h]; x; x &= x - 1, ++id) {
-                const int k = (lane + 32 * h) * 64 + __ffsll((long long)x) - 1;
-                const int s = k == m1 ? m2 : m1;
-                if (F) {
-                    atomicOr((unsigned long long *)&ix.ksig[2 * k + (s >> 6)], 1ull << (s & 63));
-                    const uint32_t next = atomicExch(reinterpret_cast<uint32_t *>(ix.cells) + 128 * k + s, (uint32_t)id);
-                    const uint64_t e0 = E[0], e1 = W == 2 ? E[1] : 0ull;
-                    ix.ent[2 * id] = make_uint4((uint32_t)e0, (uint32_t)(e0 >> 32), (uint32_t)e1, (uint32_t)(e1 >> 32));
-                    ix.ent[2 * id + 1] = make_uint4(next, (uint32_t)r, 0u, 0u);
-                    continue;
-                }
-                atomicOr((unsigned long long *)&ix.ksig[k], (unsigned long long)col_bit(s));
-                const uint32_t key = ((uint32_t)k << 12) | (uint32_t)s;
-                uint32_t p = cell_slot(key, ix.mask);
-                for (uint32_t probe = 0; probe <= ix.mask; ++probe) {
-                    const uint32_t v = atomicCAS(&ix.cells[p].x, kNoRecord, key);
-                    if (v == kNoRecord || v == key) {
-                        const uint32_t next = atomicExch(&ix.cells[p].y, (uint32_t)id);
-                        ix.ent[id] = make_uint4((uint32_t)sig, (uint32_t)(sig >> 32), next, (uint32_t)r);
-                        break;
-                    }
-                    p = (p + 1) & ix.mask;
-                }
-            }
+        const uint64_t u0 = lane < W ? res[(size_t)r * W + lane] : 0ull;
+        const uint64_t u1 = lane + 32 < W ? res[(size_t)r * W + lane + 32] : 0ull;
+        const int m = support_columns(u0, u1, cols[wid]);
+        file_result(ix, W, r, cols[wid], m, __shfl_sync(FULL, u0, 0), __shfl_sync(FULL, u0, 1));
         __syncwarp();
     }
 }
@@ -1814,7 +1713,6 @@ cudaError_t launch_dedup(const NetView &nv, const LevelArgs &a, int sm_count, cu
 #define EFM_LAUNCH(K) K<<<sm_count * 8, 256, 0, s>>>(nv, a)
     EFM_FORM(dedup_kernel, EFM_LAUNCH);
 #undef EFM_LAUNCH
-    dedup_advance_kernel<<<1, 1, 0, s>>>(a.ctr);
     return cudaGetLastError();
 }
 
@@ -1842,25 +1740,17 @@ size_t cell_table_bytes(const NetView &nv, uint64_t entries)
     return (size_t)p * 8;
 }
 
-cudaError_t launch_cells(const NetView &nv, const uint64_t *res, int64_t r0, int64_t r1, int32_t *cnt,
-                         const CellIndex &ix, int ent_stride, cudaStream_t s)
+cudaError_t launch_index(const NetView &nv, const CellIndex &ix, const uint64_t *res, int64_t n, cudaStream_t s)
 {
     cudaError_t e;
     const int W = nv.W;
-    if (r0 == 0) {
-        const size_t table = W <= 2 ? (size_t)128 * nv.N * 4 : 8 * ((size_t)ix.mask + 1);
-        if ((e = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)nv.N, s)) != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(ix.ksig, 0, 16 * (size_t)nv.N, s)) != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(ix.single, 0, 4 * (size_t)nv.N, s)) != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(ix.cells, 0xFF, table, s)) != cudaSuccess) return e;
-    }
-    if (r1 <= r0) return cudaSuccess;
-    const unsigned blocks = (unsigned)std::min<int64_t>((r1 - r0 + 3) / 4, 4096);
-    cell_count_kernel<<<blocks, 128, 0, s>>>(res, W, r0, r1, cnt);
-    if (W <= 2)
-        cell_insert_kernel<1><<<blocks, 128, 0, s>>>(res, W, r0, r1, cnt, ix, ent_stride);
-    else
-        cell_insert_kernel<0><<<blocks, 128, 0, s>>>(res, W, r0, r1, cnt, ix, ent_stride);
+    const size_t table = W <= 2 ? (size_t)128 * nv.N * 4 : 8 * ((size_t)ix.mask + 1);
+    if ((e = cudaMemsetAsync(ix.cnt, 0, sizeof(int32_t) * (size_t)nv.N, s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(ix.ksig, 0, 16 * (size_t)nv.N, s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(ix.single, 0, 4 * (size_t)nv.N, s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(ix.cells, 0xFF, table, s)) != cudaSuccess) return e;
+    if (n <= 0) return cudaSuccess;
+    index_kernel<<<(unsigned)std::min<int64_t>((n + 3) / 4, 4096), 128, 0, s>>>(ix, res, W, n);
     return cudaGetLastError();
 }
 
