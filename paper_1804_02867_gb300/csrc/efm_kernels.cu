@@ -284,6 +284,237 @@ __device__ __forceinline__ void walk_normalise(const int64_t (&t64)[EPL], int32_
     ovf = __any_sync(FULL, bad);
 }
 
+// --- narrow networks (at most 64 internal rows and 128 columns): a walk per
+// lane.  A lane's row sits in shared memory, entry m of lane l at 32 m + l (no
+// bank conflicts whatever rows the lanes touch); which entries are nonzero,
+// their signs at the pivot keys' ranks and the +-1 rows are masks in
+// registers, so a step touches the rows of column k alone unless A > 1 or no
+// +-1 entry proves the gcd to be 1.  A lane takes its next walk as soon as one
+// ends.  Bound by issue: one GB300, core-shaped network, 2^20 walks of at most
+// 30 columns: 27.0 ms with a warp per walk and 64-bit rows in registers, 4.2
+// ms this way (the whole call 28.9 -> 4.5). ---
+
+constexpr int kWalkWarps = 4;
+
+__device__ __forceinline__ int walk_pick(uint64_t x, int n)  // x mod n, n <= EFM_MAX_COLUMNS
+{
+    const uint32_t c = (uint32_t)n;
+    const uint32_t p = (0xFFFFFFFFu % c + 1u) % c;  // 2^32 mod n
+    return (int)((((uint32_t)(x >> 32) % c) * p + (uint32_t)x % c) % c);
+}
+
+struct WalkState {
+    uint64_t zm, pm, nm, um;  // nonzero rows; positive / negative entries by key rank; +-1 rows
+    uint32_t pmax;            // at least the largest magnitude
+};
+
+// The row divided by g, or rebuilt by f(row, old value) in 64 bits first (the
+// rows of rows); exact masks and magnitude.  False: an entry outside int32.
+template <typename Value>
+__device__ __noinline__ bool walk_rebuild(const NetView &nv, const uint32_t *bl, int32_t *row, uint64_t rows, WalkState &z,
+                                          Value f)
+{
+    uint64_t g = 0, mx = 0;
+    for (uint64_t x = rows; x; x &= x - 1) {
+        const int m = __ffsll((long long)x) - 1;
+        const uint64_t at = abs64(f(m));
+        if (at) g = gcd64(g, at);
+        mx = at > mx ? at : mx;
+    }
+    if (g == 0) {
+        z = WalkState{0, 0, 0, 0, 0};
+        return true;
+    }
+    if (mx / g > 2147483647ull) return false;
+    WalkState y{0, 0, 0, 0, (uint32_t)(mx / g)};
+    for (uint64_t x = rows; x; x &= x - 1) {
+        const int m = __ffsll((long long)x) - 1;
+        const int32_t v = (int32_t)(f(m) / (int64_t)g);
+        row[32 * m] = v;
+        if (v == 0) continue;
+        const uint32_t rk = bl[nv.o_rank + m];
+        y.zm |= 1ull << m;
+        if (v > 0) y.pm |= 1ull << (rk & 0xFFu);
+        else y.nm |= 1ull << ((rk >> 8) & 0xFFu);
+        if (v == 1 || v == -1) y.um |= 1ull << m;
+    }
+    z = y;
+    return true;
+}
+
+__global__ void __launch_bounds__(kWalkWarps * 32) walk_narrow_kernel(const __grid_constant__ NetView nv,
+                                                                      const __grid_constant__ LevelArgs a, int target,
+                                                                      uint64_t seed, int64_t n_walks)
+{
+    extern __shared__ int32_t s_rows[];  // per warp: M x 32 entries
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int32_t *row = s_rows + (size_t)wid * 32 * nv.M + lane;
+    const uint32_t *bl = nv.blob;
+    const uint4 *scol = reinterpret_cast<const uint4 *>(bl + nv.o_scol);
+    const uint2 *nent = reinterpret_cast<const uint2 *>(bl + nv.o_nent);
+    const int tb = target >= 0 ? nv.metptr[target] : 0, te = target >= 0 ? nv.metptr[target + 1] : 0;
+    int n_seeds = target >= 0 ? 0 : nv.N;
+    for (int q = tb; q < te; ++q) n_seeds += ent_coef(nv.metent[q]) > 0 ? 1 : 0;
+    unsigned n_walk = 0, n_exp = 0, n_ovf = 0, n_bal = 0, n_dead = 0, max_steps = 0;
+    const int64_t total = (int64_t)gridDim.x * blockDim.x;
+    int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    bool running = false;
+    WalkState z{0, 0, 0, 0, 0};
+    uint64_t U[2] = {0, 0};
+    int j = 0, pc = 0, sec = 0, s = 0;
+    if (n_seeds == 0) w = n_walks;
+    while (w < n_walks) {
+        bool ended = false;
+        if (!running) {
+            // the seed: the pick-th positive entry of the target's row
+            int pick = walk_pick(splitmix_at(seed, (uint64_t)w * 128u), n_seeds);
+            j = pick;
+            if (target >= 0)
+                for (int q = tb; q < te; ++q) {
+                    const uint32_t e = nv.metent[q];
+                    if (ent_coef(e) <= 0) continue;
+                    if (pick-- == 0) {
+                        j = ent_index(e);
+                        break;
+                    }
+                }
+            ++n_walk;
+            U[0] = j < 64 ? 1ull << j : 0ull;
+            U[1] = j < 64 ? 0ull : 1ull << (j - 64);
+            pc = 1;
+            sec = 0;
+            s = 0;
+            running = true;
+            const uint4 s1 = scol[2 * j + 1];
+            uint64_t rows = 0;
+            for (int q = (int)s1.y; q < (int)s1.z; ++q) {
+                const uint2 e = nent[q];
+                row[32 * (e.x & 63u)] = (int32_t)e.y;
+                rows |= 1ull << (e.x & 63u);
+            }
+            walk_rebuild(nv, bl, row, rows, z, [&](int m) { return (int64_t)row[32 * m]; });
+        }
+        ++s;  // this step's number
+        if (z.zm == 0) {
+            ++n_bal;
+            insert_support(a, nv.W, U, j);  // (a failure sets the error word)
+            ended = true;
+        } else if (s > 127) {  // every step adds a column or a secondary step: unreachable
+            record_diag(a.ctr, ERR_BOUNDS, 5, s, 127, 0);
+            ended = true;
+        } else {
+            const uint32_t key = mask_key(bl, nv, z.pm, z.nm);
+            const int piv = (int)(key & 0xFFFFu);
+            const int32_t bi = row[32 * piv];
+            const bool fwd = bi > 0;
+            const int lptr = (fwd ? nv.o_consptr : nv.o_prodptr) + piv;
+            const int lb = (int)bl[lptr], le = (int)bl[lptr + 1];
+            const uint32_t *list = bl + (fwd ? nv.o_consent : nv.o_prodent);
+            auto valid = [&](int q) -> bool {
+                const int k = ent_index(list[q]);
+                const uint32_t tw = bl[nv.o_twin + k];
+                if (tw != 0xFFFFFFFFu && (((tw < 64u ? U[0] : U[1]) >> (tw & 63u)) & 1ull)) return false;
+                return (((k < 64 ? U[0] : U[1]) >> (k & 63)) & 1ull) ? sec + 1 <= a.max_sec : pc + 1 <= a.max_len;
+            };
+            int cnt = 0;
+            for (int q = lb; q < le; ++q) cnt += valid(q) ? 1 : 0;
+            if (cnt == 0) {
+                ++n_dead;
+                ended = true;
+            } else {
+                int r = walk_pick(splitmix_at(seed, (uint64_t)w * 128u + (uint64_t)s), cnt);
+                int qs = lb;
+                for (int q = lb; q < le; ++q)
+                    if (valid(q) && r-- == 0) {
+                        qs = q;
+                        break;
+                    }
+                const uint32_t br = list[qs];
+                const int k = ent_index(br);
+                const uint32_t sik = (uint32_t)ent_coef(br), abi = mag(bi);
+                const uint32_t g0 = (abi == 1u || sik == 1u) ? 1u : gcd32(abi, sik);
+                const int32_t A = (int32_t)(sik / g0), C = (int32_t)(abi / g0);
+                ++n_exp;
+                if (((k < 64 ? U[0] : U[1]) >> (k & 63)) & 1ull) {
+                    ++sec;
+                } else {
+                    if (k < 64) U[0] |= 1ull << k;
+                    else U[1] |= 1ull << (k - 64);
+                    ++pc;
+                }
+                j = k;
+                const uint4 s1 = scol[2 * k + 1];
+                const int cb = (int)s1.y, ce = (int)s1.z;
+                const int ox = nv.o_colx + 10 * k;
+                const uint64_t mask = blob_u64(bl, ox + 4);
+                if ((uint64_t)A * z.pmax + (uint64_t)C * s1.x < 0x80000000ull) {
+                    uint64_t newz = 0, newp = 0, newn = 0, newu = 0;
+                    uint32_t mx = (uint32_t)A * z.pmax;
+                    for (int q = cb; q < ce; ++q) {
+                        const uint2 e = nent[q];
+                        const int m = (int)(e.x & 63u);
+                        const int32_t v = (z.zm >> m) & 1ull ? row[32 * m] : 0;
+                        const int32_t t = A * v + C * (int32_t)e.y;
+                        row[32 * m] = t;
+                        newz |= (uint64_t)(t != 0) << m;
+                        newp |= (uint64_t)(t > 0) << ((e.x >> 8) & 63u);
+                        newn |= (uint64_t)(t < 0) << ((e.x >> 16) & 63u);
+                        newu |= (uint64_t)(t == 1 || t == -1) << m;
+                        mx = max(mx, mag(t));
+                    }
+                    const uint64_t keep = z.zm & ~mask;
+                    if (A != 1)
+                        for (uint64_t x = keep; x; x &= x - 1) row[32 * (__ffsll((long long)x) - 1)] *= A;
+                    z.zm = keep | newz;
+                    z.pm = (z.pm & ~blob_u64(bl, ox)) | newp;
+                    z.nm = (z.nm & ~blob_u64(bl, ox + 2)) | newn;
+                    z.um = (A == 1 ? z.um & ~mask : 0ull) | newu;
+                    z.pmax = mx;
+                    if (z.um == 0 && z.zm != 0) {
+                        uint32_t g = 0;
+                        for (uint64_t x = z.zm; x && g != 1u; x &= x - 1)
+                            g = gcd_small(g, mag(row[32 * (__ffsll((long long)x) - 1)]));
+                        if (g != 1u)
+                            walk_rebuild(nv, bl, row, z.zm, z, [&](int m) { return (int64_t)row[32 * m]; });
+                    }
+                } else {
+                    // an entry may leave int32 before the division: in 64 bits
+                    const uint64_t zm = z.zm;
+                    const bool fit = walk_rebuild(nv, bl, row, zm | mask, z, [&](int m) {
+                        int64_t t = (zm >> m) & 1ull ? (int64_t)A * row[32 * m] : 0;
+                        if ((mask >> m) & 1ull)
+                            for (int q = cb; q < ce; ++q) {
+                                const uint2 e = nent[q];
+                                if ((int)(e.x & 63u) == m) t += (int64_t)C * (int32_t)e.y;
+                            }
+                        return t;
+                    });
+                    if (!fit) {
+                        ++n_ovf;
+                        ended = true;
+                    }
+                }
+                max_steps = max(max_steps, (unsigned)s);
+            }
+        }
+        if (ended) {
+            running = false;
+            w += total;
+        }
+    }
+    auto total_of = [&](unsigned v, int id) {
+        const unsigned t = __reduce_add_sync(FULL, v);  // (a lane's walks and steps are far below 2^27)
+        if (lane == 0 && t) atomicAdd(&a.ctr[id], (unsigned long long)t);
+    };
+    total_of(n_walk, C_SEEDS);
+    total_of(n_exp, C_EXP);
+    total_of(n_ovf, C_OVF);
+    total_of(n_bal, C_BAL);
+    total_of(n_dead, C_PRUNED);
+    const unsigned most = __reduce_max_sync(FULL, max_steps);
+    if (lane == 0 && most) atomicMax(&a.ctr[C_LEVELS], (unsigned long long)most);
+}
+
 template <int EPL>
 __global__ void __launch_bounds__(kExpandWarps * 32) walk_kernel(NetView nv, LevelArgs a, int target, uint64_t seed,
                                                                  int64_t n_walks)
@@ -1717,6 +1948,19 @@ cudaError_t launch_walks(const NetView &nv, const LevelArgs &a, int target, uint
                          cudaStream_t s)
 {
     if (n_walks <= 0) return cudaSuccess;
+    if (nv.form == 2) {
+        const size_t sm = (size_t)kWalkWarps * 32 * 4 * (size_t)std::max(nv.M, 1);
+        int per_sm = 1;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_narrow_kernel, kWalkWarps * 32, sm) != cudaSuccess ||
+            per_sm < 1) {
+            cudaGetLastError();
+            per_sm = 1;
+        }
+        const int64_t blocks = (n_walks + kWalkWarps * 32 - 1) / (kWalkWarps * 32);
+        walk_narrow_kernel<<<(int)std::min<int64_t>(blocks, (int64_t)sm_count * per_sm), kWalkWarps * 32, sm, s>>>(
+            nv, a, target, seed, n_walks);
+        return cudaGetLastError();
+    }
     const int64_t want = (n_walks + kExpandWarps - 1) / kExpandWarps;
     const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count * 8);
     switch (nv.EPL) {

@@ -67,3 +67,46 @@ def test_capped(oracle_lib, efm, max_results):
     for t, (sup, ctr) in zip(net.targets, got):
         osup, octr = oracle_lib.enumerate_pathways(net, t, oracle_lib.Limits(20, 2, max_results, 1 << 14))
         assert np.array_equal(sup, osup) and ctr == octr, (t, ctr, octr)
+
+
+EDGES = {
+    # narrow form: long columns (past the eight a lane keeps), divisors, int32 left
+    "narrow": dict(n_int=40, n_rxn=70, n_rev=15, size_range=(2, 14), coef_probs={1: 0.3, 6: 0.3, 10: 0.3, 524287: 0.1}),
+    # 64 rows, 128 columns: the last narrow network
+    "narrow-last": dict(n_int=64, n_rxn=104, n_rev=24, size_range=(2, 5), coef_probs={1: 0.6, 2: 0.2, 4: 0.2}),
+    # one row, one column more: the next two forms
+    "bits": dict(n_int=65, n_rxn=104, n_rev=24, size_range=(2, 5), coef_probs={1: 0.6, 2: 0.2, 4: 0.2}),
+    "list": dict(n_int=64, n_rxn=105, n_rev=24, size_range=(2, 5), coef_probs={1: 0.6, 2: 0.2, 4: 0.2}),
+    # one support word
+    "one-word": dict(n_int=30, n_rxn=50, n_rev=10, size_range=(2, 5), coef_probs={1: 0.5, 3: 0.5}),
+}
+
+
+def edge_network(name):
+    return synth.generate(n_targets=3, n_hubs=2, n_substrates=2, gamma=None, hub_degree=(3, 10), seed=11, name=name,
+                          **EDGES[name])
+
+
+@pytest.mark.parametrize("name", sorted(EDGES))
+def test_forms(oracle_lib, efm, name):
+    net = edge_network(name)
+    out = check(oracle_lib, efm, net, net.targets + [-1], 16, 3, 1 << 13)
+    if name == "narrow":
+        assert any(c["overflow"] for c in out)
+    with efm.Network(net) as nw:
+        for t in net.targets:
+            (got, _), = efm.enumerate_targets(nw, [t], 9, 2, 0, 1 << 16, first_k=5)
+            want, _ = oracle_lib.first_k(net, t, 5, 9, 2)
+            assert np.array_equal(got, want), (name, t)
+
+
+@pytest.mark.parametrize("name", ["narrow", "narrow-last", "one-word"])
+def test_lane_walks(oracle_lib, efm, name):
+    """A walk per lane: divisions, int32 left, both support words."""
+    net = edge_network(name)
+    with efm.Network(net) as nw:
+        for t in net.targets + [-1]:
+            for n in (1, 33, 4000):
+                sup, ctr = efm.sample_target(nw, t, 20, 3, 5, n)
+                osup, octr = oracle_lib.sample_pathways(net, t, oracle_lib.Limits(20, 3), 5, n)
+                assert np.array_equal(sup, osup) and ctr == octr, (name, t, n, ctr, octr)
