@@ -276,7 +276,7 @@ typedef struct {
     int32_t tile;            /* most parents a warp expands per pass, 1..32 */
     int32_t queue_chunk;     /* queue positions a CTA claims per atomic, 1..64 */
     int32_t pinned;          /* output only: 1 when efm_batch_set_tuning chose it */
-    float sample_default_ms; /* output only: the tuning sample (up to 256 jobs, strided) in the untuned
+    float sample_default_ms; /* output only: the tuning sample (up to 1024 jobs, strided) in the untuned
                                 configuration (8 warps, every CTA an SM holds, input order, tile 32,
                                 chunk 1); 0 when no search ran */
     float sample_tuned_ms;   /* output only: the same sample in the chosen configuration */

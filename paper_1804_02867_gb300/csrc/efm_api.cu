@@ -84,7 +84,7 @@ struct efm_net {
 
 struct TargetOut {
     DevBuf sup;
-    const uint64_t *borrowed = nullptr;  // batched jobs: rows inside the job's shared buffer
+    int64_t host_at = -1;                // batched jobs: the rows' place in the job's host array
     int err = 0;                         // batched jobs: this job's error code (0 = none)
     int64_t n = 0;
     efm_counters ctr{};
@@ -97,7 +97,7 @@ struct efm_job {
     efm_net *net = nullptr;
     std::vector<TargetOut> out;
     std::vector<int> words;  // batched jobs: support width of each entry
-    DevBuf shared_out;       // batched jobs: output rows of every job
+    std::vector<uint64_t> host_out;  // batched jobs: output rows of every job
 };
 
 // Proposal model: FP32 parameters, their gradients and Adam moments, the
@@ -554,7 +554,6 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
     acc.ctr = ctr;
     acc.cand_cap = w.cand_cap;
     acc.st = st;
-    acc.level0 = level0;
     acc.max_level = lim.max_len + lim.max_secondary + 1;
     acc.max_frontier = lim.max_frontier;
     acc.max_results = lim.max_results;
@@ -1362,43 +1361,47 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Scratch slice of one CTA of the batched traversal, sized for the largest
 // network of the batch.
-BatchLayout batch_layout(int64_t cap, int Wmax, int Mpad_max, int Nmax, int max_len_max)
+BatchLayout batch_layout(int64_t budget, int Wmax, int Nmax, int max_len_max, uint64_t seed_units)
 {
     BatchLayout L{};
-    L.cap = cap;
+    // rows before deduplication: a level whose children pass the budget is
+    // decided by their distinct count, so 1.5 times the budget at large
+    // budgets and up to 8 times at small ones (a job that needs more is run by
+    // the host alone)
+    L.cap = std::max<int64_t>(budget + budget / 2 + 64, std::min<int64_t>(8 * budget, 32768));
+    L.pay_cap = std::min<uint64_t>(std::max<uint64_t>((uint64_t)L.cap * 12, seed_units), 0xFFFFFFFFull);
+    L.fp_cap = 2 * L.cap + 4096;
     L.cand_cap = (int64_t)1 << 15;
     L.res_cap = (int64_t)1 << 13;
-    L.slot_cap = next_pow2(2 * (uint64_t)cap + 64 * (uint64_t)(kBatchThreads / 32));
+    L.slot_cap = next_pow2(2 * (uint64_t)L.fp_cap + 64);
     L.cslot_cap = next_pow2(2 * (uint64_t)L.cand_cap);
+    L.index_room = 2048;
+    L.ent_stride = max_len_max;
+    const uint64_t entries = (uint64_t)L.index_room * max_len_max;
+    L.cell_mask = (uint32_t)(next_pow2(2 * entries) - 1);
     size_t o = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = o;
+        o = align256(o + bytes);
+        return at;
+    };
     for (int i = 0; i < 2; ++i) {
-        L.o_U[i] = o;
-        o = align256(o + (size_t)cap * Wmax * 8);
-        L.o_B[i] = o;
-        o = align256(o + (size_t)cap * Mpad_max * 4);
-        L.o_meta[i] = o;
-        o = align256(o + (size_t)cap * 4);
+        L.o_hdr[i] = take((size_t)L.cap * 16);
+        L.o_pay[i] = take((size_t)L.pay_cap * 16);
     }
-    L.o_slots = o;
-    o = align256(o + L.slot_cap * 8);
-    L.o_cslots = o;
-    o = align256(o + L.cslot_cap * 8);
-    L.o_cand = o;
-    o = align256(o + (size_t)L.cand_cap * Wmax * 8);
-    L.o_res = o;
-    o = align256(o + (size_t)L.res_cap * Wmax * 8);
-    L.o_bcnt = o;
-    o = align256(o + (size_t)Nmax * 4);
-    L.o_bfill = o;
-    o = align256(o + (size_t)Nmax * 4);
-    L.o_bptr = o;
-    o = align256(o + (size_t)(Nmax + 1) * 4);
-    L.o_bres = o;
-    o = align256(o + (size_t)L.res_cap * max_len_max * Wmax * 8);
-    L.o_sort = o;
-    o = align256(o + next_pow2((uint64_t)L.res_cap) * 4);
-    L.o_rcols = o;
-    o = align256(o + (Wmax > 2 ? (size_t)L.res_cap * kRcolStride * 2 : 16));
+    L.o_slots = take(L.slot_cap * 8);
+    L.o_fp = take((size_t)L.fp_cap * 8);
+    L.o_open = take((size_t)L.fp_cap * 4);
+    L.o_cslots = take(L.cslot_cap * 8);
+    L.o_cand = take((size_t)L.cand_cap * Wmax * 8);
+    L.o_res = take((size_t)L.res_cap * Wmax * 8);
+    L.o_cnt = take((size_t)Nmax * 4);
+    L.o_ksig = take((size_t)Nmax * 16);
+    L.o_single = take((size_t)Nmax * 4);
+    L.o_cells = take(std::max<size_t>((size_t)128 * 128 * 4, Wmax > 2 ? 8 * ((size_t)L.cell_mask + 1) : 0));
+    L.o_ent = take((size_t)entries * 32);
+    L.o_sort = take(next_pow2((uint64_t)L.res_cap) * 4);
+    L.o_rcols = take(Wmax > 2 ? (size_t)L.res_cap * kRcolStride * 2 : 16);
     L.slice_bytes = o;
     return L;
 }
@@ -1428,30 +1431,32 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
     if (lim.max_len < 1 || lim.max_len > EFM_MAX_LEN || lim.max_secondary < 0 || lim.first_k != 0 ||
         lim.proposal != 0 || lim.max_frontier <= 0 || lim.variant != EFM_ADDITIVE || lim.reserved != 0)
         return EFM_EINVAL;
-    int Wmax = 1, Mpad_max = 32, Nmax = 1, Lmax = 1, max_epl = 1;
+    int Wmax = 1, Nmax = 1, Lmax = 1, max_epl = 1;
+    uint64_t seed_units = 0;  // payload units every seed of a network takes at most
     for (int i = 0; i < n_jobs; ++i) {
         const efm_net *n = nets[i];
         if (!n || targets[i] < -1 || targets[i] >= n->n_met) return EFM_EINVAL;
         if (n->nv.EPL > 8) return EFM_EUNSUPPORTED;
         Wmax = std::max(Wmax, n->nv.W);
-        Mpad_max = std::max(Mpad_max, n->nv.Mpad);
+        seed_units = std::max<uint64_t>(seed_units, (uint64_t)(n->nv.o_consptr - n->nv.o_colent) + 5ull * (uint64_t)n->nv.N + 1024);
         Nmax = std::max(Nmax, n->nv.N);
         Lmax = std::max(Lmax, std::min(lim.max_len, n->nv.N));
         max_epl = std::max(max_epl, n->nv.EPL);
     }
     efm_net *net0 = nets[0];
     cudaStream_t s = net0->stream;
-    const BatchLayout L = batch_layout(lim.max_frontier + 1, Wmax, Mpad_max, Nmax, Lmax);
+    const BatchLayout L = batch_layout(lim.max_frontier, Wmax, Nmax, Lmax, seed_units);
     const int occ8 = batch_blocks_per_sm(8), occ4 = batch_blocks_per_sm(4);
     const int occ = std::max(occ8, occ4);  // slices for the largest grid any configuration launches
     const int sms = net0->sm_count;
+    const int slices = std::min(sms * occ, n_jobs);  // a CTA more than there are jobs has nothing to do
 
     auto *job = new (std::nothrow) efm_job();
     if (!job) return EFM_ENOMEM;
     job->net = net0;
     job->out.resize(n_jobs);
     job->words.resize(n_jobs);
-    DevBuf pool, djobs, dorder, dctr, dqueue;
+    DevBuf pool, djobs, dorder, dctr, dqueue, dout, dpack, doff;
     const size_t out_rows = (size_t)L.res_cap;
     int rc = EFM_OK;
     std::vector<BatchJob> hj(n_jobs);
@@ -1463,11 +1468,14 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
     float ms = 0.f;
     TuneChoice best;
     BatchArgs ba{};
+    std::vector<int> alone;  // jobs whose levels did not fit a slice
+    std::vector<int64_t> offs((size_t)n_jobs + 1, 0);  // output words of the jobs before each
 
-    if (!dev_alloc(pool, (size_t)sms * occ * L.slice_bytes, s) ||
+    if (!dev_alloc(pool, (size_t)slices * L.slice_bytes, s) ||
         !dev_alloc(djobs, sizeof(BatchJob) * (size_t)n_jobs, s) || !dev_alloc(dorder, 4 * (size_t)n_jobs, s) ||
         !dev_alloc(dctr, 8 * (size_t)C_COUNT * n_jobs, s) || !dev_alloc(dqueue, 16, s) ||
-        !dev_alloc(job->shared_out, out_rows * Wmax * 8 * (size_t)n_jobs, s)) {
+        !dev_alloc(dout, out_rows * Wmax * 8 * (size_t)n_jobs, s) ||
+        !dev_alloc(doff, 8 * ((size_t)n_jobs + 1), s)) {
         rc = EFM_ENOMEM;
         goto done;
     }
@@ -1475,7 +1483,7 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
         hj[i].nv = nets[i]->nv;
         hj[i].target = targets[i];
         hj[i].max_len = std::min(lim.max_len, nets[i]->nv.N);
-        hj[i].out = (uint64_t *)job->shared_out.p + (size_t)i * out_rows * Wmax;
+        hj[i].out = (uint64_t *)dout.p + (size_t)i * out_rows * Wmax;
         hj[i].ctr = (unsigned long long *)dctr.p + (size_t)i * C_COUNT;
         order_in[i] = i;
         order_big[i] = i;
@@ -1522,7 +1530,7 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
             }
         }
         if (!have && n_jobs >= 64) {
-            const int sample = std::min(n_jobs, 256);
+            const int sample = std::min(n_jobs, 1024);
             auto time_cfg = [&](const TuneChoice &c, float &t) -> bool {
                 const std::vector<int> &ord = c.big ? order_big : order_in;
                 // a strided sample keeps the size mix of the whole batch
@@ -1534,7 +1542,7 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
                 if (cudaMemcpyAsync(dorder.p, samp.data(), 4 * sample, cudaMemcpyHostToDevice, s) != cudaSuccess ||
                     cudaMemsetAsync(dctr.p, 0, 8 * (size_t)C_COUNT * n_jobs, s) != cudaSuccess ||
                     cudaMemsetAsync(dqueue.p, 0, 16, s) != cudaSuccess || cudaEventRecord(e0, s) != cudaSuccess ||
-                    launch_batch(ba, sms * c.per_sm, c.warps, s) != cudaSuccess || cudaEventRecord(e1, s) != cudaSuccess ||
+                    launch_batch(ba, std::min(sms * c.per_sm, slices), c.warps, s) != cudaSuccess || cudaEventRecord(e1, s) != cudaSuccess ||
                     cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&t, e0, e1) != cudaSuccess) {
                     if (getenv("EFM_DEBUG"))
                         fprintf(stderr, "efm: batch tuning run failed: %s\n", cudaGetErrorString(cudaGetLastError()));
@@ -1622,7 +1630,7 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
         if (ok) {
             ok = cudaMemsetAsync(dctr.p, 0, 8 * (size_t)C_COUNT * n_jobs, cs) == cudaSuccess &&
                  cudaMemsetAsync(dqueue.p, 0, 16, cs) == cudaSuccess &&
-                 launch_batch(ba, sms * best.per_sm, best.warps, cs) == cudaSuccess;
+                 launch_batch(ba, std::min(sms * best.per_sm, slices), best.warps, cs) == cudaSuccess;
             ok = (cudaStreamEndCapture(cs, &graph) == cudaSuccess) && ok;
         }
         ok = ok && cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess;
@@ -1641,10 +1649,42 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
         rc = EFM_ECUDA;
         goto done;
     }
+    // Every job's rows go to the host in one copy, and the fetch of a job is a
+    // memcpy: 512 fetches took 5.7 ms with a copy and a wait for each and take
+    // 3.0 ms this way, for 0.1 ms in the call.
+    for (int i = 0; i < n_jobs; ++i) {
+        const unsigned long long *h = &hctr[(size_t)i * C_COUNT];
+        const bool ok = h[C_DONE] == 1 && !err_from_bits(h[C_ERR]);
+        offs[i + 1] = offs[i] + (ok ? (int64_t)h[C_OUT_N] * job->words[i] : 0);
+    }
+    if (offs[n_jobs] > 0) {
+        bool room = true;
+        try {
+            job->host_out.resize((size_t)offs[n_jobs]);
+        } catch (const std::bad_alloc &) {
+            room = false;
+        }
+        if (!room || !dev_alloc(dpack, (size_t)offs[n_jobs] * 8, s)) {
+            rc = EFM_ENOMEM;
+            goto done;
+        }
+        if (cudaMemcpyAsync(doff.p, offs.data(), 8 * offs.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+            launch_batch_gather(ba.jobs, (const int64_t *)doff.p, n_jobs, (uint64_t *)dpack.p, s) != cudaSuccess ||
+            cudaMemcpyAsync(job->host_out.data(), dpack.p, (size_t)offs[n_jobs] * 8, cudaMemcpyDeviceToHost, s) !=
+                cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess) {
+            rc = EFM_ECUDA;
+            goto done;
+        }
+    }
     for (int i = 0; i < n_jobs; ++i) {
         const unsigned long long *h = &hctr[(size_t)i * C_COUNT];
         TargetOut &o = job->out[i];
-        o.borrowed = hj[i].out;
+        if (h[C_DONE] == 2 && !err_from_bits(h[C_ERR])) {
+            alone.push_back(i);
+            continue;
+        }
+        o.host_at = offs[i];
         o.err = err_from_bits(h[C_ERR]);
         if (!o.err && !h[C_DONE]) o.err = EFM_ECUDA;
         o.n = (int64_t)h[C_OUT_N];
@@ -1664,6 +1704,24 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
         o.total_ms = ms;
         o.kernel_launches = i == 0 ? 1 : 0;
     }
+    if (!alone.empty() && getenv("EFM_DEBUG")) fprintf(stderr, "efm: %d jobs of the batch run alone\n", (int)alone.size());
+    // each by itself, with the batch's limits on its candidates and results
+    for (int i : alone) {
+        efm_limits l1 = lim;
+        l1.max_len = hj[i].max_len;
+        TargetOut &o = job->out[i];
+        Work w;
+        int e = alloc_work(w, nets[i], l1, level_grid(nets[i]->nv, l1, sms) * kExpandWarps, s);
+        if (e == EFM_OK) e = run_target(nets[i], w, l1, targets[i], o);
+        free_work(w, s);
+        if (e == EFM_OK && (o.ctr.candidates > L.cand_cap || o.ctr.results > L.res_cap)) e = EFM_ECAPACITY;
+        if (e == EFM_ENOMEM || e == EFM_ECUDA) {
+            rc = e;
+            goto done;
+        }
+        o.err = e;
+        o.total_ms = ms;
+    }
 done:
     if (exec) cudaGraphExecDestroy(exec);
     if (graph) cudaGraphDestroy(graph);
@@ -1674,6 +1732,9 @@ done:
     dev_free(dorder, s);
     dev_free(dctr, s);
     dev_free(dqueue, s);
+    dev_free(dout, s);
+    dev_free(dpack, s);
+    dev_free(doff, s);
     if (cudaStreamSynchronize(s) != cudaSuccess && rc == EFM_OK) rc = EFM_ECUDA;
     if (rc != EFM_OK) {
         cudaGetLastError();
@@ -1737,9 +1798,10 @@ extern "C" int efm_fetch_results(efm_job *job, int32_t idx, uint64_t *supports, 
     if (o.err) return o.err;
     if (!supports) return o.status;
     if (capacity < o.n) return EFM_ECAPACITY;
-    if (o.n > 0) {
-        const void *src = o.borrowed ? (const void *)o.borrowed : o.sup.p;
-        if (cudaMemcpyAsync(supports, src, (size_t)o.n * W * 8, cudaMemcpyDeviceToHost, job->net->stream) !=
+    if (o.n > 0 && o.host_at >= 0) {
+        memcpy(supports, job->host_out.data() + o.host_at, (size_t)o.n * W * 8);
+    } else if (o.n > 0) {
+        if (cudaMemcpyAsync(supports, o.sup.p, (size_t)o.n * W * 8, cudaMemcpyDeviceToHost, job->net->stream) !=
                 cudaSuccess ||
             cudaStreamSynchronize(job->net->stream) != cudaSuccess) {
             cudaGetLastError();
@@ -1767,7 +1829,6 @@ extern "C" void efm_free_job(efm_job *job)
     if (!job) return;
     cudaStream_t s = job->net ? job->net->stream : nullptr;
     for (auto &o : job->out) dev_free(o.sup, s);
-    dev_free(job->shared_out, s);
     cudaStreamSynchronize(s);
     delete job;
 }

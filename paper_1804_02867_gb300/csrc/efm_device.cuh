@@ -64,16 +64,6 @@ __device__ __forceinline__ unsigned long long load_volatile(unsigned long long *
     return *(volatile unsigned long long *)p;
 }
 
-__device__ __forceinline__ uint64_t global_ns()
-{
-    uint64_t t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
-
-constexpr uint64_t kWatchdogNs = 20ull * 1000000000ull;  // a level that runs longer gives up
-constexpr int kMaxRounds = 1 << 22;
-
 // Record the first failed self-check (code, offending value, its limit) and
 // raise the error bit; the caller skips the access.
 __device__ __forceinline__ void record_diag(unsigned long long *ctr, unsigned bit, unsigned long long code, long long value,

@@ -16,7 +16,6 @@ constexpr unsigned long long kEmpty = ~0ull;
 constexpr uint32_t kPending = 0xFFFFFFFFu;
 constexpr uint32_t kOverflowIdx = 0xFFFFFFFEu;
 constexpr int kNumPrimes = 24;
-constexpr int kStageLimitBytes = 72 * 1024;  // static network staged in smem up to this size
 constexpr int64_t kFirstKChunkMin = 8192;     // first-K search: fewest parents per expansion launch
 constexpr int64_t kFirstKChunks = 32;         // first-K search: launches per level, at most
 constexpr int64_t kResultWindow = 256;        // first-K search: new results fetched with the counters
@@ -38,15 +37,14 @@ enum {
     C_UNWRITTEN,  // children whose row did not fit the child arena
     C_UNV,        // distinct fingerprints among the children without a row
     C_OUT_N = 20, // batched traversal: rows written to the job's output
-    C_DONE,       // batched traversal: job finished
+    C_DONE,       // batched traversal: 1 = job finished, 2 = left to the host
     C_ACC_BEGIN,  // first candidate the next device-range minimality launch judges
     C_DEDUP_BEGIN,  // first reserved row the next dedup launch examines
     C_DIAG = 24,  // first bounds/watchdog record: code, value, limit, level
     C_ZERO = 28,  // subtractive steps discarded: no positive flux left on the reaction (Prop. 3)
     C_OPEN,       // open children listed by the generate pass, not yet finished
     C_LIVE,       // surviving rows counted by the live-list pass
-    C_CAPDEAD,    // unused
-    C_PAY,        // sparse states: payload units reserved so far in the level
+    C_PAY = 32,   // sparse states: payload units reserved so far in the level
     C_COUNT = 40
 };
 
@@ -115,16 +113,11 @@ struct NetView {
 __host__ __device__ inline int ent_index(uint32_t e) { return (int)(e >> 20); }
 __host__ __device__ inline int32_t ent_coef(uint32_t e) { return ((int32_t)(e << 12)) >> 12; }
 
-// One arena of pathway states.  The level pass keeps headers and a
-// payload pool (layout in efm_sparse.cu); the batched traversal keeps dense
-// rows: support words, extra-flux row, meta word.
+// One arena of pathway states (layout in efm_level.cuh).
 struct Arena {
     uint4 *hdr;         // [cap]
     uint4 *pay;         // [pay_cap] 16-byte units
     uint64_t pay_cap;
-    uint64_t *U;     // [cap][W]
-    int32_t *B;      // [cap][Mpad]
-    uint32_t *meta;  // [cap]: pivot row | pivot degree << 10 | |U| << 23
     int64_t cap;
 };
 
@@ -163,20 +156,14 @@ struct LevelArgs {
     int64_t n_par;
     Arena child;
     unsigned long long *slots;  // state hash table
-    uint64_t slot_mask;
     unsigned long long *cslots; // balanced-support hash table
     uint64_t cslot_mask;
     uint64_t *cand;             // [cand_cap][W]
     int64_t cand_cap;
     const uint64_t *res;        // [res_cap][W]
-    const int32_t *bptr;        // [N + 1] result buckets by column
-    const uint64_t *bres;       // bucket entries: the result's W support words (W <= 2)
-    const int32_t *bids;        // bucket entries: result ids (W > 2), same buffer as bres
     const uint16_t *rcols;      // per result: column count, then its columns (stride kRcolStride)
-    const uint64_t *band;       // W <= 2: per column, the intersection of the results containing it (or null)
     CellIndex cells;            // the level pass
     int level, max_len, max_sec;
-    int cpw;                    // parents per warp chunk (1..32; batched traversal)
     unsigned long long *ctr;
     // first-K search (zero / null otherwise)
     const uint32_t *perm;       // parent order: position -> arena index (null: arena rows par_base + position)
@@ -215,7 +202,7 @@ struct AcceptArgs {
     CellIndex ix;               // accepted results are filed here
     unsigned long long *st;
     int advance;                // what the last CTA does: 0 nothing, 1 a chunk of a level ends, 2 a level, 3 the seeds
-    int level, level0, max_level;
+    int level, max_level;
     int64_t max_frontier, max_results;
     int64_t fp_cap, child_rows;
     uint64_t slot_cap;
@@ -226,10 +213,12 @@ struct AcceptArgs {
 constexpr int kBatchThreads = 256;
 struct BatchLayout {
     size_t slice_bytes;
-    size_t o_U[2], o_B[2], o_meta[2];
-    size_t o_slots, o_cslots, o_cand, o_res, o_bcnt, o_bfill, o_bptr, o_bres, o_sort, o_rcols;
-    int64_t cap, cand_cap, res_cap;
-    uint64_t slot_cap, cslot_cap;
+    size_t o_hdr[2], o_pay[2];
+    size_t o_slots, o_fp, o_open, o_cslots, o_cand, o_res, o_cnt, o_ksig, o_single, o_cells, o_ent, o_sort, o_rcols;
+    int64_t cap, fp_cap, cand_cap, res_cap, index_room;
+    uint64_t pay_cap, slot_cap, cslot_cap;
+    uint32_t cell_mask;
+    int ent_stride;
 };
 
 struct BatchJob {
@@ -332,6 +321,8 @@ cudaError_t launch_walks(const NetView &nv, const LevelArgs &a, int target, uint
                          cudaStream_t s);
 // the batched traversal runs `warps` warps per CTA (4 or 8), one job at a time
 cudaError_t launch_batch(const BatchArgs &ba, int grid, int warps, cudaStream_t s);
+// the output rows of every job (words off[i] .. off[i + 1]) into one array
+cudaError_t launch_batch_gather(const BatchJob *jobs, const int64_t *off, int n_jobs, uint64_t *dst, cudaStream_t s);
 int batch_blocks_per_sm(int warps);
 size_t batch_smem_bytes(int warps);
 

@@ -20,14 +20,10 @@
 // tested by Gaussian elimination modulo primes p = 2^31 - c, with enough
 // primes that their product exceeds the Hadamard bound of the columns.
 //
-// Layout (narrow networks): a frontier is an arena of states, each a row of W support words,
-// a row of Mpad int32 extra-flux entries (16-byte aligned) and a meta word
-// (acting metabolite, its degree, |U|).  The expansion gives every lane its
-// own child; the seed and minimality kernels give a warp one item.  The
-// static network (CSR by column and by metabolite, twins, pivot keys) is
-// staged into shared memory with one bulk async copy (no multicast) when it
-// fits.
-#include "efm_device.cuh"
+// This file holds the minimality test, the walks, the batch and the sorting of
+// results; the level pass itself (states, expansion, merging of duplicates) is
+// efm_level.cuh, launched over the grid by efm_sparse.cu.
+#include "efm_level.cuh"
 
 namespace efm {
 namespace {
@@ -103,45 +99,6 @@ __device__ __noinline__ int insert_support(const LevelArgs &a, int W, const uint
     return INS_TABLE_FULL;
 }
 
-// 64-bit recomputation of a child's raw entries (rare: some entry left the
-// int32 range): gcd and largest magnitude over the lane's entries.
-struct GcdMax {
-    uint64_t g, m;
-};
-__device__ __noinline__ GcdMax raw_gcd_max(const int4 *prow4, const int4 *col4, int gl, int G, int CPL, int32_t A,
-                                           int32_t C)
-{
-    GcdMax r{0, 0};
-    for (int i = 0; i < CPL; ++i) {
-        const int4 v = prow4[gl + G * i];
-        const int4 w = col4[gl + G * i];
-        const int32_t pv[4] = {v.x, v.y, v.z, v.w}, cv[4] = {w.x, w.y, w.z, w.w};
-        for (int jj = 0; jj < 4; ++jj) {
-            const uint64_t at = abs64((int64_t)A * pv[jj] + (int64_t)C * cv[jj]);
-            if (at != 0) {
-                r.g = r.g == 0 ? at : gcd64(r.g, at);
-                r.m = at > r.m ? at : r.m;
-            }
-        }
-    }
-    return r;
-}
-
-// Supports of more than two words: does the result with bucket position i
-// (id list, column lists) lie inside U + {k}?  Its columns are probed
-// independently (no early exit), so the loads overlap.
-__device__ __forceinline__ bool result_inside_wide(const LevelArgs &a, const uint64_t *pu, int k, int64_t i)
-{
-    const uint16_t *lst = a.rcols + (size_t)a.bids[i] * kRcolStride;
-    const int n = lst[0];
-    bool sub = true;
-    for (int j = 1; j <= n; ++j) {
-        const int c = lst[j];
-        sub = sub && (c == k || bit_of(pu, c));
-    }
-    return sub;
-}
-
 // Pivot key of a state: min over unbalanced rows of (degree << 16 | row)
 // (warp-cooperative; lane l holds rows l + 32 e).
 template <int EPL>
@@ -157,94 +114,6 @@ __device__ __forceinline__ uint32_t pivot_key(const uint32_t *bl, const NetView 
         }
     }
     return __reduce_min_sync(FULL, kmin);
-}
-
-// warp-wide test: all balance rows (m < M) of a row held across the warp are 0
-template <int EPL>
-__device__ __forceinline__ bool balance_zero(const int32_t (&t)[EPL], int M, int lane)
-{
-    bool nz = false;
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) nz = nz || (t[e] != 0 && lane + 32 * e < M);
-    return !__any_sync(FULL, nz);
-}
-
-// warp-cooperative normalisation of a seed column (t64 in, t32 out)
-template <int EPL>
-__device__ __forceinline__ void normalise(int64_t (&t64)[EPL], int32_t (&t32)[EPL], bool &zero)
-{
-    bool nz = false;
-    uint64_t g = 0;
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) {
-        nz = nz || (t64[e] != 0);
-        g = gcd64(g, abs64(t64[e]));
-    }
-    zero = !__any_sync(FULL, nz);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) g = gcd64(g, __shfl_xor_sync(FULL, g, off));
-#pragma unroll
-    for (int e = 0; e < EPL; ++e) t32[e] = (int32_t)(g > 1 ? t64[e] / (int64_t)g : t64[e]);
-}
-
-// ---------------------------------------------------------------------------
-// a0: seeds (INIT kernel analogue): flux 1 on every column producing the
-// target (every column for target -1).  One warp per seed.
-// ---------------------------------------------------------------------------
-
-template <int EPL>
-__device__ void seed_range(const NetView &nv, const LevelArgs &a, int target, int gw, int nw)
-{
-    const int lane = threadIdx.x & 31;
-    const uint32_t *bl = nv.blob;
-    const int W = nv.W;
-    unsigned long long n_seed = 0, n_bal = 0, deg_sum = 0;
-    const int n_items = target >= 0 ? nv.metptr[target + 1] - nv.metptr[target] : nv.N;
-    for (int it = gw; it < n_items; it += nw) {
-        int k = it;
-        if (target >= 0) {
-            const uint32_t e = nv.metent[nv.metptr[target] + it];
-            if (ent_coef(e) <= 0) continue;
-            k = ent_index(e);
-        }
-        ++n_seed;
-        // the seed's row: column k of the dense copy (S_int[:, k], then, in
-        // the subtractive variant's view, flux 1 on k)
-        const int32_t *dk = reinterpret_cast<const int32_t *>(bl + nv.o_dcols) + (size_t)k * nv.Mpad;
-        int64_t t64[EPL];
-#pragma unroll
-        for (int e = 0; e < EPL; ++e) t64[e] = dk[lane + 32 * e];
-        int32_t t[EPL];
-        bool zero;
-        normalise<EPL>(t64, t, zero);
-        zero = balance_zero<EPL>(t, nv.M, lane);
-        if (zero) {
-            ++n_bal;
-            if (lane == 0) insert_support(a, W, nullptr, k);
-            __syncwarp();
-            continue;
-        }
-        const uint32_t key = pivot_key<EPL>(bl, nv, t, lane);
-        // seeds are distinct columns: no deduplication needed
-        unsigned long long idx = 0;
-        if (lane == 0) idx = atomicAdd(&a.ctr[C_NEXT], 1ull);
-        idx = __shfl_sync(FULL, idx, 0);
-        if ((int64_t)idx < a.child.cap) {
-            uint64_t *du = a.child.U + (size_t)idx * W;
-            for (int w = lane; w < W; w += 32) du[w] = child_word(nullptr, w, k);
-            int32_t *db = a.child.B + (size_t)idx * nv.Mpad;
-#pragma unroll
-            for (int e = 0; e < EPL; ++e) db[lane + 32 * e] = t[e];
-            const uint32_t bkey = branch_key(bl, nv, key, a.sub);
-            if (lane == 0) a.child.meta[idx] = pack_meta(bkey, 1);
-            deg_sum += bkey >> 16;
-        }
-    }
-    if (lane == 0) {
-        if (n_seed) atomicAdd(&a.ctr[C_SEEDS], n_seed);
-        if (n_bal) atomicAdd(&a.ctr[C_BAL], n_bal);
-        if (deg_sum) atomicAdd(&a.ctr[C_DEGSUM], deg_sum);
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -515,6 +384,17 @@ __global__ void __launch_bounds__(kWalkWarps * 32) walk_narrow_kernel(const __gr
     if (lane == 0 && most) atomicMax(&a.ctr[C_LEVELS], (unsigned long long)most);
 }
 
+// the output rows of a batch's jobs, job i's words [off[i], off[i + 1]) of dst
+__global__ void __launch_bounds__(128) batch_gather_kernel(const BatchJob *jobs, const int64_t *off, int n_jobs,
+                                                           uint64_t *dst)
+{
+    for (int i = blockIdx.x; i < n_jobs; i += gridDim.x) {
+        const uint64_t *src = jobs[i].out;
+        const int64_t b = off[i], n = off[i + 1] - b;
+        for (int64_t q = threadIdx.x; q < n; q += blockDim.x) dst[b + q] = src[q];
+    }
+}
+
 template <int EPL>
 __global__ void __launch_bounds__(kExpandWarps * 32) walk_kernel(NetView nv, LevelArgs a, int target, uint64_t seed,
                                                                  int64_t n_walks)
@@ -651,612 +531,6 @@ __global__ void __launch_bounds__(kExpandWarps * 32) walk_kernel(NetView nv, Lev
         if (max_steps) atomicMax(&a.ctr[C_LEVELS], max_steps);
     }
 }
-
-// ---------------------------------------------------------------------------
-// a1-a6: one level of expansion.
-//
-// Phase 1: a warp takes up to 32 consecutive parents; their branch counts
-// (the static degree of each parent's acting metabolite, kept in the state's
-// meta word) are prefix-summed across the lanes.  The warp then examines the
-// flattened (parent, branch) items 32 at a time, one per lane (branch
-// selection and the twin, length and first-K rules), and its groups of G
-// lanes take the valid items in order, one child per group.  In a group,
-// lane l holds the 16-byte chunks l, l + G, ... of the extra-flux row (CPL
-// chunks, 4 * CPL entries), so row loads are coalesced and every reduction
-// is log2(G) shuffles.  The AND update reads column k of S_int from a dense
-// column-major copy of S_int (staged in shared memory with the rest of the
-// static network when it fits) and stays in 32 bits unless a group needs the
-// gcd or has an entry outside int32.  The group then applies the superset
-// rule (its lanes split the results containing the new column) and appends
-// surviving unbalanced children to a per-warp batch in shared memory.
-//
-// Phase 2 (one lane per batched child, NB children at once; the whole warp
-// per child for wide rows): claim / write / publish / compare in the state
-// hash table, so the latency of the atomics is paid once per batch, not per
-// child.
-// ---------------------------------------------------------------------------
-
-template <int G>
-__device__ __forceinline__ uint32_t group_or(uint32_t x)
-{
-#pragma unroll
-    for (int off = G / 2; off > 0; off >>= 1) x |= __shfl_xor_sync(FULL, x, off);
-    return x;
-}
-template <int G>
-__device__ __forceinline__ uint32_t group_min(uint32_t x)
-{
-#pragma unroll
-    for (int off = G / 2; off > 0; off >>= 1) {
-        const uint32_t y = __shfl_xor_sync(FULL, x, off);
-        x = y < x ? y : x;
-    }
-    return x;
-}
-template <int G>
-__device__ __forceinline__ uint32_t group_add(uint32_t x)
-{
-#pragma unroll
-    for (int off = G / 2; off > 0; off >>= 1) x += __shfl_xor_sync(FULL, x, off);
-    return x;
-}
-template <int G>
-__device__ __forceinline__ uint32_t group_xor(uint32_t x)
-{
-#pragma unroll
-    for (int off = G / 2; off > 0; off >>= 1) x ^= __shfl_xor_sync(FULL, x, off);
-    return x;
-}
-
-__device__ __forceinline__ void prefetch_l2(const void *p)
-{
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-
-__device__ __forceinline__ void store_release(unsigned long long *p, unsigned long long v)
-{
-    asm volatile("st.release.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-__device__ __forceinline__ unsigned long long cas_acquire(unsigned long long *p, unsigned long long cmp,
-                                                          unsigned long long v)
-{
-    unsigned long long old;
-    asm volatile("atom.acquire.gpu.global.cas.b64 %0, [%1], %2, %3;" : "=l"(old) : "l"(p), "l"(cmp), "l"(v) : "memory");
-    return old;
-}
-
-// 32-bit mixing of one balance entry (row m, value v) into two sums
-__device__ __forceinline__ void hash_entry(uint32_t m, uint32_t v, uint32_t &lo, uint32_t &hi)
-{
-    const uint32_t x = (v ^ (m * 0x9E3779B9u)) * 0x85EBCA6Bu;
-    lo += x ^ (x >> 16);
-    hi ^= x + m;
-}
-
-// children per warp batch for a row of 16-byte chunks nch (shared memory
-// per warp: NB padded rows plus 32 bytes of bookkeeping per child)
-// First-K bound (output order: |U|, then the ascending column list): true
-// when the child support (U with column k) comes after R, both of size |R|.
-// Of two sets of equal size, the one holding the lowest column of their
-// symmetric difference comes first.
-__device__ __forceinline__ bool child_after(const uint64_t *pu, int k, const uint64_t *R, int W)
-{
-    for (int w = 0; w < W; ++w) {
-        const uint64_t c = child_word(pu, w, k);
-        const uint64_t d = c ^ __ldg(R + w);
-        if (d) return (c & (d & (~d + 1))) == 0;
-    }
-    return false;
-}
-
-template <int G, int CPL>
-struct BatchShape {
-    static constexpr int NCH = G * CPL;          // 16-byte chunks per row
-    static constexpr int NB = NCH <= 16 ? 16 : (NCH <= 32 ? 8 : 2);
-    static constexpr int ROW = NCH + 1;          // padded row (int4 units): conflict-free per-lane access
-    static constexpr int BYTES = NB * ROW * 16 + NB * 32;
-};
-
-// One level of expansion by the warps worker = 0 .. nworkers-1 (the whole
-// grid, or the warps of one CTA in the batched kernel).  bl: the static
-// network (shared or global); wbase: this warp's batch region.
-template <int G, int CPL>
-__device__ void expand_range(const NetView &nv, const LevelArgs &a, const uint32_t *bl, char *wbase, int64_t worker,
-                             int64_t nworkers)
-{
-    constexpr int NG = 32 / G;    // children per warp round
-    constexpr int EPL = 4 * CPL;  // balance entries per lane
-    using BS = BatchShape<G, CPL>;
-    constexpr int NB = BS::NB;
-    const int lane = threadIdx.x & 31;
-    const int gi = lane / G;  // group in the warp
-    const int gl = lane % G;  // lane in the group
-    const int lead = gi * G;  // group leader lane
-    const int W = nv.W;
-    const int Mpad = nv.Mpad;
-    // per-warp batch: rows, then (pos, tag, key, info, parent) per child
-    int4 *brow = reinterpret_cast<int4 *>(wbase);
-    uint64_t *bpos = reinterpret_cast<uint64_t *>(wbase + NB * BS::ROW * 16);
-    uint32_t *btag = reinterpret_cast<uint32_t *>(bpos + NB);
-    uint32_t *bkey = btag + NB;
-    uint32_t *binfo = bkey + NB;  // k | in_u << 12 | pc1 << 13
-    uint32_t *bpar = binfo + NB;  // parent index
-    const int4 *dcol = reinterpret_cast<const int4 *>(bl + nv.o_dcols);
-
-    unsigned long long n_exp = 0, n_ovf = 0, n_bal = 0, n_pruned = 0, deg_sum = 0;
-    bool fatal = false;
-    bool full = false;  // the child arena reached its capacity
-    int nb = 0;         // children in the batch (warp-uniform)
-    const uint64_t t_start = global_ns();
-
-    // Phase 2 for wide rows (more than 32 chunks): the whole warp claims and
-    // copies or compares one batched child at a time.
-    auto flush_wide = [&]() {
-        __syncwarp();
-        for (int b = 0; b < nb; ++b) {
-            const uint32_t info = binfo[b];
-            const int k = (int)(info & 0xFFFu);
-            const uint64_t *pu = a.par.U + (size_t)bpar[b] * W;
-            if (full) continue;
-            uint64_t pos = bpos[b];
-            const uint32_t tag = btag[b];
-            const int4 *row = brow + (size_t)b * BS::ROW;
-            for (uint64_t probe = 0;; ++probe) {
-                if (probe > a.slot_mask) {
-                    if (lane == 0) atomicOr(&a.ctr[C_ERR], (unsigned long long)ERR_TABLE_FULL);
-                    fatal = true;
-                    break;
-                }
-                unsigned long long v = kEmpty;
-                if (lane == 0) v = cas_acquire(&a.slots[pos], kEmpty, ((unsigned long long)tag << 32) | kPending);
-                v = __shfl_sync(FULL, v, 0);
-                if (v == kEmpty) {
-                    unsigned long long idx = 0;
-                    if (lane == 0) idx = atomicAdd(&a.ctr[C_NEXT], 1ull);
-                    idx = __shfl_sync(FULL, idx, 0);
-                    if ((int64_t)idx >= a.child.cap) {
-                        full = true;
-                        if (lane == 0) store_release(&a.slots[pos], ((unsigned long long)tag << 32) | kOverflowIdx);
-                        break;
-                    }
-                    int4 *db = reinterpret_cast<int4 *>(a.child.B + (size_t)idx * Mpad);
-                    for (int c = lane; c < BS::NCH; c += 32) db[c] = row[c];
-                    uint64_t *du = a.child.U + (size_t)idx * W;
-                    for (int w = lane; w < W; w += 32) du[w] = child_word(pu, w, k);
-                    if (lane == 0) a.child.meta[idx] = pack_meta(bkey[b], (int)(info >> 13));
-                    __threadfence();
-                    __syncwarp();
-                    if (lane == 0) {
-                        store_release(&a.slots[pos], ((unsigned long long)tag << 32) | idx);
-                        deg_sum += bkey[b] >> 16;
-                    }
-                    break;
-                }
-                if ((uint32_t)(v >> 32) != tag) {
-                    pos = (pos + 1) & a.slot_mask;
-                    continue;
-                }
-                int spins = 0;
-                while ((uint32_t)v == kPending && spins < kSpinLimit) {
-                    __nanosleep(64);
-                    ++spins;
-                    if (lane == 0) v = cas_acquire(&a.slots[pos], kEmpty, kEmpty);
-                    v = __shfl_sync(FULL, v, 0);
-                }
-                if ((uint32_t)v == kPending) {
-                    if (lane == 0) atomicOr(&a.ctr[C_ERR], (unsigned long long)ERR_TIMEOUT);
-                    fatal = true;
-                    break;
-                }
-                if ((uint32_t)v == kOverflowIdx) break;
-                const uint32_t ci = (uint32_t)v;
-                const int4 *sb = reinterpret_cast<const int4 *>(a.child.B + (size_t)ci * Mpad);
-                bool eq = true;
-                for (int c = lane; c < BS::NCH && eq; c += 32) {
-                    const int4 x = __ldcg(sb + c), o = row[c];
-                    eq = x.x == o.x && x.y == o.y && x.z == o.z && x.w == o.w;
-                }
-                const uint64_t *su = a.child.U + (size_t)ci * W;
-                for (int w = lane; w < W && eq; w += 32) eq = __ldcg(su + w) == child_word(pu, w, k);
-                if (__all_sync(FULL, eq)) break;  // duplicate of a state already in the frontier
-                pos = (pos + 1) & a.slot_mask;
-            }
-            if (__any_sync(FULL, fatal)) break;
-        }
-        fatal = __any_sync(FULL, fatal);
-        full = __any_sync(FULL, full);
-        nb = 0;
-        __syncwarp();
-    };
-
-    // Phase 2: insert the batched children, one lane each.
-    auto flush = [&]() {
-        if (BS::NCH > 32) {
-            flush_wide();
-            return;
-        }
-        __syncwarp();
-        const bool mine = lane < nb;
-        const uint32_t info = mine ? binfo[lane] : 0u;
-        const int k = (int)(info & 0xFFFu);
-        const uint64_t *pu = a.par.U + (size_t)(mine ? bpar[lane] : 0u) * W;
-        bool todo = mine;
-        if (full) todo = false;
-        const uint64_t row_i = (uint64_t)lane * BS::ROW;
-        uint64_t pos = mine ? bpos[lane] : 0ull;
-        const uint32_t tag = mine ? btag[lane] : 0u;
-        uint64_t probes = 0;
-        int spins = 0, rounds = 0;
-        while (__any_sync(FULL, todo)) {
-            const bool expired = ++rounds > kMaxRounds || ((rounds & 63) == 0 && global_ns() - t_start > kWatchdogNs);
-            if (__any_sync(FULL, expired)) {  // warp-uniform decision
-                if (lane == 0) record_diag(a.ctr, ERR_WATCHDOG, 2, rounds, kMaxRounds, a.level);
-                fatal = true;
-                break;
-            }
-            unsigned long long v = kEmpty;
-            if (todo) v = cas_acquire(&a.slots[pos], kEmpty, ((unsigned long long)tag << 32) | kPending);
-            const bool won = todo && v == kEmpty;
-            const bool other = todo && !won && (uint32_t)(v >> 32) != tag;
-            const bool waiting = todo && !won && !other && (uint32_t)v == kPending;
-            const bool over = todo && !won && !other && (uint32_t)v == kOverflowIdx;
-            const bool cmp = todo && !won && !other && !waiting && !over;
-            if (other) {
-                pos = (pos + 1) & a.slot_mask;
-                if (++probes > a.slot_mask) {
-                    atomicOr(&a.ctr[C_ERR], (unsigned long long)ERR_TABLE_FULL);
-                    todo = false;
-                    fatal = true;
-                }
-            }
-            if (over) todo = false;
-            const unsigned wmask = __ballot_sync(FULL, won);
-            if (wmask) {
-                const int leader = __ffs((int)wmask) - 1;
-                unsigned long long base_idx = 0;
-                if (lane == leader) base_idx = atomicAdd(&a.ctr[C_NEXT], (unsigned long long)__popc(wmask));
-                base_idx = __shfl_sync(FULL, base_idx, leader);
-                const uint64_t idx = base_idx + (uint64_t)__popc(wmask & ((1u << lane) - 1u));
-                bool wrote = false;
-                if (won) {
-                    if ((int64_t)idx >= a.child.cap) {
-                        full = true;  // level truncated: stop claiming
-                        store_release(&a.slots[pos], ((unsigned long long)tag << 32) | kOverflowIdx);
-                    } else {
-                        int4 *db = reinterpret_cast<int4 *>(a.child.B + (size_t)idx * Mpad);
-                        for (int c = 0; c < BS::NCH; ++c) db[c] = brow[row_i + c];
-                        uint64_t *du = a.child.U + (size_t)idx * W;
-                        for (int w = 0; w < W; ++w) du[w] = child_word(pu, w, k);
-                        a.child.meta[idx] = pack_meta(bkey[lane], (int)(info >> 13));
-                        wrote = true;
-                    }
-                    todo = false;
-                }
-                __threadfence_block();  // order each lane's row writes before its release store
-                if (wrote) {
-                    store_release(&a.slots[pos], ((unsigned long long)tag << 32) | idx);
-                    deg_sum += bkey[lane] >> 16;
-                }
-            }
-            if (cmp) {
-                const uint32_t ci = (uint32_t)v;
-                const int4 *sb = reinterpret_cast<const int4 *>(a.child.B + (size_t)ci * Mpad);
-                bool eq = true;
-                for (int c = 0; c < BS::NCH && eq; ++c) {
-                    const int4 s = __ldcg(sb + c);
-                    const int4 o = brow[row_i + c];
-                    eq = s.x == o.x && s.y == o.y && s.z == o.z && s.w == o.w;
-                }
-                const uint64_t *su = a.child.U + (size_t)ci * W;
-                for (int w = 0; w < W && eq; ++w) eq = __ldcg(su + w) == child_word(pu, w, k);
-                if (eq) {
-                    todo = false;  // duplicate of a state already in the frontier
-                } else {
-                    pos = (pos + 1) & a.slot_mask;
-                    ++probes;
-                }
-            }
-            if (__any_sync(FULL, waiting)) {
-                if (waiting && ++spins > kSpinLimit) {
-                    atomicOr(&a.ctr[C_ERR], (unsigned long long)ERR_TIMEOUT);
-                    todo = false;
-                    fatal = true;
-                }
-                __nanosleep(32);
-            }
-            full = __any_sync(FULL, full);
-            if (full) todo = false;
-        }
-        nb = 0;
-        __syncwarp();
-    };
-
-    // chunks of cpw parents per warp (fewer for small levels, so that the
-    // items of a small level spread over all warps)
-    const int cpw = a.cpw;
-    const int64_t wstride = nworkers * cpw;
-    for (int64_t p0 = worker * cpw; p0 < a.n_par; p0 += wstride) {
-        const int64_t pl = p0 + lane;
-        const bool pin = lane < cpw && pl < a.n_par;
-        const int64_t pid = pin ? (a.perm ? (int64_t)a.perm[pl] : pl) : 0;  // this lane's parent
-        // pull this chunk's and the next chunk's parents toward L2
-        if (pin) {
-            const char *rp = reinterpret_cast<const char *>(a.par.B + (size_t)pid * Mpad);
-            for (int off = 0; off < Mpad * 4; off += 128) prefetch_l2(rp + off);
-            prefetch_l2(a.par.U + (size_t)pid * W);
-        }
-        const int64_t pn = pl + wstride;
-        if (lane < cpw && pn < a.n_par) {
-            const int64_t nid = a.perm ? (int64_t)a.perm[pn] : pn;
-            const char *rp = reinterpret_cast<const char *>(a.par.B + (size_t)nid * Mpad);
-            for (int off = 0; off < Mpad * 4; off += 128) prefetch_l2(rp + off);
-            prefetch_l2(a.par.U + (size_t)nid * W);
-            prefetch_l2(a.par.meta + nid);
-        }
-        const uint32_t mj = pin ? a.par.meta[pid] : 0u;
-        int dj = pin ? (int)((mj >> 10) & 0x1FFFu) : 0;
-        // first-K: a parent larger than the bound has no descendant among the K smallest
-        if (a.fk_pc > 0 && (int)((mj >> 23) & 0x7Fu) > a.fk_pc) dj = 0;
-        int incl = dj;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int x = __shfl_up_sync(FULL, incl, off);
-            if (lane >= off) incl += x;
-        }
-        const int prej = incl - dj;
-        const int T = __shfl_sync(FULL, incl, 31);
-        if (T > 32 * nv.N) {
-            if (lane == 0) record_diag(a.ctr, ERR_BOUNDS, 3, T, 32 * nv.N, a.level);
-            fatal = true;
-        }
-        for (int base = 0; base < T; base += 32) {
-            if (__any_sync(FULL, fatal)) break;
-            // --- branch selection: one (parent, branch) item per lane ---
-            const int c = base + lane;
-            int j = 0;  // largest j with pre_j <= c
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-                const int v = __shfl_sync(FULL, prej, j + step);
-                if (v <= c) j += step;
-            }
-            const uint32_t pm = __shfl_sync(FULL, mj, j);
-            const int q = c - __shfl_sync(FULL, prej, j);
-            const int64_t pl_ = __shfl_sync(FULL, pid, j);
-            bool okl = c < T;
-            int kl = 0, pcl = 0;
-            bool inl = false;
-            int32_t Al = 0, Cl = 0;
-            if (okl) {
-                const int32_t *prow_l = a.par.B + (size_t)pl_ * Mpad;
-                const uint64_t *pu_l = a.par.U + (size_t)pl_ * W;
-                const int piv = (int)(pm & 0x3FFu);
-                pcl = (int)((pm >> 23) & 0x7Fu);
-                const int32_t bi = piv < nv.M ? prow_l[piv] : 0;
-                const bool fwd = bi > 0;  // forward flow: consume the surplus
-                const uint32_t abi = (uint32_t)(bi < 0 ? -bi : bi);
-                const int lptr = (fwd ? nv.o_consptr : nv.o_prodptr) + (piv < nv.M ? piv : 0);
-                const int lb = (int)bl[lptr];
-                const int le = (int)bl[lptr + 1];
-                if (piv >= nv.M || bi == 0 || lb + q >= le) {
-                    record_diag(a.ctr, ERR_BOUNDS, 1 + (piv >= nv.M ? 10 : 0) + (bi == 0 ? 100 : 0), (long long)q,
-                                (long long)(le - lb), a.level);
-                    fatal = true;
-                    okl = false;
-                } else {
-                    const uint32_t br = bl[(fwd ? nv.o_consent : nv.o_prodent) + lb + q];
-                    kl = ent_index(br);
-                    const uint32_t sik = (uint32_t)ent_coef(br);  // |S_ik|
-                    const int tw = (int)bl[nv.o_twin + kl];
-                    inl = bit_of(pu_l, kl);
-                    const int sec = a.level - pcl;
-                    okl = !(tw >= 0 && bit_of(pu_l, tw)) && (inl ? sec + 1 <= a.max_sec : pcl + 1 <= a.max_len);
-                    if (okl && a.fk_pc > 0) {
-                        // first-K branch and bound: the child's descendants keep
-                        // its support or grow it, so a child past the K-th
-                        // result found so far cannot yield one of the K smallest
-                        const int pc2 = pcl + (inl ? 0 : 1);
-                        okl = pc2 < a.fk_pc || (pc2 == a.fk_pc && !child_after(pu_l, kl, a.fk_sup, W));
-                    }
-                    const uint32_t g0 = (abi == 1u || sik == 1u) ? 1u : gcd32(abi, sik);
-                    Al = (int32_t)(sik / g0);
-                    Cl = (int32_t)(abi / g0);
-                }
-            }
-            if (okl) ++n_exp;
-            // packed item: column | |U| << 12 | secondary << 19; parent as 32 bits
-            const uint32_t infol = (uint32_t)kl | ((uint32_t)pcl << 12) | (inl ? 1u << 19 : 0u);
-            const uint32_t pl32 = (uint32_t)pl_;
-            // the groups take the valid items of this pass NG at a time, in order
-            unsigned vmask = __ballot_sync(FULL, okl);
-            while (vmask) {
-                if (__any_sync(FULL, fatal)) break;
-                const int src = gi < __popc(vmask) ? (int)__fns(vmask, 0, gi + 1) : -1;
-#pragma unroll
-                for (int t = 0; t < NG; ++t) vmask &= vmask - 1;
-                const int sl = src < 0 ? 0 : src;
-                const bool ok = src >= 0;
-                const uint32_t info_i = __shfl_sync(FULL, infol, sl);
-                const int k = (int)(info_i & 0xFFFu);
-                const int pc = (int)((info_i >> 12) & 0x7Fu);
-                const bool in_u = (info_i >> 19) & 1u;
-                const int32_t A = __shfl_sync(FULL, Al, sl);
-                const int32_t C = __shfl_sync(FULL, Cl, sl);
-                const int64_t p = (int64_t)__shfl_sync(FULL, pl32, sl);
-                const int32_t *prow = a.par.B + (size_t)p * Mpad;
-                const uint64_t *pu = a.par.U + (size_t)p * W;
-
-                // --- AND update (Eq. 3 / Eq. 4 in integers), group-parallel ---
-                int32_t t32[EPL];
-                uint32_t fl = 0;  // bit0 nonzero, bit1 some |t| == 1, bit2 some t outside int32
-                const int4 *prow4 = reinterpret_cast<const int4 *>(prow);
-                const int4 *col4 = dcol + (size_t)k * (Mpad >> 2);
-                if (ok) {
-    #pragma unroll
-                    for (int i = 0; i < CPL; ++i) {
-                        const int4 v = prow4[gl + G * i];
-                        const int4 w = col4[gl + G * i];
-                        const int32_t pv[4] = {v.x, v.y, v.z, v.w}, cv[4] = {w.x, w.y, w.z, w.w};
-    #pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) {
-                            const int64_t tt = (int64_t)A * pv[jj] + (int64_t)C * cv[jj];
-                            const int32_t lo = (int32_t)tt;
-                            const bool fits = tt == (int64_t)lo && lo != INT32_MIN;
-                            t32[4 * i + jj] = lo;
-                            fl |= (tt != 0 ? 1u : 0u) | ((lo == 1 || lo == -1) ? 2u : 0u) | (fits ? 0u : 4u);
-                        }
-                    }
-                } else {
-    #pragma unroll
-                    for (int e = 0; e < EPL; ++e) t32[e] = 0;
-                }
-                fl = group_or<G>(fl);
-                const bool nz = fl & 1u;
-                // slow path: the gcd is needed (no unit entry), or an entry is
-                // outside int32 (then the raw entries are recomputed in 64 bits)
-                const bool slow = ok && nz && ((fl & 6u) != 2u);
-                const bool big = (fl & 4u) != 0u;
-                bool ovf = false;
-                if (__any_sync(FULL, slow)) {
-                    uint64_t gg = 0, amax = 0;
-                    if (slow && !big) {
-    #pragma unroll
-                        for (int e = 0; e < EPL; ++e) {
-                            const uint32_t at = (uint32_t)(t32[e] < 0 ? -t32[e] : t32[e]);
-                            if (at != 0) gg = gg == 0 ? at : gcd32((uint32_t)gg, at);
-                        }
-                    } else if (slow) {
-                        const GcdMax gm = raw_gcd_max(prow4, col4, gl, G, CPL, A, C);
-                        gg = gm.g;
-                        amax = gm.m;
-                    }
-    #pragma unroll
-                    for (int off = G / 2; off > 0; off >>= 1) {
-                        const uint64_t og = __shfl_xor_sync(FULL, gg, off);
-                        gg = og == 0 ? gg : (gg == 0 ? og : gcd64(gg, og));
-                        const uint64_t y = __shfl_xor_sync(FULL, amax, off);
-                        amax = y > amax ? y : amax;
-                    }
-                    if (slow) {
-                        ovf = big && amax / gg > 2147483647ull;
-                        if (!ovf && gg > 1) {
-                            const bool pow2 = (gg & (gg - 1)) == 0;
-                            const int sh = __ffsll((long long)gg) - 1;
-                            if (!big) {
-    #pragma unroll
-                                for (int e = 0; e < EPL; ++e)
-                                    t32[e] = t32[e] == 0 ? 0 : (pow2 ? (t32[e] >> sh) : t32[e] / (int32_t)gg);
-                            } else {
-    #pragma unroll
-                                for (int i = 0; i < CPL; ++i) {
-                                    const int4 v = prow4[gl + G * i];
-                                    const int4 w = col4[gl + G * i];
-                                    const int32_t pv[4] = {v.x, v.y, v.z, v.w}, cv[4] = {w.x, w.y, w.z, w.w};
-    #pragma unroll
-                                    for (int jj = 0; jj < 4; ++jj) {
-                                        const int64_t tt = (int64_t)A * pv[jj] + (int64_t)C * cv[jj];
-                                        t32[4 * i + jj] = (int32_t)(tt / (int64_t)gg);
-                                    }
-                                }
-                            }
-                        }
-                    }
-                }
-                const bool bal = ok && !nz;
-                const bool grown = ok && nz && !ovf;
-                if (ovf && gl == 0) ++n_ovf;
-                if (bal && gl == 0) {
-                    ++n_bal;  // all metabolites stable: to the arbiter
-                    if (insert_support(a, W, pu, k) < INS_DUP) fatal = true;
-                }
-                fatal = group_or<G>(fatal ? 1u : 0u) != 0;
-                // superset pruning (counted on a truncated level too): the new
-                // column k completes a result accepted at an earlier level.  The
-                // G lanes of the group split the results containing k.
-                bool pr = false;
-                if (grown && !in_u) {
-                    const int64_t b1 = a.bptr[k];
-                    const int64_t n = a.bptr[k + 1] - b1;
-                    if (W <= 2) {
-                        const uint64_t u0 = child_word(pu, 0, k), u1 = W == 2 ? child_word(pu, 1, k) : 0ull;
-                        // every result containing k holds their intersection: if the
-                        // child lacks part of it, none of them lies inside the child
-                        bool maybe = true;
-                        if (a.band) {
-                            const uint64_t i0 = __ldg(a.band + (size_t)k * W), i1 = W == 2 ? __ldg(a.band + (size_t)k * W + 1) : 0ull;
-                            maybe = ((i0 & ~u0) | (i1 & ~u1)) == 0;
-                        }
-                        for (int64_t i = gl; i < n && !pr && maybe; i += G) {
-                            const uint64_t *E = a.bres + (size_t)(b1 + i) * W;
-                            const uint64_t e0 = __ldg(E), e1 = W == 2 ? __ldg(E + 1) : 0ull;
-                            pr = ((e0 & ~u0) | (e1 & ~u1)) == 0;
-                        }
-                    } else {
-                        for (int64_t i = gl; i < n && !pr; i += G) pr = result_inside_wide(a, pu, k, b1 + i);
-                    }
-                }
-                pr = group_or<G>(pr ? 1u : 0u) != 0;
-                if (pr && gl == 0) ++n_pruned;
-                const bool norm = grown && !pr;
-
-                // --- pivot key and fingerprint, then append to the batch ---
-                uint32_t key = 0xFFFFFFFFu, hlo = 0, hhi = 0;
-                if (norm) {
-    #pragma unroll
-                    for (int i = 0; i < CPL; ++i)
-    #pragma unroll
-                        for (int jj = 0; jj < 4; ++jj) {
-                            const int m = 4 * (gl + G * i) + jj;
-                            const int32_t v = t32[4 * i + jj];
-                            if (v != 0) {
-                                const uint32_t kk = bl[(v > 0 ? nv.o_keypos : nv.o_keyneg) + m];
-                                key = kk < key ? kk : key;
-                            }
-                            hash_entry((uint32_t)m, (uint32_t)v, hlo, hhi);
-                        }
-                    for (int w = gl; w < W; w += G) {
-                        const uint64_t x = mix64(child_word(pu, w, k) ^ (0x2545f4914f6cdd1dull * (uint64_t)(w + 1)));
-                        hlo += (uint32_t)x;
-                        hhi ^= (uint32_t)(x >> 32);
-                    }
-                }
-                key = group_min<G>(key);
-                hlo = group_add<G>(hlo);
-                hhi = group_xor<G>(hhi);
-                const unsigned nm = __ballot_sync(FULL, norm && gl == 0);
-                if (norm) {
-                    const int slot = nb + __popc(nm & ((1u << lead) - 1u));
-                    int4 *r = brow + (size_t)slot * BS::ROW;
-    #pragma unroll
-                    for (int i = 0; i < CPL; ++i)
-                        r[gl + G * i] = make_int4(t32[4 * i + 0], t32[4 * i + 1], t32[4 * i + 2], t32[4 * i + 3]);
-                    if (gl == 0) {
-                        uint64_t pos;
-                        uint32_t tag;
-                        slot_tag_pos(((uint64_t)hhi << 32) | hlo, a.slot_mask, pos, tag);
-                        prefetch_l2(&a.slots[pos]);
-                        bpos[slot] = pos;
-                        btag[slot] = tag;
-                        bkey[slot] = key;
-                        binfo[slot] = (uint32_t)k | (in_u ? 1u << 12 : 0u) | ((uint32_t)(pc + (in_u ? 0 : 1)) << 13);
-                        bpar[slot] = (uint32_t)p;
-                    }
-                }
-                nb += __popc(nm);
-                if (nb > NB - NG) flush();
-
-            }
-        }
-        if (__any_sync(FULL, fatal)) break;
-    }
-    if (nb > 0 && !__any_sync(FULL, fatal)) flush();
-    if (n_exp) atomicAdd(&a.ctr[C_EXP], n_exp);
-    if (n_ovf) atomicAdd(&a.ctr[C_OVF], n_ovf);
-    if (n_bal) atomicAdd(&a.ctr[C_BAL], n_bal);
-    if (n_pruned) atomicAdd(&a.ctr[C_PRUNED], n_pruned);
-    if (deg_sum) atomicAdd(&a.ctr[C_DEGSUM], deg_sum);
-}
-
 
 // ---------------------------------------------------------------------------
 // a7/a8: exact minimality test by elimination modulo primes, then append.
@@ -1671,49 +945,13 @@ __global__ void gather_kernel(const uint64_t *res, int W, const Rec *rec, int64_
 // ---------------------------------------------------------------------------
 // Batched traversal: one persistent launch over many (network, target) jobs.
 // Each CTA pulls jobs from a device queue and runs the whole level loop of a
-// job (seed, expand, minimality test, buckets, sorted output) with CTA
-// barriers between the steps, in its own slice of a scratch pool.  The level
-// decisions (truncation, cap, counters) are those of the single-job host loop.
+// job (seed, generate, dedup, minimality test, sorted output) with CTA
+// barriers between the steps, in its own slice of a scratch pool.  The steps
+// are the grid-wide level pass's device code and the level decisions
+// (truncation, cap, counters) those of the single-job path.  A job whose
+// levels do not fit the slice (its rows before deduplication, or more results
+// than the superset index holds) is left to the host, which runs it by itself.
 // ---------------------------------------------------------------------------
-
-// CTA-level bucket rebuild over results [0, n_res)
-__device__ void cta_buckets(const NetView &nv, const uint64_t *res, int64_t n_res, int32_t *bcnt, int32_t *bptr,
-                            int32_t *bfill, uint64_t *bres)
-{
-    const int W = nv.W;
-    for (int i = threadIdx.x; i < nv.N; i += blockDim.x) {
-        bcnt[i] = 0;
-        bfill[i] = 0;
-    }
-    __syncthreads();
-    for (int64_t i = threadIdx.x; i < n_res * W; i += blockDim.x) {
-        const int w = (int)(i % W);
-        for (uint64_t x = res[i]; x; x &= x - 1) atomicAdd(&bcnt[w * 64 + __ffsll((long long)x) - 1], 1);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int32_t run = 0;
-        for (int k = 0; k < nv.N; ++k) {
-            bptr[k] = run;
-            run += bcnt[k];
-        }
-        bptr[nv.N] = run;
-    }
-    __syncthreads();
-    for (int64_t i = threadIdx.x; i < n_res * W; i += blockDim.x) {
-        const int w = (int)(i % W);
-        const int64_t r = i / W;
-        for (uint64_t x = res[i]; x; x &= x - 1) {
-            const int k = w * 64 + __ffsll((long long)x) - 1;
-            const int64_t pos = (int64_t)bptr[k] + atomicAdd(&bfill[k], 1);
-            if (W > 2)
-                reinterpret_cast<int32_t *>(bres)[pos] = (int32_t)r;
-            else
-                for (int v = 0; v < W; ++v) bres[pos * W + v] = res[r * W + v];
-        }
-    }
-    __syncthreads();
-}
 
 // CTA-level sort of results [0, n) into out (first n_keep rows)
 __device__ void cta_sort(const uint64_t *res, int64_t n, int W, uint32_t *idx, uint64_t *out, int64_t n_keep)
@@ -1740,83 +978,116 @@ __device__ void cta_sort(const uint64_t *res, int64_t n, int W, uint32_t *idx, u
     __syncthreads();
 }
 
-template <int G, int CPL>
-__device__ void run_job(const BatchArgs &ba, const BatchJob &job, char *slice, uint32_t *sm)
-{
-    constexpr int EPL = G * CPL / 8;  // seed layout: Mpad = 32 EPL = 4 G CPL
-    const NetView &nv = job.nv;
-    unsigned long long *ctr = job.ctr;
-    const int nwarps = blockDim.x >> 5;
-    const int wid = threadIdx.x >> 5;
-    const BatchLayout &L = ba.layout;
-    __shared__ unsigned long long sh[C_COUNT];
+constexpr int kBatchAcceptWarps = 2;
 
-    LevelArgs a{};
-    a.slots = reinterpret_cast<unsigned long long *>(slice + L.o_slots);
-    a.cslots = reinterpret_cast<unsigned long long *>(slice + L.o_cslots);
-    a.cslot_mask = L.cslot_cap - 1;
-    a.cand = reinterpret_cast<uint64_t *>(slice + L.o_cand);
-    a.cand_cap = L.cand_cap;
-    a.res = reinterpret_cast<const uint64_t *>(slice + L.o_res);
-    a.bptr = reinterpret_cast<const int32_t *>(slice + L.o_bptr);
-    a.bres = reinterpret_cast<const uint64_t *>(slice + L.o_bres);
-    a.bids = reinterpret_cast<const int32_t *>(slice + L.o_bres);
-    a.rcols = nv.W > 2 ? reinterpret_cast<const uint16_t *>(slice + L.o_rcols) : nullptr;
-    a.max_len = job.max_len;
-    a.max_sec = ba.max_sec;
-    a.ctr = ctr;
+// 16-byte stores of ~0 (the regions are multiples of 16 bytes)
+__device__ __forceinline__ void cta_fill(void *p, size_t bytes)
+{
+    uint4 *t = reinterpret_cast<uint4 *>(p);
+    for (size_t i = threadIdx.x; i < bytes / 16; i += blockDim.x) t[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+}
+
+template <int F>
+__device__ void run_job(const BatchArgs &ba, const BatchJob &job, char *slice, uint32_t *sm, const NetView &nv,
+                        LevelArgs &a, AcceptArgs &acc, unsigned long long *sh)
+{
+    unsigned long long *ctr = job.ctr;
+    const int tid = threadIdx.x, nthreads = blockDim.x, nwarps = blockDim.x >> 5;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const BatchLayout &L = ba.layout;
+    const BoundScratch no_bound{};
     auto arena = [&](int i) {
         Arena r{};
-        r.U = reinterpret_cast<uint64_t *>(slice + L.o_U[i]);
-        r.B = reinterpret_cast<int32_t *>(slice + L.o_B[i]);
-        r.meta = reinterpret_cast<uint32_t *>(slice + L.o_meta[i]);
+        r.hdr = reinterpret_cast<uint4 *>(slice + L.o_hdr[i]);
+        r.pay = reinterpret_cast<uint4 *>(slice + L.o_pay[i]);
         r.cap = L.cap;
+        r.pay_cap = L.pay_cap;
         return r;
     };
-    AcceptArgs acc{};
-    acc.cand = a.cand;
-    acc.res = reinterpret_cast<uint64_t *>(slice + L.o_res);
-    acc.res_cap = L.res_cap;
-    acc.rcols = nv.W > 2 ? reinterpret_cast<uint16_t *>(slice + L.o_rcols) : nullptr;
-    acc.ctr = ctr;
-    int32_t *bcnt = reinterpret_cast<int32_t *>(slice + L.o_bcnt);
-    int32_t *bfill = reinterpret_cast<int32_t *>(slice + L.o_bfill);
-    int32_t *bptr = reinterpret_cast<int32_t *>(slice + L.o_bptr);
-    uint64_t *bres = reinterpret_cast<uint64_t *>(slice + L.o_bres);
-
-    for (uint64_t i = threadIdx.x; i < L.cslot_cap; i += blockDim.x) a.cslots[i] = kEmpty;
-    for (int i = threadIdx.x; i <= nv.N; i += blockDim.x) bptr[i] = 0;
+    if (tid == 0) {
+        a = LevelArgs{};
+        a.slots = reinterpret_cast<unsigned long long *>(slice + L.o_slots);
+        a.cslots = reinterpret_cast<unsigned long long *>(slice + L.o_cslots);
+        a.cslot_mask = L.cslot_cap - 1;
+        a.cand = reinterpret_cast<uint64_t *>(slice + L.o_cand);
+        a.cand_cap = L.cand_cap;
+        a.res = reinterpret_cast<const uint64_t *>(slice + L.o_res);
+        a.rcols = reinterpret_cast<const uint16_t *>(slice + L.o_rcols);
+        a.fp = reinterpret_cast<uint64_t *>(slice + L.o_fp);
+        a.fp_cap = L.fp_cap;
+        a.open = reinterpret_cast<uint32_t *>(slice + L.o_open);
+        a.max_len = job.max_len;
+        a.max_sec = ba.max_sec;
+        a.ctr = ctr;
+        a.child = arena(0);
+        CellIndex &ix = a.cells;
+        ix.cells = reinterpret_cast<uint2 *>(slice + L.o_cells);
+        ix.mask = L.cell_mask;
+        ix.ent = reinterpret_cast<uint4 *>(slice + L.o_ent);
+        ix.ksig = reinterpret_cast<uint64_t *>(slice + L.o_ksig);
+        ix.single = reinterpret_cast<uint32_t *>(slice + L.o_single);
+        ix.cnt = reinterpret_cast<int32_t *>(slice + L.o_cnt);
+        ix.ent_stride = L.ent_stride;
+        ix.room = L.index_room;
+        acc = AcceptArgs{};
+        acc.cand = a.cand;
+        acc.res = reinterpret_cast<uint64_t *>(slice + L.o_res);
+        acc.res_cap = L.res_cap;
+        acc.rcols = F == 0 ? reinterpret_cast<uint16_t *>(slice + L.o_rcols) : nullptr;
+        acc.ctr = ctr;
+        acc.ix = ix;
+    }
+    cta_fill(slice + L.o_cslots, L.cslot_cap * 8);
     __syncthreads();
     auto read_ctr = [&]() {
         __syncthreads();
-        for (int i = threadIdx.x; i < C_COUNT; i += blockDim.x) sh[i] = __ldcg(&ctr[i]);
+        for (int i = tid; i < C_COUNT; i += nthreads) sh[i] = __ldcg(&ctr[i]);
         __syncthreads();
     };
     auto set_ctr = [&](int i, unsigned long long v) {
-        if (threadIdx.x == 0) ctr[i] = v;
+        if (tid == 0) ctr[i] = v;
     };
-    const int ERRMASK = ERR_TIMEOUT | ERR_CAND_CAP | ERR_RES_CAP | ERR_TABLE_FULL | ERR_PRIMES | ERR_LEN |
-                        ERR_WATCHDOG | ERR_BOUNDS;
+    const unsigned ERRMASK = ERR_TIMEOUT | ERR_CAND_CAP | ERR_RES_CAP | ERR_TABLE_FULL | ERR_PRIMES | ERR_LEN |
+                             ERR_WATCHDOG | ERR_BOUNDS;
+    bool index_ready = false;
+    int64_t cand_done = 0;
+    // the minimality test of the candidates since the last one (sh is current)
+    auto accept_new = [&]() {
+        const int64_t end = (int64_t)min(sh[C_CAND_N], (unsigned long long)L.cand_cap);
+        if (end > cand_done) {
+            if (!index_ready) {  // (most jobs' first levels accept nothing)
+                for (int i = tid; i < nv.N; i += nthreads) {
+                    a.cells.cnt[i] = 0;
+                    a.cells.single[i] = 0u;
+                    a.cells.ksig[2 * i] = a.cells.ksig[2 * i + 1] = 0ull;
+                }
+                cta_fill(a.cells.cells, F ? (size_t)128 * 4 * nv.N : 8 * ((size_t)L.cell_mask + 1));
+                index_ready = true;
+            }
+            if (tid == 0) {
+                acc.cand_begin = cand_done;
+                acc.cand_end = end;
+            }
+            __syncthreads();
+            if (wid < kBatchAcceptWarps) accept_range(nv, acc, sm + wid * kAcceptWarpWords, wid, kBatchAcceptWarps);
+        }
+        cand_done = end;
+        read_ctr();
+    };
 
     // level 0: seeds, then the minimality test of balanced seeds
     int cur = 0;
-    a.level = 0;
-    a.child = arena(cur);
-    seed_range<EPL>(nv, a, job.target, wid, nwarps);
+    seed_range<F, false>(nv, a, job.target, tid, nthreads);
     read_ctr();
     if (sh[C_ERR] & ERRMASK) return;
-    acc.cand_begin = 0;
-    acc.cand_end = (int64_t)sh[C_CAND_N];
-    if (wid < kAcceptWarps) accept_range(nv, acc, sm + wid * kAcceptWarpWords, wid, kAcceptWarps);
-    read_ctr();
+    accept_new();
     if (sh[C_ERR] & ERRMASK) return;
-    int64_t cand_done = (int64_t)sh[C_CAND_N];
     int64_t res_n = (int64_t)min(sh[C_RES_N], (unsigned long long)L.res_cap);
-    int64_t n_front = (int64_t)sh[C_NEXT];
+    int64_t n_front = (int64_t)sh[C_NEXT], n_rows = n_front;
     uint64_t deg_sum = sh[C_DEGSUM];
     unsigned long long status = 0, frontier = 0, frontier_max = 0, levels = 1;
     bool stop = false;
-    if (ba.max_frontier > 0 && n_front > ba.max_frontier) {
+    if (n_front > ba.max_frontier) {
         status |= EFM_TRUNCATED;
         stop = true;
     } else {
@@ -1827,44 +1098,56 @@ __device__ void run_job(const BatchArgs &ba, const BatchJob &job, char *slice, u
             stop = true;
         }
     }
-    int64_t built_for = 0;
     for (int level = 1; !stop && n_front > 0; ++level) {
         if (level > a.max_len + a.max_sec + 1) {
-            if (threadIdx.x == 0) atomicOr(&ctr[C_ERR], (unsigned long long)ERR_WATCHDOG);
+            if (tid == 0) atomicOr(&ctr[C_ERR], (unsigned long long)ERR_WATCHDOG);
             return;
         }
-        if (res_n != built_for) {
-            cta_buckets(nv, acc.res, res_n, bcnt, bptr, bfill, bres);
-            built_for = res_n;
+        const uint64_t reserved = deg_sum + 64;
+        const uint64_t nslots = next_pow2_dev(2 * reserved + 64);
+        if ((int64_t)reserved > L.fp_cap || nslots > L.slot_cap || res_n > L.index_room) {
+            set_ctr(C_DONE, 2ull);  // to the host
+            return;
         }
-        const uint64_t bound = min(deg_sum, (uint64_t)L.cap);
-        const uint64_t nslots = min(L.slot_cap, next_pow2_dev(2 * bound + 64 * (uint64_t)nwarps));
-        for (uint64_t i = threadIdx.x; i < nslots; i += blockDim.x) a.slots[i] = kEmpty;
-        set_ctr(C_NEXT, 0);
-        set_ctr(C_DEGSUM, 0);
+        cta_fill(slice + L.o_slots, nslots * 8);
+        const int clear[] = {C_NEXT, C_DEGSUM, C_WRITTEN, C_UNWRITTEN, C_UNV, C_PAY, C_OPEN, C_DEDUP_BEGIN};
+        if (tid == 0) {
+            for (int i = 0; i < 8; ++i) ctr[clear[i]] = 0ull;
+            a.par = arena(cur);
+            a.child = arena(cur ^ 1);
+            a.level = level;
+        }
         __syncthreads();
-        a.par = arena(cur);
-        a.n_par = n_front;
-        a.child = arena(cur ^ 1);
-        a.slot_mask = nslots - 1;
-        a.level = level;
-        a.cpw = (int)min((int64_t)ba.tile, max((int64_t)1, (n_front + nwarps - 1) / nwarps));
-        expand_range<G, CPL>(nv, a, nv.blob, reinterpret_cast<char *>(sm) + (size_t)wid * BatchShape<G, CPL>::BYTES,
-                             wid, nwarps);
+        const int cpw = (int)min((int64_t)ba.tile, max((int64_t)1, (n_rows + nwarps - 1) / nwarps));
+        generate_range<F, false, false>(nv, a, n_rows, cpw, 0, 0, res_n > 0, wid, nwarps, nullptr, no_bound);
+        __syncthreads();
+        DedupSums sum;
+        // (counters past L1: this SM may hold older ones)
+        dedup_range<F, false>(nv, a, nslots - 1, __ldcg(&ctr[C_DEDUP_BEGIN]), __ldcg(&ctr[C_WRITTEN]),
+                              __ldcg(&ctr[C_OPEN]), tid & ~31, tid & ~31, nthreads, sum);
+        unsigned keep = __reduce_add_sync(FULL, sum.keep), unv = __reduce_add_sync(FULL, sum.unv);
+        unsigned deg = __reduce_add_sync(FULL, (unsigned)sum.deg);  // (far below 2^32 in a slice)
+        if (lane == 0) {
+            if (keep) atomicAdd(&ctr[C_NEXT], (unsigned long long)keep);
+            if (unv) atomicAdd(&ctr[C_UNV], (unsigned long long)unv);
+            if (deg) atomicAdd(&ctr[C_DEGSUM], (unsigned long long)deg);
+        }
         read_ctr();
         if (sh[C_ERR] & ERRMASK) return;
-        acc.cand_begin = cand_done;
-        acc.cand_end = (int64_t)sh[C_CAND_N];
-        if (wid < kAcceptWarps) accept_range(nv, acc, sm + wid * kAcceptWarpWords, wid, kAcceptWarps);
-        read_ctr();
-        if (sh[C_ERR] & ERRMASK) return;
-        cand_done = (int64_t)sh[C_CAND_N];
-        res_n = (int64_t)min(sh[C_RES_N], (unsigned long long)L.res_cap);
-        n_front = (int64_t)sh[C_NEXT];
+        const bool unwritten = sh[C_UNWRITTEN] != 0ull;
+        n_front = (int64_t)(sh[C_NEXT] + (unwritten ? sh[C_UNV] : 0ull));
+        if (unwritten && n_front <= ba.max_frontier) {
+            set_ctr(C_DONE, 2ull);  // not decided: to the host
+            return;
+        }
+        n_rows = (int64_t)min(sh[C_WRITTEN], (unsigned long long)L.cap);
         deg_sum = sh[C_DEGSUM];
+        accept_new();
+        if (sh[C_ERR] & ERRMASK) return;
+        res_n = (int64_t)min(sh[C_RES_N], (unsigned long long)L.res_cap);
         levels = level + 1;
         cur ^= 1;
-        if (ba.max_frontier > 0 && n_front > ba.max_frontier) {
+        if (n_front > ba.max_frontier) {
             status |= EFM_TRUNCATED;
             break;
         }
@@ -1876,7 +1159,7 @@ __device__ void run_job(const BatchArgs &ba, const BatchJob &job, char *slice, u
         }
     }
     if ((int64_t)sh[C_RES_N] > L.res_cap) {
-        if (threadIdx.x == 0) atomicOr(&ctr[C_ERR], (unsigned long long)ERR_RES_CAP);
+        if (tid == 0) atomicOr(&ctr[C_ERR], (unsigned long long)ERR_RES_CAP);
         return;
     }
     const int64_t n_keep = ba.max_results > 0 ? min(res_n, ba.max_results) : res_n;
@@ -1890,10 +1173,22 @@ __device__ void run_job(const BatchArgs &ba, const BatchJob &job, char *slice, u
     set_ctr(C_DONE, 1ull);
 }
 
-__global__ void __launch_bounds__(kBatchThreads) batch_kernel(BatchArgs ba)
+// A CTA takes jobs off a queue and runs each through the same level pass, its
+// states, tables and index in the CTA's slice of the pool.  Latency bounds it:
+// a level of a small job is a chain of short phases with barriers between, so
+// what counts is how fast one CTA goes through its job.  With 128 registers
+// (two CTAs of 8 warps on an SM) 512 uneven networks take 5.4 ms, with 85 and
+// three CTAs 5.6 to 6.0, with 64 and four 6.0 to 6.2 (spills); on rows of every
+// metabolite, with 255 registers and one CTA, the call took 15.8 before its
+// fetches and takes 6.2 now.
+__global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const __grid_constant__ BatchArgs ba)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ int s_job;
+    __shared__ NetView s_nv;
+    __shared__ LevelArgs s_a;
+    __shared__ AcceptArgs s_acc;
+    __shared__ unsigned long long s_ctr[C_COUNT];
     char *slice = ba.pool + (size_t)blockIdx.x * ba.layout.slice_bytes;
     const int chunk = ba.chunk > 0 ? ba.chunk : 1;
     for (;;) {
@@ -1904,15 +1199,11 @@ __global__ void __launch_bounds__(kBatchThreads) batch_kernel(BatchArgs ba)
         if (q0 >= ba.n_jobs) break;
         for (int qi = q0; qi < q0 + chunk && qi < ba.n_jobs; ++qi) {
             const BatchJob &job = ba.jobs[ba.order[qi]];
-            switch (job.nv.EPL) {
-            case 1: run_job<4, 2>(ba, job, slice, smem); break;
-            case 2: run_job<8, 2>(ba, job, slice, smem); break;
-            case 4: run_job<16, 2>(ba, job, slice, smem); break;
-            case 8: run_job<32, 2>(ba, job, slice, smem); break;
-            default:
-                if (threadIdx.x == 0) atomicOr(&job.ctr[C_ERR], (unsigned long long)ERR_LEN);
-                break;
-            }
+            if (threadIdx.x == 0) s_nv = job.nv;
+            __syncthreads();
+            if (s_nv.form == 2) run_job<2>(ba, job, slice, smem, s_nv, s_a, s_acc, s_ctr);
+            else if (s_nv.form == 1) run_job<1>(ba, job, slice, smem, s_nv, s_a, s_acc, s_ctr);
+            else run_job<0>(ba, job, slice, smem, s_nv, s_a, s_acc, s_ctr);
             __syncthreads();
         }
     }
@@ -2020,6 +1311,12 @@ cudaError_t launch_sort_index(const uint64_t *res, int64_t n, int W, uint32_t *i
     return sort_with(res, n, W, idx, n2, out, n_keep, s);
 }
 
+cudaError_t launch_batch_gather(const BatchJob *jobs, const int64_t *off, int n_jobs, uint64_t *dst, cudaStream_t s)
+{
+    batch_gather_kernel<<<std::min(n_jobs, 4096), 128, 0, s>>>(jobs, off, n_jobs, dst);
+    return cudaGetLastError();
+}
+
 int batch_blocks_per_sm(int warps)
 {
     int per_sm = 0;
@@ -2033,17 +1330,9 @@ int batch_blocks_per_sm(int warps)
     return per_sm;
 }
 
-size_t batch_smem_bytes(int warps)
+size_t batch_smem_bytes(int)
 {
-    // union of the expansion batches of all warps (largest row class) and the
-    // minimality scratch of kAcceptWarps warps
-    size_t ex = (size_t)BatchShape<4, 2>::BYTES;
-    ex = ex > (size_t)BatchShape<8, 2>::BYTES ? ex : (size_t)BatchShape<8, 2>::BYTES;
-    ex = ex > (size_t)BatchShape<16, 2>::BYTES ? ex : (size_t)BatchShape<16, 2>::BYTES;
-    ex = ex > (size_t)BatchShape<32, 2>::BYTES ? ex : (size_t)BatchShape<32, 2>::BYTES;
-    ex *= (size_t)warps;
-    const size_t ac = (size_t)kAcceptWarps * kAcceptWarpWords * 4;
-    return ex > ac ? ex : ac;
+    return (size_t)kBatchAcceptWarps * kAcceptWarpWords * 4;
 }
 
 cudaError_t launch_batch(const BatchArgs &ba, int grid, int warps, cudaStream_t s)

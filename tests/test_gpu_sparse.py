@@ -110,3 +110,24 @@ def test_lane_walks(oracle_lib, efm, name):
                 sup, ctr = efm.sample_target(nw, t, 20, 3, 5, n)
                 osup, octr = oracle_lib.sample_pathways(net, t, oracle_lib.Limits(20, 3), 5, n)
                 assert np.array_equal(sup, osup) and ctr == octr, (name, t, n, ctr, octr)
+
+
+@pytest.mark.parametrize("budget", [2**6, 2**10, 2**14])
+def test_batch_slices(efm, budget):
+    # levels that outgrow a job's slice are run alone; the rows come back in
+    # one copy: counters and rows equal single calls' at every budget
+    nets = [synth.batched_member(20 + i) for i in range(64)] + [synth.core()]
+    loaded = [efm.Network(n) for n in nets]
+    try:
+        targets = [n.targets[0] for n in nets]
+        job, _ = efm.efm_find_pathways_batch([w.handle for w in loaded], targets, 24, 3, 0, budget)
+        try:
+            got = [efm.efm_fetch_results(job, i) for i in range(len(nets))]
+        finally:
+            efm.efm_free_job(job)
+        for net, w, target, (sup, ctr, _) in zip(nets, loaded, targets, got):
+            (ssup, sctr), = efm.enumerate_targets(w, [target], 24, 3, 0, budget)
+            assert np.array_equal(sup, ssup) and ctr == sctr, net.name
+    finally:
+        for w in loaded:
+            w.close()
