@@ -613,8 +613,106 @@ __device__ bool full_rank_mod_p(const uint32_t *bl, const NetView &nv, const int
     return false;
 }
 
-// shared memory of one minimality warp: basis 64x64, columns 64, pivots 64, row map 32
-constexpr int kAcceptWarpWords = 64 * 64 + 64 + 64 + 32;
+// The same test with the rows in the lanes, for columns that touch at most 64
+// rows.  The submatrix stands in shared memory, a column of kRankStride words
+// after the other (a lane's row and a column's entry in one row are both free
+// of bank conflicts); a step finds a pivot for one column by ballot and only
+// the rows with an entry in it change, and there only the columns of the pivot
+// row's entries if the pivot is +-1.  A column without a pivot is a
+// combination of those before it, which ends the test.
+//
+// One candidate is one warp's serial chain and most levels have fewer
+// candidates than the chip has warps, so the chain's length is what counts: a
+// row of 20 columns against a basis of 20 takes 20 dependent steps of 64-bit
+// products in the streaming form above, a column here takes one.  One GB300, a
+// core query: 22.4 -> 14.6 us a launch of the test (7 us of it the launch and
+// the level state); calls: eight core targets at 2^17 9.46 -> 8.85 ms, a set of
+// seeds 3.37 -> 3.09, one core query 2.39 -> 2.27, the genome-shaped network
+// 24.3 -> 23.1.  Columns that touch more rows than that keep the streaming form.
+constexpr int kRankStride = 65;
+
+// row map of the columns and its prefix counts; returns the number of rows
+__device__ int rank_rows(const uint32_t *bl, const NetView &nv, const int *cols, int nn, uint32_t *rowmap, int *prefix,
+                         int lane)
+{
+    rowmap[lane] = 0;
+    __syncwarp();
+    for (int j = lane; j < nn; j += 32) {
+        const int col = cols[j];
+        for (int q = (int)bl[nv.o_colptr + col]; q < (int)bl[nv.o_colptr + col + 1]; ++q) {
+            const int row = ent_index(bl[nv.o_colent + q]);
+            atomicOr(&rowmap[row >> 5], 1u << (row & 31));
+        }
+    }
+    __syncwarp();
+    const int n = __popc(rowmap[lane]);
+    int sum = n;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int x = __shfl_up_sync(FULL, sum, off);
+        if (lane >= off) sum += x;
+    }
+    prefix[lane] = sum - n;
+    __syncwarp();
+    return __shfl_sync(FULL, sum, 31);
+}
+
+__device__ bool full_rank_rows(const uint32_t *bl, const NetView &nv, const int *cols, int nn, uint32_t p, uint32_t c,
+                               uint32_t *A /* [nn][kRankStride] */, const uint32_t *rowmap, const int *prefix, int lane)
+{
+    uint4 *z = reinterpret_cast<uint4 *>(A);
+    for (int i = lane; i < (nn * kRankStride + 3) / 4; i += 32) z[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+    for (int j = lane; j < nn; j += 32) {
+        const int col = cols[j];
+        for (int q = (int)bl[nv.o_colptr + col]; q < (int)bl[nv.o_colptr + col + 1]; ++q) {
+            const uint32_t e = bl[nv.o_colent + q];
+            const int row = ent_index(e);
+            const int at = prefix[row >> 5] + __popc(rowmap[row >> 5] & ((1u << (row & 31)) - 1u));
+            A[j * kRankStride + at] = to_mod(ent_coef(e), p);
+        }
+    }
+    __syncwarp();
+    unsigned free0 = FULL, free1 = FULL;  // rows that are no pivot yet
+    for (int j = 0; j < nn; ++j) {
+        const uint32_t y0 = A[j * kRankStride + lane], y1 = A[j * kRankStride + 32 + lane];
+        unsigned m0 = __ballot_sync(FULL, y0 != 0) & free0, m1 = __ballot_sync(FULL, y1 != 0) & free1;
+        if ((m0 | m1) == 0) return false;
+        const unsigned e0 = __ballot_sync(FULL, y0 == 1u || y0 == p - 1u) & m0;
+        const unsigned e1 = __ballot_sync(FULL, y1 == 1u || y1 == p - 1u) & m1;
+        const int r = e0 ? __ffs((int)e0) - 1 : e1 ? 31 + __ffs((int)e1) : m0 ? __ffs((int)m0) - 1 : 31 + __ffs((int)m1);
+        const unsigned r0 = r < 32 ? 1u << r : 0u, r1 = r < 32 ? 0u : 1u << (r - 32);
+        free0 &= ~r0;
+        free1 &= ~r1;
+        m0 &= ~r0;
+        m1 &= ~r1;
+        if ((m0 | m1) == 0) continue;
+        const uint32_t b = A[j * kRankStride + r];
+        const bool unit = b == 1u || b == p - 1u;
+        // columns to change: the pivot row's entries, or all if rows are scaled
+        // (cross-multiplied: no inverse, a chain of 60 products, is taken)
+        unsigned long long todo;
+        {
+            const bool t0 = lane > j && lane < nn && (!unit || A[lane * kRankStride + r] != 0u);
+            const bool t1 = lane + 32 > j && lane + 32 < nn && (!unit || A[(lane + 32) * kRankStride + r] != 0u);
+            todo = (unsigned long long)__ballot_sync(FULL, t0) | (unsigned long long)__ballot_sync(FULL, t1) << 32;
+        }
+        const bool a0 = (m0 >> lane) & 1u, a1 = (m1 >> lane) & 1u;
+        const uint32_t f0 = b == 1u || !unit ? y0 : p - y0, f1 = b == 1u || !unit ? y1 : p - y1;  // (y > 0 where used)
+        while (todo) {
+            uint32_t *x = A + (__ffsll((long long)todo) - 1) * kRankStride;
+            todo &= todo - 1ull;
+            const uint32_t t = x[r];
+            if (a0) x[lane] = submod(unit ? x[lane] : mulmod(x[lane], b, p, c), mulmod(f0, t, p, c), p);
+            if (a1) x[lane + 32] = submod(unit ? x[lane + 32] : mulmod(x[lane + 32], b, p, c), mulmod(f1, t, p, c), p);
+        }
+        __syncwarp();
+    }
+    return true;
+}
+
+// shared memory of one minimality warp: matrix, columns 64, pivots or prefix counts 64, row map 32
+constexpr int kAcceptWarpWords = 64 * kRankStride + 64 + 64 + 32;
 
 // Minimality test of the candidates [cand_begin, cand_end) by the warps
 // gw = 0 .. nw-1; ws: this warp's shared-memory scratch (kAcceptWarpWords).
@@ -623,7 +721,7 @@ __device__ void accept_range(const NetView &nv, const AcceptArgs &a, uint32_t *w
     const int lane = threadIdx.x & 31;
     const int W = nv.W;
     uint32_t *basis = ws;
-    int *cols = reinterpret_cast<int *>(ws + 64 * 64);
+    int *cols = reinterpret_cast<int *>(ws + 64 * kRankStride);
     int *pivcol = cols + 64;
     uint32_t *rowmap = reinterpret_cast<uint32_t *>(pivcol + 64);
     const uint32_t *bl = nv.blob;
@@ -651,9 +749,15 @@ __device__ void accept_range(const NetView &nv, const AcceptArgs &a, uint32_t *w
             continue;
         }
         bool ok = nn == 0;
-        for (int pi = 0; pi < kp && !ok; ++pi) {
+        __syncwarp();
+        const int rows = rank_rows(bl, nv, cols, nn, rowmap, pivcol, lane);
+        for (int pi = 0; pi < kp && !ok && rows >= nn; ++pi) {
             const uint32_t cc = c_prime_c[pi];
-            ok = full_rank_mod_p(bl, nv, cols, nn, 0x80000000u - cc, cc, basis, pivcol, rowmap, lane);
+            if (rows <= 64)
+                ok = full_rank_rows(bl, nv, cols, nn, 0x80000000u - cc, cc, basis, rowmap, pivcol, lane);
+            else
+                ok = full_rank_mod_p(bl, nv, cols, nn, 0x80000000u - cc, cc, basis, pivcol, rowmap, lane);
+            __syncwarp();
         }
         if (ok) {
             unsigned long long idx = 0;

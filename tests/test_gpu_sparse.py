@@ -131,3 +131,34 @@ def test_batch_slices(efm, budget):
     finally:
         for w in loaded:
             w.close()
+
+
+def ladder(steps, sides):
+    """steps rungs from one external metabolite to another, each carrying
+    1 + sides internal metabolites on; two reactions have twins with two and
+    three times their coefficients, so there are four pathways."""
+    n_int = steps * (1 + sides)
+    rxn = [[(n_int, -1)] + [(s, 1) for s in range(1 + sides)]]
+    for i in range(1, steps):
+        a, b = (i - 1) * (1 + sides), i * (1 + sides)
+        rxn.append([(a + s, -1 - s % 2) for s in range(1 + sides)] + [(b + s, 1 + s % 2) for s in range(1 + sides)])
+    a = (steps - 1) * (1 + sides)
+    rxn.append([(a + s, -1) for s in range(1 + sides)] + [(n_int + 1, 1)])
+    rxn[0] = [(m, v * (1 if m == n_int else 1 + m % (1 + sides) % 2)) for m, v in rxn[0]]
+    rxn[-1] = [(m, v * (1 if m == n_int + 1 else 1 + (m - a) % 2)) for m, v in rxn[-1]]
+    rxn.append([(m, 3 * v) for m, v in rxn[steps // 2]])
+    rxn.append([(m, 2 * v) for m, v in rxn[steps // 3]])
+    S = np.zeros((n_int + 2, len(rxn)), dtype=np.int64)
+    for j, ents in enumerate(rxn):
+        for m, v in ents:
+            S[m, j] = v
+    external = [0] * n_int + [1, 1]
+    return synth.Network.from_dense(S, [0] * len(rxn), external, [n_int + 1], f"ladder-{steps}-{sides}")
+
+
+@pytest.mark.parametrize("steps,sides", [(31, 0), (32, 0), (33, 0), (32, 1), (13, 4), (63, 0), (61, 1), (2, 40)])
+def test_rank_rows(oracle_lib, efm, steps, sides):
+    # the minimality test at 31 to 33, 64, 65 and 122 rows, and at 64 columns
+    net = ladder(steps, sides)
+    out = check(oracle_lib, efm, net, net.targets, min(64, steps + 2), 2, 1 << 12)
+    assert out[0]["results"] >= 4
