@@ -681,6 +681,21 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         out.kernel_launches += 2;
         if (manual && (rc = read_ctr())) return rc;
     }
+    int level = level0;  // last completed level (as far as the host knows)
+    if (!manual && !fs) {
+        // the first levels by one CTA while they are small; then the host has the state
+        acc.advance = 2;
+        CK(cudaEventRecord(w.ev[2], s));
+        CK(launch_small(nv, a, acc, arena(0), arena(1), kSmallBranches, s));
+        CK(cudaEventRecord(w.ev[3], s));
+        out.kernel_launches += 1;
+        if ((rc = read_ctr())) return rc;
+        float small_ms = 0.f;
+        CK(cudaEventElapsedTime(&small_ms, w.ev[2], w.ev[3]));
+        out.expand_ms += small_ms;
+        level = (int)hs[S_LEVEL];
+        cur = (level - level0) & 1;
+    }
     if (fk) {
         res_n = (int64_t)std::min<unsigned long long>(h[C_RES_N], (unsigned long long)w.res_cap);
         if (res_n > 0) {
@@ -693,11 +708,9 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         if (top.pc > 0) CK(cudaMemcpyAsync(w.fkb.p, top.kth.data(), (size_t)nv.W * 8, cudaMemcpyHostToDevice, s));
     }
     float ms = 0.f;
-    int level = level0;  // last completed level (as far as the host knows)
     int reruns = 0;
-    bool known = manual || fs;  // h holds the state
     while (!stop) {
-        if (known && hs[S_STOP] != STOP_NONE) {
+        if (hs[S_STOP] != STOP_NONE) {
             switch (hs[S_STOP]) {
             case STOP_DONE: stop = true; break;
             case STOP_CAPPED: status |= EFM_CAPPED; stop = true; break;
@@ -745,7 +758,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         if (!manual) {
             // several levels at a time while they are small: a level's launches
             // return at once when an earlier one has stopped the search
-            const uint64_t deg = known ? hs[S_DEG] : 64;
+            const uint64_t deg = hs[S_DEG];
             const int n = deg <= 65536 ? 4 : (deg <= (1u << 20) ? 2 : 1);
             CK(cudaEventRecord(w.ev[2], s));
             for (int i = 0; i < n; ++i) {
@@ -755,7 +768,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                 a.child = arena(cur ^ (i & 1) ^ 1);
                 // the level's state table: cleared by the launch itself, or, at a
                 // large level whose size the host knows, by a memset
-                a.first = n > 1 || !known;
+                a.first = n > 1;
                 if (!a.first) CK(cudaMemsetAsync(w.slots.p, 0xFF, hs[S_SLOTS] * 8, s));
                 if ((rc = launch_level(lv, grid_for(deg << (2 * i)), 2))) return rc;
             }
@@ -767,7 +780,6 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             if (done > 0) reruns = 0;
             cur ^= done & 1;
             level += done;
-            known = true;
             continue;
         }
         const int64_t n_rows = (int64_t)hs[S_NROWS];

@@ -19,6 +19,13 @@ constexpr int kNumPrimes = 24;
 constexpr int64_t kFirstKChunkMin = 8192;     // first-K search: fewest parents per expansion launch
 constexpr int64_t kFirstKChunks = 32;         // first-K search: launches per level, at most
 constexpr int64_t kResultWindow = 256;        // first-K search: new results fetched with the counters
+// Most branches of a level that one CTA runs (launch_small).  Up to there a
+// level by one CTA takes less than three launches; with 512, 1024, 2048, 4096:
+// the smallest query 0.80, 0.80, 0.84, 0.90 ms (three launches for every level:
+// 0.84), eight core targets at 2^17 8.05, 8.10, 8.20, 8.78 (8.86), a 400-row
+// network 3.93, 3.90, 4.07, 4.20 (4.13), the subtractive variant 5.85, 5.83,
+// 5.95, 6.6 (6.07).
+constexpr int kSmallBranches = 1024;
 constexpr int kWaitSpinLimit = 1 << 20;       // polls of a bounded device-side wait (with ~0.25 us sleeps)
 
 // device error bits (ctr[C_ERR])
@@ -300,6 +307,10 @@ cudaError_t launch_accept(const NetView &nv, const AcceptArgs &a, cudaStream_t s
 // minimality test of the candidates appended since the last such launch (range read on the
 // device); accepted results are filed in the index; then the level state moves on
 cudaError_t launch_accept_new(const NetView &nv, const AcceptArgs &a, int sm_count, cudaStream_t s);
+// the levels from the state's on while they have at most `limit` branches, by one CTA; the
+// parents of the first are in `first`, of the next in `second`, and so on
+cudaError_t launch_small(const NetView &nv, const LevelArgs &a, const AcceptArgs &acc, const Arena &first,
+                         const Arena &second, int limit, cudaStream_t s);
 // sort by (|U|, ascending columns); n2: n rounded up to a power of two; scratch: sort_scratch_bytes(n2)
 size_t sort_scratch_bytes(int64_t n2);
 int sort_launches(int64_t n2);

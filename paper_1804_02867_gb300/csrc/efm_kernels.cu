@@ -1277,6 +1277,93 @@ __device__ void run_job(const BatchArgs &ba, const BatchJob &job, char *slice, u
     set_ctr(C_DONE, 1ull);
 }
 
+// The levels of one search while they are small, by one CTA: from the state's
+// level on, until the search stops or a level has more than `limit` branches.
+// Latency bounds such a level: three launches of chains of dependent reads,
+// each on a cold L1.  Here a barrier ends a phase, and the network's tables and
+// the rows just written are in the SM's L1.  One GB300, with three launches for
+// every level and this way: the smallest query 0.835 -> 0.739 ms, eight core
+// targets at 2^17 8.86 -> 8.06, a 400-row network 4.13 -> 3.92, the subtractive
+// variant 6.07 -> 5.83, a set of seeds 3.09 -> 2.95.
+constexpr int kSmallWarps = 16;
+constexpr int kSmallAcceptWarps = 8;
+
+template <int F, bool SUB>
+__global__ void __launch_bounds__(kSmallWarps * 32, 1) small_kernel(const __grid_constant__ NetView nv,
+                                                                    const __grid_constant__ LevelArgs a0,
+                                                                    const __grid_constant__ AcceptArgs acc0,
+                                                                    const __grid_constant__ Arena first,
+                                                                    const __grid_constant__ Arena second, int limit)
+{
+    extern __shared__ __align__(16) uint32_t smem[];
+    __shared__ LevelArgs a;
+    __shared__ AcceptArgs acc;
+    __shared__ unsigned long long v[C_COUNT + S_COUNT];
+    const int tid = threadIdx.x, nthreads = kSmallWarps * 32, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned long long *sv = v + C_COUNT;
+    const BoundScratch no_bound{};
+    auto read_state = [&]() {
+        __syncthreads();
+        for (int i = tid; i < C_COUNT + S_COUNT; i += nthreads) v[i] = __ldcg(&a0.ctr[i]);
+        __syncthreads();
+    };
+    if (tid == 0) {
+        a = a0;
+        acc = acc0;
+    }
+    for (bool odd = false;; odd = !odd) {
+        read_state();
+        if (sv[S_STOP] != STOP_NONE || sv[S_DEG] > (unsigned long long)limit || sv[S_NROWS] > (unsigned long long)limit)
+            return;
+        const uint64_t slots = sv[S_SLOTS];
+        const int64_t n_par = (int64_t)sv[S_NROWS];
+        const bool any_result = v[C_RES_N] != 0ull;
+        cta_fill(a0.slots, slots * 8);
+        if (tid == 0) {
+            a.par = odd ? second : first;
+            a.child = odd ? first : second;
+            a.level = acc.level = (int)sv[S_LEVEL] + 1;
+            acc.child_rows = a.child.cap;
+        }
+        __syncthreads();
+        const int cpw = (int)min((int64_t)32, max((int64_t)1, (n_par + kSmallWarps - 1) / kSmallWarps));
+        generate_range<F, SUB, false>(nv, a, n_par, cpw, 0, 0, any_result, wid, kSmallWarps, nullptr, no_bound);
+        read_state();
+        DedupSums sum;
+        dedup_range<F, SUB>(nv, a, slots - 1, v[C_DEDUP_BEGIN], v[C_WRITTEN], v[C_OPEN], tid & ~31, tid & ~31, nthreads,
+                            sum);
+        const unsigned keep = __reduce_add_sync(FULL, sum.keep), unv = __reduce_add_sync(FULL, sum.unv);
+        const unsigned deg = __reduce_add_sync(FULL, (unsigned)sum.deg);  // (limit children of at most 2^13 branches)
+        if (lane == 0) {
+            if (keep) atomicAdd(&a.ctr[C_NEXT], (unsigned long long)keep);
+            if (unv) atomicAdd(&a.ctr[C_UNV], (unsigned long long)unv);
+            if (deg) atomicAdd(&a.ctr[C_DEGSUM], (unsigned long long)deg);
+        }
+        read_state();
+        // (as in the launch for one level: one that will run again is judged then)
+        const bool rerun = v[C_UNWRITTEN] != 0ull &&
+                           !(acc.max_frontier > 0 && (int64_t)(v[C_NEXT] + v[C_UNV]) > acc.max_frontier);
+        const int64_t begin = (int64_t)v[C_ACC_BEGIN], n = (int64_t)v[C_CAND_N];
+        const int64_t end = rerun ? begin : (n < acc.cand_cap ? n : acc.cand_cap);
+        if (end > begin) {
+            if (tid == 0) {
+                acc.cand_begin = begin;
+                acc.cand_end = end;
+            }
+            __syncthreads();
+            if (wid < kSmallAcceptWarps)
+                accept_range(nv, acc, smem + wid * kAcceptWarpWords, wid, kSmallAcceptWarps);
+            read_state();
+        }
+        if (tid == 0) {
+            a.ctr[C_ACC_BEGIN] = (unsigned long long)end;
+            a.ctr[C_DEDUP_BEGIN] = v[C_WRITTEN];
+            a.ctr[C_OPEN] = 0ull;
+            advance_level(acc, v);
+        }
+    }
+}
+
 // A CTA takes jobs off a queue and runs each through the same level pass, its
 // states, tables and index in the CTA's slice of the pool.  Latency bounds it:
 // a level of a small job is a chain of short phases with barriers between, so
@@ -1413,6 +1500,21 @@ cudaError_t launch_sort_index(const uint64_t *res, int64_t n, int W, uint32_t *i
                               int64_t n_keep, cudaStream_t s)
 {
     return sort_with(res, n, W, idx, n2, out, n_keep, s);
+}
+
+cudaError_t launch_small(const NetView &nv, const LevelArgs &a, const AcceptArgs &acc, const Arena &first,
+                         const Arena &second, int limit, cudaStream_t s)
+{
+    const size_t sm = (size_t)kSmallAcceptWarps * kAcceptWarpWords * 4;
+#define EFM_LAUNCH(K)                                                                                   \
+    do {                                                                                                \
+        cudaError_t e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);  \
+        if (e != cudaSuccess) return e;                                                                 \
+        K<<<1, kSmallWarps * 32, sm, s>>>(nv, a, acc, first, second, limit);                            \
+    } while (0)
+    EFM_FORM(small_kernel, EFM_LAUNCH);
+#undef EFM_LAUNCH
+    return cudaGetLastError();
 }
 
 cudaError_t launch_batch_gather(const BatchJob *jobs, const int64_t *off, int n_jobs, uint64_t *dst, cudaStream_t s)

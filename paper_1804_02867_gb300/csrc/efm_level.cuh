@@ -1463,5 +1463,15 @@ __device__ __forceinline__ void seed_range(const NetView &nv, const LevelArgs &a
     }
 }
 
+// one of a kernel's instances: form, subtractive view
+#define EFM_FORM(KERNEL, CALL)                                                    \
+    do {                                                                          \
+        if (nv.form == 2) CALL((KERNEL<2, false>));                               \
+        else if (nv.form == 1 && a.sub) CALL((KERNEL<1, true>));                  \
+        else if (nv.form == 1) CALL((KERNEL<1, false>));                          \
+        else if (a.sub) CALL((KERNEL<0, true>));                                  \
+        else CALL((KERNEL<0, false>));                                            \
+    } while (0)
+
 }  // namespace
 }  // namespace efm

@@ -249,16 +249,6 @@ int grid_of(K kernel, int sm_count)
         }                                                                         \
     } while (0)
 
-// the same for a kernel without first-K rules
-#define EFM_FORM(KERNEL, CALL)                                                    \
-    do {                                                                          \
-        if (nv.form == 2) CALL((KERNEL<2, false>));                               \
-        else if (nv.form == 1 && a.sub) CALL((KERNEL<1, true>));                  \
-        else if (nv.form == 1) CALL((KERNEL<1, false>));                          \
-        else if (a.sub) CALL((KERNEL<0, true>));                                  \
-        else CALL((KERNEL<0, false>));                                            \
-    } while (0)
-
 }  // namespace
 
 int generate_grid(const NetView &nv, bool sub, bool first_k, int sm_count)

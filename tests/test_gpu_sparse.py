@@ -162,3 +162,17 @@ def test_rank_rows(oracle_lib, efm, steps, sides):
     net = ladder(steps, sides)
     out = check(oracle_lib, efm, net, net.targets, min(64, steps + 2), 2, 1 << 12)
     assert out[0]["results"] >= 4
+
+
+@pytest.mark.parametrize("budget", [1, 30, 500, 1024, 1025, 3000])
+def test_small_levels(oracle_lib, efm, budget):
+    # searches that end, are cut or are capped at levels of one CTA and just
+    # past them, from few seeds and from many
+    for net in (synth.core(), edge_network("list"), synth.batched_member(3)):
+        check(oracle_lib, efm, net, [net.targets[0], -1], min(12, net.split_columns()), 2, budget)
+    net = edge_network("bits")
+    with efm.Network(net) as nw:
+        for cap in (1, 3):
+            (sup, ctr), = efm.enumerate_targets(nw, [net.targets[0]], 12, 2, cap, budget)
+            osup, octr = oracle_lib.enumerate_pathways(net, net.targets[0], oracle_lib.Limits(12, 2, cap, budget))
+            assert np.array_equal(sup, osup) and ctr == octr, (cap, ctr, octr)
