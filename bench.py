@@ -47,7 +47,7 @@ def workload_config(budget):
         "workload": "core-72x95 (58 internal, 114 split columns), 8 target externals",
         "max_len": MAX_LEN, "max_secondary": MAX_SEC, "max_frontier": budget,
         "support_bits": 128, "balance": "int32 x 58",
-        "l2": "frontier arenas far exceed L2 (up to 2^26 states x 276 B); L2 also flushed between steps",
+        "l2": "frontier arenas far exceed L2 (up to 2^26 states of about 100 B); L2 also flushed between steps",
         "parallelism": "replicas",
     }
 
@@ -117,8 +117,8 @@ def profile_figure(name, key):
 
 
 def profile_traffic(alg_bytes_per_launch):
-    """Per-launch DRAM traffic of the core network's level pass (generate,
-    settle and dedup kernels of one expansion launch): the DRAM-to-algorithmic
+    """Per-launch DRAM traffic of the core network's level pass (generate
+    and dedup kernels of one expansion launch): the DRAM-to-algorithmic
     ratio ncu measured on a smaller case of the same kernels (traffic grows
     with the states read and written), applied to this run's algorithmic
     bytes per launch; None without a summary for the current source."""
@@ -378,7 +378,7 @@ def run_ours(args):
         "expansions_per_step": tot_exp / args.steps / max(ws, 1),
         "results_per_step": tot_res / args.steps / max(ws, 1),
         "roofline": {
-            "kernel": "level pass: generate_narrow_kernel<8> + prune_rows_kernel + write_rows_kernel<8,2> + settle_kernel<8> + dedup_kernel",
+            "kernel": "level pass: generate_kernel<2,0,0> + dedup_kernel<2,0> + accept_kernel",
             "bound": "hbm",
             "achieved": achieved,
             "peak": float(peaks["hbm_gbs"]),
@@ -499,7 +499,7 @@ def run_genome(args):
         "config": {"workload": f"genome-1000x2500 (850 internal, 3125 split columns), {n_t} targets",
                    "max_len": 40, "max_secondary": MAX_SEC, "max_frontier": budget, "support_bits": 3136},
         "balanced_pathways_per_s": res / (tot_ms * 1e-3),
-        "roofline": {"kernel": "level pass: generate_kernel<32,7> + dedup_kernel", "bound": "hbm", "achieved": achieved,
+        "roofline": {"kernel": "level pass: generate_kernel<0,0,0> + dedup_kernel<0,0> + accept_kernel", "bound": "hbm", "achieved": achieved,
                      "peak": float(peaks["hbm_gbs"]), "unit": "GB/s", "frac": achieved / float(peaks["hbm_gbs"]),
                      "traffic": traffic, "peak_kind": f"{kind} HBM copy bandwidth", "launches": el,
                      "avg_launch_ms": ems / max(el, 1), "alg_bytes_per_launch": eb / max(el, 1)},
