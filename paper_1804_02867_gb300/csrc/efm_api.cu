@@ -827,7 +827,8 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         }
         const int64_t n_rows = (int64_t)hs[S_NROWS];
         const uint64_t par_deg = hs[S_DEG];
-        if (trace) {
+        const bool again = reruns > 0;  // the same parents as before, into a larger child arena
+        if (trace && !again) {
             // training rows: a strided sample of this frontier, through the
             // list of its surviving rows
             unsigned long long n_live = 0;
@@ -864,7 +865,8 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             chunk = std::max<int64_t>(kFirstKChunkMin, (n_rows + kFirstKChunks - 1) / kFirstKChunks);
             if (model && lim.proposal == EFM_LEARNED && n_rows > chunk) {
                 // the model's order: features of every parent, scores, and a
-                // counting sort by score (highest first)
+                // counting sort by score (highest first); it stands when the
+                // level is run again
                 const int64_t rows = (n_rows + kMlpTileRows - 1) / kMlpTileRows * kMlpTileRows;
                 if (rows > w.lx_rows) {
                     dev_free(w.lx, s);
@@ -885,14 +887,16 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                     CK(cudaMemsetAsync(w.lerr.p, 0, 4, s));
                 }
                 if ((rc = ensure_dep_tags(net))) return rc;
-                CK(launch_features(nv, arena(cur), nullptr, 0, 1, n_rows, level, lim.max_len, lim.max_secondary,
-                                   (const uint64_t *)net->dep.p, w.lx.p, 0, s));
-                CK(launch_mlp_score(w.lx.p, n_rows, model->wb.p, (const float *)model->params.p,
-                                    (float *)w.lscore.p, (unsigned *)w.lerr.p, s));
-                CK(launch_score_order((const float *)w.lscore.p, n_rows, nullptr, (unsigned *)w.lhist.p,
-                                      (uint32_t *)w.perm.p, s));
+                if (!again) {
+                    CK(launch_features(nv, arena(cur), nullptr, 0, 1, n_rows, level, lim.max_len, lim.max_secondary,
+                                       (const uint64_t *)net->dep.p, w.lx.p, 0, s));
+                    CK(launch_mlp_score(w.lx.p, n_rows, model->wb.p, (const float *)model->params.p,
+                                        (float *)w.lscore.p, (unsigned *)w.lerr.p, s));
+                    CK(launch_score_order((const float *)w.lscore.p, n_rows, nullptr, (unsigned *)w.lhist.p,
+                                          (uint32_t *)w.perm.p, s));
+                    out.kernel_launches += 6;
+                }
                 order = (const uint32_t *)w.perm.p;
-                out.kernel_launches += 6;
             }
         }
         a.par = ext ? fs->par : arena(cur);
