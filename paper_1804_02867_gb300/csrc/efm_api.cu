@@ -332,8 +332,11 @@ extern "C" void efm_free_net(efm_net *net)
 
 namespace {
 
-// Device buffers of one traversal, reused across the targets of a job.
+// Device buffers of one traversal, reused across the targets of a job, and the
+// stream they belong to: the traversal runs on it (in a batch that is the first
+// network's stream, whatever stream the searched network was loaded on).
 struct Work {
+    cudaStream_t stream = nullptr;
     DevBuf hdr[2], pay[2];  // arenas: headers, payload pools
     uint64_t pay_cap[2] = {0, 0};
     DevBuf live;                   // training traces: the surviving rows of a frontier
@@ -420,6 +423,7 @@ int alloc_work(Work &w, const efm_net *net, const efm_limits &lim, int total_war
 {
     const NetView &nv = view_of(net, lim);
     const int64_t default_cap = (int64_t)1 << 22;
+    w.stream = s;
     // a level writes a row for every surviving child before deduplication,
     // so an arena gets room for a budget-sized frontier plus duplicates; a
     // level that needs more (rows, or payload units) is run again with a
@@ -556,7 +560,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                int split_depth = 0)
 {
     const NetView &nv = view_of(net, lim);
-    cudaStream_t s = net->stream;
+    cudaStream_t s = w.stream;
     const int full_grid = level_grid(nv, lim, net->sm_count);
     unsigned long long *ctr = (unsigned long long *)w.ctr.p, *st = ctr + C_COUNT;
     unsigned long long h[C_COUNT + S_COUNT];
@@ -1091,7 +1095,7 @@ int run_first_k(efm_net *net, Work &w, const efm_limits &lim, int target, Target
         const int rc = run_target(net, w, l2, target, o, model, nullptr, seedset, n_seedset, nullptr, nullptr,
                                   kFirstKSplitDepth);
         if (rc) {
-            dev_free(o.sup, net->stream);
+            dev_free(o.sup, w.stream);
             return rc;
         }
         total_ms += o.total_ms;
@@ -1109,7 +1113,7 @@ int run_first_k(efm_net *net, Work &w, const efm_limits &lim, int target, Target
             if (depth) *depth = l2.max_len;
             return EFM_OK;
         }
-        dev_free(o.sup, net->stream);
+        dev_free(o.sup, w.stream);
     }
 }
 
@@ -1777,6 +1781,10 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
         if (e == EFM_ENOMEM || e == EFM_ECUDA) {
             rc = e;
             goto done;
+        }
+        if (e != EFM_OK) {  // as a job that fails in the launch: an error, no rows and no flags
+            dev_free(o.sup, s);
+            o = TargetOut{};
         }
         o.err = e;
         o.total_ms = ms;

@@ -141,3 +141,68 @@ def test_batch_rejects_wider_rows(efm):
     with pytest.raises(efm.EfmError) as e:
         _batch(efm, [synth.tiny(0), wide], 20, 2, 2**10)
     assert e.value.code == -6
+
+
+def two_ladders(alts, long_alts=3, long_steps=4):
+    """Many short pathways (alts^2 through two rungs) and a longer ladder whose
+    levels go on after them, to one target."""
+    n_int = 3 + long_steps + 1
+    source, target = n_int, n_int + 1
+    rxn, at = [], 0
+    for n_alts, steps in ((alts, 2), (long_alts, long_steps)):
+        rxn.append({source: -1, at: 1})
+        for i in range(steps):
+            rxn += [{at + i: -1 - q, at + i + 1: 1 + q} for q in range(n_alts)]
+        rxn.append({at + steps: -1, target: 1})
+        at += steps + 1
+    S = np.zeros((n_int + 2, len(rxn)), dtype=np.int64)
+    for j, ents in enumerate(rxn):
+        for m, v in ents.items():
+            S[m, j] = v
+    return synth.Network.from_dense(S, [0] * len(rxn), [0] * n_int + [1, 1], [target], f"two-ladders-{alts}")
+
+
+def test_batch_runs_on_one_stream(efm, capfd, monkeypatch):
+    """Networks loaded on three streams; one job has more results than a
+    job's index holds and is run by itself after the launch.  Every buffer of
+    the call belongs to the first network's stream, and the answers are those
+    of single calls."""
+    import ctypes
+
+    import torch
+
+    lib = efm.load_library()
+    seen = set()
+
+    def alloc(nbytes, stream, ctx):
+        seen.add(int(stream or 0))
+        return torch.cuda.caching_allocator_alloc(int(nbytes), 0, int(stream or 0))
+
+    def free(ptr, nbytes, stream, ctx):
+        seen.add(int(stream or 0))
+        torch.cuda.caching_allocator_delete(int(ptr))
+
+    a, f = efm._ALLOC_T(alloc), efm._FREE_T(free)
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    nets = [synth.batched_member(2), two_ladders(46), synth.batched_member(5)]
+    monkeypatch.setenv("EFM_DEBUG", "1")
+    loaded = []
+    assert lib.efm_set_allocator(ctypes.cast(a, ctypes.c_void_p), ctypes.cast(f, ctypes.c_void_p), None) == 0
+    try:
+        loaded = [efm.Network(n, s) for n, s in zip(nets, streams)]
+        seen.clear()
+        capfd.readouterr()
+        job, _ = efm.efm_find_pathways_batch([w.handle for w in loaded], [n.targets[0] for n in nets], 12, 1, 0, 1 << 12)
+        try:
+            got = [efm.efm_fetch_results(job, i) for i in range(3)]
+        finally:
+            efm.efm_free_job(job)
+        assert "1 jobs of the batch run alone" in capfd.readouterr().err
+        assert seen == {int(streams[0].cuda_stream)}
+        for n, w, (sup, ctr, _) in zip(nets, loaded, got):
+            (ssup, sctr), = efm.enumerate_targets(w, [n.targets[0]], min(12, w.n_columns), 1, 0, 1 << 12)
+            assert np.array_equal(sup, ssup) and ctr == sctr, n.name
+    finally:
+        for w in loaded:
+            w.close()
+        assert lib.efm_set_allocator(None, None, None) == 0
