@@ -59,20 +59,28 @@ struct PoolApi {
     Pool create()
     {
         int dev = 0;
+        size_t free_bytes = 0, total = 0;
         Pool pool = nullptr;
         cudaMemPoolProps props{};
-        if (cudaGetDevice(&dev) == cudaSuccess) {
+        if (cudaGetDevice(&dev) == cudaSuccess && cudaMemGetInfo(&free_bytes, &total) == cudaSuccess) {
             props.allocType = cudaMemAllocationTypePinned;
             props.location.type = cudaMemLocationTypeDevice;
             props.location.id = dev;
             if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
-                uint64_t keep = ~0ull;
+                uint64_t keep = (uint64_t)total / 8;
                 cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
                 return pool;
             }
         }
         cudaGetLastError();
         return nullptr;
+    }
+    void trim(Pool pool)
+    {
+        uint64_t keep = 0;  // (cudaMemGetInfo takes 25 us, a hundredth of a small query)
+        if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
+            cudaMemPoolTrimTo(pool, (size_t)(keep / 4)) != cudaSuccess)
+            cudaGetLastError();
     }
 };
 
@@ -139,6 +147,7 @@ struct efm_net {
     DevBuf blob_sub;
     bool has_sub = false;
     int sm_count = 0;
+    uint64_t pool_ctx = 0;  // the context it keeps the work pool of
     DevBuf dep;             // DEPTHy tags (dep_out | dep_in) per internal metabolite, for the model's features
     bool dep_ready = false;
 };
@@ -312,6 +321,7 @@ extern "C" int efm_load_network(int32_t n_met, int32_t n_rxn, const int32_t *row
         vs.form = vs.W <= 2 ? 1 : 0;
         net->has_sub = true;
     }
+    net->pool_ctx = g_pools.retain();
     *out = net;
     return EFM_OK;
 }
@@ -345,6 +355,7 @@ extern "C" void efm_free_net(efm_net *net)
     dev_free(net->metent, s);
     dev_free(net->dep, s);
     cudaStreamSynchronize(s);
+    g_pools.release(net->pool_ctx);
     delete net;
 }
 
