@@ -899,9 +899,10 @@ __device__ __forceinline__ void generate_range(const NetView &nv, const LevelArg
             if (__any_sync(FULL, fatal)) break;
             // pull the next chunk's payloads toward L2 (its headers
             // have arrived by the last round of this one)
+            // (the second line of a payload may lie past the pool's end)
             if (base + 32 >= T && meta_n != 0u) {
                 prefetch_l2(a.par.pay + off_n);
-                prefetch_l2(a.par.pay + off_n + 6);
+                if ((uint64_t)off_n + 6 < a.par.pay_cap) prefetch_l2(a.par.pay + off_n + 6);
             }
             // --- branch selection: one (parent, branch) item per lane ---
             const int c = base + lane;
