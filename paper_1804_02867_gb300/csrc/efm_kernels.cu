@@ -224,7 +224,8 @@ __global__ void __launch_bounds__(kWalkWarps * 32) walk_narrow_kernel(const __gr
     const int tb = target >= 0 ? nv.metptr[target] : 0, te = target >= 0 ? nv.metptr[target + 1] : 0;
     int n_seeds = target >= 0 ? 0 : nv.N;
     for (int q = tb; q < te; ++q) n_seeds += ent_coef(nv.metent[q]) > 0 ? 1 : 0;
-    unsigned n_walk = 0, n_exp = 0, n_ovf = 0, n_bal = 0, n_dead = 0, max_steps = 0;
+    unsigned long long n_walk = 0, n_exp = 0, n_ovf = 0, n_bal = 0, n_dead = 0;  // (walks have no upper bound)
+    unsigned max_steps = 0;
     const int64_t total = (int64_t)gridDim.x * blockDim.x;
     int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool running = false;
@@ -371,9 +372,10 @@ __global__ void __launch_bounds__(kWalkWarps * 32) walk_narrow_kernel(const __gr
             w += total;
         }
     }
-    auto total_of = [&](unsigned v, int id) {
-        const unsigned t = __reduce_add_sync(FULL, v);  // (a lane's walks and steps are far below 2^27)
-        if (lane == 0 && t) atomicAdd(&a.ctr[id], (unsigned long long)t);
+    auto total_of = [&](unsigned long long v, int id) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(FULL, v, off);
+        if (lane == 0 && v) atomicAdd(&a.ctr[id], v);
     };
     total_of(n_walk, C_SEEDS);
     total_of(n_exp, C_EXP);
