@@ -1407,7 +1407,8 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(const __grid_co
 cudaError_t launch_accept_new(const NetView &nv, const AcceptArgs &a, int sm_count, cudaStream_t s)
 {
     const size_t sm = (size_t)kAcceptWarps * kAcceptWarpWords * 4;
-    cudaFuncSetAttribute(accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = cudaFuncSetAttribute(accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
     accept_kernel<<<sm_count, kAcceptWarps * 32, sm, s>>>(nv, a);
     return cudaGetLastError();
 }
@@ -1417,11 +1418,9 @@ cudaError_t launch_accept(const NetView &nv, const AcceptArgs &a, cudaStream_t s
     const int64_t n = a.cand_end - a.cand_begin;
     if (n <= 0) return cudaSuccess;
     const size_t sm = (size_t)kAcceptWarps * kAcceptWarpWords * 4;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaFuncSetAttribute(accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        attr_set = true;
-    }
+    // (each time: the attribute belongs to the device, and to its context)
+    const cudaError_t e = cudaFuncSetAttribute(accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
     int64_t blocks = (n + kAcceptWarps - 1) / kAcceptWarps;
     if (blocks > 4096) blocks = 4096;
     accept_kernel<<<(int)blocks, kAcceptWarps * 32, sm, s>>>(nv, a);

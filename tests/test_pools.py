@@ -102,7 +102,8 @@ from paper_1804_02867_gb300 import efmgraph, synth
 net = synth.core()
 def run():
     w = efmgraph.Network(net, 0)
-    return w, efmgraph.enumerate_targets(w, net.targets[:2], 20, 2, 0, 1 << 14)
+    sampled = efmgraph.sample_target(w, net.targets[4], 20, 2, 7, 1 << 12)  # before any traversal
+    return w, [sampled] + efmgraph.enumerate_targets(w, net.targets[:2], 20, 2, 0, 1 << 14)
 w, want = run()
 cu, dev = ctypes.CDLL("libcuda.so.1"), ctypes.c_int()
 assert cu.cuInit(0) == 0 and cu.cuDeviceGet(ctypes.byref(dev), 0) == 0
@@ -110,6 +111,7 @@ assert cu.cuDevicePrimaryCtxReset(dev) == 0  # this process's own context; nothi
 for _ in range(2):
     w, got = run()
     w.close()
+    assert len(want[0][0]) > 0  # the walks' minimality test ran
     assert all(np.array_equal(a[0], b[0]) and a[1] == b[1] for a, b in zip(want, got))
 print("same")
 """
