@@ -224,8 +224,8 @@ __global__ void __launch_bounds__(kWalkWarps * 32) walk_narrow_kernel(const __gr
     const int tb = target >= 0 ? nv.metptr[target] : 0, te = target >= 0 ? nv.metptr[target + 1] : 0;
     int n_seeds = target >= 0 ? 0 : nv.N;
     for (int q = tb; q < te; ++q) n_seeds += ent_coef(nv.metent[q]) > 0 ? 1 : 0;
-    unsigned long long n_walk = 0, n_exp = 0, n_ovf = 0, n_bal = 0, n_dead = 0;  // (walks have no upper bound)
-    unsigned max_steps = 0;
+    // (64-bit counters in the lanes cost 1.6 %: a lane adds 32-bit ones up before they wrap)
+    unsigned n_walk = 0, n_exp = 0, n_ovf = 0, n_bal = 0, n_dead = 0, max_steps = 0;
     const int64_t total = (int64_t)gridDim.x * blockDim.x;
     int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool running = false;
@@ -370,6 +370,14 @@ __global__ void __launch_bounds__(kWalkWarps * 32) walk_narrow_kernel(const __gr
         if (ended) {
             running = false;
             w += total;
+            if ((n_walk | n_exp) >> 31) {
+                atomicAdd(&a.ctr[C_SEEDS], (unsigned long long)n_walk);
+                atomicAdd(&a.ctr[C_EXP], (unsigned long long)n_exp);
+                atomicAdd(&a.ctr[C_OVF], (unsigned long long)n_ovf);
+                atomicAdd(&a.ctr[C_BAL], (unsigned long long)n_bal);
+                atomicAdd(&a.ctr[C_PRUNED], (unsigned long long)n_dead);
+                n_walk = n_exp = n_ovf = n_bal = n_dead = 0;
+            }
         }
     }
     auto total_of = [&](unsigned long long v, int id) {
