@@ -306,17 +306,18 @@ int efm_fetch_results(efm_job *job, int32_t job_target_idx, uint64_t *supports, 
 /* Measurements of one target's traversal, for the benchmark's roofline:
  *  total_ms          device time of the whole traversal (CUDA events on the
  *                    network's stream, seeds to sorted results)
- *  expand_ms         summed device time of the expansion launches: the
- *                    generate kernel and the passes that finish its level
- *                    (prune, row, settle and dedup passes), event to event
- *  expand_launches   number of expansion launches (one per level, or per
- *                    chunk of a first-K level)
+ *  expand_ms         summed device time of the expansion launches, event to
+ *                    event: each level's generate and dedup passes, its
+ *                    minimality test and the clearing of its state table
+ *  expand_launches   number of expansion launches: one per level (also where
+ *                    one kernel runs several small ones), per chunk of a
+ *                    first-K level, and again for a level that ran again with
+ *                    a larger work area
  *  expand_bytes      algorithmic bytes those launches must move: each parent
  *                    state read once, each new distinct state written once
- *                    (state = 8 W + 4 M + 4 bytes; beyond 64 internal
- *                    metabolites a header and the payload of its columns and
- *                    unbalanced entries), 16 bytes of hash slot traffic per
- *                    child
+ *                    (state = a 16-byte header and the 16-byte units that its
+ *                    columns and unbalanced entries take), 16 bytes of hash
+ *                    slot traffic per child
  *  kernel_launches   every kernel this library launched for the target
  * Any output pointer may be NULL. */
 int efm_job_timing(const efm_job *job, int32_t job_target_idx, double *total_ms, double *expand_ms,

@@ -573,6 +573,7 @@ struct FrontierStart {
     int64_t r0, r1;
     int level;
     uint64_t deg_sum;
+    uint64_t units;  // payload units of their states, about
 };
 
 // split_depth (first-K only): a level over the frontier budget does not end
@@ -734,6 +735,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         x[S_LEVEL] = (unsigned long long)level0;
         x[S_NROWS] = x[S_NFRONT] = (unsigned long long)n;
         x[S_DEG] = fs->deg_sum;
+        x[S_UNITS] = fs->units;
         x[S_RESERVED] = fs->deg_sum + 64;
         x[S_SLOTS] = next_pow2(2 * x[S_RESERVED] + 64);
         if (lim.max_frontier > 0 && n > lim.max_frontier) {
@@ -820,7 +822,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                     return EFM_ENOMEM;
                 const int back[] = {C_EXP, C_OVF, C_BAL, C_PRUNED, C_ZERO};
                 for (int i = 0; i < 5; ++i) h[back[i]] = hs[S_SNAP + i];
-                const int clear[] = {C_NEXT, C_DEGSUM, C_WRITTEN, C_UNWRITTEN, C_UNV, C_PAY, C_DEDUP_BEGIN, C_OPEN};
+                const int clear[] = {C_NEXT, C_DEGSUM, C_WRITTEN, C_UNWRITTEN, C_UNV, C_PAY, C_KEPT, C_DEDUP_BEGIN, C_OPEN};
                 for (int i : clear) h[i] = 0;
                 h[C_COUNT + S_STOP] = STOP_NONE;
                 CK(cudaMemcpyAsync(ctr, h, sizeof(h), cudaMemcpyHostToDevice, s));
@@ -859,7 +861,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             continue;
         }
         const int64_t n_rows = (int64_t)hs[S_NROWS];
-        const uint64_t par_deg = hs[S_DEG];
+        const uint64_t par_deg = hs[S_DEG], par_units = hs[S_UNITS];
         const bool again = reruns > 0;  // the same parents as before, into a larger child arena
         if (trace && !again) {
             // training rows: a strided sample of this frontier, through the
@@ -1000,7 +1002,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             const int64_t par0 = ext ? fs->r0 : 0;
             for (int64_t p = 0; rc2 == EFM_OK && p < parts; ++p) {
                 FrontierStart sub{par_arena, par0 + n_rows * p / parts, par0 + n_rows * (p + 1) / parts, level - 1,
-                                  par_deg};
+                                  par_deg, par_units / (uint64_t)parts};
                 if (sub.r1 <= sub.r0) continue;
                 TargetOut so;
                 const std::vector<uint64_t> known_top = top.rows;
@@ -1423,7 +1425,7 @@ extern "C" int efm_sample_pathways(efm_net *net, int32_t target, const efm_limit
     cudaEventElapsedTime(&ms, w.ev[0], w.ev[2]);
     o.expand_ms = ms;  // the walk kernel
     o.expand_launches = n_walks > 0 ? 1 : 0;
-    o.kernel_launches = 2 + (res_n > 0 ? 2 : 0);
+    o.kernel_launches = (n_walks > 0 ? 1 : 0) + (h[C_CAND_N] > 0 ? 1 : 0) + (res_n > 0 ? sort_launches((int64_t)n2) : 0);
     o.n = res_n;
     efm_counters &c = o.ctr;
     memset(&c, 0, sizeof(c));

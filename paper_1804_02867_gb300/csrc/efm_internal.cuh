@@ -51,7 +51,8 @@ enum {
     C_ZERO = 28,  // subtractive steps discarded: no positive flux left on the reaction (Prop. 3)
     C_OPEN,       // open children listed by the generate pass, not yet finished
     C_LIVE,       // surviving rows counted by the live-list pass
-    C_PAY = 32,   // sparse states: payload units reserved so far in the level
+    C_PAY = 32,   // payload units reserved so far in the level
+    C_KEPT,       // payload units that its distinct states take
     C_COUNT = 40
 };
 
@@ -65,7 +66,7 @@ enum {
     S_NROWS,      // its arena rows (the next level's parents)
     S_NFRONT,     // its distinct states
     S_DEG,        // sum of their branch counts
-    S_UNITS,      // payload units of its rows
+    S_UNITS,      // payload units of its distinct states
     S_SLOTS,      // next level: slots of the state table (a power of two)
     S_RESERVED,   // next level: rows that may be reserved
     S_BLK,        // next level: rows a warp reserves at a time
@@ -73,7 +74,7 @@ enum {
     S_FRONTIER,   // sum and largest of the levels' distinct states
     S_FRONTIER_MAX,
     S_BYTES,      // algorithmic bytes of the expansions so far
-    S_EXPANDS,    // levels expanded
+    S_EXPANDS,    // expansion launches: levels, chunks of a first-K level and levels run again
     S_TICKET,     // CTAs of the running minimality launch that are done
     S_SNAP,       // C_EXP, C_OVF, C_BAL, C_PRUNED, C_ZERO when the running level began
     S_COUNT = S_SNAP + 8

@@ -817,11 +817,17 @@ __device__ void advance_level(const AcceptArgs &a, const unsigned long long *v)
     unsigned long long *c = a.ctr, *st = a.st;
     const unsigned long long *sv = v + C_COUNT;
     auto get = [&](int i) { return v[i]; };
-    if (a.advance == 1) return;
     const bool seeds = a.advance == 3;
+    if (!seeds) st[S_EXPANDS] = sv[S_EXPANDS] + 1;
+    if (a.advance == 1) return;
     const uint64_t next = get(C_NEXT), unv = get(C_UNV), written = seeds ? next : get(C_WRITTEN);
     const uint64_t deg = get(C_DEGSUM), units = get(C_PAY), unwritten = get(C_UNWRITTEN);
     const uint64_t front = next + (unwritten ? unv : 0ull);
+    const uint64_t kept = seeds ? units : get(C_KEPT);  // (seeds take what they reserve)
+    // algorithmic bytes: the header and payload of every distinct parent and
+    // new state, 16 bytes of slot traffic per child
+    if (!seeds)
+        st[S_BYTES] = sv[S_BYTES] + 16 * (sv[S_NFRONT] + sv[S_UNITS] + next + kept + (get(C_EXP) - sv[S_SNAP]));
     unsigned long long stop = STOP_NONE;
     if (get(C_ERR)) {
         stop = STOP_ERROR;
@@ -834,20 +840,11 @@ __device__ void advance_level(const AcceptArgs &a, const unsigned long long *v)
         st[S_STOP] = STOP_RERUN;  // the counters stay as they are for the host
         return;
     }
-    if (!seeds) {
-        // algorithmic bytes: a header and the payload units of an average row,
-        // per distinct parent and new state; 16 bytes of slot traffic per child
-        const uint64_t prow = sv[S_NROWS], pfront = sv[S_NFRONT];
-        st[S_BYTES] = sv[S_BYTES] + 16 * (pfront + next) + (prow ? 16 * (uint64_t)((double)sv[S_UNITS] * pfront / prow) : 0ull) +
-                       (written ? 16 * (uint64_t)((double)units * next / written) : 0ull) +
-                       16 * (get(C_EXP) - sv[S_SNAP]);
-        st[S_EXPANDS] = sv[S_EXPANDS] + 1;
-    }
     st[S_LEVEL] = (unsigned long long)a.level;
     st[S_NROWS] = written < (uint64_t)a.child_rows ? written : (uint64_t)a.child_rows;
     st[S_NFRONT] = front;
     st[S_DEG] = deg;
-    st[S_UNITS] = units;
+    st[S_UNITS] = kept;
     if (stop == STOP_NONE) {
         st[S_FRONTIER] = sv[S_FRONTIER] + front;
         if (front > sv[S_FRONTIER_MAX]) st[S_FRONTIER_MAX] = front;
@@ -874,9 +871,9 @@ __device__ void advance_level(const AcceptArgs &a, const unsigned long long *v)
     for (int i = 0; i < 5; ++i) st[S_SNAP + i] = get(snap[i]);
     if (stop == STOP_NONE && (int64_t)get(C_RES_N) > a.ix.room) stop = STOP_INDEX;
     if (stop == STOP_NONE && ((int64_t)reserved > a.fp_cap || slots > a.slot_cap)) stop = STOP_TABLES;
-    const int clear[] = {C_NEXT, C_DEGSUM, C_WRITTEN, C_UNWRITTEN, C_UNV, C_PAY, C_DEDUP_BEGIN};
+    const int clear[] = {C_NEXT, C_DEGSUM, C_WRITTEN, C_UNWRITTEN, C_UNV, C_PAY, C_KEPT, C_DEDUP_BEGIN};
     if (stop == STOP_NONE || stop == STOP_INDEX || stop == STOP_TABLES)
-        for (int i = 0; i < 7; ++i) c[clear[i]] = 0ull;
+        for (int i = 0; i < 8; ++i) c[clear[i]] = 0ull;
     st[S_STOP] = stop;
 }
 
@@ -1240,7 +1237,7 @@ __device__ void run_job(const BatchArgs &ba, const BatchJob &job, char *slice, u
         dedup_range<F, false>(nv, a, nslots - 1, __ldcg(&ctr[C_DEDUP_BEGIN]), __ldcg(&ctr[C_WRITTEN]),
                               __ldcg(&ctr[C_OPEN]), tid & ~31, tid & ~31, nthreads, sum);
         unsigned keep = __reduce_add_sync(FULL, sum.keep), unv = __reduce_add_sync(FULL, sum.unv);
-        unsigned deg = __reduce_add_sync(FULL, (unsigned)sum.deg);  // (far below 2^32 in a slice)
+        unsigned deg = __reduce_add_sync(FULL, (unsigned)sum.deg_units);  // (far below 2^32 in a slice)
         if (lane == 0) {
             if (keep) atomicAdd(&ctr[C_NEXT], (unsigned long long)keep);
             if (unv) atomicAdd(&ctr[C_UNV], (unsigned long long)unv);
@@ -1343,10 +1340,12 @@ __global__ void __launch_bounds__(kSmallWarps * 32, 1) small_kernel(const __grid
         dedup_range<F, SUB>(nv, a, slots - 1, v[C_DEDUP_BEGIN], v[C_WRITTEN], v[C_OPEN], tid & ~31, tid & ~31, nthreads,
                             sum);
         const unsigned keep = __reduce_add_sync(FULL, sum.keep), unv = __reduce_add_sync(FULL, sum.unv);
-        const unsigned deg = __reduce_add_sync(FULL, (unsigned)sum.deg);  // (limit children of at most 2^13 branches)
+        const unsigned units = __reduce_add_sync(FULL, (unsigned)(sum.deg_units >> 32));
+        const unsigned deg = __reduce_add_sync(FULL, (unsigned)sum.deg_units);  // (limit children of at most 2^13 branches)
         if (lane == 0) {
             if (keep) atomicAdd(&a.ctr[C_NEXT], (unsigned long long)keep);
             if (unv) atomicAdd(&a.ctr[C_UNV], (unsigned long long)unv);
+            if (units) atomicAdd(&a.ctr[C_KEPT], (unsigned long long)units);
             if (deg) atomicAdd(&a.ctr[C_DEGSUM], (unsigned long long)deg);
         }
         read_state();

@@ -1261,7 +1261,9 @@ __device__ __noinline__ uint64_t finish_open(const NetView &nv, const LevelArgs 
 
 struct DedupSums {
     unsigned keep = 0, unv = 0;
-    unsigned long long deg = 0;
+    // the kept states' branches, and their payload units << 32: a lane takes at
+    // most 2^32 / (1216 CTAs x 256) rows of 8191 branches, a warp's sum fits 32 bits
+    unsigned long long deg_units = 0;
 };
 
 // Insert a warp's rows (lane: row i, fingerprint f, kDeadFp for none, header
@@ -1288,7 +1290,8 @@ __device__ __forceinline__ void dedup_insert(const LevelArgs &a, uint64_t mask, 
             if (v == kEmpty) {  // first of its state
                 if (written) {
                     ++sum.keep;
-                    sum.deg += (h.y >> 10) & 0x1FFFu;
+                    const int u = support_units<F>((int)((h.y >> 23) & 0x7Fu)) + entry_units<F>((int)(h.z & 0x7FFu));
+                    sum.deg_units += ((h.y >> 10) & 0x1FFFu) | (unsigned long long)u << 32;
                 } else {
                     ++sum.unv;
                 }

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256, 6) dedup_kernel(const __grid_constant__ N
     dedup_range<F, SUB>(nv, a, a.st[S_SLOTS] - 1, a.ctr[C_DEDUP_BEGIN], a.ctr[C_WRITTEN], a.ctr[C_OPEN],
                         (uint64_t)blockIdx.x * blockDim.x + in_cta,
                         stride - blockDim.x - (uint64_t)blockIdx.x * blockDim.x + in_cta, stride, sum);
-    unsigned long long deg = sum.deg, n_unv = sum.unv, n_keep = sum.keep;
+    unsigned long long deg = sum.deg_units, n_unv = sum.unv, n_keep = sum.keep;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         deg += __shfl_xor_sync(FULL, deg, off);
@@ -81,14 +81,16 @@ __global__ void __launch_bounds__(256, 6) dedup_kernel(const __grid_constant__ N
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        unsigned long long k = 0, d = 0, u = 0;
+        unsigned long long k = 0, d = 0, u = 0, p = 0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
             k += s_keep[w];
-            d += s_deg[w];
+            d += (uint32_t)s_deg[w];
+            p += s_deg[w] >> 32;
             u += s_unv[w];
         }
         if (k) atomicAdd(&a.ctr[C_NEXT], k);
         if (d) atomicAdd(&a.ctr[C_DEGSUM], d);
+        if (p) atomicAdd(&a.ctr[C_KEPT], p);
         if (u) atomicAdd(&a.ctr[C_UNV], u);
     }
 }

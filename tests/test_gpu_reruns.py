@@ -105,3 +105,35 @@ def test_trace_takes_a_level_once(efm, capfd, monkeypatch):
         finally:
             efm.efm_model_free(m)
         assert (n, pos) == (want, want), budget  # every state lies inside a pathway
+
+
+@pytest.mark.gpu
+def test_timing_counts_what_ran(efm, capfd, monkeypatch):
+    """expand_launches and expand_bytes of a search whose states are known: 6^l
+    states of 81 entries at level l (43 units and a header each), the children
+    of the last level balanced; with a small budget, levels run again count
+    again; a first-K search counts its chunks."""
+    net = ladders(*RERUN["bits"])
+    state = 16 * (1 + 2 + 41)
+    want = sum(state * (6 ** l + (6 ** (l + 1) if l < 5 else 0)) + 16 * 6 ** min(l + 1, 5) for l in range(6))
+    monkeypatch.setenv("EFM_DEBUG", "1")
+    with efm.Network(net) as nw:
+        (_, _, t), = efm.enumerate_targets(nw, net.targets, 10, 1, 0, 1 << 17, timing=True)
+        assert (t["expand_launches"], t["expand_bytes"]) == (6, want)
+        capfd.readouterr()
+        (_, _, t), = efm.enumerate_targets(nw, net.targets, 10, 1, 0, 8000, timing=True)
+        again = len(re.findall(r"stop 4", capfd.readouterr().err))
+        assert again > 0 and t["expand_launches"] == 6 + again and t["expand_bytes"] > want
+    net = ladders((21, 3, 0))  # 9261 states before the last level: two chunks
+    with efm.Network(net) as nw:
+        capfd.readouterr()
+        (sup, _, t), = efm.enumerate_targets(nw, net.targets, 5, 1, 0, 1 << 15, first_k=21 ** 3, timing=True)
+        err = capfd.readouterr().err
+    assert len(sup) == 21 ** 3
+    lines = len(re.findall(r"efm: level", err))
+    runs = len(re.findall(r"efm: level 0 .* children so far 0 ", err))
+    assert runs == 5 and t["expand_launches"] == lines - runs
+    core = synth.core()
+    with efm.Network(core) as nw:  # walks, minimality test, a sort of two results
+        sup, _, t = efm.sample_target(nw, core.targets[4], 20, 2, 7, 1 << 12, timing=True)
+    assert len(sup) == 2 and t["kernel_launches"] == 1 + 1 + 3
