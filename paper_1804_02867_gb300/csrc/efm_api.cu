@@ -256,6 +256,7 @@ extern "C" int efm_load_network(int32_t n_met, int32_t n_rxn, const int32_t *row
     nv.Mpad = prep.Mpad;
     nv.form = nv.W > 2 ? 0 : (prep.narrow ? 2 : 1);
     nv.n_met = n_met;
+    nv.long_cols = has_long_columns(prep, nv.form == 2 ? kNarrowCol : kListCol, nv.form == 2 ? nv.N : kListMean);
     cudaStream_t s = net->stream;
     int rc = EFM_OK;
     if (!dev_alloc(net->blob, blob.size() * 4, s) || !dev_alloc(net->metptr, mptr.size() * 4, s) ||
@@ -319,6 +320,7 @@ extern "C" int efm_load_network(int32_t n_met, int32_t n_rxn, const int32_t *row
         vs.Mpad = sub.Mpad;
         vs.o_scol = sub.o_scol;
         vs.form = vs.W <= 2 ? 1 : 0;
+        vs.long_cols = has_long_columns(prep, kListCol - 1, kListMean);  // (a flux entry more)
         net->has_sub = true;
     }
     net->pool_ctx = g_pools.retain();

@@ -112,11 +112,28 @@ struct NetView {
     // masks and the values in row order), 1 = bitset support and a list of entries (at most 128
     // columns), 0 = column list and a list of entries
     int form;
+    int long_cols;  // long children are common: see has_long_columns
     int o_rank, o_keyr, o_colx, o_nent;  // narrow: see efm_netprep.h
     const int32_t *metptr;     // full S rows over split columns (seeds), [n_met + 1]
     const uint32_t *metent;    // packed (column, coefficient)
     int n_met;
 };
+
+// Entries that a lane of the generate pass takes at most: of a column (kept in
+// registers on narrow networks), and 64 of a list.  Longer children are left to
+// the dedup pass, a warp each, or, in the instances of the kernels for networks
+// where they are common (any column past the line; or, lists, columns so long
+// that states pass 64 entries within a few levels), taken by a lane all the same.
+// One GB300, dense rows (before sparse states), a lane each in the dedup pass, a
+// warp each there, a lane each in the generate pass: 90 reactions of 10 to 20
+// metabolites on 60 rows at 2^18 3.0, 5.5, 7.5 and 2.4 ms; 500 of 30 to 80 on 300
+// rows 23, 40, 53 and 12; 100 of 20 to 60 on 100 rows 4.6, 11.7, 15.9 and 4.5 (at
+// 2^14, where a level has few children, 1.5, 3.7, 3.2 and 2.1).  On the core-shaped
+// network, whose columns are short, the code for them costs 14 % (spills: 467 and
+// 533 ms at 2^26).  A warp each is right for the rare ones of other networks: a
+// small level waits for one lane's chain (eight core targets at 2^17 7.8 -> 6.7 ms,
+// subtractive 5.8 -> 4.6, a 400-row network 3.8 -> 3.4).
+constexpr int kNarrowCol = 8, kListCol = 32, kListMean = 8;
 
 __host__ __device__ inline int ent_index(uint32_t e) { return (int)(e >> 20); }
 __host__ __device__ inline int32_t ent_coef(uint32_t e) { return ((int32_t)(e << 12)) >> 12; }

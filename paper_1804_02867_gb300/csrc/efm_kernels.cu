@@ -1230,7 +1230,7 @@ __device__ void run_job(const BatchArgs &ba, const BatchJob &job, char *slice, u
         }
         __syncthreads();
         const int cpw = (int)min((int64_t)ba.tile, max((int64_t)1, (n_rows + nwarps - 1) / nwarps));
-        generate_range<F, false, false>(nv, a, n_rows, cpw, 0, 0, res_n > 0, wid, nwarps, nullptr, no_bound);
+        generate_range<F, false, false, true>(nv, a, n_rows, cpw, 0, 0, res_n > 0, wid, nwarps, nullptr, no_bound);
         __syncthreads();
         DedupSums sum;
         // (counters past L1: this SM may hold older ones)
@@ -1334,7 +1334,7 @@ __global__ void __launch_bounds__(kSmallWarps * 32, 1) small_kernel(const __grid
         }
         __syncthreads();
         const int cpw = (int)min((int64_t)32, max((int64_t)1, (n_par + kSmallWarps - 1) / kSmallWarps));
-        generate_range<F, SUB, false>(nv, a, n_par, cpw, 0, 0, any_result, wid, kSmallWarps, nullptr, no_bound);
+        generate_range<F, SUB, false, true>(nv, a, n_par, cpw, 0, 0, any_result, wid, kSmallWarps, nullptr, no_bound);
         read_state();
         DedupSums sum;
         dedup_range<F, SUB>(nv, a, slots - 1, v[C_DEDUP_BEGIN], v[C_WRITTEN], v[C_OPEN], tid & ~31, tid & ~31, nthreads,

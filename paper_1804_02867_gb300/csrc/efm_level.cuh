@@ -274,9 +274,9 @@ struct Child {
     int32_t pv;     // the entry of that key
     uint32_t om;    // OR of the magnitudes
     uint32_t g;     // gcd of the entries (1 as soon as it is known to be 1)
-    uint64_t rh;    // slow_child only
+    uint64_t rh;    // wide_child only
     bool zflux;     // the flux of k is not positive any more (Prop. 3)
-    bool ovf;       // an entry outside int32 after the division (slow_child only)
+    bool ovf;       // an entry outside int32 after the division (wide_child only)
 };
 
 // Column entries: words [cb, ce) of the column CSR, rows ascending; in the
@@ -410,6 +410,64 @@ __device__ __forceinline__ void fast_child(const NetView &nv, const uint32_t *bl
     r.zflux = zflux;
 }
 
+// One child of any number of entries, when every one is known to fit int32
+// (networks whose reactions have dozens of metabolites, where states have as
+// many entries): the coefficients from the dense copy of S_int, the rows that
+// the parent has as bits in local memory, the entries written one after the
+// other.
+template <bool SUB>
+__device__ __noinline__ void long_child(const NetView &nv, const uint32_t *bl, const uint4 *pe, int np, int32_t A,
+                                        int32_t C, int cb, int ce, int k, uint4 *dst, Child &r)
+{
+    const int2 *p2 = reinterpret_cast<const int2 *>(pe);
+    int2 *d2 = reinterpret_cast<int2 *>(dst);
+    const int32_t *col = reinterpret_cast<const int32_t *>(bl + nv.o_dcols) + (size_t)k * nv.Mpad;
+    const int rows = nv.M + (SUB ? nv.N : 0);  // at most EFM_MAX_INTERNAL
+    uint32_t has[EFM_MAX_INTERNAL / 32];
+    for (int w = 0; 32 * w < rows; ++w) has[w] = 0u;
+    uint32_t key = kPadKey, om = 0, g = 0;
+    int32_t pv = 0;
+    bool zflux = false;
+    int n = 0;
+    auto put = [&](uint32_t kk, int32_t t) {
+        const uint32_t at = mag(t);
+        om |= at;
+        if (g != 1u) g = gcd_small(g, at);
+        if (kk < key) {
+            key = kk;
+            pv = t;
+        }
+        if (d2) d2[n] = make_int2((int)kk, t);
+        ++n;
+    };
+    for (int i = 0; i < np; ++i) {
+        const int2 e = p2[i];
+        const int row = e.x & 0xFFFF;
+        const int32_t cv = col[row];
+        has[row >> 5] |= 1u << (row & 31);
+        const int32_t t = A * e.y + C * cv;
+        if (SUB && row == nv.M + k && t <= 0) zflux = true;
+        if (t != 0) put(cv == 0 ? (uint32_t)e.x : entry_key<SUB>(nv, bl, row, t > 0), t);
+    }
+    const int nq = ce - cb + (SUB ? 1 : 0);
+    for (int q = 0; q < nq; ++q) {
+        int row;
+        int32_t cv;
+        column_entry<SUB>(nv, bl, cb, ce, q, k, row, cv);
+        if ((has[row >> 5] >> (row & 31)) & 1u) continue;
+        const int32_t t = C * cv;
+        if (SUB && row >= nv.M && t <= 0) zflux = true;
+        put(entry_key<SUB>(nv, bl, row, t > 0), t);
+    }
+    if (d2 && (n & 1)) d2[n] = make_int2((int)kPadKey, 0);
+    r.n = n;
+    r.key = key;
+    r.pv = pv;
+    r.om = om;
+    r.g = g;
+    r.zflux = zflux;
+}
+
 // --- narrow networks ---
 
 // values below row r in a state with nonzero rows zm
@@ -419,11 +477,11 @@ struct NarrowMasks {
     uint64_t zm, pm, nm;
 };
 
-constexpr int kNarrowCol = 8;  // column entries the fast path keeps in registers
-
-// One child of a narrow network, when every entry is known to fit int32 and
-// the column has at most kNarrowCol entries: the masks follow from the rows of
-// column k alone, the other values are copied (times A) to their places.
+// One child of a narrow network, when every entry is known to fit int32: the
+// masks follow from the rows of column k alone, the other values are copied
+// (times A) to their places.  LONG: a column of more than kNarrowCol entries,
+// whose new values are computed twice instead of kept.
+template <bool LONG = false>
 __device__ __forceinline__ void narrow_child(const NetView &nv, const uint32_t *bl, const uint4 *pp, int32_t A,
                                              int32_t C, int cb, int nc, int k, int32_t *dst, Child &r, NarrowMasks &z)
 {
@@ -432,24 +490,37 @@ __device__ __forceinline__ void narrow_child(const NetView &nv, const uint32_t *
     const int ox = nv.o_colx + 10 * k;
     const uint64_t mask = blob_u64(bl, ox + 4);
     const uint2 *ent = reinterpret_cast<const uint2 *>(bl + nv.o_nent) + cb;
-    int32_t t[kNarrowCol];
+    int32_t t[LONG ? 1 : kNarrowCol];
     uint32_t om = 0, mn = 0xFFFFFFFFu;  // OR of the magnitudes; smallest magnitude less one
     uint64_t newz = 0, newp = 0, newn = 0;
-#pragma unroll
-    for (int q = 0; q < kNarrowCol; ++q) {
-        t[q] = 0;
-        if (q < nc) {
+    auto value = [&](const uint2 &e) -> int32_t {  // the child's, on a row of column k
+        const int row = (int)(e.x & 63u);
+        int32_t v = 0;
+        if ((zm >> row) & 1ull) v = vals[value_at(zm, row)];
+        return A * v + C * (int32_t)e.y;
+    };
+    auto note = [&](const uint2 &e, int32_t x) {
+        newz |= (uint64_t)(x != 0) << (e.x & 63u);
+        newp |= (uint64_t)(x > 0) << ((e.x >> 8) & 63u);
+        newn |= (uint64_t)(x < 0) << ((e.x >> 16) & 63u);
+        const uint32_t a = mag(x);
+        om |= a;
+        mn = min(mn, a - 1u);
+    };
+    if (LONG) {
+        for (int q = 0; q < nc; ++q) {
             const uint2 e = ent[q];
-            const int row = (int)(e.x & 63u);
-            int32_t v = 0;
-            if ((zm >> row) & 1ull) v = vals[value_at(zm, row)];
-            t[q] = A * v + C * (int32_t)e.y;
-            newz |= (uint64_t)(t[q] != 0) << row;
-            newp |= (uint64_t)(t[q] > 0) << ((e.x >> 8) & 63u);
-            newn |= (uint64_t)(t[q] < 0) << ((e.x >> 16) & 63u);
-            const uint32_t a = mag(t[q]);
-            om |= a;
-            mn = min(mn, a - 1u);
+            note(e, value(e));
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < kNarrowCol; ++q) {
+            t[q] = 0;
+            if (q < nc) {
+                const uint2 e = ent[q];
+                t[q] = value(e);
+                note(e, t[q]);
+            }
         }
     }
     const uint64_t keep = zm & ~mask;
@@ -480,16 +551,23 @@ __device__ __forceinline__ void narrow_child(const NetView &nv, const uint32_t *
     if ((om & 1u) && (g & (g - 1u)) == 0u) g = 1u;
     const int piv = (int)(r.key & 63u);
     int32_t pv = 0;
-#pragma unroll
-    for (int q = 0; q < kNarrowCol; ++q) {
-        if (q < nc) {
-            const int row = (int)(ent[q].x & 63u);
-            if (row == piv) pv = t[q];
-            if (t[q] != 0) {
-                if (g != 1u) g = gcd_small(g, mag(t[q]));
-                if (dst) dst[value_at(z.zm, row)] = t[q];
-            }
+    auto place = [&](const uint2 &e, int32_t x) {
+        const int row = (int)(e.x & 63u);
+        if (row == piv) pv = x;
+        if (x != 0) {
+            if (g != 1u) g = gcd_small(g, mag(x));
+            if (dst) dst[value_at(z.zm, row)] = x;
         }
+    };
+    if (LONG) {
+        for (int q = 0; q < nc; ++q) {
+            const uint2 e = ent[q];
+            place(e, value(e));
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < kNarrowCol; ++q)
+            if (q < nc) place(ent[q], t[q]);
     }
     if (g != 1u)
         for (uint64_t x = keep; x && g != 1u; x &= x - 1) g = gcd_small(g, mag(A * vals[value_at(zm, __ffsll((long long)x) - 1)]));
@@ -499,6 +577,12 @@ __device__ __forceinline__ void narrow_child(const NetView &nv, const uint32_t *
     r.zflux = false;
     if (dst)
         for (int i = r.n; i & 3; ++i) dst[i] = 0;
+}
+
+__device__ __noinline__ void narrow_child_long(const NetView &nv, const uint32_t *bl, const uint4 *pp, int32_t A,
+                                               int32_t C, int cb, int nc, int k, int32_t *dst, Child &r, NarrowMasks &z)
+{
+    narrow_child<true>(nv, bl, pp, A, C, cb, nc, k, dst, r, z);
 }
 
 // gcd and exact division of the children below: most are there for a common
@@ -518,64 +602,100 @@ __device__ __forceinline__ int32_t div_any(int64_t t, uint64_t g)
     return (int32_t)(t / (int64_t)g);
 }
 
-// Any child of a narrow network, in 64 bits (see slow_child).
-__device__ __noinline__ void slow_narrow(const NetView &nv, const uint32_t *bl, const uint4 *pp, int32_t A, int32_t C,
-                                         int cb, int ce, int k, int32_t *dst, Child &r, NarrowMasks &z)
+// does x / g leave int32?
+__device__ __forceinline__ bool past_int32(uint64_t x, uint64_t g) { return x > 2147483647ull && x / g > 2147483647ull; }
+
+// gcd over a warp (g: 0 for a lane without an entry).  Mostly small numbers that
+// share a small divisor: Euclid against the smallest, all lanes at once, ends
+// after a step or two.
+__device__ __forceinline__ uint64_t warp_gcd(uint64_t g)
+{
+    if (__any_sync(FULL, (g >> 32) != 0)) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) g = gcd64(g, __shfl_xor_sync(FULL, g, off));
+        return g;
+    }
+    uint32_t x = (uint32_t)g;
+    for (;;) {
+        const uint32_t m = __reduce_min_sync(FULL, x - 1u) + 1u;  // (less one: no entry counts as the largest)
+        if (m == 1u) return 1ull;
+        const uint32_t rest = x % m;
+        if (!__any_sync(FULL, rest != 0u)) return m;
+        x = rest ? rest : (x ? m : 0u);
+    }
+}
+
+__device__ __forceinline__ uint64_t warp_sum(uint64_t x)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(FULL, x, off);
+    return x;
+}
+
+// Any child of a narrow network, in 64 bits, by one warp: lane l holds rows l
+// and l + 32 (see wide_child).
+__device__ __forceinline__ void wide_narrow(const NetView &nv, const uint32_t *bl, const uint4 *pp, int32_t A, int32_t C,
+                                         int cb, int k, int32_t *dst, Child &r, NarrowMasks &z, int lane)
 {
     const uint64_t zm = reinterpret_cast<const uint64_t *>(pp)[1];
     const int32_t *vals = reinterpret_cast<const int32_t *>(pp + 3);
-    const uint2 *ent = reinterpret_cast<const uint2 *>(bl + nv.o_nent);
+    const uint2 *ent = reinterpret_cast<const uint2 *>(bl + nv.o_nent) + cb;
     const uint64_t mask = blob_u64(bl, nv.o_colx + 10 * k + 4);
-    uint64_t g = 0, mx = 0;
+    int64_t t[2];
+    uint64_t g = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int row = lane + 32 * h;
+        t[h] = 0;
+        if ((zm >> row) & 1ull) t[h] = (int64_t)A * vals[value_at(zm, row)];
+        if ((mask >> row) & 1ull) t[h] += (int64_t)C * (int32_t)ent[value_at(mask, row)].y;  // (rows ascend in the column)
+        g = gcd_any(g, abs64(t[h]));
+    }
     r.n = 0;
     r.key = kPadKey;
     r.pv = 0;
     r.om = 0;
     r.rh = 0;
+    r.g = 1;
     r.zflux = r.ovf = false;
     z.zm = z.pm = z.nm = 0;
-    for (int pass = 0; pass < 2; ++pass) {
-        int q = cb;  // rows ascend in the column and in the state
-        for (uint64_t x = zm | mask; x; x &= x - 1) {
-            const int row = __ffsll((long long)x) - 1;
-            int64_t t = 0;
-            if ((zm >> row) & 1ull) t = (int64_t)A * vals[value_at(zm, row)];
-            while (q < ce && (int)(ent[q].x & 63u) < row) ++q;
-            if (q < ce && (int)(ent[q].x & 63u) == row) t += (int64_t)C * (int32_t)ent[q].y;
-            if (t == 0) continue;
-            if (pass == 0) {
-                const uint64_t at = abs64(t);
-                g = gcd_any(g, at);
-                mx = at > mx ? at : mx;
-                continue;
-            }
-            const int32_t v = div_any(t, g);
-            const uint32_t kk = bl[(v > 0 ? nv.o_keypos : nv.o_keyneg) + row];
-            const uint32_t rk = bl[nv.o_rank + row];
-            z.zm |= 1ull << row;
-            if (v > 0) z.pm |= 1ull << (rk & 0xFFu);
-            else z.nm |= 1ull << ((rk >> 8) & 0xFFu);
-            r.om |= mag(v);
-            r.rh += (uint64_t)(int64_t)v * row_hash(row);
-            if (kk < r.key) {
-                r.key = kk;
-                r.pv = v;
-            }
-            if (dst) dst[r.n] = v;
-            ++r.n;
-        }
-        if (pass == 0) {
-            if (g == 0) return;  // balanced (key stays kPadKey)
-            if (mx / g > 2147483647ull) {
-                r.ovf = true;
-                r.key = 0;
-                return;
-            }
-        }
+    if (!__any_sync(FULL, g != 0)) return;  // balanced (key stays kPadKey)
+    g = warp_gcd(g);
+    if (__any_sync(FULL, past_int32(abs64(t[0]), g) || past_int32(abs64(t[1]), g))) {
+        r.ovf = true;
+        r.key = 0;
+        return;
     }
-    r.g = 1;
-    if (dst)
-        for (int i = r.n; i & 3; ++i) dst[i] = 0;
+    int32_t v[2];
+    uint64_t pm = 0, nm = 0, rh = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int row = lane + 32 * h;
+        v[h] = div_any(t[h], g);
+        z.zm |= (uint64_t)__ballot_sync(FULL, v[h] != 0) << (32 * h);
+        if (v[h] == 0) continue;
+        const uint32_t rk = bl[nv.o_rank + row];
+        if (v[h] > 0) pm |= 1ull << (rk & 0xFFu);
+        else nm |= 1ull << ((rk >> 8) & 0xFFu);
+        rh += (uint64_t)(int64_t)v[h] * row_hash(row);
+    }
+    r.om = __reduce_or_sync(FULL, mag(v[0]) | mag(v[1]));
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        z.pm |= (uint64_t)__reduce_or_sync(FULL, (uint32_t)(pm >> (32 * h))) << (32 * h);
+        z.nm |= (uint64_t)__reduce_or_sync(FULL, (uint32_t)(nm >> (32 * h))) << (32 * h);
+    }
+    r.rh = warp_sum(rh);
+    r.n = __popcll(z.zm);
+    r.key = mask_key(bl, nv, z.pm, z.nm);
+    const int piv = (int)(r.key & 63u);
+    r.pv = __shfl_sync(FULL, piv < 32 ? v[0] : v[1], piv & 31);
+    if (dst) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (v[h] != 0) dst[value_at(z.zm, lane + 32 * h)] = v[h];
+        if (lane < ((4 - r.n) & 3)) dst[r.n + lane] = 0;
+    }
 }
 
 // payload units of n entries (values on narrow networks)
@@ -585,90 +705,134 @@ __device__ __forceinline__ int entry_units(int n)
     return F == 2 ? (n + 3) >> 2 : (n + 1) >> 1;
 }
 
-// Any child: entries in 64 bits, the gcd and the range over all of them,
-// then the divided entries.  The rare child that may leave int32, shares a
-// divisor, or is long.
+// Any child, by one warp: the entries in 64 bits, a lane each; the gcd and the
+// range over all of them, then the divided entries.  For the child that may
+// leave int32, shares a divisor, or has more entries than a lane of the
+// generate pass takes: rare where reactions have a few metabolites, every
+// child where they have dozens.
 template <bool SUB>
-__device__ __noinline__ void slow_child(const NetView &nv, const uint32_t *bl, const uint4 *pe, int np, int32_t A,
-                                        int32_t C, int cb, int ce, int k, uint4 *dst, Child &r)
+__device__ __forceinline__ void wide_child(const NetView &nv, const uint32_t *bl, const uint4 *pe, int np, int32_t A,
+                                        int32_t C, int cb, int ce, int k, uint4 *dst, Child &r, int lane)
 {
     const int2 *p2 = reinterpret_cast<const int2 *>(pe);
     int2 *d2 = reinterpret_cast<int2 *>(dst);
-    const int nq = ce - cb + (SUB ? 1 : 0);
-    uint32_t matched[(EFM_MAX_INTERNAL + 32) / 32];
-    for (int i = 0; 32 * i < nq; ++i) matched[i] = 0;
+    const int nq = ce - cb + (SUB ? 1 : 0);  // at most 1024
+    // the child's value at parent entry i; at: its place in the column (-1: none)
+    auto parent_entry = [&](int i, int &row, int &at) -> int64_t {
+        const int2 e = p2[i];
+        row = e.x & 0xFFFF;
+        int lo = 0, hi = nq;  // first column entry with a row >= row (they ascend)
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            int rq;
+            int32_t vq;
+            column_entry<SUB>(nv, bl, cb, ce, mid, k, rq, vq);
+            if (rq < row) lo = mid + 1;
+            else hi = mid;
+        }
+        int64_t t = (int64_t)A * e.y;
+        at = -1;
+        if (lo < nq) {
+            int rq;
+            int32_t vq;
+            column_entry<SUB>(nv, bl, cb, ce, lo, k, rq, vq);
+            if (rq == row) {
+                t += (int64_t)C * vq;
+                at = lo;
+            }
+        }
+        return t;
+    };
+    uint32_t matched = 0;  // lane w: which of the column entries 32 w .. 32 w + 31 the parent has
     uint64_t g = 0, mx = 0;
+    bool unbal = false, zflux = false;
+    auto see = [&](int row, int64_t t) {
+        if (SUB && row == nv.M + k && t <= 0) zflux = true;
+        if (t == 0) return;
+        const uint64_t at = abs64(t);
+        g = gcd_any(g, at);
+        mx = at > mx ? at : mx;
+        if (!SUB || row < nv.M) unbal = true;
+    };
+    for (int i0 = 0; i0 < np; i0 += 32) {
+        int row = 0, at = -1;
+        if (i0 + lane < np) {
+            const int64_t t = parent_entry(i0 + lane, row, at);
+            see(row, t);
+        }
+        for (int w = 0; 32 * w < nq; ++w) {
+            const uint32_t m = __reduce_or_sync(FULL, at >= 0 && (at >> 5) == w ? 1u << (at & 31) : 0u);
+            if (lane == w) matched |= m;
+        }
+    }
+    // the column entries that the parent does not have
+    auto fresh = [&](int q0) -> bool {
+        const uint32_t w = __shfl_sync(FULL, matched, q0 >> 5);
+        return q0 + lane < nq && !((w >> lane) & 1u);
+    };
+    for (int q0 = 0; q0 < nq; q0 += 32)
+        if (fresh(q0)) {
+            int row;
+            int32_t cv;
+            column_entry<SUB>(nv, bl, cb, ce, q0 + lane, k, row, cv);
+            see(row, (int64_t)C * cv);
+        }
     r.n = 0;
     r.key = kPadKey;
     r.pv = 0;
     r.om = 0;
     r.rh = 0;
-    r.zflux = r.ovf = false;
-    int nbal = 0;
-    for (int pass = 0; pass < 2; ++pass) {
-        auto take = [&](int row, int64_t t) {
-            if (SUB && row == nv.M + k && t <= 0) r.zflux = true;
-            if (t == 0) return;
-            if (pass == 0) {
-                const uint64_t at = abs64(t);
-                g = gcd_any(g, at);
-                mx = at > mx ? at : mx;
-                if (!SUB || row < nv.M) ++nbal;
-                return;
-            }
+    r.g = 1;
+    r.zflux = __any_sync(FULL, zflux);
+    r.ovf = false;
+    if (!__any_sync(FULL, unbal)) return;  // balanced (key stays kPadKey)
+    g = warp_gcd(g);
+    if (__any_sync(FULL, past_int32(mx, g))) {
+        r.ovf = true;
+        r.key = 0;
+        return;
+    }
+    uint32_t key = kPadKey, om = 0;
+    int32_t pv = 0;
+    uint64_t rh = 0;
+    int n = 0;
+    auto put = [&](int row, int64_t t) {
+        const unsigned m = __ballot_sync(FULL, t != 0);
+        if (t != 0) {
             const int32_t v = div_any(t, g);
             const uint32_t kk = entry_key<SUB>(nv, bl, row, v > 0);
-            r.om |= mag(v);
-            r.rh += (uint64_t)(int64_t)v * row_hash(row);
-            if (kk < r.key) {
-                r.key = kk;
-                r.pv = v;
+            om |= mag(v);
+            rh += (uint64_t)(int64_t)v * row_hash(row);
+            if (kk < key) {
+                key = kk;
+                pv = v;
             }
-            if (d2) d2[r.n] = make_int2((int)kk, v);
-            ++r.n;
-        };
-        for (int i = 0; i < np; ++i) {
-            const int2 e = p2[i];
-            const int row = e.x & 0xFFFF;
-            int64_t t = (int64_t)A * e.y;
-            int lo = 0, hi = nq;  // first column entry with a row >= row (they ascend)
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                int rq;
-                int32_t vq;
-                column_entry<SUB>(nv, bl, cb, ce, mid, k, rq, vq);
-                if (rq < row) lo = mid + 1;
-                else hi = mid;
-            }
-            if (lo < nq) {
-                int rq;
-                int32_t vq;
-                column_entry<SUB>(nv, bl, cb, ce, lo, k, rq, vq);
-                if (rq == row) {
-                    t += (int64_t)C * vq;
-                    matched[lo >> 5] |= 1u << (lo & 31);
-                }
-            }
-            take(row, t);
+            if (d2) d2[n + __popc(m & ((1u << lane) - 1u))] = make_int2((int)kk, v);
         }
-        for (int q = 0; q < nq; ++q) {
-            if ((matched[q >> 5] >> (q & 31)) & 1u) continue;
-            int row;
-            int32_t cv;
-            column_entry<SUB>(nv, bl, cb, ce, q, k, row, cv);
-            take(row, (int64_t)C * cv);
-        }
-        if (pass == 0) {
-            if (nbal == 0) return;  // balanced (key stays kPadKey)
-            if (mx / g > 2147483647ull) {
-                r.ovf = true;
-                r.key = 0;
-                return;
-            }
-        }
+        n += __popc(m);
+    };
+    for (int i0 = 0; i0 < np; i0 += 32) {
+        int row = 0, at;
+        int64_t t = 0;
+        if (i0 + lane < np) t = parent_entry(i0 + lane, row, at);
+        put(row, t);
     }
-    r.g = 1;
-    if (d2 && (r.n & 1)) d2[r.n] = make_int2((int)kPadKey, 0);
+    for (int q0 = 0; q0 < nq; q0 += 32) {
+        int row = 0;
+        int64_t t = 0;
+        if (fresh(q0)) {
+            int32_t cv;
+            column_entry<SUB>(nv, bl, cb, ce, q0 + lane, k, row, cv);
+            t = (int64_t)C * cv;
+        }
+        put(row, t);
+    }
+    r.n = n;
+    r.key = __reduce_min_sync(FULL, key);
+    r.pv = __shfl_sync(FULL, pv, __ffs((int)__ballot_sync(FULL, key == r.key)) - 1);  // (keys are distinct)
+    r.om = __reduce_or_sync(FULL, om);
+    r.rh = warp_sum(rh);
+    if (d2 && lane == 0 && (n & 1)) d2[n] = make_int2((int)kPadKey, 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -844,8 +1008,9 @@ __device__ __forceinline__ void write_support(uint4 *dst, const uint4 *pp, int p
 // ---------------------------------------------------------------------------
 // One level by the warps worker = 0 .. nworkers-1: parents are arena rows
 // (a.perm, or a.par_base on), cpw of them a warp and chunk; blk / pay_blk: rows
-// and payload units a warp reserves at a time, at least a round's.
-template <int F, bool SUB, bool FK>
+// and payload units a warp reserves at a time, at least a round's.  LONG: see
+// NetView::long_cols.
+template <int F, bool SUB, bool FK, bool LONG>
 __device__ __forceinline__ void generate_range(const NetView &nv, const LevelArgs &a, int64_t n_par, int cpw, int blk,
                                                int pay_blk, bool any_result, int64_t worker, int64_t nworkers,
                                                CapScratch *cap, const BoundScratch &bound)
@@ -1077,12 +1242,22 @@ __device__ __forceinline__ void generate_range(const NetView &nv, const LevelArg
                 uint4 hd = make_uint4((uint32_t)off, 0u, 0u, 0u);  // an open child: where its payload may go
                 // (what the parent and the column hold is read again where it is
                 // needed, from L1, rather than kept in registers)
-                const bool fast = fits && (F == 2 ? ce - cb <= kNarrowCol : np <= 64 && ce - cb + (SUB ? 1 : 0) <= 32);
-                if (fast) {
+                const int nc = ce - cb + (SUB ? 1 : 0);
+                const bool is_long = F == 2 ? nc > kNarrowCol : (np > 64 || nc > kListCol);
+                if (fits && (LONG || !is_long)) {
                     Child m;
                     NarrowMasks z;
-                    if (F == 2) {
-                        narrow_child(nv, bl, pp, A, C, cb, ce - cb, k, reinterpret_cast<int32_t *>(de), m, z);
+                    if (LONG && is_long) {  // (copies: what a call takes by reference lives in local memory)
+                        Child lm;
+                        NarrowMasks lz;
+                        if (F == 2)
+                            narrow_child_long(nv, bl, pp, A, C, cb, nc, k, reinterpret_cast<int32_t *>(de), lm, lz);
+                        else
+                            long_child<SUB>(nv, bl, pp + support_units<F>(pc), np, A, C, cb, ce, k, de, lm);
+                        m = lm;
+                        if (F == 2) z = lz;
+                    } else if (F == 2) {
+                        narrow_child(nv, bl, pp, A, C, cb, nc, k, reinterpret_cast<int32_t *>(de), m, z);
                     } else {
                         const uint4 s0 = scol[2 * k];
                         fast_child<SUB>(nv, bl, pp + support_units<F>(pc), np, A, C, cb, ce,
@@ -1189,73 +1364,109 @@ __device__ bool same_state(const uint4 *px, const uint4 *py, int pc, int n, int 
     return __all_sync(FULL, same);
 }
 
-// An open child of reserved row i: balanced (to the arbiter), or one whose
-// update needs 64 bits, a division or more entries than the generate pass
-// takes (about one in a thousand).  Returns its fingerprint (kDeadFp: none)
-// and its header; live rows without a payload count as unwritten.
-template <int F, bool SUB>
-__device__ __noinline__ uint64_t finish_open(const NetView &nv, const LevelArgs &a, uint64_t f, uint64_t i, uint4 &h)
+// An open child that balances, to the arbiter (one lane).
+template <int F>
+__device__ __noinline__ void finish_balanced(const NetView &nv, const LevelArgs &a, uint64_t f)
+{
+    const uint4 ph = a.par.hdr[(uint32_t)f];
+    atomicAdd(&a.ctr[C_BAL], 1ull);
+    insert_candidate<F>(a, nv.W, a.par.pay + ph.x, (int)((ph.y >> 23) & 0x7Fu),
+                        (f & kOpenInU) ? -1 : (int)((f >> 32) & 0xFFFu));  // (a failure sets the error word)
+}
+
+// What any other open child needs: its parent, and A and C from the pivot's
+// entry and the coefficient of k in the pivot's row.
+struct OpenChild {
+    const uint4 *pp;
+    int pc, np, k, cb, ce;
+    bool in_u;
+    int32_t A, C;
+};
+
+__device__ __forceinline__ OpenChild open_child(const NetView &nv, const LevelArgs &a, uint64_t f)
 {
     const uint32_t *bl = nv.blob;
     const uint4 ph = a.par.hdr[(uint32_t)f];
-    const uint4 *pp = a.par.pay + ph.x;
-    const int pc = (int)((ph.y >> 23) & 0x7Fu), np = (int)(ph.z & 0x7FFu);
-    const int k = (int)((f >> 32) & 0xFFFu);
-    const bool in_u = (f & kOpenInU) != 0;
-    h = i < (uint64_t)a.child.cap ? a.child.hdr[i] : make_uint4(0u, 0u, 0u, 0u);
-    uint4 *dst = h.z ? a.child.pay + h.x : nullptr;
-    const uint32_t off = h.x;
-    h = make_uint4(0u, 0u, 0u, 0u);
-    if (f & kOpenBal) {
-        atomicAdd(&a.ctr[C_BAL], 1ull);
-        insert_candidate<F>(a, nv.W, pp, pc, in_u ? -1 : k);  // (a failure sets the error word)
-        return kDeadFp;
-    }
-    const int cb = (int)bl[nv.o_colptr + k], ce = (int)bl[nv.o_colptr + k + 1];
-    // A and C from the pivot's entry and the coefficient of k in the pivot's row
+    OpenChild o;
+    o.pp = a.par.pay + ph.x;
+    o.pc = (int)((ph.y >> 23) & 0x7Fu);
+    o.np = (int)(ph.z & 0x7FFu);
+    o.k = (int)((f >> 32) & 0xFFFu);
+    o.in_u = (f & kOpenInU) != 0;
+    o.cb = (int)bl[nv.o_colptr + o.k];
+    o.ce = (int)bl[nv.o_colptr + o.k + 1];
     const int piv = (int)(ph.y & 0x3FFu);
-    uint32_t sik = 1;
-    for (int q = cb; q < ce; ++q) {
-        const uint32_t e = bl[nv.o_colent + q];
-        if (ent_index(e) == piv) sik = mag(ent_coef(e));
-    }
-    const uint32_t abi = mag((int32_t)ph.w), g0 = gcd32(abi, sik);
-    const int32_t A = (int32_t)(sik / g0), C = (f & kOpenSub) ? -(int32_t)(abi / g0) : (int32_t)(abi / g0);
-    const int pc2 = pc + (in_u ? 0 : 1);
+    const uint32_t sik =
+        mag(reinterpret_cast<const int32_t *>(bl + nv.o_dcols)[(size_t)o.k * nv.Mpad + piv]);
+    const uint32_t abi = mag((int32_t)ph.w), g0 = abi == 1u || sik == 1u ? 1u : gcd_small(abi, sik);
+    o.A = (int32_t)(sik / g0);
+    o.C = (f & kOpenSub) ? -(int32_t)(abi / g0) : (int32_t)(abi / g0);
+    return o;
+}
+
+// Reserved row i's payload, if it has one, and its header cleared.
+__device__ __forceinline__ uint4 *open_payload(const LevelArgs &a, uint64_t i, uint32_t &off)
+{
+    const uint4 h = i < (uint64_t)a.child.cap ? a.child.hdr[i] : make_uint4(0u, 0u, 0u, 0u);
+    off = h.x;
+    return h.z ? a.child.pay + h.x : nullptr;
+}
+
+template <bool SUB>
+__device__ __forceinline__ uint4 child_header(const NetView &nv, uint32_t off, const Child &m, int pc)
+{
+    return make_uint4(off, pack_meta(branch_key(nv.blob, nv, m.key, SUB ? 1 : 0), pc),
+                      (uint32_t)m.n | ((uint32_t)max_bits(m.om) << 11), (uint32_t)m.pv);
+}
+
+// Any other open child, of reserved row i, by one warp: one whose update needs
+// 64 bits, a division or more entries than the generate pass takes.  Returns its fingerprint (kDeadFp: none) and its
+// header; live rows without a payload count as unwritten.
+template <int F, bool SUB>
+__device__ __noinline__ uint64_t finish_open(const NetView &nv, const LevelArgs &a, uint64_t f, uint64_t i, uint4 &h,
+                                             int lane)
+{
+    const uint32_t *bl = nv.blob;
+    const OpenChild o = open_child(nv, a, f);
+    const int pc2 = o.pc + (o.in_u ? 0 : 1), k2 = o.in_u ? -1 : o.k;
+    uint32_t off;
+    uint4 *dst = open_payload(a, i, off);
+    uint4 *de = dst ? dst + support_units<F>(pc2) : nullptr;
+    h = make_uint4(0u, 0u, 0u, 0u);
     Child m;
     NarrowMasks z;
-    uint4 *de = dst ? dst + support_units<F>(pc2) : nullptr;
     if (F == 2)
-        slow_narrow(nv, bl, pp, A, C, cb, ce, k, reinterpret_cast<int32_t *>(de), m, z);
+        wide_narrow(nv, bl, o.pp, o.A, o.C, o.cb, o.k, reinterpret_cast<int32_t *>(de), m, z, lane);
     else
-        slow_child<SUB>(nv, bl, pp + support_units<F>(pc), np, A, C, cb, ce, k, de, m);
+        wide_child<SUB>(nv, bl, o.pp + support_units<F>(o.pc), o.np, o.A, o.C, o.cb, o.ce, o.k, de, m, lane);
     if (SUB && m.zflux) {
-        atomicAdd(&a.ctr[C_ZERO], 1ull);
+        if (lane == 0) atomicAdd(&a.ctr[C_ZERO], 1ull);
         return kDeadFp;
     }
     if (m.key >= kFluxKey) {
-        atomicAdd(&a.ctr[C_BAL], 1ull);
-        insert_candidate<F>(a, nv.W, pp, pc, in_u ? -1 : k);
+        if (lane == 0) finish_balanced<F>(nv, a, f);
         return kDeadFp;
     }
     if (m.ovf) {
-        atomicAdd(&a.ctr[C_OVF], 1ull);
+        if (lane == 0) atomicAdd(&a.ctr[C_OVF], 1ull);
         return kDeadFp;
     }
     if (f & (kOpenPruned | kOpenDead)) {
-        if (f & kOpenPruned) atomicAdd(&a.ctr[C_PRUNED], 1ull);
+        if (lane == 0 && (f & kOpenPruned)) atomicAdd(&a.ctr[C_PRUNED], 1ull);
         return kDeadFp;
     }
-    const uint64_t uh = support_hash_of<F>(pp, in_u ? -1 : k);
+    const uint64_t uh = support_hash_of<F>(o.pp, k2);
     if (dst) {
-        write_support<F>(dst, pp, pc, in_u ? -1 : k, m.rh, uh, z);
-        h = make_uint4(off, pack_meta(branch_key(bl, nv, m.key, SUB ? 1 : 0), pc2),
-                       (uint32_t)m.n | ((uint32_t)max_bits(m.om) << 11), (uint32_t)m.pv);
-        a.child.hdr[i] = h;
-    } else {
+        h = child_header<SUB>(nv, off, m, pc2);
+        if (lane == 0) {
+            write_support<F>(dst, o.pp, o.pc, k2, m.rh, uh, z);
+            a.child.hdr[i] = h;
+        }
+    } else if (lane == 0) {
         atomicAdd(&a.ctr[C_UNWRITTEN], 1ull);
     }
     __threadfence();  // the row is complete before its slot is taken
+    __syncwarp();
     return state_fp(m.rh, uh);
 }
 
@@ -1355,13 +1566,34 @@ __device__ __forceinline__ void dedup_range(const NetView &nv, const LevelArgs &
     const int lane = threadIdx.x & 31;
     end = end < (uint64_t)a.fp_cap ? end : (uint64_t)a.fp_cap;
     const uint64_t row_cap = (uint64_t)a.child.cap;
-    for (uint64_t q0 = t_open; q0 < n_open; q0 += stride) {
+    // as many open children to a warp as there are for each, at most 32: the
+    // balanced ones a lane each, the others by the warp, one after the other
+    const uint64_t warps = stride >> 5;
+    const uint64_t per = min((uint64_t)32, max((uint64_t)1, (n_open + warps - 1) / warps));
+    for (uint64_t q0 = (t_open >> 5) * per; q0 < n_open; q0 += warps * per) {
         uint64_t i = 0, f = kDeadFp;
         uint4 h = make_uint4(0u, 0u, 0u, 0u);
-        if (q0 + lane < n_open) {
+        if ((uint64_t)lane < per && q0 + lane < n_open) {
             i = a.open[q0 + lane];
-            f = finish_open<F, SUB>(nv, a, a.fp[i], i, h);
-            if (h.y == 0u && i < row_cap) a.child.hdr[i] = h;
+            f = a.fp[i];
+            if (f & kOpenBal) {
+                finish_balanced<F>(nv, a, f);
+                f = kDeadFp;
+                if (i < row_cap) a.child.hdr[i] = h;
+            }
+        }
+        __syncwarp();
+        for (unsigned m = __ballot_sync(FULL, f != kDeadFp); m; m &= m - 1) {
+            const int src = __ffs((int)m) - 1;
+            const uint64_t row = __shfl_sync(FULL, i, src);
+            uint4 hc;
+            const uint64_t fc = finish_open<F, SUB>(nv, a, __shfl_sync(FULL, f, src), row, hc, lane);
+            if (lane == src) {
+                f = fc;
+                h = hc;
+                if (h.y == 0u && row < row_cap) a.child.hdr[row] = h;
+            }
+            __syncwarp();
         }
         dedup_insert<F>(a, mask, i, f, h, lane, sum);
     }

@@ -317,4 +317,13 @@ inline int prepare_network(int32_t n_met, int32_t n_rxn, const int32_t *row_ptr,
     return EFM_OK;
 }
 
+// Does a column have more entries than `limit`, or do they have more than
+// `mean` on average?
+inline int has_long_columns(const NetPrep &p, int limit, int mean)
+{
+    for (int k = 0; k < p.N; ++k)
+        if (p.blob[p.o_colptr + k + 1] - p.blob[p.o_colptr + k] > (uint32_t)limit) return 1;
+    return p.N > 0 && p.blob[p.o_colptr + p.N] - p.blob[p.o_colptr] > (uint64_t)mean * (uint64_t)p.N;
+}
+
 }  // namespace efm

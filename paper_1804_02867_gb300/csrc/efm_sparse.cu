@@ -11,7 +11,7 @@ constexpr int kGenWarps = 8;      // warps per CTA
 // network at a 2^26 budget; 24 warps 537.
 constexpr int kGenBlocks = 5;
 
-template <int F, bool SUB, bool FK>
+template <int F, bool SUB, bool FK, bool LONG>
 __global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks) generate_kernel(const __grid_constant__ NetView nv,
                                                                               const __grid_constant__ LevelArgs a)
 {
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks) generate_kernel(co
     // parents per warp and chunk: fewer at small levels, so that their items
     // spread over all warps
     const int cpw = (int)min((int64_t)32, max((int64_t)1, (n_par + a.warps - 1) / a.warps));
-    generate_range<F, SUB, FK>(nv, a, n_par, cpw, blk, pay_blk, any_result, (int64_t)blockIdx.x * kGenWarps + wid,
+    generate_range<F, SUB, FK, LONG>(nv, a, n_par, cpw, blk, pay_blk, any_result, (int64_t)blockIdx.x * kGenWarps + wid,
                                (int64_t)gridDim.x * kGenWarps, s_cap + (FK ? wid : 0), s_bound);
 }
 
@@ -234,21 +234,22 @@ int grid_of(K kernel, int sm_count)
     return sm_count * per_sm;
 }
 
-// one of the kernel's instances: form, subtractive view, first-K rules
+// one of the kernel's instances: form, subtractive view, first-K rules, long columns
+#define EFM_GENERATE_OF(CALL, F, SUB, FK)                                         \
+    do {                                                                          \
+        if (nv.long_cols) CALL((generate_kernel<F, SUB, FK, true>));              \
+        else CALL((generate_kernel<F, SUB, FK, false>));                          \
+    } while (0)
 #define EFM_GENERATE(CALL)                                                        \
     do {                                                                          \
-        if (nv.form == 2) {                                                       \
-            if (first_k) CALL((generate_kernel<2, false, true>));                 \
-            else CALL((generate_kernel<2, false, false>));                        \
-        } else if (nv.form == 1) {                                                \
-            if (sub) CALL((generate_kernel<1, true, false>));                     \
-            else if (first_k) CALL((generate_kernel<1, false, true>));            \
-            else CALL((generate_kernel<1, false, false>));                        \
-        } else {                                                                  \
-            if (sub) CALL((generate_kernel<0, true, false>));                     \
-            else if (first_k) CALL((generate_kernel<0, false, true>));            \
-            else CALL((generate_kernel<0, false, false>));                        \
-        }                                                                         \
+        if (nv.form == 2 && first_k) EFM_GENERATE_OF(CALL, 2, false, true);       \
+        else if (nv.form == 2) EFM_GENERATE_OF(CALL, 2, false, false);            \
+        else if (nv.form == 1 && sub) EFM_GENERATE_OF(CALL, 1, true, false);      \
+        else if (nv.form == 1 && first_k) EFM_GENERATE_OF(CALL, 1, false, true);  \
+        else if (nv.form == 1) EFM_GENERATE_OF(CALL, 1, false, false);            \
+        else if (sub) EFM_GENERATE_OF(CALL, 0, true, false);                      \
+        else if (first_k) EFM_GENERATE_OF(CALL, 0, false, true);                  \
+        else EFM_GENERATE_OF(CALL, 0, false, false);                              \
     } while (0)
 
 }  // namespace

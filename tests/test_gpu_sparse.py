@@ -176,3 +176,34 @@ def test_small_levels(oracle_lib, efm, budget):
             (sup, ctr), = efm.enumerate_targets(nw, [net.targets[0]], 12, 2, cap, budget)
             osup, octr = oracle_lib.enumerate_pathways(net, net.targets[0], oracle_lib.Limits(12, 2, cap, budget))
             assert np.array_equal(sup, osup) and ctr == octr, (cap, ctr, octr)
+
+
+LONG = {
+    # columns past the 8 entries of a narrow lane; with common divisors; leaving int32
+    "narrow": dict(n_int=60, n_rxn=90, n_rev=20, size_range=(7, 20), coef_probs={1: 0.5, 2: 0.3, 3: 0.2}),
+    "narrow-even": dict(n_int=30, n_rxn=50, n_rev=10, size_range=(8, 12), coef_probs={2: 0.4, 4: 0.4, 6: 0.2}),
+    "narrow-large": dict(n_int=40, n_rxn=60, n_rev=10, size_range=(8, 12), coef_probs={1: 0.3, 999: 0.4, 524287: 0.3}),
+    # columns past 32 entries, states past 64; bitsets and lists
+    "bits": dict(n_int=100, n_rxn=100, n_rev=20, size_range=(28, 60), coef_probs={1: 0.5, 2: 0.3, 3: 0.2}),
+    "bits-even": dict(n_int=100, n_rxn=100, n_rev=20, size_range=(30, 40), coef_probs={2: 0.4, 4: 0.4, 6: 0.2}),
+    "list": dict(n_int=300, n_rxn=500, n_rev=100, size_range=(30, 80), coef_probs={1: 0.5, 2: 0.3, 3: 0.2}),
+    "list-large": dict(n_int=90, n_rxn=130, n_rev=10, size_range=(31, 36), coef_probs={1: 0.3, 999: 0.4, 524287: 0.3}),
+}
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("name", sorted(LONG))
+def test_long_columns(oracle_lib, efm, name, variant):
+    # reactions of dozens of metabolites: at budgets that one CTA's levels reach and past them
+    net = synth.generate(n_targets=3, n_hubs=3, n_substrates=2, gamma=None, hub_degree=(5, 20), seed=77, name=name,
+                         **LONG[name])
+    max_len, targets = (12, net.targets[:2]) if variant == 0 else (6, net.targets[:1])
+    for budget in (300, 3000):
+        with efm.Network(net) as nw:
+            got = efm.enumerate_targets(nw, targets, max_len, 2, 0, budget, variant=variant)
+        seen = 0
+        for t, (sup, ctr) in zip(targets, got):
+            osup, octr = oracle_lib.enumerate_pathways(net, t, oracle_lib.Limits(max_len, 2, 0, budget, subtractive=bool(variant)))
+            assert np.array_equal(sup, osup) and ctr == octr, (t, budget, ctr, octr)
+            seen = max(seen, octr["frontier_max"])
+        assert seen > 20
