@@ -770,6 +770,14 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         CK(cudaEventRecord(w.ev[3], s));
         out.kernel_launches += 1;
         if ((rc = read_ctr())) return rc;
+        if (hs[S_PENDING]) {
+            acc.level = (int)hs[S_LEVEL] + 1;
+            acc.child_rows = w.rows[(acc.level - level0) & 1];
+            CK(launch_accept_new(nv, acc, net->sm_count, s));
+            CK(cudaEventRecord(w.ev[3], s));
+            out.kernel_launches += 1;
+            if ((rc = read_ctr())) return rc;
+        }
         float small_ms = 0.f;
         CK(cudaEventElapsedTime(&small_ms, w.ev[2], w.ev[3]));
         out.expand_ms += small_ms;

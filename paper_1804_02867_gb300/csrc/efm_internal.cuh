@@ -26,6 +26,10 @@ constexpr int64_t kResultWindow = 256;        // first-K search: new results fet
 // network 3.93, 3.90, 4.07, 4.20 (4.13), the subtractive variant 5.85, 5.83,
 // 5.95, 6.6 (6.07).
 constexpr int kSmallBranches = 1024;
+// Most new balanced supports that its eight warps judge; more are left to the
+// grid: 1000 supports of 61 columns 7.9 ms by one CTA and 1.3 by the grid, 900
+// of 31 columns 2.0 and 0.9, 60 of 61 columns 1.1 either way.
+constexpr int kSmallCandidates = 64;
 constexpr int kWaitSpinLimit = 1 << 20;       // polls of a bounded device-side wait (with ~0.25 us sleeps)
 
 // device error bits (ctr[C_ERR])
@@ -76,6 +80,7 @@ enum {
     S_BYTES,      // algorithmic bytes of the expansions so far
     S_EXPANDS,    // expansion launches: levels, chunks of a first-K level and levels run again
     S_TICKET,     // CTAs of the running minimality launch that are done
+    S_PENDING,    // 1: launch_small left the minimality test of a level to the grid
     S_SNAP,       // C_EXP, C_OVF, C_BAL, C_PRUNED, C_ZERO when the running level began
     S_COUNT = S_SNAP + 8
 };

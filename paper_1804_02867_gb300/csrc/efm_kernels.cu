@@ -818,6 +818,7 @@ __device__ void advance_level(const AcceptArgs &a, const unsigned long long *v)
     const unsigned long long *sv = v + C_COUNT;
     auto get = [&](int i) { return v[i]; };
     const bool seeds = a.advance == 3;
+    st[S_PENDING] = 0ull;
     if (!seeds) st[S_EXPANDS] = sv[S_EXPANDS] + 1;
     if (a.advance == 1) return;
     const uint64_t next = get(C_NEXT), unv = get(C_UNV), written = seeds ? next : get(C_WRITTEN);
@@ -1285,7 +1286,9 @@ __device__ void run_job(const BatchArgs &ba, const BatchJob &job, char *slice, u
 }
 
 // The levels of one search while they are small, by one CTA: from the state's
-// level on, until the search stops or a level has more than `limit` branches.
+// level on, until the search stops, a level has more than `limit` branches, or
+// one has more new balanced supports than a few warps should judge (S_PENDING:
+// the grid then ends that level).
 // Latency bounds such a level: three launches of chains of dependent reads,
 // each on a cold L1.  Here a barrier ends a phase, and the network's tables and
 // the rows just written are in the SM's L1.  One GB300, with three launches for
@@ -1354,6 +1357,10 @@ __global__ void __launch_bounds__(kSmallWarps * 32, 1) small_kernel(const __grid
                            !(acc.max_frontier > 0 && (int64_t)(v[C_NEXT] + v[C_UNV]) > acc.max_frontier);
         const int64_t begin = (int64_t)v[C_ACC_BEGIN], n = (int64_t)v[C_CAND_N];
         const int64_t end = rerun ? begin : (n < acc.cand_cap ? n : acc.cand_cap);
+        if (end - begin > kSmallCandidates) {
+            if (tid == 0) a0.st[S_PENDING] = 1ull;
+            return;
+        }
         if (end > begin) {
             if (tid == 0) {
                 acc.cand_begin = begin;

@@ -87,6 +87,37 @@ def test_level_run_again_on_the_grid(oracle_lib, efm, form, capfd, monkeypatch):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("max_results", [0, 10])
+@pytest.mark.parametrize("spec", [((8, 2, 0),), ((9, 2, 0), (2, 5, 0)), ((17, 2, 0), (3, 4, 0)), ((30, 2, 1),)])
+def test_small_levels_with_many_results(oracle_lib, efm, spec, max_results):
+    """64, 81, 289 and 900 balanced children at a level that one CTA runs (its
+    warps judge up to 64 of them), as the last level and with more to come."""
+    net = ladders(*spec)
+    with efm.Network(net) as nw:
+        got = efm.enumerate_targets(nw, net.targets * 2, 10, 1, max_results, 1 << 12)
+    osup, octr = oracle_lib.enumerate_pathways(net, net.targets[0], oracle_lib.Limits(10, 1, max_results, 1 << 12))
+    assert octr["balanced"] >= 64
+    for sup, ctr in got:
+        assert np.array_equal(sup, osup) and ctr == octr, (ctr, octr)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("spec", [((46, 2, 0), (3, 4, 0)), ((55, 2, 0), (4, 5, 0))])
+def test_index_grows(oracle_lib, efm, spec, capfd, monkeypatch):
+    """More results at one level than the superset rule's index has room for,
+    and levels after it: bitset form and list form."""
+    net = ladders(*spec)
+    monkeypatch.setenv("EFM_DEBUG", "1")
+    with efm.Network(net) as nw:
+        assert (nw.n_columns > 128) == (spec[0][0] == 55)
+        capfd.readouterr()
+        (sup, ctr), = efm.enumerate_targets(nw, net.targets, 10, 1, 0, 1 << 13)
+    assert STOP_INDEX in stops(capfd.readouterr().err)
+    osup, octr = oracle_lib.enumerate_pathways(net, net.targets[0], oracle_lib.Limits(10, 1, 0, 1 << 13))
+    assert np.array_equal(sup, osup) and ctr == octr, (ctr, octr)
+
+
+@pytest.mark.gpu
 def test_trace_takes_a_level_once(efm, capfd, monkeypatch):
     """A first-K search with every pathway among its K: the traced levels hold
     6^0 + ... + 6^5 states (the seed's level among them), whether or not
