@@ -1445,7 +1445,16 @@ cudaError_t launch_walks(const NetView &nv, const LevelArgs &a, int target, uint
                          cudaStream_t s)
 {
     if (n_walks <= 0) return cudaSuccess;
-    if (nv.form == 2) {
+    // A lane takes a walk in several times the time of a warp, so few walks go to
+    // a warp each.  Kernel times of n walks by warps grow with n, by lanes they
+    // are level until the chip is full: they meet at 68 walks an SM on the
+    // smallest network (one row a lane of the warp; 0.046 against 0.124 ms at
+    // 1000 walks, 0.173 / 0.130 at 16000), at half of that on the core-shaped one
+    // (two rows; 0.103 / 0.193 at 1000, 0.259 / 0.193 at 8000), and where
+    // reactions are long, whose rows a lane takes one by one, at 110 (0.148 /
+    // 0.916 at 1000, 0.828 / 0.943 at 16000, 1.63 / 0.99 at 32000).
+    const int64_t few = (int64_t)sm_count * (nv.long_cols ? 220 : 68) / nv.EPL;
+    if (nv.form == 2 && n_walks >= few) {
         const size_t sm = (size_t)kWalkWarps * 32 * 4 * (size_t)std::max(nv.M, 1);
         int per_sm = 1;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, walk_narrow_kernel, kWalkWarps * 32, sm) != cudaSuccess ||

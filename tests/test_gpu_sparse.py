@@ -112,6 +112,19 @@ def test_lane_walks(oracle_lib, efm, name):
                 assert np.array_equal(sup, osup) and ctr == octr, (name, t, n, ctr, octr)
 
 
+@pytest.mark.parametrize("name,n", [("one-word", 10000), ("one-word", 12000), ("narrow-last", 5000),
+                                    ("narrow-last", 6000), ("narrow", 16000), ("narrow", 18000)])
+def test_walk_kernels(oracle_lib, efm, name, n):
+    """A warp per walk below the line and a lane per walk above it (152 SMs):
+    one and two rows a lane, short and long columns."""
+    net = edge_network(name)
+    with efm.Network(net) as nw:
+        for t in net.targets[:2] + [-1]:
+            sup, ctr = efm.sample_target(nw, t, 20, 3, 5, n)
+            osup, octr = oracle_lib.sample_pathways(net, t, oracle_lib.Limits(20, 3), 5, n)
+            assert np.array_equal(sup, osup) and ctr == octr, (t, ctr, octr)
+
+
 @pytest.mark.parametrize("budget", [2**6, 2**10, 2**14])
 def test_batch_slices(efm, budget):
     # levels that outgrow a job's slice are run alone; the rows come back in
