@@ -219,7 +219,7 @@ extern "C" int efm_load_network(int32_t n_met, int32_t n_rxn, const int32_t *row
     if (!out) return EFM_EINVAL;
     *out = nullptr;
     NetPrep prep;
-    const int prc = prepare_network(n_met, n_rxn, row_ptr, col_idx, coef, reversible, external, prep);
+    const int prc = prepare_network(n_met, n_rxn, row_ptr, col_idx, coef, reversible, external, prep, false, false);
     if (prc != EFM_OK) return prc;
     auto *net = new (std::nothrow) efm_net();
     if (!net) return EFM_ENOMEM;
@@ -248,7 +248,6 @@ extern "C" int efm_load_network(int32_t n_met, int32_t n_rxn, const int32_t *row
     nv.o_keyr = prep.o_keyr;
     nv.o_colx = prep.o_colx;
     nv.o_nent = prep.o_nent;
-    nv.blob_words = (int)blob.size();
     nv.M = prep.M;
     nv.N = prep.N;
     nv.W = prep.W;
@@ -313,7 +312,6 @@ extern "C" int efm_load_network(int32_t n_met, int32_t n_rxn, const int32_t *row
         NetView &vs = net->nv_sub;
         vs = nv;
         vs.blob = (const uint32_t *)net->blob_sub.p;
-        vs.blob_words = (int)sub.blob.size();
         vs.o_dcols = sub.o_dcols;
         vs.o_hbits = sub.o_hbits;
         vs.EPL = sub.EPL;
@@ -450,7 +448,7 @@ const NetView &view_of(const efm_net *net, const efm_limits &lim)
     return lim.variant == EFM_SUBTRACTIVE ? net->nv_sub : net->nv;
 }
 
-int alloc_work(Work &w, const efm_net *net, const efm_limits &lim, int total_warps, cudaStream_t s)
+int alloc_work(Work &w, const efm_net *net, const efm_limits &lim, cudaStream_t s)
 {
     const NetView &nv = view_of(net, lim);
     const int64_t default_cap = (int64_t)1 << 22;
@@ -762,7 +760,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         if (manual && (rc = read_ctr())) return rc;
     }
     int level = level0;  // last completed level (as far as the host knows)
-    if (!manual && !fs) {
+    if (!manual) {
         // the first levels by one CTA while they are small; then the host has the state
         acc.advance = 2;
         CK(cudaEventRecord(w.ev[2], s));
@@ -851,8 +849,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             CK(cudaEventRecord(w.ev[2], s));
             for (int i = 0; i < n; ++i) {
                 const int lv = level + 1 + i;
-                const bool ext = fs && lv == level0 + 1;
-                a.par = ext ? fs->par : arena(cur ^ (i & 1));
+                a.par = arena(cur ^ (i & 1));  // (a part of a split level is first-K)
                 a.child = arena(cur ^ (i & 1) ^ 1);
                 // the level's state table: cleared by the launch itself, or, at a
                 // large level whose size the host knows, by a memset
@@ -995,7 +992,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             // first-K: the level's parents in parts of about half the
             // budget's worth of children, each run to the end
             Work w2;
-            int rc2 = alloc_work(w2, net, lim, full_grid * kExpandWarps, s);
+            int rc2 = alloc_work(w2, net, lim, s);
             if (rc2 == EFM_ENOMEM) {
                 // no room for a second work area: the answer stays uncertified
                 free_work(w2, s);
@@ -1185,8 +1182,7 @@ extern "C" int efm_find_pathways(efm_net *net, const int32_t *targets, int32_t n
     job->net = net;
     job->out.resize(n_targets);
     Work w;
-    const int total_warps = level_grid(view_of(net, lim), lim, net->sm_count) * kExpandWarps;
-    int rc = alloc_work(w, net, lim, total_warps, net->stream);
+    int rc = alloc_work(w, net, lim, net->stream);
     int flags = 0;
     for (int i = 0; rc == EFM_OK && i < n_targets; ++i) {
         rc = lim.first_k > 0 ? run_first_k(net, w, lim, targets[i], job->out[i], mdl, nullptr)
@@ -1233,8 +1229,7 @@ extern "C" int efm_find_pathways_from(efm_net *net, const int32_t *columns, int3
     cudaStream_t s = net->stream;
     Work w;
     DevBuf cols;
-    const int total_warps = level_grid(view_of(net, lim), lim, net->sm_count) * kExpandWarps;
-    int rc = alloc_work(w, net, lim, total_warps, s);
+    int rc = alloc_work(w, net, lim, s);
     if (rc == EFM_OK && !dev_alloc(cols, (size_t)n_columns * 4, s)) rc = EFM_ENOMEM;
     if (rc == EFM_OK && cudaMemcpyAsync(cols.p, columns, (size_t)n_columns * 4, cudaMemcpyHostToDevice, s) != cudaSuccess)
         rc = EFM_ECUDA;
@@ -1382,7 +1377,7 @@ extern "C" int efm_sample_pathways(efm_net *net, int32_t target, const efm_limit
     job->out.resize(1);
     TargetOut &o = job->out[0];
     Work w;
-    int rc = alloc_work(w, net, lim, 0, s);
+    int rc = alloc_work(w, net, lim, s);
     unsigned long long h[C_COUNT];
     auto fail = [&](int code) {
         cudaGetLastError();
@@ -1815,7 +1810,7 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
         l1.max_len = hj[i].max_len;
         TargetOut &o = job->out[i];
         Work w;
-        int e = alloc_work(w, nets[i], l1, level_grid(nets[i]->nv, l1, sms) * kExpandWarps, s);
+        int e = alloc_work(w, nets[i], l1, s);
         if (e == EFM_OK) e = run_target(nets[i], w, l1, targets[i], o);
         free_work(w, s);
         if (e == EFM_OK && (o.ctr.candidates > L.cand_cap || o.ctr.results > L.res_cap)) e = EFM_ECAPACITY;
@@ -2244,8 +2239,7 @@ extern "C" int efm_model_trace(efm_model *m, efm_net *net, const int32_t *target
     for (int i = 0; i < n_targets; ++i)
         if (targets[i] < -1 || targets[i] >= net->n_met) return EFM_EINVAL;
     Work w;
-    const int total_warps = level_grid(net->nv, lim, net->sm_count) * kExpandWarps;
-    int rc = alloc_work(w, net, lim, total_warps, net->stream);
+    int rc = alloc_work(w, net, lim, net->stream);
     for (int i = 0; rc == EFM_OK && i < n_targets; ++i) {
         TargetOut ans;
         int depth = lim.max_len;

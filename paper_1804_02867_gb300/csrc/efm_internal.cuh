@@ -100,7 +100,6 @@ enum : unsigned long long {
 // coefficient a signed 20-bit value.
 struct NetView {
     const uint32_t *blob;  // device
-    int blob_words;        // multiple of 4
     int M, N, W, Mpad, EPL;
     int o_colptr, o_colent;    // S_int by column: rows with coefficients
     int o_consptr, o_consent;  // per internal row: consuming columns, |coef|

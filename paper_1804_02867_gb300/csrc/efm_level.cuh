@@ -587,8 +587,7 @@ __device__ __noinline__ void narrow_child_long(const NetView &nv, const uint32_t
 
 // gcd and exact division of the children below: most are there for a common
 // divisor and fit 32 bits, where both take a fraction of the 64-bit time (one
-// such child holds up a small level: 1 to 2 % of a call, eight core targets at
-// 2^17 8.06 -> 7.92 ms, the smallest query 0.739 -> 0.729)
+// such child holds up a small level)
 __device__ __forceinline__ uint64_t gcd_any(uint64_t g, uint64_t x)
 {
     if (g == 1ull) return 1ull;

@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(kFeatWarps * 32) features_kernel(NetView nv, A
             atomicAdd(&emb[wid][h & 63u], (h & 64u) ? 1.f : -1.f);
             colsum += (float)k;
         };
-        // the state's columns (layout in efm_sparse.cu), then its entries; flux
+        // the state's columns (layout in efm_level.cuh), then its entries; flux
         // entries (rows past M) are not balance rows
         const uint4 hd = par.hdr[p];
         const uint4 *pay = par.pay + hd.x;

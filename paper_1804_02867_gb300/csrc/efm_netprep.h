@@ -24,8 +24,8 @@
 //    orders), its row-space mask, sum_m S_int[m][k] R[m], max |S_int[m][k]|
 //    and whether the gcd of its entries is 1; per entry of the column CSR its
 //    row, the row's two ranks and the coefficient;
-//  - wide networks: per column, the lane masks of the rows it consumes and
-//    of the rows it produces (the first-K length-cap rule);
+//  - wide networks, on request: per column, the lane masks of the rows it
+//    consumes and of the rows it produces;
 //  - per column, what the AND update of a sparse state reads at once
 //    (kScolWords = 8 words): sum_m S_int[m][k] R[m] (2 words; with the flux
 //    rows also R[M + k]), the mask of its rows modulo 64 (2), its largest
@@ -95,9 +95,11 @@ struct NetPrep {
 // carry their flux vector after the extra flux: a row holds M + N entries
 // and the dense copy of column k is S_int[:, k] followed by the unit vector
 // e_k (flux 1 on k); EFM_EUNSUPPORTED when M + N exceeds EFM_MAX_INTERNAL.
+// lane_masks: also the lane masks of wide networks, which no kernel reads
+// (0.8 MB on a genome-shaped network; the library leaves them out).
 inline int prepare_network(int32_t n_met, int32_t n_rxn, const int32_t *row_ptr, const int32_t *col_idx,
                            const int32_t *coef, const uint8_t *reversible, const uint8_t *external, NetPrep &out,
-                           bool flux_rows = false)
+                           bool flux_rows = false, bool lane_masks = true)
 {
     if (n_met <= 0 || n_rxn <= 0 || !row_ptr || !reversible || !external) return EFM_EINVAL;
     if (row_ptr[0] != 0) return EFM_EINVAL;
@@ -178,8 +180,7 @@ inline int prepare_network(int32_t n_met, int32_t n_rxn, const int32_t *row_ptr,
             for (auto &e : l) blob.push_back(ent_pack(e.first, e.second));
     };
     put_csr(col, out.o_colptr, out.o_colent);
-    // [o_consptr, o_hbits): the expansion's sparse tables (branch lists, twins,
-    // keys), 16-byte aligned so that one bulk copy can stage them
+    // the branch lists, twins and keys, 16-byte aligned
     while (blob.size() % 4) blob.push_back(0);
     put_csr(cons, out.o_consptr, out.o_consent);
     put_csr(prod, out.o_prodptr, out.o_prodent);
@@ -261,11 +262,11 @@ inline int prepare_network(int32_t n_met, int32_t n_rxn, const int32_t *row_ptr,
             }
     }
     // wide networks (not narrow, additive rows): the rows column k consumes
-    // and produces, as lane masks of the expansion's row layout.  Lane l of
+    // and produces, as lane masks of a row in 4-entry chunks.  Lane l of
     // a group of G = min(32, 4 EPL) lanes holds the rows 4 (l + G i) + j for
     // i < 8 EPL / G and j < 4, at bit 4 i + j of its mask word.
     out.o_fixc = out.o_fixp = 0;
-    if (!out.narrow && !flux_rows) {
+    if (lane_masks && !out.narrow && !flux_rows) {
         const int G = std::min(32, 4 * EPL);
         const int CPL = EPL * 8 / G;
         out.o_fixc = (int)blob.size();
