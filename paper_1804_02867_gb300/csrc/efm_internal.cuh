@@ -134,8 +134,8 @@ struct NetView {
 // rows 23, 40, 53 and 12; 100 of 20 to 60 on 100 rows 4.6, 11.7, 15.9 and 4.5 (at
 // 2^14, where a level has few children, 1.5, 3.7, 3.2 and 2.1).  On the core-shaped
 // network, whose columns are short, the code for them costs 14 % (spills: 467 and
-// 533 ms at 2^26).  A warp each is right for the rare ones of other networks: a
-// small level waits for one lane's chain (eight core targets at 2^17 7.8 -> 6.7 ms,
+// 533 ms at 2^26).  A warp each is right for the few of other networks (see
+// kWarpOpen): a small level waits for one lane's chain (eight core targets at 2^17 7.8 -> 6.7 ms,
 // subtractive 5.8 -> 4.6, a 400-row network 3.8 -> 3.4).
 constexpr int kNarrowCol = 8, kListCol = 32, kListMean = 8;
 

@@ -697,6 +697,66 @@ __device__ __forceinline__ void wide_narrow(const NetView &nv, const uint32_t *b
     }
 }
 
+// The same by one lane (see slow_child).
+__device__ __noinline__ void slow_narrow(const NetView &nv, const uint32_t *bl, const uint4 *pp, int32_t A, int32_t C,
+                                         int cb, int ce, int k, int32_t *dst, Child &r, NarrowMasks &z)
+{
+    const uint64_t zm = reinterpret_cast<const uint64_t *>(pp)[1];
+    const int32_t *vals = reinterpret_cast<const int32_t *>(pp + 3);
+    const uint2 *ent = reinterpret_cast<const uint2 *>(bl + nv.o_nent);
+    const uint64_t mask = blob_u64(bl, nv.o_colx + 10 * k + 4);
+    uint64_t g = 0, mx = 0;
+    r.n = 0;
+    r.key = kPadKey;
+    r.pv = 0;
+    r.om = 0;
+    r.rh = 0;
+    r.zflux = r.ovf = false;
+    z.zm = z.pm = z.nm = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        int q = cb;  // rows ascend in the column and in the state
+        for (uint64_t x = zm | mask; x; x &= x - 1) {
+            const int row = __ffsll((long long)x) - 1;
+            int64_t t = 0;
+            if ((zm >> row) & 1ull) t = (int64_t)A * vals[value_at(zm, row)];
+            while (q < ce && (int)(ent[q].x & 63u) < row) ++q;
+            if (q < ce && (int)(ent[q].x & 63u) == row) t += (int64_t)C * (int32_t)ent[q].y;
+            if (t == 0) continue;
+            if (pass == 0) {
+                const uint64_t at = abs64(t);
+                g = gcd_any(g, at);
+                mx = at > mx ? at : mx;
+                continue;
+            }
+            const int32_t v = div_any(t, g);
+            const uint32_t kk = bl[(v > 0 ? nv.o_keypos : nv.o_keyneg) + row];
+            const uint32_t rk = bl[nv.o_rank + row];
+            z.zm |= 1ull << row;
+            if (v > 0) z.pm |= 1ull << (rk & 0xFFu);
+            else z.nm |= 1ull << ((rk >> 8) & 0xFFu);
+            r.om |= mag(v);
+            r.rh += (uint64_t)(int64_t)v * row_hash(row);
+            if (kk < r.key) {
+                r.key = kk;
+                r.pv = v;
+            }
+            if (dst) dst[r.n] = v;
+            ++r.n;
+        }
+        if (pass == 0) {
+            if (g == 0) return;  // balanced (key stays kPadKey)
+            if (past_int32(mx, g)) {
+                r.ovf = true;
+                r.key = 0;
+                return;
+            }
+        }
+    }
+    r.g = 1;
+    if (dst)
+        for (int i = r.n; i & 3; ++i) dst[i] = 0;
+}
+
 // payload units of n entries (values on narrow networks)
 template <int F>
 __device__ __forceinline__ int entry_units(int n)
@@ -832,6 +892,91 @@ __device__ __forceinline__ void wide_child(const NetView &nv, const uint32_t *bl
     r.om = __reduce_or_sync(FULL, om);
     r.rh = warp_sum(rh);
     if (d2 && lane == 0 && (n & 1)) d2[n] = make_int2((int)kPadKey, 0);
+}
+
+// The same by one lane: where many such children come to a warp, 32 chains side
+// by side take less than 32 one after the other.
+template <bool SUB>
+__device__ __noinline__ void slow_child(const NetView &nv, const uint32_t *bl, const uint4 *pe, int np, int32_t A,
+                                        int32_t C, int cb, int ce, int k, uint4 *dst, Child &r)
+{
+    const int2 *p2 = reinterpret_cast<const int2 *>(pe);
+    int2 *d2 = reinterpret_cast<int2 *>(dst);
+    const int nq = ce - cb + (SUB ? 1 : 0);
+    uint32_t matched[(EFM_MAX_INTERNAL + 32) / 32];
+    for (int i = 0; 32 * i < nq; ++i) matched[i] = 0;
+    uint64_t g = 0, mx = 0;
+    r.n = 0;
+    r.key = kPadKey;
+    r.pv = 0;
+    r.om = 0;
+    r.rh = 0;
+    r.zflux = r.ovf = false;
+    int nbal = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        auto take = [&](int row, int64_t t) {
+            if (SUB && row == nv.M + k && t <= 0) r.zflux = true;
+            if (t == 0) return;
+            if (pass == 0) {
+                const uint64_t at = abs64(t);
+                g = gcd_any(g, at);
+                mx = at > mx ? at : mx;
+                if (!SUB || row < nv.M) ++nbal;
+                return;
+            }
+            const int32_t v = div_any(t, g);
+            const uint32_t kk = entry_key<SUB>(nv, bl, row, v > 0);
+            r.om |= mag(v);
+            r.rh += (uint64_t)(int64_t)v * row_hash(row);
+            if (kk < r.key) {
+                r.key = kk;
+                r.pv = v;
+            }
+            if (d2) d2[r.n] = make_int2((int)kk, v);
+            ++r.n;
+        };
+        for (int i = 0; i < np; ++i) {
+            const int2 e = p2[i];
+            const int row = e.x & 0xFFFF;
+            int64_t t = (int64_t)A * e.y;
+            int lo = 0, hi = nq;  // first column entry with a row >= row (they ascend)
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                int rq;
+                int32_t vq;
+                column_entry<SUB>(nv, bl, cb, ce, mid, k, rq, vq);
+                if (rq < row) lo = mid + 1;
+                else hi = mid;
+            }
+            if (lo < nq) {
+                int rq;
+                int32_t vq;
+                column_entry<SUB>(nv, bl, cb, ce, lo, k, rq, vq);
+                if (rq == row) {
+                    t += (int64_t)C * vq;
+                    matched[lo >> 5] |= 1u << (lo & 31);
+                }
+            }
+            take(row, t);
+        }
+        for (int q = 0; q < nq; ++q) {
+            if ((matched[q >> 5] >> (q & 31)) & 1u) continue;
+            int row;
+            int32_t cv;
+            column_entry<SUB>(nv, bl, cb, ce, q, k, row, cv);
+            take(row, (int64_t)C * cv);
+        }
+        if (pass == 0) {
+            if (nbal == 0) return;  // balanced (key stays kPadKey)
+            if (past_int32(mx, g)) {
+                r.ovf = true;
+                r.key = 0;
+                return;
+            }
+        }
+    }
+    r.g = 1;
+    if (d2 && (r.n & 1)) d2[r.n] = make_int2((int)kPadKey, 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -1418,10 +1563,11 @@ __device__ __forceinline__ uint4 child_header(const NetView &nv, uint32_t off, c
                       (uint32_t)m.n | ((uint32_t)max_bits(m.om) << 11), (uint32_t)m.pv);
 }
 
-// Any other open child, of reserved row i, by one warp: one whose update needs
-// 64 bits, a division or more entries than the generate pass takes.  Returns its fingerprint (kDeadFp: none) and its
+// Any other open child, of reserved row i, by one warp (WARP) or one lane: one
+// whose update needs 64 bits, a division or more entries than the generate pass
+// takes.  Returns its fingerprint (kDeadFp: none) and its
 // header; live rows without a payload count as unwritten.
-template <int F, bool SUB>
+template <int F, bool SUB, bool WARP>
 __device__ __noinline__ uint64_t finish_open(const NetView &nv, const LevelArgs &a, uint64_t f, uint64_t i, uint4 &h,
                                              int lane)
 {
@@ -1434,40 +1580,53 @@ __device__ __noinline__ uint64_t finish_open(const NetView &nv, const LevelArgs 
     h = make_uint4(0u, 0u, 0u, 0u);
     Child m;
     NarrowMasks z;
-    if (F == 2)
+    const bool one = !WARP || lane == 0;
+    if (!WARP && F == 2)
+        slow_narrow(nv, bl, o.pp, o.A, o.C, o.cb, o.ce, o.k, reinterpret_cast<int32_t *>(de), m, z);
+    else if (!WARP)
+        slow_child<SUB>(nv, bl, o.pp + support_units<F>(o.pc), o.np, o.A, o.C, o.cb, o.ce, o.k, de, m);
+    else if (F == 2)
         wide_narrow(nv, bl, o.pp, o.A, o.C, o.cb, o.k, reinterpret_cast<int32_t *>(de), m, z, lane);
     else
         wide_child<SUB>(nv, bl, o.pp + support_units<F>(o.pc), o.np, o.A, o.C, o.cb, o.ce, o.k, de, m, lane);
     if (SUB && m.zflux) {
-        if (lane == 0) atomicAdd(&a.ctr[C_ZERO], 1ull);
+        if (one) atomicAdd(&a.ctr[C_ZERO], 1ull);
         return kDeadFp;
     }
     if (m.key >= kFluxKey) {
-        if (lane == 0) finish_balanced<F>(nv, a, f);
+        if (one) finish_balanced<F>(nv, a, f);
         return kDeadFp;
     }
     if (m.ovf) {
-        if (lane == 0) atomicAdd(&a.ctr[C_OVF], 1ull);
+        if (one) atomicAdd(&a.ctr[C_OVF], 1ull);
         return kDeadFp;
     }
     if (f & (kOpenPruned | kOpenDead)) {
-        if (lane == 0 && (f & kOpenPruned)) atomicAdd(&a.ctr[C_PRUNED], 1ull);
+        if (one && (f & kOpenPruned)) atomicAdd(&a.ctr[C_PRUNED], 1ull);
         return kDeadFp;
     }
     const uint64_t uh = support_hash_of<F>(o.pp, k2);
     if (dst) {
         h = child_header<SUB>(nv, off, m, pc2);
-        if (lane == 0) {
+        if (one) {
             write_support<F>(dst, o.pp, o.pc, k2, m.rh, uh, z);
             a.child.hdr[i] = h;
         }
-    } else if (lane == 0) {
+    } else if (one) {
         atomicAdd(&a.ctr[C_UNWRITTEN], 1ull);
     }
     __threadfence();  // the row is complete before its slot is taken
-    __syncwarp();
+    if (WARP) __syncwarp();
     return state_fp(m.rh, uh);
 }
+
+// Open children that a warp takes one after the other; more go to a lane each.
+// With 0, 2, 4, 8, 16: the smallest query 0.684, 0.665, 0.663, 0.686, 0.731 ms,
+// subtractive 5.16, 4.57, 4.56, 4.55, 4.55, a 400-row network 3.51, 3.28, 3.28,
+// 3.28, 3.27, six targets of a 200-row network of even coefficients at 2^18 5.37,
+// 4.81, 4.59, 4.55, 4.91; with all of them by warps a batch of 64 networks of 12
+// rows took 3.5, by lanes 2.4.
+constexpr uint64_t kWarpOpen = 4;
 
 struct DedupSums {
     unsigned keep = 0, unv = 0;
@@ -1566,7 +1725,8 @@ __device__ __forceinline__ void dedup_range(const NetView &nv, const LevelArgs &
     end = end < (uint64_t)a.fp_cap ? end : (uint64_t)a.fp_cap;
     const uint64_t row_cap = (uint64_t)a.child.cap;
     // as many open children to a warp as there are for each, at most 32: the
-    // balanced ones a lane each, the others by the warp, one after the other
+    // balanced ones a lane each, the others by the warp, one after the other, or,
+    // if they are more than a few, a lane each as well
     const uint64_t warps = stride >> 5;
     const uint64_t per = min((uint64_t)32, max((uint64_t)1, (n_open + warps - 1) / warps));
     for (uint64_t q0 = (t_open >> 5) * per; q0 < n_open; q0 += warps * per) {
@@ -1579,14 +1739,19 @@ __device__ __forceinline__ void dedup_range(const NetView &nv, const LevelArgs &
                 finish_balanced<F>(nv, a, f);
                 f = kDeadFp;
                 if (i < row_cap) a.child.hdr[i] = h;
+            } else if (per > kWarpOpen) {
+                uint4 hc;
+                f = finish_open<F, SUB, false>(nv, a, f, i, hc, lane);
+                h = hc;
+                if (h.y == 0u && i < row_cap) a.child.hdr[i] = h;
             }
         }
         __syncwarp();
-        for (unsigned m = __ballot_sync(FULL, f != kDeadFp); m; m &= m - 1) {
+        for (unsigned m = per > kWarpOpen ? 0u : __ballot_sync(FULL, f != kDeadFp); m; m &= m - 1) {
             const int src = __ffs((int)m) - 1;
             const uint64_t row = __shfl_sync(FULL, i, src);
             uint4 hc;
-            const uint64_t fc = finish_open<F, SUB>(nv, a, __shfl_sync(FULL, f, src), row, hc, lane);
+            const uint64_t fc = finish_open<F, SUB, true>(nv, a, __shfl_sync(FULL, f, src), row, hc, lane);
             if (lane == src) {
                 f = fc;
                 h = hc;
