@@ -324,11 +324,6 @@ int efm_job_timing(const efm_job *job, int32_t job_target_idx, double *total_ms,
                    int64_t *expand_launches, double *expand_bytes, int64_t *kernel_launches);
 
 void efm_free_job(efm_job *job);
-
-/* Frees a network.  The device memory of a call's work area is kept for the
- * next call (unless efm_set_allocator replaced the allocator): at most an
- * eighth of the device's memory between calls, and a thirty-second
- * once the last network of a context is freed. */
 void efm_free_net(efm_net *net);
 
 /* Sort supports into the output order of efm_fetch_results (by |U|, then

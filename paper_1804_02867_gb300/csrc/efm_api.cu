@@ -59,28 +59,20 @@ struct PoolApi {
     Pool create()
     {
         int dev = 0;
-        size_t free_bytes = 0, total = 0;
         Pool pool = nullptr;
         cudaMemPoolProps props{};
-        if (cudaGetDevice(&dev) == cudaSuccess && cudaMemGetInfo(&free_bytes, &total) == cudaSuccess) {
+        if (cudaGetDevice(&dev) == cudaSuccess) {
             props.allocType = cudaMemAllocationTypePinned;
             props.location.type = cudaMemLocationTypeDevice;
             props.location.id = dev;
             if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
-                uint64_t keep = (uint64_t)total / 8;
+                uint64_t keep = ~0ull;
                 cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
                 return pool;
             }
         }
         cudaGetLastError();
         return nullptr;
-    }
-    void trim(Pool pool)
-    {
-        uint64_t keep = 0;  // (cudaMemGetInfo takes 25 us, a hundredth of a small query)
-        if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess ||
-            cudaMemPoolTrimTo(pool, (size_t)(keep / 4)) != cudaSuccess)
-            cudaGetLastError();
     }
 };
 
@@ -147,7 +139,6 @@ struct efm_net {
     DevBuf blob_sub;
     bool has_sub = false;
     int sm_count = 0;
-    uint64_t pool_ctx = 0;  // the context it keeps the work pool of
     DevBuf dep;             // DEPTHy tags (dep_out | dep_in) per internal metabolite, for the model's features
     bool dep_ready = false;
 };
@@ -321,7 +312,6 @@ extern "C" int efm_load_network(int32_t n_met, int32_t n_rxn, const int32_t *row
         vs.long_cols = has_long_columns(prep, kListCol - 1, kListMean);  // (a flux entry more)
         net->has_sub = true;
     }
-    net->pool_ctx = g_pools.retain();
     *out = net;
     return EFM_OK;
 }
@@ -355,7 +345,6 @@ extern "C" void efm_free_net(efm_net *net)
     dev_free(net->metent, s);
     dev_free(net->dep, s);
     cudaStreamSynchronize(s);
-    g_pools.release(net->pool_ctx);
     delete net;
 }
 

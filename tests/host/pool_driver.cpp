@@ -4,17 +4,13 @@
 //   ctx I       the current context (0: none)
 //   fail 0|1    whether making a pool fails
 //   get         -> pool P (0: the default pool)
-//   retain      -> id I
-//   release I   -> trims: the pools trimmed by it
 #include <cstdio>
 #include <cstring>
-#include <string>
 
 #include "efm_pool.h"
 
 static unsigned long long g_ctx = 0;
 static int g_fail = 0, g_made = 0;
-static std::string g_trims;
 
 struct FakeApi {
     using Pool = int *;
@@ -24,7 +20,6 @@ struct FakeApi {
         return g_ctx != 0;
     }
     Pool create() { return g_fail ? nullptr : new int(++g_made); }
-    void trim(Pool p) { g_trims += " " + std::to_string(*p); }
 };
 
 int main()
@@ -32,7 +27,6 @@ int main()
     static efm::WorkPools<FakeApi> pools;
     char cmd[16];
     while (std::scanf("%15s", cmd) == 1) {
-        unsigned long long x = 0;
         if (!std::strcmp(cmd, "ctx")) {
             if (std::scanf("%llu", &g_ctx) != 1) return 2;
             std::printf("ok\n");
@@ -42,13 +36,6 @@ int main()
         } else if (!std::strcmp(cmd, "get")) {
             int *p = pools.get();
             std::printf("pool %d\n", p ? *p : 0);
-        } else if (!std::strcmp(cmd, "retain")) {
-            std::printf("id %llu\n", (unsigned long long)pools.retain());
-        } else if (!std::strcmp(cmd, "release")) {
-            if (std::scanf("%llu", &x) != 1) return 2;
-            g_trims.clear();
-            pools.release(x);
-            std::printf("trims%s\n", g_trims.c_str());
         } else {
             return 2;
         }
