@@ -30,62 +30,19 @@ struct DevBuf {
     size_t bytes = 0;
 };
 
-// The calls' work areas come from a stream-ordered pool of their own, one per
-// device, which keeps what a call frees for the next.  In the default pool the
-// small buffers that outlive a call (networks, results) come to lie between
-// the large ones, and a call then has its arenas mapped anew: in a process with
-// a dozen networks four genome-shaped targets took 35.6 ms a call, and take 22.6
-// with this pool (alone in a process 22.7 either way).
-cudaMemPool_t work_pool()
-{
-    static std::mutex mu;
-    static std::map<int, cudaMemPool_t> pools;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = pools.find(dev);
-    if (it != pools.end()) return it->second;
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    cudaMemPool_t pool = nullptr;
-    uint64_t keep = ~0ull;
-    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
-        cudaGetLastError();
-        pool = nullptr;  // the default pool then
-    } else {
-        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    }
-    pools[dev] = pool;
-    return pool;
-}
-
-// work: part of a call's work area, freed before the call returns
-bool dev_alloc(DevBuf &b, size_t bytes, cudaStream_t s, bool work = false)
+bool dev_alloc(DevBuf &b, size_t bytes, cudaStream_t s)
 {
     b.bytes = bytes ? bytes : 16;
     if (g_alloc) {
         b.p = g_alloc(b.bytes, (uintptr_t)s, g_ctx);
         return b.p != nullptr;
     }
-    cudaMemPool_t pool = work ? work_pool() : nullptr;
-    if (pool && cudaMallocFromPoolAsync(&b.p, b.bytes, pool, s) == cudaSuccess) return true;
-    if (!pool && cudaMallocAsync(&b.p, b.bytes, s) == cudaSuccess) return true;
-    // once more without what the pools keep unused
-    cudaGetLastError();
-    cudaMemPool_t other = nullptr;
-    int dev = 0;
-    if (cudaStreamSynchronize(s) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetDefaultMemPool(&other, dev) == cudaSuccess) {
-        cudaMemPoolTrimTo(other, 0);
-        if (work_pool()) cudaMemPoolTrimTo(work_pool(), 0);
-        if ((pool ? cudaMallocFromPoolAsync(&b.p, b.bytes, pool, s) : cudaMallocAsync(&b.p, b.bytes, s)) == cudaSuccess)
-            return true;
+    if (cudaMallocAsync(&b.p, b.bytes, s) != cudaSuccess) {
+        cudaGetLastError();
+        b.p = nullptr;
+        return false;
     }
-    cudaGetLastError();
-    b.p = nullptr;
-    return false;
+    return true;
 }
 
 void dev_free(DevBuf &b, cudaStream_t s)
@@ -381,7 +338,7 @@ bool alloc_arena(Work &w, int i, int64_t rows, uint64_t units, cudaStream_t s)
     free_arena(w, i, s);
     const size_t F = (size_t)rows;
     units = std::min<uint64_t>(units, 0xFFFFFFFFull);  // a header's offset has 32 bits
-    if (!dev_alloc(w.hdr[i], F * 16, s, true) || !dev_alloc(w.pay[i], units * 16, s, true)) return false;
+    if (!dev_alloc(w.hdr[i], F * 16, s) || !dev_alloc(w.pay[i], units * 16, s)) return false;
     w.rows[i] = rows;
     w.pay_cap[i] = units;
     return true;
@@ -394,13 +351,13 @@ bool ensure_level_tables(Work &w, uint64_t reserved, cudaStream_t s)
         dev_free(w.fp, s);
         const int64_t cap = std::max<int64_t>((int64_t)reserved, w.fp_cap + w.fp_cap / 2);
         dev_free(w.open, s);
-        if (!dev_alloc(w.fp, (size_t)cap * 8, s, true) || !dev_alloc(w.open, (size_t)cap * 4, s, true)) return false;
+        if (!dev_alloc(w.fp, (size_t)cap * 8, s) || !dev_alloc(w.open, (size_t)cap * 4, s)) return false;
         w.fp_cap = cap;
     }
     const uint64_t need = next_pow2(2 * reserved + 64);
     if (need > w.slot_cap) {
         dev_free(w.slots, s);
-        if (!dev_alloc(w.slots, need * 8, s, true)) return false;
+        if (!dev_alloc(w.slots, need * 8, s)) return false;
         w.slot_cap = need;
     }
     return true;
@@ -441,14 +398,14 @@ int alloc_work(Work &w, const efm_net *net, const efm_limits &lim, cudaStream_t 
     bool ok = alloc_arena(w, 0, rows, units, s) && alloc_arena(w, 1, rows, units, s);
     // (a start: a level that needs more makes them grow)
     ok = ok && ensure_level_tables(w, std::min<uint64_t>(2 * (uint64_t)rows, 1u << 19), s);
-    ok = ok && dev_alloc(w.cslots, w.cslot_cap * 8, s, true);
-    ok = ok && dev_alloc(w.cand, (size_t)w.cand_cap * W * 8, s, true);
-    ok = ok && dev_alloc(w.res, (size_t)w.res_cap * W * 8, s, true);
-    ok = ok && dev_alloc(w.bcnt, (size_t)nv.N * 4, s, true);
-    ok = ok && dev_alloc(w.ctr, (C_COUNT + S_COUNT) * 8, s, true);
-    if (nv.W > 2) ok = ok && dev_alloc(w.rcols, (size_t)w.res_cap * kRcolStride * 2, s, true);
-    ok = ok && dev_alloc(w.ksig, (size_t)nv.N * 16, s, true) && dev_alloc(w.csingle, (size_t)nv.N * 4, s, true);
-    if (lim.first_k > 0) ok = ok && dev_alloc(w.fkb, W * 8, s, true);
+    ok = ok && dev_alloc(w.cslots, w.cslot_cap * 8, s);
+    ok = ok && dev_alloc(w.cand, (size_t)w.cand_cap * W * 8, s);
+    ok = ok && dev_alloc(w.res, (size_t)w.res_cap * W * 8, s);
+    ok = ok && dev_alloc(w.bcnt, (size_t)nv.N * 4, s);
+    ok = ok && dev_alloc(w.ctr, (C_COUNT + S_COUNT) * 8, s);
+    if (nv.W > 2) ok = ok && dev_alloc(w.rcols, (size_t)w.res_cap * kRcolStride * 2, s);
+    ok = ok && dev_alloc(w.ksig, (size_t)nv.N * 16, s) && dev_alloc(w.csingle, (size_t)nv.N * 4, s);
+    if (lim.first_k > 0) ok = ok && dev_alloc(w.fkb, W * 8, s);
     for (auto &e : w.ev) ok = ok && cudaEventCreate(&e) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -613,8 +570,8 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             dev_free(w.cent, s);
             dev_free(w.cells, s);
             w.cent_cap = 0;
-            if (!dev_alloc(w.cent, (size_t)need * (nv.W <= 2 ? 32 : 16), s, true) ||
-                !dev_alloc(w.cells, cell_table_bytes(nv, (uint64_t)need), s, true))
+            if (!dev_alloc(w.cent, (size_t)need * (nv.W <= 2 ? 32 : 16), s) ||
+                !dev_alloc(w.cells, cell_table_bytes(nv, (uint64_t)need), s))
                 return EFM_ENOMEM;
             w.cent_cap = need;
         }
@@ -849,7 +806,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
             if (n_rows > w.live_cap) {
                 dev_free(w.live, s);
                 const int64_t cap = std::max<int64_t>(n_rows, 2 * w.live_cap);
-                if (!dev_alloc(w.live, (size_t)cap * 4, s, true)) return EFM_ENOMEM;
+                if (!dev_alloc(w.live, (size_t)cap * 4, s)) return EFM_ENOMEM;
                 w.live_cap = cap;
             }
             CK(launch_live_list((const uint4 *)w.hdr[cur].p, n_rows, (uint32_t *)w.live.p, ctr + C_LIVE, net->sm_count, s));
@@ -885,18 +842,18 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
                     dev_free(w.lx, s);
                     dev_free(w.lscore, s);
                     const int64_t cap = std::max<int64_t>(rows, 2 * w.lx_rows);
-                    if (!dev_alloc(w.lx, (size_t)cap * kMlpFeatures * 2, s, true) || !dev_alloc(w.lscore, (size_t)cap * 4, s, true))
+                    if (!dev_alloc(w.lx, (size_t)cap * kMlpFeatures * 2, s) || !dev_alloc(w.lscore, (size_t)cap * 4, s))
                         return EFM_ENOMEM;
                     w.lx_rows = cap;
                 }
                 if (n_rows > w.perm_cap) {
                     dev_free(w.perm, s);
                     const int64_t cap = std::max<int64_t>(n_rows, 2 * w.perm_cap);
-                    if (!dev_alloc(w.perm, (size_t)cap * 4, s, true)) return EFM_ENOMEM;
+                    if (!dev_alloc(w.perm, (size_t)cap * 4, s)) return EFM_ENOMEM;
                     w.perm_cap = cap;
                 }
                 if (!w.lhist.p) {
-                    if (!dev_alloc(w.lhist, 4096 * 4, s, true) || !dev_alloc(w.lerr, 4, s, true)) return EFM_ENOMEM;
+                    if (!dev_alloc(w.lhist, 4096 * 4, s) || !dev_alloc(w.lerr, 4, s)) return EFM_ENOMEM;
                     CK(cudaMemsetAsync(w.lerr.p, 0, 4, s));
                 }
                 if ((rc = ensure_dep_tags(net))) return rc;
@@ -1048,7 +1005,7 @@ int run_target(efm_net *net, Work &w, const efm_limits &lim, int target, TargetO
         const uint64_t n2 = next_pow2((uint64_t)std::max<int64_t>(res_n, 1));
         if (n2 > w.sort_cap) {
             dev_free(w.sortidx, s);
-            if (!dev_alloc(w.sortidx, sort_scratch_bytes((int64_t)n2), s, true)) return EFM_ENOMEM;
+            if (!dev_alloc(w.sortidx, sort_scratch_bytes((int64_t)n2), s)) return EFM_ENOMEM;
             w.sort_cap = n2;
         }
         if (!dev_alloc(out.sup, (size_t)std::max<int64_t>(n_keep, 1) * nv.W * 8, s)) return EFM_ENOMEM;
@@ -1390,7 +1347,7 @@ extern "C" int efm_sample_pathways(efm_net *net, int32_t target, const efm_limit
     if ((int64_t)h[C_RES_N] > w.res_cap) return fail(EFM_ECAPACITY);
     const int64_t res_n = (int64_t)h[C_RES_N];
     const uint64_t n2 = next_pow2((uint64_t)std::max<int64_t>(res_n, 1));
-    if (!dev_alloc(w.sortidx, sort_scratch_bytes((int64_t)n2), s, true) || !dev_alloc(o.sup, (size_t)std::max<int64_t>(res_n, 1) * nv.W * 8, s))
+    if (!dev_alloc(w.sortidx, sort_scratch_bytes((int64_t)n2), s) || !dev_alloc(o.sup, (size_t)std::max<int64_t>(res_n, 1) * nv.W * 8, s))
         return fail(EFM_ENOMEM);
     if (launch_sort_results((const uint64_t *)w.res.p, res_n, nv.W, w.sortidx.p, (int64_t)n2,
                             (uint64_t *)o.sup.p, res_n, s) != cudaSuccess ||
@@ -1541,11 +1498,11 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
     std::vector<int> alone;  // jobs whose levels did not fit a slice
     std::vector<int64_t> offs((size_t)n_jobs + 1, 0);  // output words of the jobs before each
 
-    if (!dev_alloc(pool, (size_t)slices * L.slice_bytes, s, true) ||
-        !dev_alloc(djobs, sizeof(BatchJob) * (size_t)n_jobs, s, true) || !dev_alloc(dorder, 4 * (size_t)n_jobs, s, true) ||
-        !dev_alloc(dctr, 8 * (size_t)C_COUNT * n_jobs, s, true) || !dev_alloc(dqueue, 16, s, true) ||
-        !dev_alloc(dout, out_rows * Wmax * 8 * (size_t)n_jobs, s, true) ||
-        !dev_alloc(doff, 8 * ((size_t)n_jobs + 1), s, true)) {
+    if (!dev_alloc(pool, (size_t)slices * L.slice_bytes, s) ||
+        !dev_alloc(djobs, sizeof(BatchJob) * (size_t)n_jobs, s) || !dev_alloc(dorder, 4 * (size_t)n_jobs, s) ||
+        !dev_alloc(dctr, 8 * (size_t)C_COUNT * n_jobs, s) || !dev_alloc(dqueue, 16, s) ||
+        !dev_alloc(dout, out_rows * Wmax * 8 * (size_t)n_jobs, s) ||
+        !dev_alloc(doff, 8 * ((size_t)n_jobs + 1), s)) {
         rc = EFM_ENOMEM;
         goto done;
     }
@@ -1734,7 +1691,7 @@ extern "C" int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targ
         } catch (const std::bad_alloc &) {
             room = false;
         }
-        if (!room || !dev_alloc(dpack, (size_t)offs[n_jobs] * 8, s, true)) {
+        if (!room || !dev_alloc(dpack, (size_t)offs[n_jobs] * 8, s)) {
             rc = EFM_ENOMEM;
             goto done;
         }
