@@ -21,6 +21,7 @@ from __future__ import annotations
 
 import argparse
 import concurrent.futures as cf
+import gc
 import hashlib
 import json
 import os
@@ -99,30 +100,45 @@ def measured_peaks():
         return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0}, "fallback"
 
 
-def profile_figure(name, key):
+LEVEL_SOURCES = ("efm_level.cuh", "efm_sparse.cu")  # the generate and dedup kernels
+
+
+def source_hash(sources):
+    h = hashlib.sha256()
+    for f in sources:
+        h.update(open(os.path.join(ROOT, "paper_1804_02867_gb300", "csrc", f), "rb").read())
+    return h.hexdigest()[:16]
+
+
+def profile_figure(name, key, sources=("efm_kernels.cu",), tag="kernel_source_sha256_16"):
     """A figure from a committed ncu summary under profiles/, if that summary
-    was taken on the current kernel source (else None)."""
+    was taken on the current kernel source (else None): its line `tag` has to
+    name the hash of `sources`."""
     path = os.path.join(ROOT, "profiles", name)
-    src = os.path.join(ROOT, "paper_1804_02867_gb300", "csrc", "efm_kernels.cu")
     try:
         text = open(path).read()
-        sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
+        sha = source_hash(sources)
     except OSError:
         return None
-    m_sha = re.search(r"kernel_source_sha256_16:\s*([0-9a-f]+)", text)
+    m_sha = re.search(re.escape(tag) + r":\s*([0-9a-f]+)", text)
     m_val = re.search(re.escape(key) + r":\s*([0-9.eE+]+)", text)
     if not m_sha or not m_val or m_sha.group(1) != sha:
         return None
     return float(m_val.group(1))
 
 
+def traffic_ratio(name):
+    """DRAM bytes per algorithmic byte of the level pass, from its summary."""
+    return profile_figure(name, "dram_to_algorithmic_ratio", LEVEL_SOURCES, "level_source_sha256_16")
+
+
 def profile_traffic(alg_bytes_per_launch):
-    """Per-launch DRAM traffic of the core network's level pass (generate
-    and dedup kernels of one expansion launch): the DRAM-to-algorithmic
-    ratio ncu measured on a smaller case of the same kernels (traffic grows
-    with the states read and written), applied to this run's algorithmic
-    bytes per launch; None without a summary for the current source."""
-    ratio = profile_figure("level_pass_core.md", "dram_to_algorithmic_ratio")
+    """Per-launch DRAM traffic of the core network's level pass: the
+    DRAM-to-algorithmic ratio ncu measured over a smaller search's launches
+    (traffic grows with the states read and written), applied to this run's
+    algorithmic bytes per launch; None without a summary for the current
+    source."""
+    ratio = traffic_ratio("level_pass_core.md")
     return ratio * alg_bytes_per_launch if ratio else None
 
 
@@ -378,7 +394,7 @@ def run_ours(args):
         "expansions_per_step": tot_exp / args.steps / max(ws, 1),
         "results_per_step": tot_res / args.steps / max(ws, 1),
         "roofline": {
-            "kernel": "level pass: generate_kernel<2,0,0> + dedup_kernel<2,0> + accept_kernel",
+            "kernel": "level pass: generate_kernel<2,0,0,0> + dedup_kernel<2,0> + accept_kernel",
             "bound": "hbm",
             "achieved": achieved,
             "peak": float(peaks["hbm_gbs"]),
@@ -488,9 +504,9 @@ def run_genome(args):
     nw.close()
     peaks, kind = measured_peaks()
     achieved = eb / (ems * 1e-3) / 1e9 if ems else 0.0
-    # DRAM traffic: the ratio ncu measured on one launch of this kernel,
+    # DRAM traffic: the ratio ncu measured on a smaller search's launches,
     # applied to this run's algorithmic bytes per launch
-    ratio = profile_figure("level_pass_genome.md", "dram_to_algorithmic_ratio")
+    ratio = traffic_ratio("level_pass_genome.md")
     traffic = ratio * eb / el if ratio and el else None
     line = {
         "metric": METRIC, "value": exp / (tot_ms * 1e-3), "unit": UNIT, "n_gpus": 1, "steps": args.steps,
@@ -499,7 +515,7 @@ def run_genome(args):
         "config": {"workload": f"genome-1000x2500 (850 internal, 3125 split columns), {n_t} targets",
                    "max_len": 40, "max_secondary": MAX_SEC, "max_frontier": budget, "support_bits": 3136},
         "balanced_pathways_per_s": res / (tot_ms * 1e-3),
-        "roofline": {"kernel": "level pass: generate_kernel<0,0,0> + dedup_kernel<0,0> + accept_kernel", "bound": "hbm", "achieved": achieved,
+        "roofline": {"kernel": "level pass: generate_kernel<0,0,0,0> + dedup_kernel<0,0> + accept_kernel", "bound": "hbm", "achieved": achieved,
                      "peak": float(peaks["hbm_gbs"]), "unit": "GB/s", "frac": achieved / float(peaks["hbm_gbs"]),
                      "traffic": traffic, "peak_kind": f"{kind} HBM copy bandwidth", "launches": el,
                      "avg_launch_ms": ems / max(el, 1), "alg_bytes_per_launch": eb / max(el, 1)},
@@ -540,34 +556,35 @@ def run_batched(args):
 
     for _ in range(max(1, args.warmup)):
         batch_once()  # includes the autotuner's sample runs the first time
-    torch.cuda.synchronize()
-    tot_ms = 0.0
-    exp = res = 0
-    for _ in range(args.steps):
+    tune = efmgraph.efm_batch_tuning()
+
+    def timed():
+        torch.cuda.synchronize()
         ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         ev0.record(stream)
         e, r = batch_once()
         ev1.record(stream)
         ev1.synchronize()
-        tot_ms += ev0.elapsed_time(ev1)
+        return ev0.elapsed_time(ev1), e, r
+
+    # the tuned batch and the untuned launch configuration (8 warps per job,
+    # every CTA an SM holds, input order, tile 32, queue chunk 1) in turn.  4096
+    # fetches make some 30 000 Python objects: the collector would stop every
+    # other step for 30 ms, in one arm or the other
+    gc.collect()
+    gc.disable()
+    tot_ms = default_ms = 0.0
+    exp = res = 0
+    for _ in range(args.steps):
+        t, e, r = timed()
+        tot_ms += t
         exp += e
         res += r
-    tune = efmgraph.efm_batch_tuning()
-    # the same batch in the untuned launch configuration (8 warps per job,
-    # every CTA an SM holds, input order, tile 32, queue chunk 1)
-    efmgraph.efm_batch_set_tuning(ctas_per_sm=0, largest_first=0, warps_per_job=8, tile=32, queue_chunk=1)
-    try:
-        batch_once()
-        torch.cuda.synchronize()
-        ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        ev0.record(stream)
-        for _ in range(args.steps):
-            batch_once()
-        ev1.record(stream)
-        ev1.synchronize()
-        default_ms = ev0.elapsed_time(ev1) / args.steps
-    finally:
-        efmgraph.efm_batch_set_tuning(None)
+        efmgraph.efm_batch_set_tuning(ctas_per_sm=0, largest_first=0, warps_per_job=8, tile=32, queue_chunk=1)
+        try:
+            default_ms += timed()[0] / args.steps
+        finally:
+            efmgraph.efm_batch_set_tuning(None)
     # the same jobs as sequential single-job calls (one pass)
     torch.cuda.synchronize()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -581,6 +598,7 @@ def run_batched(args):
     ev1.record(stream)
     ev1.synchronize()
     seq_ms = ev0.elapsed_time(ev1)
+    gc.enable()
     for h in loaded:
         h.close()
     value = exp / (tot_ms * 1e-3)

@@ -261,7 +261,12 @@ int efm_sample_pathways(efm_net *net, int32_t target, const efm_limits *limits, 
  *  out              one job handle with n_jobs entries for efm_fetch_results
  * Per-job device errors (capacity, bounded waits) are reported by
  * efm_fetch_results for that entry.  Per job at most 2^15 distinct balanced
- * supports and 2^13 results. */
+ * supports and 2^13 results.  A slice holds 1.5 max_frontier rows before
+ * deduplication (8 max_frontier up to a budget of 2^12) and 2048 results in its
+ * superset index: a job that outgrows it is left by the launch and runs by
+ * itself after it, on the same stream, with the same answer.  At budgets of
+ * 2^12 that is a job in some hundreds, at 2^14 one in 16, from 2^15 on one in
+ * five; such batches gain less. */
 int efm_find_pathways_batch(efm_net *const *nets, const int32_t *targets, int32_t n_jobs, const efm_limits *limits,
                             const efm_model *model, efm_job **out);
 
